@@ -7,61 +7,105 @@
 
 namespace moehub {
 
-// One warp per token: the token's logits sit in registers (EP/32 per lane); K rounds of a shuffle
-// arg-max on (value, lowest index); then the softmax weights of the picks.  ls: [tokens][EP] logits
-// in shared memory.
+// The fp32 chain on bf16 data: acc + x * w with the exact product and one rounding - the same bits as widening both
+// operands to fp32 and one fused multiply-add, without the widening instructions.  lo / hi: the half of a 32-bit word.
+__device__ __forceinline__ float fma_bf16_lo(uint32_t x, uint32_t w, float acc) {
+  float d;
+  asm("{\n\t.reg .b16 xl, xh, wl, wh;\n\t"
+      "mov.b32 {xl, xh}, %1;\n\tmov.b32 {wl, wh}, %2;\n\t"
+      "fma.rn.f32.bf16 %0, xl, wl, %3;\n\t}"
+      : "=f"(d) : "r"(x), "r"(w), "f"(acc));
+  return d;
+}
+__device__ __forceinline__ float fma_bf16_hi(uint32_t x, uint32_t w, float acc) {
+  float d;
+  asm("{\n\t.reg .b16 xl, xh, wl, wh;\n\t"
+      "mov.b32 {xl, xh}, %1;\n\tmov.b32 {wl, wh}, %2;\n\t"
+      "fma.rn.f32.bf16 %0, xh, wh, %3;\n\t}"
+      : "=f"(d) : "r"(x), "r"(w), "f"(acc));
+  return d;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {  // a shared-memory load by its 32-bit shared address
+  uint4 r;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr));
+  return r;
+}
+
+// A float as an unsigned number of the same order (-0 and +0 equal), so that an integer reduction finds the maximum.
+__device__ __forceinline__ unsigned order_key(float v) {
+  const unsigned u = __float_as_uint(v + 0.0f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+// Maximum / minimum / sum over the G neighbouring lanes of a token (a whole warp: one instruction for the integers).
+template <int G> __device__ __forceinline__ unsigned group_max(unsigned v) {
+  if (G == 32) return __reduce_max_sync(0xffffffffu, v);
+#pragma unroll
+  for (int off = G / 2; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, off));
+  return v;
+}
+template <int G> __device__ __forceinline__ unsigned group_min(unsigned v) {
+  if (G == 32) return __reduce_min_sync(0xffffffffu, v);
+#pragma unroll
+  for (int off = G / 2; off > 0; off >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, off));
+  return v;
+}
+template <int G> __device__ __forceinline__ float group_sum(float v) {
+#pragma unroll
+  for (int off = G / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// G lanes per token (8, 16 or a whole warp): the token's logits sit in registers (NJ per lane, experts lane + G j);
+// K rounds of an arg-max (largest value, then lowest index), then the softmax weights of the picks.  ls: rows of
+// `pitch` logits (shared or global memory); row tl is token t0 + tl.
 // s_hist (shared memory, [E], or nullptr): every pick is also counted per expert.
-template <int EP>
 // tp > 1 (expert + tensor parallelism, paper Section VII): every pick is listed once per TP shard, as the
 // virtual expert e*tp + s with the pick's weight, so that the dispatch stores the row into every shard's region.
-__device__ __forceinline__ void select_topk(const float* ls, int tvalid, int t0, int E, int K, int renorm,
+template <int G, int NJ>
+__device__ __forceinline__ void select_topk(const float* ls, int pitch, int tvalid, int t0, int E, int K, int renorm,
                                             int* __restrict__ topk_idx, float* __restrict__ topk_w, int* s_hist, int tp) {
-  constexpr int NJ = (EP + 31) / 32;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  for (int tl = warp; tl < tvalid; tl += blockDim.x / 32) {
+  constexpr int PER_WARP = 32 / G;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % G, sub = threadIdx.x % 32 / G;
+  for (int base = warp * PER_WARP; base < tvalid; base += blockDim.x / 32 * PER_WARP) {
+    const int tl = base + sub;
+    const bool live = tl < tvalid;  // (the other tokens of the warp keep it in the shuffles)
+    const float* row = ls + (live ? tl : base) * pitch;
     float v[NJ];
+    unsigned key[NJ];  // 0: no expert, or picked already
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-      const int e = lane + 32 * j;
-      v[j] = (e < E) ? ls[tl * EP + e] : -FLT_MAX;
+      const int e = lane + G * j;
+      v[j] = (e < E) ? row[e] : -FLT_MAX;
+      key[j] = (e < E) ? max(order_key(v[j]), 1u) : 0u;
     }
-    unsigned taken = 0;
-    float my_v = 0.0f;
+    float my_v = 0.0f, m = 0.0f;
     int my_e = 0;
     for (int k = 0; k < K; ++k) {
-      float bv = -FLT_MAX;
-      int be = 0x7fffffff;
+      unsigned bk = key[0];
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        const int e = lane + 32 * j;
-        const bool ok = (e < E) && !((taken >> j) & 1u);
-        if (ok && (be == 0x7fffffff || v[j] > bv)) { bv = v[j]; be = e; }
-      }
+      for (int j = 1; j < NJ; ++j) bk = max(bk, key[j]);
+      bk = group_max<G>(bk);
+      unsigned be = 0xffffffffu;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-        const int oe = __shfl_xor_sync(0xffffffffu, be, off);
-        const bool other = (oe != 0x7fffffff) && (be == 0x7fffffff || ov > bv || (ov == bv && oe < be));
-        if (other) { bv = ov; be = oe; }
-      }
-      if ((be & 31) == lane) taken |= 1u << (be >> 5);
-      if (lane == k) { my_v = bv; my_e = be; }
+      for (int j = NJ - 1; j >= 0; --j)
+        if (key[j] == bk) be = (unsigned)(lane + G * j);
+      be = group_min<G>(be);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j)
+        if (be == (unsigned)(lane + G * j)) key[j] = 0u;
+      const float bv = row[be];
+      if (k == 0) m = bv;
+      if (lane == k) { my_e = (int)be; my_v = bv; }
     }
-    const float m = __shfl_sync(0xffffffffu, my_v, 0);
     float z = 0.0f;
 #pragma unroll
     for (int j = 0; j < NJ; ++j)
-      if (lane + 32 * j < E) z += expf(v[j] - m);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) z += __shfl_xor_sync(0xffffffffu, z, off);
+      if (lane + G * j < E) z += expf(v[j] - m);
+    z = group_sum<G>(z);
     float p = (lane < K) ? expf(my_v - m) / z : 0.0f;
-    if (renorm) {
-      float s = p;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      p = p / s;
-    }
-    if (lane < K) {
+    if (renorm) p = p / group_sum<G>(p);
+    if (lane < K && live) {
       for (int sh = 0; sh < tp; ++sh) {
         const size_t o = ((size_t)(t0 + tl) * K + lane) * tp + sh;
         topk_idx[o] = my_e * tp + sh;

@@ -207,14 +207,6 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 // token's row of x per step with two TMA copies, kRfBufs - 1 chunks ahead, and each chain reads its rows from
 // shared memory (128-byte swizzle: 16-byte unit u of row r sits at u ^ (r % 8)).  Exact values go back into
 // the logit rows; then the common selection.
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {  // a shared-memory load by its 32-bit shared address
-  uint4 r;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr));
-  return r;
-}
-__device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
-
 template <int TPC>
 __global__ void __launch_bounds__(TPC * 16, 1)
 route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
@@ -241,7 +233,6 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   const int lane = threadIdx.x % 32, l16 = threadIdx.x % 16, half = lane / 16;
   const int tl = threadIdx.x / 16;  // this half-warp's token inside the block
   const bool live = tl < tvalid;
-  const unsigned hmask = 0xffffu << (16 * half);
   if (threadIdx.x == 0) {
     for (int b = 0; b < kRfBufs; ++b) {
       mbar_init(smem_u32(&s_full[b]), 1);
@@ -420,14 +411,14 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
           for (int q = 0; q < 8; ++q) {
             const uint4 xa = lds128(xb + xo[q]);
             const uint4 wa = lds128(wb + wo[q]);
-            acc = __fmaf_rn(bf16_lo(xa.x), bf16_lo(wa.x), acc);
-            acc = __fmaf_rn(bf16_hi(xa.x), bf16_hi(wa.x), acc);
-            acc = __fmaf_rn(bf16_lo(xa.y), bf16_lo(wa.y), acc);
-            acc = __fmaf_rn(bf16_hi(xa.y), bf16_hi(wa.y), acc);
-            acc = __fmaf_rn(bf16_lo(xa.z), bf16_lo(wa.z), acc);
-            acc = __fmaf_rn(bf16_hi(xa.z), bf16_hi(wa.z), acc);
-            acc = __fmaf_rn(bf16_lo(xa.w), bf16_lo(wa.w), acc);
-            acc = __fmaf_rn(bf16_hi(xa.w), bf16_hi(wa.w), acc);
+            acc = fma_bf16_lo(xa.x, wa.x, acc);
+            acc = fma_bf16_hi(xa.x, wa.x, acc);
+            acc = fma_bf16_lo(xa.y, wa.y, acc);
+            acc = fma_bf16_hi(xa.y, wa.y, acc);
+            acc = fma_bf16_lo(xa.z, wa.z, acc);
+            acc = fma_bf16_hi(xa.z, wa.z, acc);
+            acc = fma_bf16_lo(xa.w, wa.w, acc);
+            acc = fma_bf16_hi(xa.w, wa.w, acc);
           }
         }
         __syncwarp();
@@ -486,7 +477,7 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
     __syncthreads();
     return;
   }
-  select_topk<kRfEP>(ls, tvalid, t0, E, K, renorm, topk_idx, topk_w, prep.hist ? s_hist : nullptr, tp);
+  select_topk<32, kRfEP / 32>(ls, kRfEP, tvalid, t0, E, K, renorm, topk_idx, topk_w, prep.hist ? s_hist : nullptr, tp);
   route_prep_end(prep, s_hist);
 }
 

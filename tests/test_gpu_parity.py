@@ -212,6 +212,33 @@ def test_router_every_kernel_shape(shape):
         Hh.check_route(idx, tw, ridx, rw)
 
 
+# The chain kernel where its shapes end: expert counts at the edges of its lane grids and clusters (8 / 16 / 32 / 64 /
+# 128 / 192 / 256), one token, token counts around its blocks, one, two and eight chains per thread, an h range shorter
+# than a box and one that ends inside a box and inside a stage; and the filter just past its first batch size.
+CHAIN_SHAPES = [
+    # (T, H, E, K, dtype)
+    (1, 8, 8, 8, BF16), (1, 4, 1, 1, FP32), (17, 72, 9, 2, BF16), (5000, 72, 8, 2, BF16), (5000, 36, 16, 3, FP32),
+    (3, 584, 33, 4, BF16), (1, 2056, 64, 8, BF16), (601, 584, 31, 5, BF16), (4700, 72, 61, 4, BF16), (4700, 36, 64, 4, FP32),
+    (1, 584, 256, 8, BF16), (9, 292, 193, 32, FP32), (129, 136, 128, 6, BF16), (768, 136, 192, 8, BF16),
+    (769, 136, 192, 8, BF16), (768, 68, 256, 8, FP32), (769, 68, 256, 8, FP32),
+]
+
+
+@pytest.mark.parametrize("shape", CHAIN_SHAPES, ids=lambda s: f"T{s[0]}_H{s[1]}_E{s[2]}_K{s[3]}_d{s[4]}")
+def test_router_chain_kernel_edges(shape):
+    T, H, E, K, dtype = shape
+    w = inputs.Workload("router_edges", T=T, H=H, E=E, R=1, K=K, F=8, dtype=dtype, zipf_s=1.0, seed=13, identity_experts=True)
+    x, wr, bias, *_ = Hh.oracle_inputs(w, with_experts=False)
+    ridx, rw, _ = oracle.route(x, wr, bias, K, dtype)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    idx = torch.empty((T, K), dtype=torch.int32, device="cuda")
+    tw = torch.empty((T, K), dtype=torch.float32, device="cuda")
+    plan.moe_route(Hh.to_dev(x), Hh.to_dev(wr), Hh.to_dev(bias), idx, tw)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    Hh.check_route(idx, tw, ridx, rw)
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

@@ -257,7 +257,7 @@ static int ffn_dispatch(moe_plan* p, const void* recv, const int* tile_expert, c
                         cudaStream_t st) {
   if (p->cfg.dtype == MOE_DTYPE_BF16 && p->cfg.ffn_kernel != 1)
     return launch_ffn_tc(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
-  return launch_ffn_simt(p, recv, tile_expert, wg, wu, wd, out_rows, st);
+  return launch_ffn_simt(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
 }
 
 int moe_expert_ffn(moe_plan_t* p, const void* d_recv, const int32_t* d_tile_expert, const void* d_wg,

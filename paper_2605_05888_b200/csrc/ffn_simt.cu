@@ -1,11 +1,11 @@
-// Step 3 of the MoE layer (paper Section II-A, expert computation) on plain fp32 FMA units.
+// Step 3 of the MoE layer (paper Section II-A, expert computation) on plain fp32 FMA units: S = silu(A*Wg^T) .* (A*Wu^T)
+// into the intermediate buffer, then O = S*Wd^T, two launches.  Tiles without an owner exit at once, so the weights of
+// experts that received no rows are never read.
 //
-// Used for dtype fp32 (a tensor-core tf32 product cannot meet the 1e-4 error bound) and as a
-// second, independent device implementation to check the tcgen05 kernel against.  Two launches:
-// S = silu(A*Wg^T) .* (A*Wu^T) into the intermediate buffer, then O = S*Wd^T.  A CTA owns one
-// 128-row tile of one expert and 64 output columns; tiles without an owner exit at once, so the
-// weights of experts that received no rows are never read.
-#include "common.cuh"
+// Two kernels.  ffn_fp32_kernel is the path of dtype fp32 (a tensor-core tf32 product cannot meet the 1e-4 error
+// bound).  ffn_simt_kernel, slow and simple, is a second, independent device implementation to check the tcgen05
+// kernel against on bf16 data (ffn_kernel = 1).
+#include "tc_common.cuh"
 
 namespace moehub {
 
@@ -89,6 +89,246 @@ ffn_simt_kernel(const XT* __restrict__ A, int lda, const int* __restrict__ tile_
     }
 }
 
+// ---- dtype fp32 ----------------------------------------------------------------------------------------
+// Bound by fp32 FMA issue (128 per clock and SM).  A CTA computes 8 TM rows of a tile x 16 TN columns (GEMM1: half of
+// them gate, half up columns of the same f); a warp has 2 TM rows, a lane TM x TN results.  Operands stay in their
+// natural K-major rows: TMA brings 128 bytes (32 k) of every row per stage (128-byte swizzle), a lane reads 16 bytes
+// (4 k) of its TM rows and TN columns - two pipe cycles each, lanes of a warp being 2 row groups x 16 column groups -
+// for TM x TN x 4 FMAs, k ascending.  (Packed FMAs, fma.rn.f32x2 on pairs of k, halve the instructions but ran at 66
+// FMAs per clock and SM where scalar ones reach 85 in the same register-only loop.)  A lane of the first warp issues
+// the copies on the side (a warp of its own would cost the others a third of their registers); the warps wait per
+// stage on its mbarrier.  A warp whose rows a partly filled tile does not have leaves at once.
+// Measured against the plain 128 x 64 kernel above on fp32 data (both GEMMs): T 1000, H 1024, 16 experts, top-2,
+// F 2048: 1295 -> 793 us; T 256, H 128, 8 experts, top-2, F 256: 77 -> 28 us.
+constexpr int kF32Warps = 4;
+constexpr int kF32Threads = 32 * kF32Warps;
+constexpr int kF32K = 32;  // k per stage
+constexpr int kF32Stages = 4;
+template <int TM, int TN> constexpr int kF32StageBytes = (kF32Warps * 2 * TM + 16 * TN) * kF32K * 4;
+
+struct Fp32Params {
+  const int* tile_expert;  // [P]
+  const int* tile_count;   // [P] rows per tile, or nullptr
+  const int* rows_done;
+  int total_rows;
+  int E, tp, N, Kd;        // experts (TP shards counted), columns of the result, length of the sums
+  float* C;                // [P * 128, N]
+  unsigned long long wait_ns;
+  int* status;
+};
+
+__device__ __forceinline__ float4 lds_k4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+
+template <int TM, int TN, bool SWIGLU>
+__global__ void __launch_bounds__(kF32Threads, 2)
+ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b1,
+                const __grid_constant__ CUtensorMap map_b2, const Fp32Params p) {
+  constexpr int BM = kF32Warps * 2 * TM, BN = 16 * TN;  // rows and columns of B per CTA
+  constexpr int NOUT = SWIGLU ? BN / 2 : BN;             // columns of the result per CTA
+  constexpr int kA = BM * kF32K * 4, kStage = kF32StageBytes<TM, TN>;
+  constexpr int kParts = kTileRows / BM;
+  __shared__ unsigned long long s_full[kF32Stages], s_empty[kF32Stages];
+  __shared__ int s_abort;
+  extern __shared__ uint8_t f32_dyn[];
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(f32_dyn) + 1023) & ~(uintptr_t)1023);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int tile = blockIdx.x / kParts, part = blockIdx.x % kParts;
+  const int n0 = blockIdx.y * NOUT;
+  pdl_wait();
+  pdl_trigger();
+  const int e = p.tile_expert[tile];
+  if (e < 0 || e >= p.E) return;  // no owner, or no expert at all (a caller's own table): nothing of the weights is read
+  int rows = kTileRows;
+  if (p.tile_count != nullptr && *p.rows_done >= p.total_rows) rows = p.tile_count[tile];
+  rows = min(rows - part * BM, BM);
+  if (rows <= 0) return;
+  const int live_warps = (rows + 2 * TM - 1) / (2 * TM);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kF32Stages; ++s) {
+      mbar_init(smem_u32(&s_full[s]), 1);
+      mbar_init(smem_u32(&s_empty[s]), live_warps);
+    }
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (warp >= live_warps) return;
+  volatile int* abort_flag = &s_abort;
+  const int nk = (p.Kd + kF32K - 1) / kF32K;
+  const size_t row0 = (size_t)tile * kTileRows + part * BM;
+  int issued = 0, fill = 0;  // copies issued so far (by the first thread), the stage the next one goes to
+  auto issue = [&]() {
+    const uint32_t bar = smem_u32(&s_full[fill]), dst = smem_u32(ring) + (uint32_t)(fill * kStage);
+    const int kc = issued * kF32K;
+    mbar_expect_tx(bar, (uint32_t)kStage);  // rows and columns outside a matrix arrive as zeros
+    tma_load_2d(dst, &map_a, bar, kc, (int)row0);
+    if (SWIGLU) {
+      tma_load_3d(dst + kA, &map_b1, bar, kc, n0, e);
+      tma_load_3d(dst + kA + (kStage - kA) / 2, &map_b2, bar, kc, n0, e);
+    } else {
+      tma_load_4d(dst + kA, &map_b1, bar, kc, n0, e % p.tp, e / p.tp);
+    }
+    ++issued;
+    if (++fill == kF32Stages) fill = 0;
+  };
+  if (threadIdx.x == 0)
+    for (int k = 0; k < min(kF32Stages - 1, nk); ++k) issue();
+  bool failed = false;
+  float acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
+  const int r0 = warp * 2 * TM + lane % 2, c0 = lane / 2;  // rows r0 + 2 i, columns of B c0 + 16 j
+  // the swizzle's row bits: a lane's rows r0 + 2 i take four values of (row % 8), its columns c0 + 16 j only one
+  uint32_t aoff[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) aoff[i] = (uint32_t)((r0 + 2 * i) & 7) << 4;
+  const uint32_t boff = (uint32_t)(c0 & 7) << 4;
+  int b = 0;
+  uint32_t phase = 0;
+  for (int k = 0; k < nk; ++k) {
+    if (!mbar_wait(smem_u32(&s_full[b]), phase, abort_flag, p.wait_ns)) {
+      failed = true;
+      break;
+    }
+    const uint32_t a_base = smem_u32(ring) + (uint32_t)(b * kStage) + (uint32_t)r0 * 128u;
+    const uint32_t b_base = smem_u32(ring) + (uint32_t)(b * kStage + kA) + (uint32_t)c0 * 128u;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      if (half == 1 && issued > 0 && issued < nk) {  // the first thread: refill the stage used up in the last iteration
+        if (k > 0 && !mbar_wait(smem_u32(&s_empty[fill]), (uint32_t)((k - 1) / kF32Stages) & 1u, abort_flag, p.wait_ns)) failed = true;
+        else issue();
+      }
+#pragma unroll
+      for (int uu = 0; uu < kF32K / 8; ++uu) {
+        const uint32_t u = (uint32_t)(half * (kF32K / 8) + uu) << 4;
+        float4 bv[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) bv[j] = lds_k4(b_base + (boff ^ u) + (uint32_t)j * 16u * 128u);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const float4 av = lds_k4(a_base + (aoff[i & 3] ^ u) + (uint32_t)i * 2u * 128u);
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.x, bv[j].x, acc[i][j]);
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.y, bv[j].y, acc[i][j]);
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.z, bv[j].z, acc[i][j]);
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.w, bv[j].w, acc[i][j]);
+        }
+      }
+    }
+    failed = __any_sync(0xffffffffu, failed);
+    if (failed) break;
+    if (lane == 0) mbar_arrive(smem_u32(&s_empty[b]));
+    if (++b == kF32Stages) { b = 0; phase ^= 1u; }
+  }
+  if (failed) {
+    s_abort = 1;
+    set_status(p.status, MOE_ERR_TIMEOUT, kWaitMbarTma);
+    // no copy may still be landing when the CTA's shared memory goes away (only the first thread has issued any)
+    for (int g = max(0, issued - kF32Stages); g < issued; ++g) {
+      const unsigned long long ts = globaltimer();
+      while (!mbar_try(smem_u32(&s_full[g % kF32Stages]), (uint32_t)(g / kF32Stages) & 1u))
+        if (globaltimer() - ts > p.wait_ns + 1000000ull) break;
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    if (r0 + 2 * i >= rows) continue;
+    float* crow = p.C + (row0 + r0 + 2 * i) * p.N;
+#pragma unroll
+    for (int j = 0; j < (SWIGLU ? TN / 2 : TN); ++j) {
+      const int n = n0 + c0 + 16 * j;
+      if (n >= p.N) continue;
+      float v = acc[i][j];
+      if (SWIGLU) v = v / (1.0f + expf(-v)) * acc[i][SWIGLU ? TN / 2 + j : j];
+      crow[n] = v;
+    }
+  }
+}
+
+// fp32 tensor, innermost dimension first, rows of 32 elements by box_rows, 128-byte swizzle.
+static int make_map_f32(EncodeTiledFn enc, CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims,
+                        const cuuint64_t* strides, int box_rows) {
+  cuuint32_t box[4] = {(cuuint32_t)kF32K, (cuuint32_t)box_rows, 1, 1}, estr[4] = {1, 1, 1, 1};
+  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
+}
+
+template <int TM, int TN, bool SWIGLU>
+static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
+                            const Fp32Params& q, cudaStream_t st) {
+  constexpr int BM = kF32Warps * 2 * TM, BN = 16 * TN, NOUT = SWIGLU ? BN / 2 : BN;
+  const cuuint64_t E = (cuuint64_t)p->cfg.E, K = (cuuint64_t)q.Kd, N = (cuuint64_t)q.N, tp = (cuuint64_t)p->tp;
+  CUtensorMap ma, mb1, mb2;
+  int rc;
+  const cuuint64_t adims[2] = {K, (cuuint64_t)p->P * kTileRows}, astr[1] = {K * 4};
+  if ((rc = make_map_f32(enc, &ma, A, 2, adims, astr, BM)) != MOE_OK) return rc;
+  if (SWIGLU) {  // gate / up rows of a TP shard are contiguous: [E * tp, F / tp, H]
+    const cuuint64_t dims[3] = {K, N, E}, str[2] = {K * 4, N * K * 4};
+    if ((rc = make_map_f32(enc, &mb1, b1, 3, dims, str, BN / 2)) != MOE_OK) return rc;
+    if ((rc = make_map_f32(enc, &mb2, b2, 3, dims, str, BN / 2)) != MOE_OK) return rc;
+  } else {       // a shard of the down matrix is a column slice of it
+    const cuuint64_t dims[4] = {K, N, tp, E / tp}, str[3] = {K * tp * 4, K * 4, N * K * tp * 4};
+    if ((rc = make_map_f32(enc, &mb1, b1, 4, dims, str, BN)) != MOE_OK) return rc;
+    mb2 = mb1;
+  }
+  auto kern = ffn_fp32_kernel<TM, TN, SWIGLU>;
+  constexpr size_t smem = 1024 + (size_t)kF32Stages * kF32StageBytes<TM, TN>;
+  static SmemAttrOnce once;
+  if (ensure_dynamic_smem(kern, smem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
+  const dim3 grid((unsigned)(p->P * (kTileRows / BM)), (unsigned)((q.N + NOUT - 1) / NOUT));
+  p->launches += 1;
+  return launch_pdl(kern, grid, dim3(kF32Threads), smem, st, ma, mb1, mb2, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+}
+
+// Both GEMMs of an fp32 plan.
+static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu, const void* wd,
+                       void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st) {
+  const moe_config_t& c = p->cfg;
+  EncodeTiledFn enc;
+  int rc = get_encoder(p, &enc);
+  if (rc != MOE_OK) return rc;
+  Fp32Params q;
+  q.tile_expert = tile_expert;
+  q.tile_count = tile_count;
+  q.rows_done = rows_done;
+  q.total_rows = c.T * c.K;
+  q.E = c.E;
+  q.tp = p->tp;
+  q.wait_ns = kDefaultWaitNs;  // the waits are on this CTA's own copies: nothing a caller's limit is meant for
+  q.status = p->s.status;
+  const int sms = p->sm_count > 0 ? p->sm_count : 148;
+  // 8 x 8 results per lane (64 x 128 per CTA) want experts with enough rows and enough CTAs; otherwise 4 x 4 (32 x 64).
+  // Measured, us, 8 x 8 / 4 x 4: 250 rows per expert, GEMM1 of 624 CTAs 121 / 133, of 312 37 / 43, GEMM2 of 156
+  // 114 / 77; 125 rows per expert, GEMM1 of 1504 CTAs 508 / 511, GEMM2 of 376 349 / 278; 66 rows 97 / 84; 12 rows 183 / 125.
+  const long long blocks = (long long)c.T * c.K / 64 + c.E;  // 64-row blocks, about
+  const bool many_rows = (long long)c.T * c.K >= 192ll * c.E;
+  mark(p, 3, st);
+  q.N = c.F;
+  q.Kd = c.H;
+  q.C = (float*)p->s.inter;
+  if (many_rows && blocks * ((c.F + 63) / 64) >= 2 * sms) rc = launch_fp32_gemm<8, 8, true>(p, enc, recv, wg, wu, q, st);
+  else rc = launch_fp32_gemm<4, 4, true>(p, enc, recv, wg, wu, q, st);
+  if (rc != 0) return rc;
+  mark(p, 4, st);
+  q.N = c.H;
+  q.Kd = c.F;
+  q.C = (float*)out_rows;
+  if (many_rows && blocks * ((c.H + 127) / 128) >= 2 * sms) return launch_fp32_gemm<8, 8, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  return launch_fp32_gemm<4, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+}
+
 template <typename XT>
 static int launch_typed(moe_plan* p, const void* recv, const int* tile_expert, const void* wg,
                         const void* wu, const void* wd, void* out_rows, cudaStream_t st) {
@@ -110,11 +350,11 @@ static int launch_typed(moe_plan* p, const void* recv, const int* tile_expert, c
 }
 
 int launch_ffn_simt(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu,
-                    const void* wd, void* out_rows, cudaStream_t st) {
+                    const void* wd, void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st) {
   if (p->P == 0 || p->cfg.T == 0) return 0;
   if (p->cfg.dtype == MOE_DTYPE_BF16)
     return launch_typed<__nv_bfloat16>(p, recv, tile_expert, wg, wu, wd, out_rows, st);
-  return launch_typed<float>(p, recv, tile_expert, wg, wu, wd, out_rows, st);
+  return launch_fp32(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
 }
 
 }  // namespace moehub

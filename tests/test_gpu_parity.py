@@ -239,6 +239,37 @@ def test_router_chain_kernel_edges(shape):
     Hh.check_route(idx, tw, ridx, rw)
 
 
+# The fp32 expert kernel where its tiles end: both tile sizes (few and many blocks), experts with 1 to 300 rows (so that
+# warps, half tiles and whole tiles are left out), widths that are no multiple of its column blocks and sums whose
+# length is no multiple of its stages, TP shards, and tiles computed whole because no row counts are given.
+FP32_FFN = [
+    # (T, H, E, K, F, tp, zipf_s)
+    (1, 4, 2, 1, 4, 1, 0.0), (40, 36, 4, 2, 68, 1, 1.2), (300, 132, 3, 2, 100, 1, 1.2), (1200, 260, 8, 2, 1284, 1, 1.2),
+    (700, 516, 16, 3, 1028, 1, 1.0), (129, 100, 6, 2, 264, 2, 1.0),
+]
+
+
+@pytest.mark.parametrize("case", FP32_FFN, ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}")
+def test_fp32_expert_kernel_edges(case):
+    T, H, E, K, F, tp, zipf = case
+    w = inputs.Workload("fp32_edges", T=T, H=H, E=E, R=1, K=K, F=F, dtype=FP32, zipf_s=zipf, seed=17)
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    ref = Hh.oracle_layer_for(w, x, wr, bias, wg, wu, wd)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, tp_shards=tp)
+    y = torch.empty((T, H), dtype=torch.float32, device="cuda")
+    args = [Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)]
+    plan.moe_layer(*args, y)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    Hh.assert_output_close(Hh.to_host_f64(y), ref["y"], FP32)
+    # the same rows without the counters: every tile computed whole, the same bytes in the rows there are
+    rows = torch.empty((plan.P * 128, H), dtype=torch.float32, device="cuda")
+    plan.moe_expert_ffn(plan.layer_tensor(2), plan.layer_tensor(4), *args[3:], rows)
+    torch.cuda.synchronize()
+    used = plan.layer_tensor(6).flatten().long()
+    assert torch.equal(rows[used], plan.layer_tensor(7)[used])
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

@@ -121,7 +121,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
   int* work_counter = prm.work_counter + (phase == 2 ? 1 : 0);
   int first_claim = 0;
   if (threadIdx.x == 0 && !producer_cta) first_claim = atomicAdd(work_counter, 1);  // in flight while the work list is built
-  build_worklist(wl, prm.tile_expert, prm.P, E, (F + 127) / 128, (H + 255) / 256, prm.lag, prm.fused, 1, prm.hot_min,
+  build_worklist(wl, reinterpret_cast<uint16_t*>(stage_base), prm.tile_expert, prm.P, E, (F + 127) / 128, (H + 255) / 256, prm.lag, prm.fused, 1, prm.hot_min,
                  prm.hist, prm.hot_first);
   tc_fence_before();
   __syncthreads();

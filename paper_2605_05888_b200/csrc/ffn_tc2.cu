@@ -117,7 +117,7 @@ ffn_tc2_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   pdl_wait();  // everything above needs no global data and overlaps the predecessor's tail
-  build_worklist(wl, prm.tile_expert, prm.P, E, (F + 127) / 128, (H + 255) / 256, prm.lag, prm.fused, 2);
+  build_worklist(wl, reinterpret_cast<uint16_t*>(stage_base), prm.tile_expert, prm.P, E, (F + 127) / 128, (H + 255) / 256, prm.lag, prm.fused, 2);
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers exist before anything arrives on them

@@ -79,10 +79,11 @@ typedef struct {
   int32_t renormalize;          /* 0: w = softmax prob. of the picked experts; 1: / their sum */
   int32_t dispatch_mode;        /* MOE_DISPATCH_*                                            */
   int32_t identity_experts;     /* 1: moe_layer skips the FFN (expert output = expert input)  */
-  int32_t ffn_kernel;           /* 0: tensor-core (tcgen05) kernel, one CTA per tile, for bf16,
-                                   SIMT for fp32; 1: SIMT fp32-FMA kernel for either dtype
-                                   (check path); 2: tensor-core kernel on CTA pairs
-                                   (cta_group::2, two tiles per MMA; bf16)                    */
+  int32_t ffn_kernel;           /* 0: tensor-core (tcgen05) kernel for bf16 - one CTA per tile, or
+                                   CTA pairs (cta_group::2, two tiles of an expert per item)
+                                   where experts have more than one tile of rows on average -
+                                   and the fp32-FMA kernel for fp32; 1: plain SIMT fp32-FMA
+                                   kernel for bf16 (check path); 2: always CTA pairs (bf16)   */
   int32_t ffn_split;            /* 1: one launch per expert GEMM; 2: both GEMMs in one persistent
                                    launch (per-tile status counters gate GEMM2); 0: choose
                                    (one launch when E <= 64; with more, smaller experts two
@@ -108,7 +109,7 @@ typedef struct {
                                    reads each row's source information and stores the result at
                                    the token's own position [t*K+k], the combine kernel then reads
                                    K consecutive rows per token).  Push needs bf16 and the
-                                   one-CTA-per-tile tensor-core kernel (ffn_kernel 0)            */
+                                   tensor-core kernel of ffn_kernel 0                            */
   int32_t tp_shards;            /* expert + tensor parallelism (Section VII): S > 1 cuts every expert's
                                    FFN into S slices of its width F (gate/up rows [s*F/S, (s+1)*F/S),
                                    the matching columns of the down matrix), gives every slice a
@@ -362,7 +363,7 @@ int moe_layer_buffer(moe_plan_t* plan, int which, void** out_ptr);
  * dispatch CTA, [1] the moment the global counter reached all T*K assignments, [2 + p] the moment
  * tile p's counter reached 128 rows (0: the tile never filled).  Disabled (the default) the kernels
  * are unchanged.  The flag is host-side state of the plan.
- * While enabled, the tensor-core expert kernel (one CTA per tile, bf16) also writes a timeline of its
+ * While enabled, the tensor-core expert kernel (bf16; always the one with one CTA per tile then) also writes a timeline of its
  * work items: uint64 [P * (ceil(F/128) + ceil(H/256))][4] (moe_layer_buffer, which = 9), one entry
  * per position of its item list in the order the items were claimed: [0] the moment the item's
  * producer had seen its tile ready and began to load, [1] the moment its MMAs were complete, [2] what

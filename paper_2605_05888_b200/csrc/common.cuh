@@ -222,6 +222,12 @@ template <> struct Vec16<__nv_bfloat16> {
   }
 };
 
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {  // a shared-memory load by its 32-bit shared address
+  uint4 r;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr));
+  return r;
+}
+
 // Programmatic dependent launch: the kernels of the layer (all but the first, the router: starting
 // it while the previous layer call drains measured slower) are launched so that they may start while
 // their predecessor in the stream is still draining.  pdl_wait() blocks until the predecessor has

@@ -85,7 +85,10 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   uint8_t* stage_base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   TcShared* sh = reinterpret_cast<TcShared*>(stage_base + kStages * kStageBytes);
-  __shared__ __align__(16) WorkList wl;  // a producer CTA keeps the dispatch's bookkeeping (with its mbarriers) here first
+  // a producer CTA keeps the dispatch's bookkeeping (with its mbarriers) here first
+  __shared__ __align__(16) union { WorkList wl; OrdShared ord; } list_or_dispatch;
+  WorkList& wl = list_or_dispatch.wl;
+  __shared__ int row_count[kMaxExperts];  // rows per expert when the list was built from row counts, else -1
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nseg = 2 * E;
@@ -115,14 +118,14 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
     // dispatch's bookkeeping sits in the work list's place; every bulk copy has completed when the call
     // returns.  Afterwards the CTA takes no work item: it only goes through the common tear-down.
     __syncthreads();
-    dispatch_ordered_cta<kTcThreads>(ov.ord, *reinterpret_cast<OrdShared*>(&wl), stage_base, (int)blockIdx.x, ov.n_dispatch);
+    dispatch_ordered_cta<kTcThreads>(ov.ord, list_or_dispatch.ord, stage_base, (int)blockIdx.x, ov.n_dispatch);
     __syncthreads();
   }
   int* work_counter = prm.work_counter + (phase == 2 ? 1 : 0);
   int first_claim = 0;
   if (threadIdx.x == 0 && !producer_cta) first_claim = atomicAdd(work_counter, 1);  // in flight while the work list is built
-  build_worklist(wl, reinterpret_cast<uint16_t*>(stage_base), prm.tile_expert, prm.P, E, (F + 127) / 128, (H + 255) / 256, prm.lag, prm.fused, 1, prm.hot_min,
-                 prm.hist, prm.hot_first);
+  build_worklist(wl, *reinterpret_cast<WorkScratch*>(stage_base), prm.tile_expert, prm.P, E, (F + 127) / 128, (H + 255) / 256, prm.lag, prm.fused, 1, prm.hot_min,
+                 prm.hist, prm.hot_first, row_count);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -218,7 +221,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
         // Rows the tile will hold, when the work list was built from the experts' row counts: the threshold of
         // its status counter (a partly filled last tile is ready as soon as ITS rows have arrived).
         int tile_rows = -1;
-        if (wl.count[it.e] >= 0) tile_rows = min(kTileRows, wl.count[it.e] - (it.tile - wl.estart[it.e]) * kTileRows);
+        if (row_count[it.e] >= 0) tile_rows = min(kTileRows, row_count[it.e] - (it.tile - wl.estart[it.e]) * kTileRows);
         if (it.type == 0 && tile_count != nullptr && tile_rows >= 0 && ov.gate_all) {
           if (ld_acquire(rows_done) < total_rows) {
             const unsigned long long t0 = globaltimer();
@@ -564,38 +567,11 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
 }
 
 // ---- host side ------------------------------------------------------------------------------
-// bf16 tensor [E, rows, cols], box [1, box_rows, 64].
-static int make_map_3d(EncodeTiledFn enc, CUtensorMap* m, const void* base, uint64_t E, uint64_t rows, uint64_t cols,
-                       uint32_t box_rows) {
-  cuuint64_t dims[3] = {cols, rows, E};
-  cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
-  cuuint32_t box[3] = {(cuuint32_t)kBK, box_rows, 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
-}
-
 OrderedParams make_ordered_params(moe_plan* p, const void* x, const int* topk_idx, void* recv, int* expert_count,
                                   int* tile_expert, int* src_info, int* slot_of, int* tile_count, int* rows_done);
 
 // overlap_x / overlap_idx != nullptr: the overlapped form - the launch that runs the GEMM1 items also
 // dispatches x (ordered scheme, into recv and the plan's own dispatch outputs) on its first CTAs.
-// The down matrices [E, H, F*tp] seen as [E, tp, H, F]: shard s of an expert is the column slice [s*F, (s+1)*F).
-// Box [1, 1, box_rows, 64].
-static int make_map_wd(EncodeTiledFn enc, CUtensorMap* m, const void* base, uint64_t experts, uint64_t tp, uint64_t rows,
-                       uint64_t cols, uint32_t box_rows) {
-  cuuint64_t dims[4] = {cols, rows, tp, experts};
-  cuuint64_t strides[3] = {cols * tp * 2, cols * 2, rows * cols * tp * 2};
-  cuuint32_t box[4] = {(cuuint32_t)kBK, box_rows, 1, 1};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
-}
-
 int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu,
                   const void* wd, void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st,
                   const void* overlap_x, const int* overlap_idx, const int* push_src) {
@@ -610,12 +586,7 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   if ((rc = make_map_3d(enc, &bg, wg, c.E, c.F, c.H, 128)) != MOE_OK) return rc;
   if ((rc = make_map_3d(enc, &bu, wu, c.E, c.F, c.H, 128)) != MOE_OK) return rc;
   if ((rc = make_map_2d(enc, &a2, p->s.inter, pool_rows, c.F, kTileRows)) != MOE_OK) return rc;
-  if (c.ffn_kernel == 2) {  // the pair kernel: 3-D map, no TP shards
-    if (p->tp != 1) return MOE_ERR_UNSUPPORTED;
-    if ((rc = make_map_3d(enc, &bd, wd, c.E, c.H, c.F, 128)) != MOE_OK) return rc;
-  } else if ((rc = make_map_wd(enc, &bd, wd, c.E / p->tp, p->tp, c.H, c.F, 256)) != MOE_OK) {
-    return rc;
-  }
+  if ((rc = make_map_wd(enc, &bd, wd, c.E / p->tp, p->tp, c.H, c.F, 256)) != MOE_OK) return rc;
   CUtensorMap a1t, a2t;  // the first kThinRows rows of a tile, for tiles computed the other way round
   if ((rc = make_map_2d(enc, &a1t, recv, pool_rows, c.H, kThinRows)) != MOE_OK) return rc;
   if ((rc = make_map_2d(enc, &a2t, p->s.inter, pool_rows, c.F, kThinRows)) != MOE_OK) return rc;
@@ -628,22 +599,26 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   // the single launch measures 2-3 % slower than two, also with items handed out dynamically, so the
   // default splits there.
   const int fused = c.ffn_split == 2 ? 1 : (c.ffn_split == 1 ? 0 : (c.E <= 64 ? 1 : 0));
-  const bool pairs = c.ffn_kernel == 2;  // opt-in: the CTA-pair kernel
-  if (pairs && push_src != nullptr) return MOE_ERR_UNSUPPORTED;
-  const int workers = pairs ? grid / 2 : grid;
+  if (c.ffn_kernel == 2 && (push_src != nullptr || p->tp != 1)) return MOE_ERR_UNSUPPORTED;  // asked for by number: the plain layer only
+  // CTA pairs by default where experts have more than one tile of rows on average (a pair reads an expert's weights once
+  // per two tiles and pads the rows to 32 instead of 128) and the sums are long enough for the pair's unhidden epilogue.
+  // Measured, layer time one CTA / pair: 137 rows per expert (H 2048, F 1408) 1.05, 256 (H 4096, F 14336) 1.045, 192
+  // (H 4096, F 1024) 1.03-1.07; 128 rows 0.95-1.01; 64 rows 0.95; 250 rows with H 1024 0.94.  The options that only the
+  // other kernel has (in-launch dispatch, interleaving, work-item timeline, no narrow form) keep it.
+  const bool pairs = c.ffn_kernel == 2 || (c.ffn_kernel == 0 && (long long)c.T * c.K > (long long)kTileRows * c.E && c.H >= 1536 &&
+                                           c.F >= 1024 && overlap_x == nullptr && c.ffn_hot_min_tiles <= 0 &&
+                                           c.ffn_thin_tiles >= 0 && !p->trace);
   if (p->P > kMaxListTiles) return MOE_ERR_UNSUPPORTED;  // the work list lives in the kernel's shared memory
   if ((long long)p->P * (NB1 + NB2) >= (1ll << kThinShift)) return MOE_ERR_UNSUPPORTED;  // item index field of the ring
-  // The one-CTA kernel puts its counters back to zero itself; the pair kernel has static item assignment
-  // and no last-one-out step, so its GEMM1 counters are cleared here (also for a call without counters,
-  // which no dispatch preceded).
-  if ((tile_count == nullptr || pairs) &&
+  // The kernels put their counters back to zero themselves; a call without counters may come before any dispatch.
+  if (tile_count == nullptr &&
       cudaMemsetAsync(p->s.gemm1_done, 0, sizeof(int) * (size_t)(p->P + 4), st) != cudaSuccess)
     return MOE_ERR_CUDA;
   mark(p, 3, st);
   FfnParams prm;
   prm.tile_expert = tile_expert;
   prm.P = (int)p->P;
-  prm.lag = 2 * workers;
+  prm.lag = 2 * grid;
   prm.fused = fused;
   // Interleaving (opt-in, two-launch form only).  Measured on the DeepSeek-like layer it changes nothing:
   // every kind of item there takes 57-75 us whether the kinds are mixed or not, because none of them is
@@ -670,8 +645,13 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   prm.hot_first = 0;
   prm.band = 0;
   prm.push_src = push_src;
+  if (pairs) {
+    rc = launch_ffn_pair(p, recv, wg, wu, wd, prm, st);
+    if (rc != 0) return rc;
+    return cudaGetLastError() == cudaSuccess ? 0 : MOE_ERR_CUDA;
+  }
   OverlapParams ov = {};
-  const bool overlap = overlap_x != nullptr && !pairs;
+  const bool overlap = overlap_x != nullptr;
   if (overlap) {
     Scratch& s = p->s;
     ov.ord = make_ordered_params(p, overlap_x, overlap_idx, s.recv, s.expert_count, s.tile_expert, s.src_info, s.slot_of,
@@ -686,7 +666,6 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   }
   auto launch = [&](int phase) -> int {
     prm.phase = phase;
-    if (pairs) return launch_ffn_tc2_kernel(a1, bg, bu, a2, bd, prm, grid, st);
     OverlapParams ovp = {};
     if (overlap && phase != 2) {
       // The launch that carries the dispatch: its work list comes from the row counts (no tile owner is

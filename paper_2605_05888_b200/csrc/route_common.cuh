@@ -25,12 +25,6 @@ __device__ __forceinline__ float fma_bf16_hi(uint32_t x, uint32_t w, float acc) 
       : "=f"(d) : "r"(x), "r"(w), "f"(acc));
   return d;
 }
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {  // a shared-memory load by its 32-bit shared address
-  uint4 r;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr));
-  return r;
-}
-
 // A float as an unsigned number of the same order (-0 and +0 equal), so that an integer reduction finds the maximum.
 __device__ __forceinline__ unsigned order_key(float v) {
   const unsigned u = __float_as_uint(v + 0.0f);

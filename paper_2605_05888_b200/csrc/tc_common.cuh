@@ -32,13 +32,15 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// The hardware suspends the thread until the phase completes or the time hint (nanoseconds) has passed.
+constexpr uint32_t kTryHintNs = 20000;
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(kTryHintNs) : "memory");
   return ok != 0;
 }
 // Bounded wait.  Returns false when the time limit ran out or another role already gave up.
@@ -180,14 +182,18 @@ struct WorkList {
   int estart[kMaxExperts + 1];
   int seg_start[2 * kMaxExperts + 1];
   int seg_info[2 * kMaxExperts];
-  int cursor[kMaxExperts];
-  int order[kMaxExperts];      // the experts in the order their segments are placed
-  int count[kMaxExperts];      // rows per expert when the list was built from row counts, else -1
-  int units[kMaxExperts + 1];  // units (tiles, or pairs of them) of the experts placed before position i
-  int after[kMaxExperts];      // the position whose GEMM1 segment the GEMM2 segment of position q follows
   int n1;
   int n_hot[2];
   uint16_t tiles[kMaxListTiles];
+};
+// What only the building needs (it lies in the operand stages, which are not in use yet).
+struct WorkScratch {
+  int cursor[kMaxExperts];
+  int order[kMaxExperts];      // the experts in the order their segments are placed
+  int units[kMaxExperts + 1];  // units (tiles, or pairs of them) of the experts placed before position i
+  int after[kMaxExperts];      // the position whose GEMM1 segment the GEMM2 segment of position q follows
+  int n_hot_experts;
+  uint16_t owner[kMaxListTiles];  // tile_expert, 0xffff: unused
 };
 
 // All threads of the CTA call this (it synchronises the CTA).  pair = 2 counts one item per PAIR of
@@ -198,22 +204,22 @@ struct WorkList {
 // owns the consecutive tiles [estart[e], estart[e + 1]) (the layout of the ordered dispatch), which is known
 // before a single row has been dispatched.  hot_first: experts are placed by descending row count (the
 // experts whose first tiles fill earliest come first) instead of by index.
-// raw: shared-memory scratch of P entries (the operand stages, not in use yet).
+// count: [kMaxExperts] rows per expert, filled in when the list is built from them (else -1), or nullptr.
 //
 // Every step but the scatter of the tiles is a prefix sum or a binary search per expert, because this stands in front
 // of every expert launch: a serial walk over the experts with dependent shared-memory reads, and tile owners fetched
 // from global memory 32 at a time, took 12-14 us with 60 experts (expert launch of one Qwen-like token 53.7 -> 45.4 us,
 // of 512 tokens 190.8 -> 178.7; both launches of the 128-token DeepSeek-like layer 2382 -> 2319).
-__device__ __forceinline__ void build_worklist(WorkList& wl, uint16_t* raw, const int* __restrict__ tile_expert, int P, int E,
+__device__ __forceinline__ void build_worklist(WorkList& wl, WorkScratch& ws, const int* __restrict__ tile_expert, int P, int E,
                                                int NB1, int NB2, int lag, int fused, int pair, int hot_min = 0,
-                                               const int* __restrict__ hist = nullptr, int hot_first = 0) {
+                                               const int* __restrict__ hist = nullptr, int hot_first = 0, int* count = nullptr) {
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid % 32;
   constexpr int kPer = kMaxExperts / 32;  // experts per lane in the scans
   constexpr int kAhead = 4;               // tile owners fetched at once
   for (int e = tid; e < kMaxExperts; e += nthr) {
-    wl.cursor[e] = (hist != nullptr && e < E) ? (hist[e] + kTileRows - 1) / kTileRows : 0;
-    wl.count[e] = (hist != nullptr && e < E) ? hist[e] : -1;
-    wl.order[e] = e;
+    ws.cursor[e] = (hist != nullptr && e < E) ? (hist[e] + kTileRows - 1) / kTileRows : 0;
+    if (count != nullptr) count[e] = (hist != nullptr && e < E) ? hist[e] : -1;
+    ws.order[e] = e;
   }
   __syncthreads();
   if (hist == nullptr) {
@@ -225,30 +231,57 @@ __device__ __forceinline__ void build_worklist(WorkList& wl, uint16_t* raw, cons
       for (int i = 0; i < kAhead; ++i) {
         const int p = p0 + i * nthr;
         const bool used = e[i] >= 0 && e[i] < E;
-        if (p < P) raw[p] = used ? (uint16_t)e[i] : (uint16_t)0xffff;
-        if (used) atomicAdd(&wl.cursor[e[i]], 1);
+        if (p < P) ws.owner[p] = used ? (uint16_t)e[i] : (uint16_t)0xffff;
+        if (used) atomicAdd(&ws.cursor[e[i]], 1);
       }
     }
   } else if (hot_first) {
     // position of expert e = experts with more rows, or as many and a lower index
     for (int e = tid; e < E; e += nthr) {
-      const int c = wl.count[e];
+      const int c = count[e];
       int rank = 0;
       for (int o = 0; o < E; ++o) {
-        const int co = wl.count[o];
+        const int co = count[o];
         rank += (co > c || (co == c && o < e)) ? 1 : 0;
       }
-      wl.order[rank] = e;
+      ws.order[rank] = e;
     }
   }
   __syncthreads();
+  if (hot_min > 0 && !fused) {  // order: the hot experts, then the cold ones, each in index order
+    if (tid < 32) {
+      int hot[kPer], sum = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int e = lane * kPer + i;
+        hot[i] = e < E && ws.cursor[e] >= hot_min ? 1 : 0;
+        sum += hot[i];
+      }
+      int incl = sum;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += n;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      int run = incl - sum;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int e = lane * kPer + i;
+        if (e < E) ws.order[hot[i] ? run : total + e - run] = e;
+        run += hot[i];
+      }
+      if (lane == 0) ws.n_hot_experts = total;
+    }
+    __syncthreads();
+  }
   if (tid < 64) {  // warp 0: tiles of the experts before expert e; warp 1: units of the experts placed before position e
     const bool units = tid >= 32;
     int c[kPer], sum = 0;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
       const int e = lane * kPer + i;
-      c[i] = e < E ? wl.cursor[units ? wl.order[e] : e] : 0;
+      c[i] = e < E ? ws.cursor[units ? ws.order[e] : e] : 0;
       if (units) c[i] = (c[i] + pair - 1) / pair;
       sum += c[i];
     }
@@ -259,7 +292,7 @@ __device__ __forceinline__ void build_worklist(WorkList& wl, uint16_t* raw, cons
       if (lane >= off) incl += n;
     }
     int run = incl - sum;
-    int* dst = units ? wl.units : wl.estart;
+    int* dst = units ? ws.units : wl.estart;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
       const int e = lane * kPer + i;
@@ -269,82 +302,61 @@ __device__ __forceinline__ void build_worklist(WorkList& wl, uint16_t* raw, cons
     if (lane == 31) dst[E] = incl;
   }
   __syncthreads();
-  auto tiles_of = [&](int e) { return wl.estart[e + 1] - wl.estart[e]; };
   if (tid < 32) {
     if (hist != nullptr) {
       const int total = min(wl.estart[E], kMaxListTiles);
       for (int t = lane; t < total; t += 32) wl.tiles[t] = (uint16_t)t;  // regions are consecutive tiles
     } else {
-      for (int e = lane; e < E; e += 32) wl.cursor[e] = wl.estart[e];
+      for (int e = lane; e < E; e += 32) ws.cursor[e] = wl.estart[e];
       __syncwarp();
       // stable scatter, 32 tiles at a time: the same list in every CTA
       for (int p0 = 0; p0 < P; p0 += 32) {
         const int p = p0 + lane;
-        const unsigned e = p < P ? raw[p] : 0xffffu;
+        const unsigned e = p < P ? ws.owner[p] : 0xffffu;
         const unsigned peers = __match_any_sync(0xffffffffu, e);
-        if (e != 0xffffu) wl.tiles[wl.cursor[e] + __popc(peers & ((1u << lane) - 1u))] = (uint16_t)p;
+        if (e != 0xffffu) wl.tiles[ws.cursor[e] + __popc(peers & ((1u << lane) - 1u))] = (uint16_t)p;
         __syncwarp();
-        if (e != 0xffffu && lane == __ffs(peers) - 1) wl.cursor[e] += __popc(peers);
+        if (e != 0xffffu && lane == __ffs(peers) - 1) ws.cursor[e] += __popc(peers);
         __syncwarp();
       }
     }
   } else if (tid < 64) {
-    const int* units = wl.units;
+    const int* units = ws.units;
     const int total = units[E];
-    if (!fused && hot_min > 0) {
-      if (lane == 0) {  // two passes per GEMM: hot experts, then cold ones
-        int pos = 0, nseg = 0;
-        for (int g = 0; g < 2; ++g) {
-          const int nb = g == 0 ? NB1 : NB2;
-          const int begin = pos;
-          for (int cold = 0; cold < 2; ++cold) {
-            for (int e = 0; e < E; ++e) {
-              const int m = tiles_of(e);
-              if ((m >= hot_min ? 0 : 1) != cold) continue;
-              wl.seg_start[nseg] = pos;
-              wl.seg_info[nseg++] = e | (g << 16);
-              pos += (m + pair - 1) / pair * nb;
-            }
-            if (cold == 0) wl.n_hot[g] = pos - begin;
-          }
-          if (g == 0) wl.n1 = pos;
+    // Position q's GEMM2 segment goes behind position after[q]'s GEMM1 segment: the first one at least `lag` GEMM1
+    // items on.  The last positions keep their GEMM2 segments for the end of the list, so that they too have `lag`
+    // items between the two (without that their GEMM2 items waited up to half an item for the intermediate).
+    for (int q = lane; q < E; q += 32) {
+      int after = E - 1;
+      if (fused && (long long)NB2 * (units[max(E - 1, q + 1)] - units[q + 1]) >= lag) {
+        int lo = q, hi = E - 1;  // first i > q with NB1 * (units up to i - units up to q) >= lag; none: the last position
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) / 2;
+          if ((long long)NB1 * (units[mid + 1] - units[q + 1]) >= lag) hi = mid; else lo = mid;
         }
-        wl.seg_start[nseg] = pos;  // nseg == 2E
+        after = hi;
       }
-    } else {
-      // Position q's GEMM2 segment goes behind position after[q]'s GEMM1 segment: the first one at least `lag` GEMM1
-      // items on.  The last positions keep their GEMM2 segments for the end of the list, so that they too have `lag`
-      // items between the two (without that their GEMM2 items waited up to half an item for the intermediate).
-      for (int q = lane; q < E; q += 32) {
-        int after = E - 1;
-        if (fused && (long long)NB2 * (units[max(E - 1, q + 1)] - units[q + 1]) >= lag) {
-          int lo = q, hi = E - 1;  // first i > q with NB1 * (units up to i - units up to q) >= lag; none: the last position
-          while (hi - lo > 1) {
-            const int mid = (lo + hi) / 2;
-            if ((long long)NB1 * (units[mid + 1] - units[q + 1]) >= lag) hi = mid; else lo = mid;
-          }
-          after = hi;
-        }
-        wl.after[q] = after;
+      ws.after[q] = after;
+    }
+    __syncwarp();
+    for (int i = lane; i < E; i += 32) {
+      int before = 0, hi = E;  // GEMM2 segments in front of position i's GEMM1 segment: those with after[q] < i
+      while (before < hi) {
+        const int mid = (before + hi) / 2;
+        if (ws.after[mid] < i) before = mid + 1; else hi = mid;
       }
-      __syncwarp();
-      for (int i = lane; i < E; i += 32) {
-        int before = 0, hi = E;  // GEMM2 segments in front of position i's GEMM1 segment: those with after[q] < i
-        while (before < hi) {
-          const int mid = (before + hi) / 2;
-          if (wl.after[mid] < i) before = mid + 1; else hi = mid;
-        }
-        wl.seg_start[i + before] = NB1 * units[i] + NB2 * units[before];
-        wl.seg_info[i + before] = wl.order[i];
-        const int seg2 = wl.after[i] + 1 + i;
-        wl.seg_start[seg2] = NB1 * units[wl.after[i] + 1] + NB2 * units[i];
-        wl.seg_info[seg2] = wl.order[i] | (1 << 16);
-      }
-      if (lane == 0) {
-        wl.n_hot[0] = wl.n_hot[1] = -1;  // no interleaving
-        wl.n1 = fused ? 0 : NB1 * total;
-        wl.seg_start[2 * E] = (NB1 + NB2) * total;
-      }
+      wl.seg_start[i + before] = NB1 * units[i] + NB2 * units[before];
+      wl.seg_info[i + before] = ws.order[i];
+      const int seg2 = ws.after[i] + 1 + i;
+      wl.seg_start[seg2] = NB1 * units[ws.after[i] + 1] + NB2 * units[i];
+      wl.seg_info[seg2] = ws.order[i] | (1 << 16);
+    }
+    if (lane == 0) {
+      const bool split = !fused && hot_min > 0;
+      wl.n_hot[0] = split ? NB1 * units[ws.n_hot_experts] : -1;  // -1: no interleaving
+      wl.n_hot[1] = split ? NB2 * units[ws.n_hot_experts] : -1;
+      wl.n1 = fused ? 0 : NB1 * total;
+      wl.seg_start[2 * E] = (NB1 + NB2) * total;
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the scratch becomes the target of TMA loads
@@ -402,8 +414,8 @@ struct ClockProbe {
 };
 
 // The CTA-pair (cta_group::2) kernel lives in ffn_tc2.cu.
-int launch_ffn_tc2_kernel(const CUtensorMap& a1, const CUtensorMap& bg, const CUtensorMap& bu, const CUtensorMap& a2,
-                          const CUtensorMap& bd, const FfnParams& prm, int grid, cudaStream_t st);
+int launch_ffn_pair(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, FfnParams prm,
+                    cudaStream_t st);
 
 // ---- tensor maps (host side) ---------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -431,6 +443,31 @@ inline int make_map_2d(EncodeTiledFn enc, CUtensorMap* m, const void* base, uint
   cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
+}
+// bf16 tensor [E, rows, cols], box [1, box_rows, 64].
+inline int make_map_3d(EncodeTiledFn enc, CUtensorMap* m, const void* base, uint64_t E, uint64_t rows, uint64_t cols,
+                       uint32_t box_rows) {
+  cuuint64_t dims[3] = {cols, rows, E};
+  cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
+  cuuint32_t box[3] = {(cuuint32_t)kBK, box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
+}
+// The down matrices [E, H, F*tp] seen as [E, tp, H, F]: shard s of an expert is the column slice [s*F, (s+1)*F).
+// Box [1, 1, box_rows, 64].
+inline int make_map_wd(EncodeTiledFn enc, CUtensorMap* m, const void* base, uint64_t experts, uint64_t tp, uint64_t rows,
+                       uint64_t cols, uint32_t box_rows) {
+  cuuint64_t dims[4] = {cols, rows, tp, experts};
+  cuuint64_t strides[3] = {cols * tp * 2, cols * 2, rows * cols * tp * 2};
+  cuuint32_t box[4] = {(cuuint32_t)kBK, box_rows, 1, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;

@@ -270,6 +270,56 @@ def test_fp32_expert_kernel_edges(case):
     assert torch.equal(rows[used], plan.layer_tensor(7)[used])
 
 
+# The CTA-pair expert kernel where its items end: an expert's rows around 16, 32, 128 (one tile), 129, 256 (a pair of
+# tiles) and 257, all experts the same so that every count is met; in the paged layout (tiles of an expert apart) and
+# the ordered one; H and F that end inside its 512- and 256-column blocks and inside a k-block; one and two launches.
+@pytest.mark.parametrize("split", [1, 2])
+@pytest.mark.parametrize("mode", [B.DISPATCH_ATOMIC_PAGED, B.DISPATCH_ATOMIC_ORDERED])
+@pytest.mark.parametrize("rows", [1, 16, 17, 33, 112, 127, 128, 129, 145, 255, 256, 257, 300])
+def test_pair_expert_kernel_row_counts(rows, mode, split):
+    E, H, F = 3, (200, 776, 1032)[rows % 3], (72, 392, 520)[rows % 3]
+    w = inputs.Workload("pair_rows", T=rows, H=H, E=E, R=1, K=E, F=F, dtype=BF16, seed=19)   # K = E: every expert gets every token
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    ref = Hh.oracle_layer_for(w, x, wr, bias, wg, wu, wd)
+    args = [Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)]
+    ys = []
+    for kernel in (2, 0):
+        plan = Hh.make_plan(w, mode, ffn_kernel=kernel, ffn_split=split)
+        for _ in range(2):      # twice: the second call meets the counters as the first one left them
+            y = torch.empty((w.T, w.H), dtype=torch.bfloat16, device="cuda")
+            plan.layer_tensor(2).fill_(float("nan"))   # rows that are not there must not reach the others
+            plan.moe_layer(*args, y)
+            torch.cuda.synchronize()
+            assert plan.moe_last_status() == (0, 0)
+        Hh.assert_output_close(Hh.to_host_f64(y), ref["y"], BF16)
+        ys.append(y)
+    assert torch.equal(ys[0], ys[1])     # the same sums in the same order: the same bytes as one CTA per tile
+
+
+# Where the default takes the pair kernel: skewed experts (empty ones and ones of several tiles), TP shards, the push
+# epilogue and a call without counters give the bytes of the one-CTA kernel (asked for with ffn_thin_tiles = -1).
+@pytest.mark.parametrize("tp,combine", [(1, 0), (1, 1), (2, 0), (2, 1)])
+def test_pair_expert_kernel_by_default(tp, combine):
+    w = inputs.Workload("pair_default", T=900, H=1544, E=12, R=1, K=3, F=2064, dtype=BF16, zipf_s=1.2, seed=23)
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    args = [Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)]
+    ys = []
+    for thin in (0, -1):
+        plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_ORDERED, tp_shards=tp, combine_mode=combine, ffn_thin_tiles=thin)
+        y = torch.empty((w.T, w.H), dtype=torch.bfloat16, device="cuda")
+        plan.moe_layer(*args, y)
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == (0, 0)
+        ys.append(y)
+        if combine == 0:
+            rows = torch.empty((plan.P * 128, w.H), dtype=torch.bfloat16, device="cuda")
+            plan.moe_expert_ffn(plan.layer_tensor(2), plan.layer_tensor(4), *args[3:], rows)
+            torch.cuda.synchronize()
+            used = plan.layer_tensor(6).flatten().long()
+            assert torch.equal(rows[used], plan.layer_tensor(7)[used])
+    assert torch.equal(ys[0], ys[1])
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

@@ -33,11 +33,13 @@ constexpr int kRfEP = 256;           // experts covered (the accumulator's colum
 constexpr float kRfEps = 1.5f * 1.1920929e-7f;  // 1.5 * 2^-23
 constexpr int kRfChunk = 64;         // h per staged chunk: 128 bytes of a row
 constexpr int kRfBufs = 3;           // staged chunks in flight
+constexpr int kRfAhead = 8;          // chunks of x asked for ahead of that, into L2
 constexpr int kRfWBytes = kRfEP * kRfChunk * 2;  // one chunk of every expert's row: 32 KB
-// shared memory of the refine kernel for TPC tokens per CTA (half a warp each): kRfBufs buffers of one chunk of Wr
+// shared memory of the refine kernel for tpc tokens per CTA (half a warp each): kRfBufs buffers of one chunk of Wr
 // and of the tokens' rows of x (written by TMA, 128-byte swizzle), the tokens' logit rows, the list of chains
+__host__ __device__ constexpr int rf_x_bytes(int tpc) { return (tpc * kRfChunk * 2 + 1023) & ~1023; }  // buffers start on 1024 bytes
 constexpr size_t rf_smem(int tpc) {
-  return 1024 + (size_t)kRfBufs * (kRfWBytes + tpc * kRfChunk * 2) + (size_t)tpc * kRfEP * 4 + (size_t)tpc * kRfEP * 2;
+  return 1024 + (size_t)kRfBufs * (kRfWBytes + rf_x_bytes(tpc)) + (size_t)tpc * kRfEP * 4 + (size_t)tpc * kRfEP * 2;
 }
 
 // M = 128 tokens, N = 128 experts per MMA
@@ -197,7 +199,7 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 
 
 // ---- (2) candidates, exact chains, selection ----------------------------------------------------------
-// A CTA takes TPC tokens, half a warp each (a warp runs two tokens in lockstep) for everything that is per
+// A CTA takes tpc tokens, half a warp each (a warp runs two tokens in lockstep) for everything that is per
 // token: the row of approximate logits (+ bias) into shared memory; |x_t| from the row of x; the K-th largest
 // approximate logit by K rounds of a 16-lane arg-max; the threshold; the candidates.  The chains of all
 // tokens of the CTA are then numbered through and thread s runs chain s (so no lane idles because its token
@@ -207,29 +209,34 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 // token's row of x per step with two TMA copies, kRfBufs - 1 chunks ahead, and each chain reads its rows from
 // shared memory (128-byte swizzle: 16-byte unit u of row r sits at u ^ (r % 8)).  Exact values go back into
 // the logit rows; then the common selection.
-template <int TPC>
-__global__ void __launch_bounds__(TPC * 16, 1)
+// What bounds it: shared memory (ncu, T 8192, H 7168, 256 experts: its pipe 65 % busy with 5.4 wavefronts per 16-byte load
+// and another 11 % with the TMA writes; issue slots 48 %).  Whole router call, us, before / after the numbering by e % 8,
+// CTAs of any even token count (T 8192: 147 CTAs of 56 tokens instead of 128 of 64) and x asked for ahead: T 2048 113 /
+// 108, T 4096 147 / 131, T 6000 262 / 176, T 8192 258 / 225, T 16384 508 / 438; Zipf bias T 8192 249 / 243.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT * 16, 1)
 route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                     const __nv_bfloat16* __restrict__ x, const float* __restrict__ bias, const float* __restrict__ logits,
-                    const float* __restrict__ wnorm2, int T, int H, int E, int K, int renorm, int* __restrict__ topk_idx,
+                    const float* __restrict__ wnorm2, int tpc, int T, int H, int E, int K, int renorm, int* __restrict__ topk_idx,
                     float* __restrict__ topk_w, const PrepArgs prep, int tp, unsigned long long wait_ns,
                     int* __restrict__ status) {
-  constexpr int NT = TPC * 16;
-  constexpr int kXBytes = TPC * kRfChunk * 2;
+  const int NT = tpc * 16;
+  const int kXBytes = rf_x_bytes(tpc);
   __shared__ int s_hist[kRouteMaxExperts];
-  __shared__ int s_ncand[TPC];
-  __shared__ float s_eps[TPC];
+  __shared__ unsigned char s_ncand[MAXT][8];  // a token's candidates per bucket (expert % 8)
+  __shared__ int s_total[8];
+  __shared__ float s_eps[MAXT];
   __shared__ unsigned long long s_full[kRfBufs];
   __shared__ unsigned long long s_empty[kRfBufs];  // a buffer may be refilled once every warp has left it
   __shared__ int s_abort;
   extern __shared__ uint8_t rf_dyn[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(rf_dyn) + 1023) & ~(uintptr_t)1023);
   uint8_t* w_stage = base;                                              // [kRfBufs][256 experts][128 bytes]
-  uint8_t* x_stage = base + (size_t)kRfBufs * kRfWBytes;                // [kRfBufs][TPC tokens][128 bytes]
-  float* ls = reinterpret_cast<float*>(x_stage + (size_t)kRfBufs * kXBytes);  // [TPC][256] logits: approximate, exact where a chain ran
-  unsigned short* chains = reinterpret_cast<unsigned short*>(ls + (size_t)TPC * kRfEP);  // [TPC * 256]: token << 8 | expert
-  const int t0 = blockIdx.x * TPC;
-  const int tvalid = min(TPC, T - t0);
+  uint8_t* x_stage = base + (size_t)kRfBufs * kRfWBytes;                // [kRfBufs][tpc tokens][128 bytes]
+  float* ls = reinterpret_cast<float*>(x_stage + (size_t)kRfBufs * kXBytes);  // [tpc][256] logits: approximate, exact where a chain ran
+  unsigned short* chains = reinterpret_cast<unsigned short*>(ls + (size_t)tpc * kRfEP);  // [tpc * 256]: token << 8 | expert; 0xffff: none
+  const int t0 = blockIdx.x * tpc;
+  const int tvalid = min(tpc, T - t0);
   const int lane = threadIdx.x % 32, l16 = threadIdx.x % 16, half = lane / 16;
   const int tl = threadIdx.x / 16;  // this half-warp's token inside the block
   const bool live = tl < tvalid;
@@ -263,6 +270,7 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   float xn2 = 0.0f, wm2 = 0.0f;
   if (live) {
     const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)(t0 + tl) * H);
+#pragma unroll 8
     for (int q = l16; q < H / 8; q += 16) {
       float f[8];
       Vec16<__nv_bfloat16>::unpack(__ldg(xr + q), f);
@@ -321,9 +329,11 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
       return;
     }
     const uint32_t bar = smem_u32(&s_full[b]);
-    mbar_expect_tx(bar, (uint32_t)(kRfWBytes + kXBytes));
+    mbar_expect_tx(bar, (uint32_t)(kRfWBytes + tpc * kRfChunk * 2));
     tma_load_2d(smem_u32(w_stage + (size_t)b * kRfWBytes), &map_w, bar, ch * kRfChunk, 0);   // rows past E, columns past H: zeros
     tma_load_2d(smem_u32(x_stage + (size_t)b * kXBytes), &map_x, bar, ch * kRfChunk, t0);    // rows past T: zeros
+    if (ch + kRfAhead < nchunk)  // x comes from HBM (Wr stays in L2): ask for it well before its turn
+      asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(&map_x), "r"((ch + kRfAhead) * kRfChunk), "r"(t0) : "memory");
     ++issued;
   };
   // candidates of the first round, while the approximate logits are still in registers (later rounds, which are
@@ -349,40 +359,59 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
         }
       }
     }
-    int n_cand = __popc(cand);
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) n_cand += __shfl_xor_sync(0xffffffffu, n_cand, off);
-    if (l16 == 0) s_ncand[tl] = n_cand;
+    // The CTA's chains are numbered so that lane l of a warp gets an expert with e % 8 == l % 8: the eight lanes that
+    // read shared memory together then read eight different 16-byte units whatever their rows are (numbered token by
+    // token, their units met in a bank two and a half times on average).  Chain number i of bucket b is slot 8 i + b; a
+    // bucket is in token order, so neighbouring lanes also read (nearly) the same token's row.  What a bucket has beyond
+    // an eighth of the chains (popular experts) takes the slots that other buckets leave free.
+    const int bucket = l16 & 7;  // of all of this lane's experts l16 + 16 j
+    const int mine = __popc(cand), other = __shfl_xor_sync(0xffffffffu, mine, 8);  // lanes l16 and l16 ^ 8 share a bucket
+    if (l16 < 8) s_ncand[tl][bucket] = (unsigned char)(mine + other);
     __syncthreads();
-    int first = 0, total = 0;
-    for (int i = 0; i < TPC; ++i) {
-      const int n = s_ncand[i];
+    int first = l16 < 8 ? 0 : other, in_bucket = 0;
+    for (int i = 0; i < tpc; ++i) {
+      const int n = s_ncand[i][bucket];
       if (i < tl) first += n;
-      total += n;
+      in_bucket += n;
     }
+    if (tl == 0 && l16 < 8) s_total[bucket] = in_bucket;
+    int total = 0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) total += __shfl_sync(0xffffffffu, in_bucket, b);
     if (total == 0) break;  // no token of the CTA asks for more (CTA-uniform)
-    {  // this token's chains: lanes in order, each lane its experts in order
-      int mine = __popc(cand), before = mine;
+    const int rows = (total + 7) / 8;
+    total = 8 * rows;
+    int over = 0;  // chains beyond `rows` in the buckets before this lane's
 #pragma unroll
-      for (int off = 1; off < 16; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, before, off, 16);
-        if (l16 >= off) before += o;
-      }
-      int pos = first + before - mine;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if ((cand >> j) & 1u) chains[pos++] = (unsigned short)((tl << 8) | (l16 + 16 * j));
-      done |= cand;
+    for (int b = 0; b < 8; ++b) {
+      const int n = __shfl_sync(0xffffffffu, in_bucket, b);
+      if (b < bucket) over += max(0, n - rows);
     }
+    for (int i = threadIdx.x; i < total; i += NT) chains[i] = 0xffff;
+    __syncthreads();
+    for (int j = 0, pos = first; j < 16; ++j) {
+      if (!((cand >> j) & 1u)) continue;
+      int slot = 8 * pos + bucket;
+      if (pos >= rows) {
+        int o = over + pos - rows;
+        for (int b = 0; b < 8; ++b) {
+          const int n = s_total[b], free = max(0, rows - n);
+          if (o < free) { slot = 8 * (n + o) + b; break; }
+          o -= free;
+        }
+      }
+      ++pos;
+      chains[slot] = (unsigned short)((tl << 8) | (l16 + 16 * j));
+    }
+    done |= cand;
     __syncthreads();
     const int passes = (total + NT - 1) / NT;
     for (int p = 0; p < passes; ++p) {
       const int sidx = p * NT + threadIdx.x;
       int e = -1, tk = 0;
-      if (sidx < total) {
-        const unsigned short c = chains[sidx];
-        e = c & 0xff;
-        tk = c >> 8;
+      if (sidx < total && chains[sidx] != 0xffff) {
+        e = chains[sidx] & 0xff;
+        tk = chains[sidx] >> 8;
       }
       // shared-memory byte offsets of the eight 16-byte units of this chain's two rows inside a buffer (swizzled)
       uint32_t wo[8], xo[8];
@@ -507,22 +536,27 @@ int launch_route_filter(moe_plan* p, const void* x, const void* wr, const float*
                        (const __nv_bfloat16*)wr, c.T, c.H, p->route_E, p->s.route_logits, p->s.route_wnorm2, wait_ns,
                        p->s.status) != cudaSuccess)
     return MOE_ERR_CUDA;
-  // Tokens per CTA: every CTA streams all of Wr once, so as many tokens as still fill the GPU with CTAs.
-  static SmemAttrOnce once_b[3];
-  auto refine = [&](auto kern, int tpc) -> int {
+  // Tokens per CTA (even: a warp has two): the time is about (waves of CTAs over the SMs) x (tokens + what streaming all
+  // of Wr costs a CTA, 10 tokens' worth).
+  const int sms = p->sm_count > 0 ? p->sm_count : 148;
+  int tpc = 64;
+  long long best = 1ll << 60;
+  for (int i = 64; i >= 12; i -= 2) {  // (8 tokens per CTA measure slower than 16: T 1024 117 against 110 us)
+    const long long ctas = (c.T + i - 1) / i, cost = (ctas + sms - 1) / sms * (i + 10);
+    if (cost < best) { best = cost; tpc = i; }
+  }
+  static SmemAttrOnce once_b[2];
+  auto refine = [&](auto kern, SmemAttrOnce& attr) -> int {
     CUtensorMap mxb;  // the tokens' rows of x, one CTA's worth per box
     int r = make_map_2d(enc, &mxb, x, (uint64_t)c.T, (uint64_t)c.H, (uint32_t)tpc);
     if (r != MOE_OK) return r;
-    if (ensure_dynamic_smem(kern, rf_smem(tpc), p->device, once_b[tpc / 32]) != cudaSuccess) return MOE_ERR_CUDA;
+    if (ensure_dynamic_smem(kern, rf_smem(tpc), p->device, attr) != cudaSuccess) return MOE_ERR_CUDA;
     return launch_pdl(kern, dim3((c.T + tpc - 1) / tpc), dim3(tpc * 16), rf_smem(tpc), st, mw, mxb, (const __nv_bfloat16*)x, bias,
-                      (const float*)p->s.route_logits, (const float*)p->s.route_wnorm2, c.T, c.H, p->route_E, p->route_K,
+                      (const float*)p->s.route_logits, (const float*)p->s.route_wnorm2, tpc, c.T, c.H, p->route_E, p->route_K,
                       c.renormalize, topk_idx, topk_w, prep, p->tp, wait_ns, p->s.status) == cudaSuccess
                ? 0 : MOE_ERR_CUDA;
   };
-  const int sms = p->sm_count > 0 ? p->sm_count : 148;
-  if (c.T >= 48 * sms) rc = refine(route_refine_kernel<64>, 64);
-  else if (c.T >= 24 * sms) rc = refine(route_refine_kernel<32>, 32);
-  else rc = refine(route_refine_kernel<16>, 16);
+  rc = tpc > 32 ? refine(route_refine_kernel<64>, once_b[0]) : refine(route_refine_kernel<32>, once_b[1]);
   if (rc != 0) return rc;
   p->launches += 2;
   return 0;

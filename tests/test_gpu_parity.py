@@ -320,6 +320,31 @@ def test_pair_expert_kernel_by_default(tp, combine):
     assert torch.equal(ys[0], ys[1])
 
 
+# The refine kernel's numbering of the chains: token counts that give its CTAs 12 to 64 tokens (a whole wave on 148 SMs),
+# with every token's candidates in ONE class of experts modulo eight (its bucket overflows into the others' free slots),
+# with two classes, and with more candidates than a CTA has threads (every expert the same: all 256 are candidates).
+@pytest.mark.parametrize("T", [1300, 3000, 5500, 8000, 9500])
+@pytest.mark.parametrize("case", ["one_class", "two_classes", "all_equal"])
+def test_router_filter_chain_numbering(T, case):
+    H, E, K = 64, 256, 8
+    w = inputs.Workload("numbering", T=T, H=H, E=E, R=1, K=K, F=8, dtype=BF16, seed=29, identity_experts=True)
+    x, wr, _, *_ = Hh.oracle_inputs(w, with_experts=False)
+    bias = np.zeros(E, np.float32)
+    if case == "all_equal":
+        wr[:] = wr[0]
+    else:
+        keep = (np.arange(E) % 8 == 3) if case == "one_class" else (np.arange(E) % 4 == 1)
+        bias[~keep] = -50.0
+    ridx, rw, _ = oracle.route(x, wr, bias, K, BF16)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    idx = torch.empty((T, K), dtype=torch.int32, device="cuda")
+    tw = torch.empty((T, K), dtype=torch.float32, device="cuda")
+    plan.moe_route(Hh.to_dev(x), Hh.to_dev(wr), Hh.to_dev(bias), idx, tw)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    Hh.check_route(idx, tw, ridx, rw)
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

@@ -417,6 +417,11 @@ struct ClockProbe {
 int launch_ffn_pair(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, FfnParams prm,
                     cudaStream_t st);
 
+// A handful of tokens: plain FMAs, every SM streams weights (ffn_few.cu).
+constexpr int kFewMaxTokens = 5;
+int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
+                   const int* push_src, cudaStream_t st);
+
 // ---- tensor maps (host side) ---------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,

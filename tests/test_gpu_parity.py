@@ -345,6 +345,47 @@ def test_router_filter_chain_numbering(T, case):
     Hh.check_route(idx, tw, ridx, rw)
 
 
+# The kernel for a handful of tokens: one to five tokens (an expert with one to five rows; six go to the tensor cores),
+# H and F that end inside a lane's vectors and a warp's columns, few and many experts (more tiles than the table's first
+# 256 entries), TP shards, the push epilogue, and a call whose rows never become available.
+FEW = [
+    # (T, H, E, K, F, tp, combine)
+    (1, 1032, 8, 2, 520, 1, 0), (2, 1288, 4, 4, 776, 1, 0), (3, 1024, 2, 2, 512, 1, 1), (4, 1544, 6, 3, 1056, 2, 0),
+    (5, 1032, 5, 5, 520, 1, 1), (5, 1024, 256, 8, 512, 1, 0), (5, 1032, 128, 16, 1040, 2, 1), (6, 1032, 8, 2, 520, 1, 0),
+]
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("case", FEW, ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}_push{c[6]}")
+def test_few_tokens_kernel(case, mode):
+    T, H, E, K, F, tp, combine = case
+    w = inputs.Workload("few", T=T, H=H, E=E, R=1, K=K, F=F, dtype=BF16, zipf_s=1.2, seed=31)
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    ref = Hh.oracle_layer_for(w, x, wr, bias, wg, wu, wd)
+    plan = Hh.make_plan(w, mode, tp_shards=tp, combine_mode=combine)
+    y = torch.empty((T, H), dtype=torch.bfloat16, device="cuda")
+    plan.layer_tensor(2).fill_(float("nan"))     # rows that are not there must not reach the others
+    plan.moe_layer(*[Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)], y)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    Hh.assert_output_close(Hh.to_host_f64(y), ref["y"], BF16)
+
+
+def test_few_tokens_kernel_wait_runs_out_and_reports_it():
+    w = inputs.Workload("few_wait", T=2, H=1024, E=4, R=1, K=2, F=512, dtype=BF16, seed=31)
+    _, _, _, wg, wu, wd = Hh.oracle_inputs(w)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, wait_limit_ns=1_000_000)
+    rows = plan.P * 128
+    recv, out = (torch.zeros((rows, w.H), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    te = torch.full((plan.P,), -1, dtype=torch.int32, device="cuda")
+    te[0] = 1
+    counts, done = torch.zeros(plan.P, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    plan.moe_expert_ffn(recv, te, Hh.to_dev(wg), Hh.to_dev(wu), Hh.to_dev(wd), out, counts, done)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status()[0] == -6       # MOE_ERR_TIMEOUT; the context stays usable
+    assert torch.count_nonzero(out) == 0
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

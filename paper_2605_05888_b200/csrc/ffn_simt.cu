@@ -94,16 +94,20 @@ ffn_simt_kernel(const XT* __restrict__ A, int lda, const int* __restrict__ tile_
 // them gate, half up columns of the same f); a warp has 2 TM rows, a lane TM x TN results.  Operands stay in their
 // natural K-major rows: TMA brings 128 bytes (32 k) of every row per stage (128-byte swizzle), a lane reads 16 bytes
 // (4 k) of its TM rows and TN columns - two pipe cycles each, lanes of a warp being 2 row groups x 16 column groups -
-// for TM x TN x 4 FMAs, k ascending.  (Packed FMAs, fma.rn.f32x2 on pairs of k, halve the instructions but ran at 66
-// FMAs per clock and SM where scalar ones reach 85 in the same register-only loop.)  A lane of the first warp issues
-// the copies on the side (a warp of its own would cost the others a third of their registers); the warps wait per
-// stage on its mbarrier.  A warp whose rows a partly filled tile does not have leaves at once.
-// Measured against the plain 128 x 64 kernel above on fp32 data (both GEMMs): T 1000, H 1024, 16 experts, top-2,
-// F 2048: 1295 -> 793 us; T 256, H 128, 8 experts, top-2, F 256: 77 -> 28 us.
+// for TM x TN x 2 packed FMAs (fma.rn.f32x2 on pairs of neighbouring k: a result is the sum of its even and its odd k).
+// With scalar FMAs half of them found their accumulator in the register bank of the operand that changes (the four k of
+// a 16-byte load alternate between the banks) and ran at two thirds of the rate; an aligned pair spans both banks.  A
+// lane of the first warp issues the copies on the side (a warp of its own would cost the others a third of their
+// registers); the warps wait per stage on its mbarrier.  A warp whose rows a partly filled tile does not have leaves at
+// once.
+// Measured against the plain 128 x 64 kernel above on fp32 data: T 1000, H 1024, 16 experts, top-2,
+// F 2048: whole layer 1311 -> 735 us (801 with scalar FMAs); T 256, H 128, 8 experts, top-2, F 256: 96 -> 35 us.
 constexpr int kF32Warps = 4;
 constexpr int kF32Threads = 32 * kF32Warps;
 constexpr int kF32K = 32;  // k per stage
-constexpr int kF32Stages = 4;
+// stages and CTAs per SM: 8 x 8 results fill the registers with two CTAs, smaller tiles fit three
+template <int TM, int TN> constexpr int kF32Stages = TM * TN == 32 ? 3 : 4;
+template <int TM, int TN> constexpr int kF32Ctas = TM * TN == 64 ? 2 : 3;
 template <int TM, int TN> constexpr int kF32StageBytes = (kF32Warps * 2 * TM + 16 * TN) * kF32K * 4;
 
 struct Fp32Params {
@@ -117,21 +121,26 @@ struct Fp32Params {
   int* status;
 };
 
-__device__ __forceinline__ float4 lds_k4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-  return v;
+__device__ __forceinline__ void lds_k4(uint32_t addr, unsigned long long& lo, unsigned long long& hi) {
+  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "r"(addr));
+}
+__device__ __forceinline__ void fma_x2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float sum_x2(unsigned long long v) {
+  return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
 }
 
 template <int TM, int TN, bool SWIGLU>
-__global__ void __launch_bounds__(kF32Threads, 2)
+__global__ void __launch_bounds__(kF32Threads, kF32Ctas<TM, TN>)
 ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b1,
                 const __grid_constant__ CUtensorMap map_b2, const Fp32Params p) {
   constexpr int BM = kF32Warps * 2 * TM, BN = 16 * TN;  // rows and columns of B per CTA
   constexpr int NOUT = SWIGLU ? BN / 2 : BN;             // columns of the result per CTA
   constexpr int kA = BM * kF32K * 4, kStage = kF32StageBytes<TM, TN>;
+  constexpr int kStages = kF32Stages<TM, TN>;
   constexpr int kParts = kTileRows / BM;
-  __shared__ unsigned long long s_full[kF32Stages], s_empty[kF32Stages];
+  __shared__ unsigned long long s_full[kStages], s_empty[kStages];
   __shared__ int s_abort;
   extern __shared__ uint8_t f32_dyn[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(f32_dyn) + 1023) & ~(uintptr_t)1023);
@@ -148,7 +157,7 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   if (rows <= 0) return;
   const int live_warps = (rows + 2 * TM - 1) / (2 * TM);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kF32Stages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&s_full[s]), 1);
       mbar_init(smem_u32(&s_empty[s]), live_warps);
     }
@@ -173,16 +182,16 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       tma_load_4d(dst + kA, &map_b1, bar, kc, n0, e % p.tp, e / p.tp);
     }
     ++issued;
-    if (++fill == kF32Stages) fill = 0;
+    if (++fill == kStages) fill = 0;
   };
   if (threadIdx.x == 0)
-    for (int k = 0; k < min(kF32Stages - 1, nk); ++k) issue();
+    for (int k = 0; k < min(kStages - 1, nk); ++k) issue();
   bool failed = false;
-  float acc[TM][TN];
+  unsigned long long acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0ull;
   const int r0 = warp * 2 * TM + lane % 2, c0 = lane / 2;  // rows r0 + 2 i, columns of B c0 + 16 j
   // the swizzle's row bits: a lane's rows r0 + 2 i take four values of (row % 8), its columns c0 + 16 j only one
   uint32_t aoff[4];
@@ -201,41 +210,38 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
       if (half == 1 && issued > 0 && issued < nk) {  // the first thread: refill the stage used up in the last iteration
-        if (k > 0 && !mbar_wait(smem_u32(&s_empty[fill]), (uint32_t)((k - 1) / kF32Stages) & 1u, abort_flag, p.wait_ns)) failed = true;
+        if (k > 0 && !mbar_wait(smem_u32(&s_empty[fill]), (uint32_t)((k - 1) / kStages) & 1u, abort_flag, p.wait_ns)) failed = true;
         else issue();
       }
 #pragma unroll
       for (int uu = 0; uu < kF32K / 8; ++uu) {
         const uint32_t u = (uint32_t)(half * (kF32K / 8) + uu) << 4;
-        float4 bv[TN];
+        unsigned long long bl[TN], bh[TN];
 #pragma unroll
-        for (int j = 0; j < TN; ++j) bv[j] = lds_k4(b_base + (boff ^ u) + (uint32_t)j * 16u * 128u);
+        for (int j = 0; j < TN; ++j) lds_k4(b_base + (boff ^ u) + (uint32_t)j * 16u * 128u, bl[j], bh[j]);
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
-          const float4 av = lds_k4(a_base + (aoff[i & 3] ^ u) + (uint32_t)i * 2u * 128u);
+          unsigned long long al, ah;
+          lds_k4(a_base + (aoff[i & 3] ^ u) + (uint32_t)i * 2u * 128u, al, ah);
 #pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.x, bv[j].x, acc[i][j]);
+          for (int j = 0; j < TN; ++j) fma_x2(acc[i][j], al, bl[j]);
 #pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.y, bv[j].y, acc[i][j]);
-#pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.z, bv[j].z, acc[i][j]);
-#pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = __fmaf_rn(av.w, bv[j].w, acc[i][j]);
+          for (int j = 0; j < TN; ++j) fma_x2(acc[i][j], ah, bh[j]);
         }
       }
     }
     failed = __any_sync(0xffffffffu, failed);
     if (failed) break;
     if (lane == 0) mbar_arrive(smem_u32(&s_empty[b]));
-    if (++b == kF32Stages) { b = 0; phase ^= 1u; }
+    if (++b == kStages) { b = 0; phase ^= 1u; }
   }
   if (failed) {
     s_abort = 1;
     set_status(p.status, MOE_ERR_TIMEOUT, kWaitMbarTma);
     // no copy may still be landing when the CTA's shared memory goes away (only the first thread has issued any)
-    for (int g = max(0, issued - kF32Stages); g < issued; ++g) {
+    for (int g = max(0, issued - kStages); g < issued; ++g) {
       const unsigned long long ts = globaltimer();
-      while (!mbar_try(smem_u32(&s_full[g % kF32Stages]), (uint32_t)(g / kF32Stages) & 1u))
+      while (!mbar_try(smem_u32(&s_full[g % kStages]), (uint32_t)(g / kStages) & 1u))
         if (globaltimer() - ts > p.wait_ns + 1000000ull) break;
     }
     return;
@@ -248,8 +254,8 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     for (int j = 0; j < (SWIGLU ? TN / 2 : TN); ++j) {
       const int n = n0 + c0 + 16 * j;
       if (n >= p.N) continue;
-      float v = acc[i][j];
-      if (SWIGLU) v = v / (1.0f + expf(-v)) * acc[i][SWIGLU ? TN / 2 + j : j];
+      float v = sum_x2(acc[i][j]);
+      if (SWIGLU) v = v / (1.0f + expf(-v)) * sum_x2(acc[i][SWIGLU ? TN / 2 + j : j]);
       crow[n] = v;
     }
   }
@@ -284,7 +290,7 @@ static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const
     mb2 = mb1;
   }
   auto kern = ffn_fp32_kernel<TM, TN, SWIGLU>;
-  constexpr size_t smem = 1024 + (size_t)kF32Stages * kF32StageBytes<TM, TN>;
+  constexpr size_t smem = 1024 + (size_t)kF32Stages<TM, TN> * kF32StageBytes<TM, TN>;
   static SmemAttrOnce once;
   if (ensure_dynamic_smem(kern, smem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
   const dim3 grid((unsigned)(p->P * (kTileRows / BM)), (unsigned)((q.N + NOUT - 1) / NOUT));
@@ -309,23 +315,27 @@ static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, co
   q.wait_ns = kDefaultWaitNs;  // the waits are on this CTA's own copies: nothing a caller's limit is meant for
   q.status = p->s.status;
   const int sms = p->sm_count > 0 ? p->sm_count : 148;
-  // 8 x 8 results per lane (64 x 128 per CTA) want experts with enough rows and enough CTAs; otherwise 4 x 4 (32 x 64).
-  // Measured, us, 8 x 8 / 4 x 4: 250 rows per expert, GEMM1 of 624 CTAs 121 / 133, of 312 37 / 43, GEMM2 of 156
-  // 114 / 77; 125 rows per expert, GEMM1 of 1504 CTAs 508 / 511, GEMM2 of 376 349 / 278; 66 rows 97 / 84; 12 rows 183 / 125.
-  const long long blocks = (long long)c.T * c.K / 64 + c.E;  // 64-row blocks, about
-  const bool many_rows = (long long)c.T * c.K >= 192ll * c.E;
+  // Results per lane: 8 x 8 (64 x 128 per CTA) for experts with many rows, 4 x 8 (32 x 128) for experts with about a tile,
+  // both where that gives enough CTAs; otherwise 4 x 4 (32 x 64).  Measured, whole layer, us, 8 x 8 / 4 x 8 / 4 x 4: 500 rows
+  // per expert 357 / 382 / 383, 250 rows (H 512, F 1024) 248 / 242 / 215, 125 rows 787 / 735 / 766, 66 rows 157 / 143 / 138,
+  // 37 rows 470 / 409 / 365.
+  const long long rows = (long long)c.T * c.K, blocks = rows / 64 + c.E;  // 64-row blocks, about
+  const int shape = rows >= 192ll * c.E ? 2 : rows >= 96ll * c.E ? 1 : 0;
   mark(p, 3, st);
   q.N = c.F;
   q.Kd = c.H;
   q.C = (float*)p->s.inter;
-  if (many_rows && blocks * ((c.F + 63) / 64) >= 2 * sms) rc = launch_fp32_gemm<8, 8, true>(p, enc, recv, wg, wu, q, st);
+  const bool enough1 = blocks * ((c.F + 63) / 64) >= 2 * sms, enough2 = blocks * ((c.H + 127) / 128) >= 3 * sms / 2;
+  if (shape == 2 && enough1) rc = launch_fp32_gemm<8, 8, true>(p, enc, recv, wg, wu, q, st);
+  else if (shape == 1 && enough1) rc = launch_fp32_gemm<4, 8, true>(p, enc, recv, wg, wu, q, st);
   else rc = launch_fp32_gemm<4, 4, true>(p, enc, recv, wg, wu, q, st);
   if (rc != 0) return rc;
   mark(p, 4, st);
   q.N = c.H;
   q.Kd = c.F;
   q.C = (float*)out_rows;
-  if (many_rows && blocks * ((c.H + 127) / 128) >= 2 * sms) return launch_fp32_gemm<8, 8, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (shape == 2 && enough2) return launch_fp32_gemm<8, 8, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (shape == 1 && enough2) return launch_fp32_gemm<4, 8, false>(p, enc, p->s.inter, wd, nullptr, q, st);
   return launch_fp32_gemm<4, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
 }
 

@@ -12,11 +12,13 @@
 //      threshold; every expert at or above it is a candidate and gets its exact chain; the exact values
 //      replace the approximate ones and the usual selection runs on the row.
 //
-// Why the picks are the exact ones.  Error model: every fp32 addition, in whatever order and whether rounded
-// to nearest or truncated, is off by at most 2^-23 of a magnitude that never exceeds S = sum_h |x_h * w_eh|.
-// A sum of H products has H - 1 additions, so |l~ - exact sum| <= H * 2^-23 * S, and the chain (rounded to
-// nearest) is within H * 2^-24 * S of it: |l~ - l| <= eps = 1.5 * H * 2^-23 * S, with S <= |x_t| * max_e |w_e|
-// (Cauchy-Schwarz) computed from the data of the call.  The K experts with the largest l~ have l >= kth~ - eps
+// Why the picks are the exact ones.  Error model: every fp32 addition, whether rounded to nearest or truncated, is
+// off by at most 2^-23 of the sum of the magnitudes that have gone into it, which never exceeds S = sum_h |x_h * w_eh|.
+// An MMA adds 16 products to an accumulator: 17 additions, in whatever order; an accumulator takes at most
+// n = 4 * ceil(H / 256) MMAs, and the four meet in 3 more additions.  Over the accumulators' shares of S that is
+// |l~ - exact sum| <= (17 n + 3) * 2^-23 * S, and the chain (rounded to nearest) is within H * 2^-24 * S of the exact
+// sum: |l~ - l| <= eps = (H / 2 + 17 n + 3) * 2^-23 * S, with S <= |x_t| * max_e |w_e| (Cauchy-Schwarz) computed from
+// the data of the call.  The K experts with the largest l~ have l >= kth~ - eps
 // and every expert below the threshold kth~ - 2 eps has l < kth~ - eps, so none of those can be among the K
 // largest l, ties included.  The kernel checks the model on every candidate (both values are at hand) and
 // reports MOE_ERR_INTERNAL if |l~ - l| ever exceeded eps.
@@ -30,7 +32,7 @@
 namespace moehub {
 
 constexpr int kRfEP = 256;           // experts covered (the accumulator's columns)
-constexpr float kRfEps = 1.5f * 1.1920929e-7f;  // 1.5 * 2^-23
+constexpr float kRfUlp = 1.1920929e-7f;  // 2^-23
 constexpr int kRfChunk = 64;         // h per staged chunk: 128 bytes of a row
 constexpr int kRfBufs = 3;           // staged chunks in flight
 constexpr int kRfAhead = 8;          // chunks of x asked for ahead of that, into L2
@@ -211,8 +213,9 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 // the logit rows; then the common selection.
 // What bounds it: shared memory (ncu, T 8192, H 7168, 256 experts: its pipe 65 % busy with 5.4 wavefronts per 16-byte load
 // and another 11 % with the TMA writes; issue slots 48 %).  Whole router call, us, before / after the numbering by e % 8,
-// CTAs of any even token count (T 8192: 147 CTAs of 56 tokens instead of 128 of 64) and x asked for ahead: T 2048 113 /
-// 108, T 4096 147 / 131, T 6000 262 / 176, T 8192 258 / 225, T 16384 508 / 438; Zipf bias T 8192 249 / 243.
+// CTAs of any even token count (T 8192: 147 CTAs of 56 tokens instead of 128 of 64) and x asked for ahead / with the
+// error bound counted per MMA (before: H * 2^-23 * S for the approximate logit too, half a candidate more per token): T 2048
+// 113 / 108 / 107, T 4096 147 / 131 / 130, T 6000 262 / 176 / 169, T 8192 258 / 225 / 213, T 16384 508 / 438 / 414.
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT * 16, 1)
 route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
@@ -310,7 +313,7 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   // (plus a sliver) below the K-th largest approximate logit - half the window the proof needs, so about ten
   // candidates instead of twelve and hardly ever more than sixteen.  The missing half is made up afterwards with
   // the exact values: see the end of the round.
-  const float eps = kRfEps * (float)H * sqrtf(xn2 * wm2) * 1.0001f + 4.0e-7f * (1.0f + fabsf(kth));
+  const float eps = kRfUlp * (0.5f * (float)H + 68.0f * (float)((H + 255) / 256) + 3.0f) * sqrtf(xn2 * wm2) * 1.0001f + 4.0e-7f * (1.0f + fabsf(kth));
   if (l16 == 0) s_eps[tl] = eps;
   float thr = kth - eps - 1.0e-3f * (1.0f + fabsf(kth));
   unsigned done = 0;  // bit j: the chain of expert l16 + 16 j has been run

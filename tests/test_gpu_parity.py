@@ -351,7 +351,8 @@ def test_router_filter_chain_numbering(T, case):
 FEW = [
     # (T, H, E, K, F, tp, combine)
     (1, 1032, 8, 2, 520, 1, 0), (2, 1288, 4, 4, 776, 1, 0), (3, 1024, 2, 2, 512, 1, 1), (4, 1544, 6, 3, 1056, 2, 0),
-    (5, 1032, 5, 5, 520, 1, 1), (5, 1024, 256, 8, 512, 1, 0), (5, 1032, 128, 16, 1040, 2, 1), (6, 1032, 8, 2, 520, 1, 0),
+    (5, 1032, 5, 5, 520, 1, 1), (5, 1024, 256, 8, 512, 1, 0), (5, 1032, 128, 16, 1040, 2, 1), (6, 1032, 8, 2, 520, 1, 0), (1, 256, 8, 2, 256, 1, 0),
+    (4, 264, 40, 6, 264, 1, 1),
 ]
 
 

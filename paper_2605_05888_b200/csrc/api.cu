@@ -322,7 +322,9 @@ int moe_layer(moe_plan_t* p, const void* d_x, const void* d_wr, const float* d_b
   // The router puts the dispatch's counters and tables into their start state on the side (and counts the
   // rows per expert for the ordered scheme), so no reset launch stands between it and the dispatch.
   const bool prepared = p->cfg.T > 0;
-  const PrepArgs prep = make_prep(p, s.expert_count, s.tile_expert, s.src_info, s.tile_count, s.rows_done);
+  const bool few = few_layer_applies(p);
+  const PrepArgs prep = make_prep(p, s.expert_count, s.tile_expert, s.src_info, s.tile_count, s.rows_done,
+                                  p->cfg.dispatch_mode == MOE_DISPATCH_ATOMIC_ORDERED && !few);
   auto cuda_failed = [&](int step) {
     p->cuda_error = (int)cudaGetLastError();
     p->cuda_error_step = step;
@@ -330,6 +332,12 @@ int moe_layer(moe_plan_t* p, const void* d_x, const void* d_wr, const float* d_b
   };
   if (launch_route(p, d_x, d_wr, d_bias, s.topk_idx, s.topk_w, prepared ? &prep : nullptr, st)) return cuda_failed(1);
   mark(p, 1, st);
+  if (few) {  // a handful of tokens: two more launches do the rest
+    mark(p, 2, st);
+    if (launch_few_layer(p, d_x, d_wg, d_wu, d_wd, d_y, st)) return cuda_failed(3);
+    mark(p, 6, st);
+    return MOE_OK;
+  }
   // Overlapped form: the dispatch runs inside the expert kernel's launch (ordered scheme, tensor-core kernel).
   const moe_config_t& c = p->cfg;
   const bool overlap = c.overlap != 0 && prepared && c.dispatch_mode == MOE_DISPATCH_ATOMIC_ORDERED &&

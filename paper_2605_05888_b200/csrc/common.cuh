@@ -164,7 +164,8 @@ int launch_route_filter(moe_plan* p, const void* x, const void* wr, const float*
 int launch_dispatch(moe_plan* p, const void* x, const int* topk_idx, void* recv, int* expert_count,
                     int* tile_expert, int* src_info, int* slot_of, int* tile_count, int* rows_done,
                     bool prepared, cudaStream_t st);
-PrepArgs make_prep(moe_plan* p, int* expert_count, int* tile_expert, int* src_info, int* tile_count, int* rows_done);
+// ordered: an ordered dispatch follows (it wants the rows per expert and writes some of the tables itself).
+PrepArgs make_prep(moe_plan* p, int* expert_count, int* tile_expert, int* src_info, int* tile_count, int* rows_done, bool ordered);
 // staged: rows holds assignment (t, k) at row t*K+k (push-style combine); slot_of then only tells dropped assignments.
 int launch_combine(moe_plan* p, const void* rows, const int* slot_of, const float* topk_w, void* y,
                    cudaStream_t st, bool staged = false);
@@ -178,6 +179,9 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
                   const void* wu, const void* wd, void* out_rows, const int* tile_count,
                   const int* rows_done, cudaStream_t st, const void* overlap_x = nullptr,
                   const int* overlap_idx = nullptr, const int* push_src = nullptr);
+// A handful of tokens: everything of the layer that follows the router, dispatch and combine included (ffn_few.cu).
+bool few_layer_applies(const moe_plan* p);
+int launch_few_layer(moe_plan* p, const void* x, const void* wg, const void* wu, const void* wd, void* y, cudaStream_t st);
 
 // ---- element helpers ---------------------------------------------------------------------------
 __device__ __forceinline__ float to_float(float v) { return v; }

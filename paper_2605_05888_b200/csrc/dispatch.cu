@@ -379,7 +379,7 @@ dispatch_ordered_kernel(const OrderedParams prm, int* __restrict__ hist_rw, int*
   }
 }
 
-PrepArgs make_prep(moe_plan* p, int* expert_count, int* tile_expert, int* src_info, int* tile_count, int* rows_done) {
+PrepArgs make_prep(moe_plan* p, int* expert_count, int* tile_expert, int* src_info, int* tile_count, int* rows_done, bool ordered) {
   const moe_config_t& c = p->cfg;
   const int P = (int)p->P;
   PrepArgs a = {};
@@ -390,7 +390,7 @@ PrepArgs make_prep(moe_plan* p, int* expert_count, int* tile_expert, int* src_in
   add(rows_done, 1, 0);
   add(tile_count, P, 0);
   add(p->s.gemm1_done, P + 4, 0);
-  if (c.dispatch_mode == MOE_DISPATCH_ATOMIC_ORDERED && c.T > 0) {
+  if (ordered && c.T > 0) {
     add(p->s.row_pointer, c.E, 0);  // expert_count, tile_expert and the empty slots' source info are written by the dispatch
     a.hist = p->s.hist;
   } else {  // (an empty batch in the ordered scheme launches no dispatch: its outputs get their start state here)
@@ -462,7 +462,8 @@ int launch_dispatch(moe_plan* p, const void* x, const int* topk_idx, void* recv,
   // Per-call start state (and, for the ordered scheme, the rows per expert): done by the kernel before this
   // call when `prepared`, else by one small launch here.
   if (!prepared) {
-    const PrepArgs prep = make_prep(p, expert_count, tile_expert, src_info, tile_count, rows_done);
+    const PrepArgs prep = make_prep(p, expert_count, tile_expert, src_info, tile_count, rows_done,
+                                    c.dispatch_mode == MOE_DISPATCH_ATOMIC_ORDERED);
     const long long work = max((long long)p->P * kTileRows, (long long)c.T * c.K);
     const int grid = (int)max(1ll, min((long long)4 * p->sm_count, (work + 4 * kDispThreads - 1) / (4 * kDispThreads)));
     launch_pdl(prep_count_kernel, dim3(grid), dim3(kDispThreads), 0, st, prep, topk_idx, c.T * c.K, c.K);

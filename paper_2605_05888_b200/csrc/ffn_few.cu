@@ -6,8 +6,9 @@
 // up row of it, or a row of the down matrix), reads it in 16-byte vectors, eight loads in flight per lane, and forms the
 // dot products with all of the expert's rows (at most R, which come from L1) on plain fp32 FMAs; CTAs walk the columns
 // of one tile with a stride, so the work spreads over all SMs whatever the number of experts.
-// Measured, layer time, us, before / now: one Qwen-like token 57.7 / 41.3, one Mixtral-like 209.6 / 140 (705 MB of weights:
-// 109 at the copy rate), one DeepSeek-like 187 / 152; the rule in launch_ffn_tc has more.
+// Measured, layer time, us, tensor-core kernels / this / with dispatch and combine taken in (second half of the file): one
+// Qwen-like token 57.7 / 41.3 / 31, one Mixtral-like 209.6 / 140 / 125 (705 MB of weights: 109 at the copy rate), one
+// DeepSeek-like 187 / 152 / 147; the rule in launch_ffn_tc has more.
 #include "tc_common.cuh"
 #include "route_common.cuh"
 
@@ -34,58 +35,69 @@ struct FewParams {
   int* status;
 };
 
+// One column of the result for R rows, a + off[r]: lane r returns row r's value (gate and up rows w1, w2: the activated
+// product).
+template <int R, bool SWIGLU>
+__device__ __forceinline__ float few_dots(const __nv_bfloat16* __restrict__ w1, const __nv_bfloat16* __restrict__ w2,
+                                          const __nv_bfloat16* a, const int (&off)[R], int Kd) {
+  const int lane = threadIdx.x % 32;
+  float acc1[R], acc2[SWIGLU ? R : 1];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    acc1[r] = 0.0f;
+    if (SWIGLU) acc2[r] = 0.0f;
+  }
+  for (int k0 = lane * 8; k0 < Kd; k0 += 256 * kFewUnroll) {
+    uint4 v1[kFewUnroll], v2[SWIGLU ? kFewUnroll : 1];
+#pragma unroll
+    for (int i = 0; i < kFewUnroll; ++i) {
+      const int k = k0 + 256 * i;
+      v1[i] = make_uint4(0, 0, 0, 0);
+      if (k < Kd) v1[i] = __ldcs(reinterpret_cast<const uint4*>(w1 + k));
+      if (SWIGLU) {
+        v2[i] = make_uint4(0, 0, 0, 0);
+        if (k < Kd) v2[i] = __ldcs(reinterpret_cast<const uint4*>(w2 + k));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kFewUnroll; ++i) {
+      const int k = k0 + 256 * i;
+      if (k >= Kd) break;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint4 x = *reinterpret_cast<const uint4*>(a + off[r] + k);
+        const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+        const uint32_t g[4] = {v1[i].x, v1[i].y, v1[i].z, v1[i].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc1[r] = fma_bf16_hi(xw[q], g[q], fma_bf16_lo(xw[q], g[q], acc1[r]));
+        if (SWIGLU) {
+          const uint32_t u[4] = {v2[i].x, v2[i].y, v2[i].z, v2[i].w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc2[r] = fma_bf16_hi(xw[q], u[q], fma_bf16_lo(xw[q], u[q], acc2[r]));
+        }
+      }
+    }
+  }
+  float mine = 0.0f;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float s1 = group_sum<32>(acc1[r]);
+    const float s2 = SWIGLU ? group_sum<32>(acc2[r]) : 0.0f;
+    if (lane == r) mine = SWIGLU ? silu_mul(s1, s2) : s1;
+  }
+  return mine;
+}
+
 // The columns of one tile, for at most R of its rows: those past `rows` are multiplied too (they are in the pool) and
 // not stored.
 template <int R, bool SWIGLU>
-__device__ __forceinline__ void few_columns(const FewParams& p, const __nv_bfloat16* __restrict__ a, size_t base, int tile, int rows) {
+__device__ __forceinline__ void few_columns(const FewParams& p, const __nv_bfloat16* a, size_t base, int tile, int rows) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  int off[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) off[r] = r * p.Kd;
   for (int n = blockIdx.x * kFewWarps + warp; n < p.N; n += gridDim.x * kFewWarps) {
-    const __nv_bfloat16* w1 = p.b1 + base + (size_t)n * p.ldb;
-    const __nv_bfloat16* w2 = SWIGLU ? p.b2 + base + (size_t)n * p.ldb : nullptr;
-    float acc1[R], acc2[SWIGLU ? R : 1];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      acc1[r] = 0.0f;
-      if (SWIGLU) acc2[r] = 0.0f;
-    }
-    for (int k0 = lane * 8; k0 < p.Kd; k0 += 256 * kFewUnroll) {
-      uint4 v1[kFewUnroll], v2[SWIGLU ? kFewUnroll : 1];
-#pragma unroll
-      for (int i = 0; i < kFewUnroll; ++i) {
-        const int k = k0 + 256 * i;
-        v1[i] = make_uint4(0, 0, 0, 0);
-        if (k < p.Kd) v1[i] = __ldcs(reinterpret_cast<const uint4*>(w1 + k));
-        if (SWIGLU) {
-          v2[i] = make_uint4(0, 0, 0, 0);
-          if (k < p.Kd) v2[i] = __ldcs(reinterpret_cast<const uint4*>(w2 + k));
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < kFewUnroll; ++i) {
-        const int k = k0 + 256 * i;
-        if (k >= p.Kd) break;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const uint4 x = *reinterpret_cast<const uint4*>(a + (size_t)r * p.Kd + k);
-          const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-          const uint32_t g[4] = {v1[i].x, v1[i].y, v1[i].z, v1[i].w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) acc1[r] = fma_bf16_hi(xw[q], g[q], fma_bf16_lo(xw[q], g[q], acc1[r]));
-          if (SWIGLU) {
-            const uint32_t u[4] = {v2[i].x, v2[i].y, v2[i].z, v2[i].w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc2[r] = fma_bf16_hi(xw[q], u[q], fma_bf16_lo(xw[q], u[q], acc2[r]));
-          }
-        }
-      }
-    }
-    float mine = 0.0f;  // lane r: row r
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float s1 = group_sum<32>(acc1[r]);
-      const float s2 = SWIGLU ? group_sum<32>(acc2[r]) : 0.0f;
-      if (lane == r) mine = SWIGLU ? silu_mul(s1, s2) : s1;
-    }
+    const float mine = few_dots<R, SWIGLU>(p.b1 + base + (size_t)n * p.ldb, SWIGLU ? p.b2 + base + (size_t)n * p.ldb : nullptr, a, off, p.Kd);
     if (lane < rows) {
       long long row = (long long)tile * kTileRows + lane;
       if (!SWIGLU && p.push_src != nullptr) {  // push-style combine: to the token's own position
@@ -150,13 +162,21 @@ ffn_few_kernel(const FewParams p) {
   else few_columns<R, SWIGLU>(p, a, base, tile, rows);
 }
 
-template <int R>
-static int launch_few(moe_plan* p, FewParams q, const void* recv, const void* wg, const void* wu, const void* wd, void* out,
-                      const int* push_src, cudaStream_t st) {
+static int few_tiles(const moe_plan* p) { return min(p->cfg.T * p->cfg.K, p->cfg.E); }  // at most this many are used
+static dim3 few_grid(const moe_plan* p, int columns) {  // CTAs per tile: up to eight per SM in all
+  const int sms = p->sm_count > 0 ? p->sm_count : 148, tiles = few_tiles(p);
+  return dim3(max(1, min((8 * sms + tiles - 1) / tiles, (columns + kFewWarps - 1) / kFewWarps)), tiles);
+}
+
+bool few_applies(const moe_plan* p) {
   const moe_config_t& c = p->cfg;
-  const int tiles = (int)min((long long)c.T * c.K, (long long)p->P);  // at most this many are used
-  const int sms = p->sm_count > 0 ? p->sm_count : 148;
-  const int per_tile = max(1, (8 * sms + tiles - 1) / tiles);          // CTAs per tile: up to eight per SM in all
+  return c.ffn_kernel == 0 && c.T <= kFewMaxTokens && c.H >= 256 && c.F >= 256 && c.ffn_hot_min_tiles <= 0 && c.ffn_thin_tiles >= 0 &&
+         c.ffn_split == 0 && !p->trace;
+}
+
+template <int R>
+static int launch_few_gate_up(moe_plan* p, FewParams q, const void* recv, const void* wg, const void* wu, cudaStream_t st) {
+  const moe_config_t& c = p->cfg;
   q.expert_stride = (size_t)c.F * p->tp * c.H;
   q.A = (const __nv_bfloat16*)recv;
   q.b1 = (const __nv_bfloat16*)wg;
@@ -166,22 +186,33 @@ static int launch_few(moe_plan* p, FewParams q, const void* recv, const void* wg
   q.N = c.F;
   q.Kd = c.H;
   q.C = (__nv_bfloat16*)p->s.inter;
-  q.push_src = nullptr;
-  const int g1 = min(per_tile, (c.F + kFewWarps - 1) / kFewWarps), g2 = min(per_tile, (c.H + kFewWarps - 1) / kFewWarps);
-  if (launch_pdl(ffn_few_kernel<R, true>, dim3(g1, tiles), dim3(kFewThreads), 0, st, q) != cudaSuccess) return MOE_ERR_CUDA;
-  mark(p, 4, st);
+  p->launches += 1;
+  return launch_pdl(ffn_few_kernel<R, true>, few_grid(p, c.F), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+}
+
+template <int R>
+static int launch_few_down(moe_plan* p, FewParams q, const void* wd, void* out, const int* push_src, cudaStream_t st) {
+  const moe_config_t& c = p->cfg;
+  q.expert_stride = (size_t)c.F * p->tp * c.H;
   q.A = (const __nv_bfloat16*)p->s.inter;
   q.b1 = (const __nv_bfloat16*)wd;
-  q.b2 = nullptr;
   q.shard_offset = (size_t)c.F;
   q.ldb = c.F * p->tp;
   q.N = c.H;
   q.Kd = c.F;
   q.C = (__nv_bfloat16*)out;
   q.push_src = push_src;
-  if (launch_pdl(ffn_few_kernel<R, false>, dim3(g2, tiles), dim3(kFewThreads), 0, st, q) != cudaSuccess) return MOE_ERR_CUDA;
-  p->launches += 2;
-  return 0;
+  p->launches += 1;
+  return launch_pdl(ffn_few_kernel<R, false>, few_grid(p, c.H), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+}
+
+template <int R>
+static int launch_few(moe_plan* p, const FewParams& q, const void* recv, const void* wg, const void* wu, const void* wd, void* out,
+                      const int* push_src, cudaStream_t st) {
+  int rc = launch_few_gate_up<R>(p, q, recv, wg, wu, st);
+  if (rc != 0) return rc;
+  mark(p, 4, st);
+  return launch_few_down<R>(p, q, wd, out, push_src, st);
 }
 
 int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
@@ -200,7 +231,316 @@ int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu
   if (T <= 1) return launch_few<1>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
   if (T <= 2) return launch_few<2>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
   if (T <= 4) return launch_few<4>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
-  return launch_few<8>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
+  return launch_few<kFewMaxTokens>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
+}
+
+// ---- the whole layer behind the router ----------------------------------------------------------------
+// With at most kFewMaxTokens tokens every CTA can resolve all addresses for itself from the picks: used experts in
+// ascending order, each with one tile, rows in (token, k) order.  So the dispatch has no launch of its own: the gate/up
+// kernel reads the token's row where it is, and one CTA per tile leaves the rows and the tables where a dispatch would
+// have put them.  The down kernel's CTAs hold a column for every used tile, so they also form the combined output.
+// Each kernel costs about 4 us of launch, ramp and drain whatever it does: three instead of five.
+// Measured, layer time, us, five launches / this: H 512, F 512, 32 experts, K 4: one token 20.8 / 14.0, five 29.8 / 23.0;
+// H 1024, F 1024, 64 experts, K 8: 36.1 / 24.9, 65.5 / 59.7; Qwen-like: 42.5 / 30.9, 84.2 / 73.1; H 256, F 256: 19.8 / 14.0.
+constexpr long long kFewDownBytes = 64ll << 20;
+constexpr int kFewAssign = kFewMaxTokens * 32;  // most assignments (token, k)
+
+struct FewLayerParams {
+  const __nv_bfloat16* x;  // [T, H]
+  const __nv_bfloat16* w1; // gate rows, or the down matrix
+  const __nv_bfloat16* w2; // up rows
+  size_t expert_stride, shard_offset;
+  int tp, ldb;
+  int T, H, K, E, F;
+  int tile_step;           // tiles per expert of the static regions; 0: the used experts' tiles follow one another
+  const int* topk_idx;     // [T, K]
+  const float* topk_w;     // [T, K]
+  __nv_bfloat16* inter;    // [P * 128, F]
+  __nv_bfloat16* out;      // [P * 128, H], or the staging rows of the push-style combine
+  int push;
+  __nv_bfloat16* y;        // [T, H]
+  __nv_bfloat16* recv;     // what a dispatch leaves behind
+  int *expert_count, *tile_expert, *src_info, *slot_of, *tile_count, *rows_done;
+  int* status;
+};
+
+struct FewPicks {
+  int idx[kFewAssign];     // the picked expert per assignment, -1: none
+  int used[kMaxExperts];   // the used experts, ascending
+  int mark[kMaxExperts];
+  int warp_used[kFewWarps];
+};
+
+// Every thread of the CTA calls; returns the number of used experts.
+__device__ __forceinline__ int few_picks(const FewLayerParams& p, FewPicks& s) {
+  static_assert(kMaxExperts == kFewThreads, "a thread per expert");
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  s.mark[tid] = 0;
+  __syncthreads();
+  if (tid < p.T * p.K) {
+    int e = __ldcg(p.topk_idx + tid);  // (may run before the wait on the previous kernel: from L2)
+    if (e < 0 || e >= p.E) e = -1;
+    s.idx[tid] = e;
+    if (e >= 0) s.mark[e] = 1;
+  }
+  __syncthreads();
+  const bool mine = s.mark[tid] != 0;
+  const unsigned b = __ballot_sync(0xffffffffu, mine);
+  if (lane == 0) s.warp_used[warp] = __popc(b);
+  __syncthreads();
+  int before = 0, n = 0;
+#pragma unroll
+  for (int w = 0; w < kFewWarps; ++w) {
+    if (w < warp) before += s.warp_used[w];
+    n += s.warp_used[w];
+  }
+  if (mine) s.used[before + __popc(b & ((1u << lane) - 1u))] = tid;
+  __syncthreads();
+  return n;
+}
+
+// A warp lists the assignments of expert e in ascending order, at most kFewMaxTokens of them (an expert is picked at
+// most once per token); returns how many.
+__device__ __forceinline__ int few_rows(const FewLayerParams& p, const FewPicks& s, int e, int* list) {
+  const int lane = threadIdx.x % 32;
+  int n = 0;
+  __syncwarp();
+  for (int base = 0; base < p.T * p.K; base += 32) {
+    const bool hit = base + lane < p.T * p.K && s.idx[base + lane] == e;
+    const unsigned b = __ballot_sync(0xffffffffu, hit);
+    const int at = n + __popc(b & ((1u << lane) - 1u));
+    if (hit && at < kFewMaxTokens) list[at] = base + lane;
+    n += __popc(b);
+  }
+  __syncwarp();
+  return min(n, kFewMaxTokens);
+}
+
+template <int R>
+__device__ __forceinline__ void few_gate_up(const FewLayerParams& p, size_t base, int tile, const int* list, int rows) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  int off[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) off[r] = list[r < rows ? r : 0] / p.K * p.H;
+  for (int n = blockIdx.x * kFewWarps + warp; n < p.F; n += gridDim.x * kFewWarps) {
+    const size_t at = base + (size_t)n * p.ldb;
+    const float mine = few_dots<R, true>(p.w1 + at, p.w2 + at, p.x, off, p.H);
+    if (lane < rows) p.inter[((size_t)tile * kTileRows + lane) * p.F + n] = __float2bfloat16_rn(mine);
+  }
+}
+
+// Grid: (CTAs per tile, T * K): blockIdx.y is the used expert's number.
+template <int R>
+__global__ void __launch_bounds__(kFewThreads)
+few_gate_up_kernel(const FewLayerParams p) {
+  __shared__ FewPicks s;
+  __shared__ int s_list[kFewWarps][kFewMaxTokens];
+  pdl_wait();
+  pdl_trigger();
+  const int n_used = few_picks(p, s);
+  const int u = blockIdx.y;
+  if (u >= n_used) return;
+  const int warp = threadIdx.x / 32;
+  const int e = s.used[u], tile = p.tile_step > 0 ? e * p.tile_step : u;
+  const int* list = s_list[warp];
+  const int rows = min(few_rows(p, s, e, s_list[warp]), R);
+  if (blockIdx.x == gridDim.x - 1) {  // this tile's rows and table entries, for whoever looks at them after the layer
+    const int vec = p.H / 8;
+    for (int i = threadIdx.x; i < rows * vec; i += kFewThreads) {
+      const int r = i / vec, v = i - r * vec;
+      reinterpret_cast<uint4*>(p.recv + ((size_t)tile * kTileRows + r) * p.H)[v] =
+          reinterpret_cast<const uint4*>(p.x + (size_t)(list[r] / p.K) * p.H)[v];
+    }
+    if ((int)threadIdx.x < rows) {
+      const int slot = tile * kTileRows + threadIdx.x;
+      p.src_info[slot] = list[threadIdx.x];
+      p.slot_of[list[threadIdx.x]] = slot;
+    }
+    if (threadIdx.x == 0) {
+      p.expert_count[e] = rows;
+      p.tile_expert[tile] = e;
+      p.tile_count[tile] = rows;
+    }
+    if (u == 0)
+      for (int a = threadIdx.x; a < p.T * p.K; a += kFewThreads) {
+        if (a == 0) *p.rows_done = p.T * p.K;
+        if (s.idx[a] < 0) {  // not an expert: reported, adds nothing
+          set_status(p.status, MOE_ERR_ARG, a / p.K);
+          p.slot_of[a] = -1;
+        }
+      }
+  }
+  const size_t base = (size_t)(e / p.tp) * p.expert_stride + (size_t)(e % p.tp) * p.shard_offset;
+  if (rows == 1) few_gate_up<1>(p, base, tile, list, rows);
+  else if (R >= 2 && rows == 2) few_gate_up<(R < 2 ? R : 2)>(p, base, tile, list, rows);
+  else if (R >= 4 && rows <= 4) few_gate_up<(R < 4 ? R : 4)>(p, base, tile, list, rows);
+  else few_gate_up<R>(p, base, tile, list, rows);
+}
+
+// The first 4 KB of a weight row on their way into L2.
+__device__ __forceinline__ void few_prefetch(const __nv_bfloat16* w, int Kd) {
+  const int k = (threadIdx.x % 32) * 64;
+  if (k < Kd) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + k));
+}
+
+template <int R>
+__device__ __forceinline__ float few_down(const FewLayerParams& p, const __nv_bfloat16* w, int tile, int rows) {
+  int off[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) off[r] = (r < rows ? r : 0) * p.F;
+  return few_dots<R, false>(w, nullptr, p.inter + (size_t)tile * kTileRows * p.F, off, p.F);
+}
+
+// A CTA holds kFewWarps / S columns, a column's used tiles being dealt to S warps; the CTA then adds up each token's K
+// values in ascending k, rounded to the storage type as they are in `out`.
+template <int R, int S>
+__global__ void __launch_bounds__(kFewThreads, 3)
+few_down_kernel(const FewLayerParams p) {
+  constexpr int C = kFewWarps / S;
+  __shared__ FewPicks s;
+  __shared__ int s_list[kFewWarps][kFewMaxTokens];
+  __shared__ float s_val[C][kFewAssign];
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = warp / S, part = warp % S;
+  // The picks are the router's, complete before the gate/up kernel let this one start: they need no wait.
+  const int n_used = few_picks(p, s);
+  auto weights = [&](int e, int n) {
+    return p.w1 + (size_t)(e / p.tp) * p.expert_stride + (size_t)(e % p.tp) * p.shard_offset + (size_t)n * p.ldb;
+  };
+  if (part < n_used && (int)blockIdx.x * C + c < p.H) few_prefetch(weights(s.used[part], blockIdx.x * C + c), p.F);
+  pdl_wait();
+  pdl_trigger();
+  for (int n0 = blockIdx.x * C; n0 < p.H; n0 += gridDim.x * C) {
+    const int n = n0 + c;
+    for (int a = lane + 32 * part; a < p.T * p.K; a += 32 * S)
+      if (s.idx[a] < 0) s_val[c][a] = 0.0f;
+    for (int u = part; u < n_used && n < p.H; u += S) {
+      const int e = s.used[u], tile = p.tile_step > 0 ? e * p.tile_step : u;
+      const int rows = min(few_rows(p, s, e, s_list[warp]), R);
+      if (u + S < n_used) few_prefetch(weights(s.used[u + S], n), p.F);
+      else if (n + (int)gridDim.x * C < p.H) few_prefetch(weights(s.used[part], n + gridDim.x * C), p.F);
+      const __nv_bfloat16* w = weights(e, n);
+      float v;
+      if (rows == 1) v = few_down<1>(p, w, tile, rows);
+      else if (R >= 2 && rows == 2) v = few_down<(R < 2 ? R : 2)>(p, w, tile, rows);
+      else if (R >= 4 && rows <= 4) v = few_down<(R < 4 ? R : 4)>(p, w, tile, rows);
+      else v = few_down<R>(p, w, tile, rows);
+      if (lane < rows) {
+        const int a = s_list[warp][lane];
+        const __nv_bfloat16 b = __float2bfloat16_rn(v);
+        p.out[(p.push ? (size_t)a : (size_t)tile * kTileRows + lane) * p.H + n] = b;
+        s_val[c][a] = __bfloat162float(b);
+      }
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < p.T * C) {
+      const int t = threadIdx.x / C, cc = threadIdx.x % C;
+      if (n0 + cc < p.H) {
+        float acc = 0.0f;
+        for (int k = 0; k < p.K; ++k) acc = __fmaf_rn(p.topk_w[t * p.K + k], s_val[cc][t * p.K + k], acc);
+        p.y[(size_t)t * p.H + n0 + cc] = __float2bfloat16_rn(acc);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// The rows are read again for every column and live in L1, so the gate/up kernel asks for most of it: launched behind the
+// router while that still runs, it otherwise gets what its ring of shared memory left (Mixtral-like layer, one token:
+// 139 us without this, 128 with it; two tokens 246 and 223).
+template <typename Kern>
+static void few_prefer_l1(Kern kern, int device, SmemAttrOnce& once) {
+  if (device >= 0 && device < 64 && once.set[device]) return;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 8) != cudaSuccess) cudaGetLastError();  // a hint only
+  if (device >= 0 && device < 64) once.set[device] = 1;
+}
+
+template <int R>
+static int launch_few_layer(moe_plan* p, FewLayerParams q, const void* wd, cudaStream_t st) {
+  const moe_config_t& c = p->cfg;
+  static SmemAttrOnce once;
+  few_prefer_l1(few_gate_up_kernel<R>, p->device, once);
+  if (launch_pdl(few_gate_up_kernel<R>, few_grid(p, c.F), dim3(kFewThreads), 0, st, q) != cudaSuccess) return MOE_ERR_CUDA;
+  p->launches += 1;
+  mark(p, 4, st);
+  const int tiles = few_tiles(p);
+  // The combined form for one token, and for more while the down matrices are small: its warps wait for the slowest
+  // tile of their column, which costs more than a launch when experts have unequal row counts and long columns.  Measured,
+  // down (+ 5 us for the combine launch) / combined, us, by the down matrices' bytes: one token 23 MB 14.3 / 14.3, 235 MB
+  // 45.1 / 45.1; two or more 46 MB 18.4 / 20.4, 84 MB 24.6 / 28.7, 115 MB 34.8 / 38.9, 940 MB 129 / 188.
+  if (c.T > 1 && (long long)tiles * c.H * c.F * 2 > kFewDownBytes) {
+    FewParams d = {};
+    d.tp = p->tp;
+    d.tile_expert = q.tile_expert;
+    d.P = (int)p->P;
+    d.E = c.E;
+    d.tile_count = q.tile_count;
+    d.rows_done = q.rows_done;
+    d.total_rows = c.T * c.K;
+    d.wait_ns = kDefaultWaitNs;
+    d.status = q.status;
+    int rc = launch_few_down<R>(p, d, wd, q.out, q.push ? q.src_info : nullptr, st);
+    if (rc != 0) return rc;
+    mark(p, 5, st);
+    return launch_combine(p, q.out, q.slot_of, q.topk_w, q.y, st, q.push) ? MOE_ERR_CUDA : 0;
+  }
+  q.w1 = (const __nv_bfloat16*)wd;
+  q.w2 = nullptr;
+  q.shard_offset = (size_t)c.F;
+  q.ldb = c.F * p->tp;
+  const int sms = p->sm_count > 0 ? p->sm_count : 148;
+  const int S = tiles >= 8 ? 8 : tiles >= 4 ? 4 : tiles >= 2 ? 2 : 1;  // warps per column: as many as there are tiles for
+  const int grid = min(8 * sms, (c.H + kFewWarps / S - 1) / (kFewWarps / S));
+  auto kern = S == 1 ? few_down_kernel<R, 1> : S == 2 ? few_down_kernel<R, 2> : S == 4 ? few_down_kernel<R, 4> : few_down_kernel<R, 8>;
+  if (launch_pdl(kern, dim3(grid), dim3(kFewThreads), 0, st, q) != cudaSuccess) return MOE_ERR_CUDA;
+  p->launches += 1;
+  mark(p, 5, st);
+  return 0;
+}
+
+// Four or five tokens with very long columns keep the separate dispatch: its launch saved is nothing there, and the rows
+// taken from where the tokens are cost the gate/up kernel about 2 % (F 14336: 332 us with a dispatch, 339 without; F 6400
+// and five tokens: 230 and 219).
+bool few_layer_applies(const moe_plan* p) {
+  const moe_config_t& c = p->cfg;
+  return c.T > 0 && (c.T <= 3 || c.F <= 8192) && c.dtype == MOE_DTYPE_BF16 && !c.identity_experts && c.overlap == 0 && few_applies(p);
+}
+
+int launch_few_layer(moe_plan* p, const void* x, const void* wg, const void* wu, const void* wd, void* y, cudaStream_t st) {
+  const moe_config_t& c = p->cfg;
+  Scratch& s = p->s;
+  FewLayerParams q = {};
+  q.x = (const __nv_bfloat16*)x;
+  q.w1 = (const __nv_bfloat16*)wg;
+  q.w2 = (const __nv_bfloat16*)wu;
+  q.expert_stride = (size_t)c.F * p->tp * c.H;
+  q.shard_offset = (size_t)c.F * c.H;
+  q.tp = p->tp;
+  q.ldb = c.H;
+  q.T = c.T;
+  q.H = c.H;
+  q.K = c.K;
+  q.E = c.E;
+  q.F = c.F;
+  q.tile_step = c.dispatch_mode == MOE_DISPATCH_ATOMIC_STATIC ? (int)(p->cap_rows / kTileRows) : 0;
+  q.topk_idx = s.topk_idx;
+  q.topk_w = s.topk_w;
+  q.inter = (__nv_bfloat16*)s.inter;
+  q.out = (__nv_bfloat16*)s.out_rows;
+  q.push = c.combine_mode == 1;
+  q.y = (__nv_bfloat16*)y;
+  q.recv = (__nv_bfloat16*)s.recv;
+  q.expert_count = s.expert_count;
+  q.tile_expert = s.tile_expert;
+  q.src_info = s.src_info;
+  q.slot_of = s.slot_of;
+  q.tile_count = s.tile_count;
+  q.rows_done = s.rows_done;
+  q.status = s.status;
+  mark(p, 3, st);
+  if (c.T <= 1) return launch_few_layer<1>(p, q, wd, st);
+  if (c.T <= 2) return launch_few_layer<2>(p, q, wd, st);
+  if (c.T <= 4) return launch_few_layer<4>(p, q, wd, st);
+  return launch_few_layer<kFewMaxTokens>(p, q, wd, st);
 }
 
 }  // namespace moehub

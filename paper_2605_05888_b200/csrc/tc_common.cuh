@@ -419,6 +419,7 @@ int launch_ffn_pair(moe_plan* p, const void* recv, const void* wg, const void* w
 
 // A handful of tokens: plain FMAs, every SM streams weights (ffn_few.cu).
 constexpr int kFewMaxTokens = 5;
+bool few_applies(const moe_plan* p);
 int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
                    const int* push_src, cudaStream_t st);
 

@@ -352,7 +352,7 @@ FEW = [
     # (T, H, E, K, F, tp, combine)
     (1, 1032, 8, 2, 520, 1, 0), (2, 1288, 4, 4, 776, 1, 0), (3, 1024, 2, 2, 512, 1, 1), (4, 1544, 6, 3, 1056, 2, 0),
     (5, 1032, 5, 5, 520, 1, 1), (5, 1024, 256, 8, 512, 1, 0), (5, 1032, 128, 16, 1040, 2, 1), (6, 1032, 8, 2, 520, 1, 0), (1, 256, 8, 2, 256, 1, 0),
-    (4, 264, 40, 6, 264, 1, 1),
+    (4, 264, 40, 6, 264, 1, 1), (3, 4096, 4, 2, 2064, 1, 0), (2, 2048, 24, 4, 2064, 1, 1), (1, 2048, 16, 16, 1040, 1, 0),
 ]
 
 
@@ -370,6 +370,46 @@ def test_few_tokens_kernel(case, mode):
     torch.cuda.synchronize()
     assert plan.moe_last_status() == (0, 0)
     Hh.assert_output_close(Hh.to_host_f64(y), ref["y"], BF16)
+
+
+# Up to five tokens the layer resolves the addresses and combines inside the two expert kernels: the tables it leaves are
+# a dispatch's, and the result is, byte for byte, that of the steps called one after the other.
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("case", [c for c in FEW if c[0] <= 5], ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}_push{c[6]}")
+def test_few_tokens_layer_equals_its_steps(case, mode):
+    T, H, E, K, F, tp, combine = case
+    w = inputs.Workload("few", T=T, H=H, E=E, R=1, K=K, F=F, dtype=BF16, zipf_s=1.2, seed=32)
+    x, wr, bias, wg, wu, wd = (Hh.to_dev(a) for a in Hh.oracle_inputs(w))
+    plan = Hh.make_plan(w, mode, tp_shards=tp, combine_mode=combine)
+    y, y2 = (torch.full((T, H), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    for i in range(9):
+        if i not in (8, 9):
+            plan.layer_tensor(i).zero_()
+    plan.moe_layer(x, wr, bias, wg, wu, wd, y)
+    down = 1 if T == 1 or min(T * K * tp, E * tp) * H * (F // tp) * 2 <= 64 << 20 else 2  # combined, or with a combine behind it
+    assert plan.moe_last_launch_count() == (1 if E <= 64 else 2) + 1 + down
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    left = [plan.layer_tensor(i).clone() for i in range(8)]
+    idx, tw, recv, cnt, te, src, slot, rows = left
+    recv2, rows2 = torch.zeros_like(recv), torch.zeros_like(rows)
+    cnt2, te2, src2, slot2 = (torch.empty_like(a) for a in (cnt, te, src, slot))
+    tiles, done = torch.empty(plan.P, dtype=torch.int32, device="cuda"), torch.empty(1, dtype=torch.int32, device="cuda")
+    plan.moe_dispatch(x, idx, recv2, cnt2, te2, src2, slot2, tiles, done)
+    if combine:
+        plan.moe_expert_ffn_push(recv2, te2, src2, wg, wu, wd, rows2, tiles, done)
+        plan.moe_combine_staged(rows2, slot2, tw, y2)
+    else:
+        plan.moe_expert_ffn(recv2, te2, wg, wu, wd, rows2, tiles, done)
+        plan.moe_combine(rows2, slot2, tw, y2)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    assert torch.equal(y, y2) and torch.equal(cnt, cnt2)
+    flat, s, s2 = torch.arange(idx.numel(), device="cuda", dtype=torch.int32), slot.flatten().long(), slot2.flatten().long()
+    assert torch.equal(src[s], flat) and int((src >= 0).sum()) == flat.numel()
+    assert torch.equal(te[s // 128], idx.flatten()) and int((te >= 0).sum()) == int((cnt > 0).sum())
+    assert torch.equal(recv[s], recv2[s2])
+    assert torch.equal(rows, rows2) if combine else torch.equal(rows[s], rows2[s2])
 
 
 def test_few_tokens_kernel_wait_runs_out_and_reports_it():

@@ -82,7 +82,7 @@ typedef struct {
   int32_t ffn_kernel;           /* 0: tensor-core (tcgen05) kernel for bf16 - one CTA per tile, or
                                    CTA pairs (cta_group::2, two tiles of an expert per item)
                                    where experts have more than one tile of rows on average, or
-                                   plain FMAs for up to five tokens - and the fp32-FMA kernel for fp32; 1: plain SIMT fp32-FMA
+                                   plain FMAs for up to five tokens (small layers: 32) - and the fp32-FMA kernel for fp32; 1: plain SIMT fp32-FMA
                                    kernel for bf16 (check path); 2: always CTA pairs (bf16)   */
   int32_t ffn_split;            /* 1: one launch per expert GEMM; 2: both GEMMs in one persistent
                                    launch (per-tile status counters gate GEMM2); 0: choose

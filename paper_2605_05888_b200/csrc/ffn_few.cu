@@ -1,4 +1,5 @@
-// Step 3 of the MoE layer (paper Section II-A, expert computation) for a handful of tokens in bf16: decoding.
+// Step 3 of the MoE layer (paper Section II-A, expert computation) for a handful of tokens in bf16 (decoding), and for
+// small layers of some tens of tokens.
 //
 // Bound by reading the picked experts' weights once.  The tensor-core kernels hand out blocks of 128 or 256 weight rows
 // per CTA, which leaves most SMs without work when few experts have rows (one Qwen-like token: 44 blocks for 148 SMs,
@@ -16,6 +17,7 @@ namespace moehub {
 
 constexpr int kFewThreads = 256;
 constexpr int kFewWarps = kFewThreads / 32;
+constexpr int kFewAssign = 256;  // most assignments (token, k): a thread per assignment
 constexpr int kFewUnroll = 4;  // 16-byte vectors per lane, matrix and pass
 
 struct FewParams {
@@ -88,10 +90,11 @@ __device__ __forceinline__ float few_dots(const __nv_bfloat16* __restrict__ w1, 
   return mine;
 }
 
-// The columns of one tile, for at most R of its rows: those past `rows` are multiplied too (they are in the pool) and
-// not stored.
+// The columns of one tile, for `rows` (at most R) of its rows from r0 on: those past them are multiplied too (the tile
+// has them) and not stored.
 template <int R, bool SWIGLU>
-__device__ __forceinline__ void few_columns(const FewParams& p, const __nv_bfloat16* a, size_t base, int tile, int rows) {
+__device__ __forceinline__ void few_columns(const FewParams& p, size_t base, int tile, int r0, int rows) {
+  const __nv_bfloat16* a = p.A + ((size_t)tile * kTileRows + r0) * p.Kd;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   int off[R];
 #pragma unroll
@@ -99,7 +102,7 @@ __device__ __forceinline__ void few_columns(const FewParams& p, const __nv_bfloa
   for (int n = blockIdx.x * kFewWarps + warp; n < p.N; n += gridDim.x * kFewWarps) {
     const float mine = few_dots<R, SWIGLU>(p.b1 + base + (size_t)n * p.ldb, SWIGLU ? p.b2 + base + (size_t)n * p.ldb : nullptr, a, off, p.Kd);
     if (lane < rows) {
-      long long row = (long long)tile * kTileRows + lane;
+      long long row = (long long)tile * kTileRows + r0 + lane;
       if (!SWIGLU && p.push_src != nullptr) {  // push-style combine: to the token's own position
         row = __ldcg(p.push_src + row);
         if (row >= p.total_rows) row = -1;
@@ -148,29 +151,43 @@ ffn_few_kernel(const FewParams p) {
       }
       __nanosleep(64);
     }
-    s_rows = ready ? min(R, p.tile_count[tile]) : 0;
+    s_rows = ready ? min(kTileRows, p.tile_count[tile]) : 0;
   }
   __syncthreads();
   const int rows = s_rows;
   if (rows <= 0) return;
   const int e = p.tile_expert[tile];
   const size_t base = (size_t)(e / p.tp) * p.expert_stride + (size_t)(e % p.tp) * p.shard_offset;
-  const __nv_bfloat16* a = p.A + (size_t)tile * kTileRows * p.Kd;
-  if (rows == 1) few_columns<1, SWIGLU>(p, a, base, tile, rows);
-  else if (R >= 2 && rows == 2) few_columns<(R < 2 ? R : 2), SWIGLU>(p, a, base, tile, rows);
-  else if (R >= 4 && rows <= 4) few_columns<(R < 4 ? R : 4), SWIGLU>(p, a, base, tile, rows);
-  else few_columns<R, SWIGLU>(p, a, base, tile, rows);
+  if (rows == 1) few_columns<1, SWIGLU>(p, base, tile, 0, rows);
+  else if (R >= 2 && rows == 2) few_columns<(R < 2 ? R : 2), SWIGLU>(p, base, tile, 0, rows);
+  else if (R >= 4 && rows <= 4) few_columns<(R < 4 ? R : 4), SWIGLU>(p, base, tile, 0, rows);
+  else few_columns<R, SWIGLU>(p, base, tile, 0, min(rows, R));
+  for (int r0 = R; r0 < rows;) {  // more rows than tokens: a caller's routing that names an expert twice for a token
+    const int n = R < 8 || rows - r0 < 8 ? 1 : 8;  // (or more than 8 tokens)
+    if (n == 1) few_columns<1, SWIGLU>(p, base, tile, r0, 1);
+    else few_columns<(R < 8 ? 1 : 8), SWIGLU>(p, base, tile, r0, 8);
+    r0 += n;
+  }
 }
 
-static int few_tiles(const moe_plan* p) { return min(p->cfg.T * p->cfg.K, p->cfg.E); }  // at most this many are used
-static dim3 few_grid(const moe_plan* p, int columns) {  // CTAs per tile: up to eight per SM in all
-  const int sms = p->sm_count > 0 ? p->sm_count : 148, tiles = few_tiles(p);
+static dim3 few_grid(const moe_plan* p, int tiles, int columns) {  // CTAs per tile: up to eight per SM in all
+  const int sms = p->sm_count > 0 ? p->sm_count : 148;
   return dim3(max(1, min((8 * sms + tiles - 1) / tiles, (columns + kFewWarps - 1) / kFewWarps)), tiles);
 }
 
+// Up to five tokens: measured, layer time tensor cores / plain FMAs (four and five launches, without what the second half
+// of the file saves): one token 1.23 (256 experts of 88 MB) to 1.81 (32 of 6 MB), five 1.03-1.21, six 0.93-1.22, eight
+// 0.92-1.11 (an expert's rows share a weight's load but not its FMAs).
+// More tokens while the layer is so small that launches and latencies are what it costs, by the number of dot products;
+// measured, layer time, us, tensor cores / plain FMAs with three launches: H 256, F 256, K 2: T 8 28.8 / 13.3, T 32 28.8 /
+// 16.8 (49 thousand); H 512, F 512, K 2: T 16 32.9 / 23.6 (49), T 32 32.9 / 30.0 (98); H 1024, F 512, K 2: T 16 39.1 / 29.6
+// (66), T 32 39.1 / 39.3 (131); H 512, F 512, K 4, 32 experts: T 8 35.0 / 30.0 (49), T 12 35.5 / 36.3 (74); H 512, F 256, K 8,
+// 64 experts: T 8 41.2 / 37.1 (66), T 12 40.8 / 46.5 (98).
+constexpr long long kFewDots = 65536;
 bool few_applies(const moe_plan* p) {
   const moe_config_t& c = p->cfg;
-  return c.ffn_kernel == 0 && c.T <= kFewMaxTokens && c.H >= 256 && c.F >= 256 && c.ffn_hot_min_tiles <= 0 && c.ffn_thin_tiles >= 0 &&
+  const long long dots = (long long)c.T * c.K * (c.H + 2ll * c.F);
+  return c.ffn_kernel == 0 && (c.T <= 5 || (c.T <= kFewMaxTokens && c.T * c.K <= kFewAssign && dots <= kFewDots)) && c.H >= 256 && c.F >= 256 && c.ffn_hot_min_tiles <= 0 && c.ffn_thin_tiles >= 0 &&
          c.ffn_split == 0 && !p->trace;
 }
 
@@ -187,7 +204,7 @@ static int launch_few_gate_up(moe_plan* p, FewParams q, const void* recv, const 
   q.Kd = c.H;
   q.C = (__nv_bfloat16*)p->s.inter;
   p->launches += 1;
-  return launch_pdl(ffn_few_kernel<R, true>, few_grid(p, c.F), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+  return launch_pdl(ffn_few_kernel<R, true>, few_grid(p, (int)min((long long)c.T * c.K, (long long)p->P), c.F), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
 }
 
 template <int R>
@@ -203,7 +220,7 @@ static int launch_few_down(moe_plan* p, FewParams q, const void* wd, void* out, 
   q.C = (__nv_bfloat16*)out;
   q.push_src = push_src;
   p->launches += 1;
-  return launch_pdl(ffn_few_kernel<R, false>, few_grid(p, c.H), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+  return launch_pdl(ffn_few_kernel<R, false>, few_grid(p, (int)min((long long)c.T * c.K, (long long)p->P), c.H), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
 }
 
 template <int R>
@@ -231,11 +248,12 @@ int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu
   if (T <= 1) return launch_few<1>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
   if (T <= 2) return launch_few<2>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
   if (T <= 4) return launch_few<4>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
-  return launch_few<kFewMaxTokens>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
+  if (T <= 5) return launch_few<5>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
+  return launch_few<8>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
 }
 
 // ---- the whole layer behind the router ----------------------------------------------------------------
-// With at most kFewMaxTokens tokens every CTA can resolve all addresses for itself from the picks: used experts in
+// With so few tokens every CTA can resolve all addresses for itself from the picks: used experts in
 // ascending order, each with one tile, rows in (token, k) order.  So the dispatch has no launch of its own: the gate/up
 // kernel reads the token's row where it is, and one CTA per tile leaves the rows and the tables where a dispatch would
 // have put them.  The down kernel's CTAs hold a column for every used tile, so they also form the combined output.
@@ -243,7 +261,6 @@ int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu
 // Measured, layer time, us, five launches / this: H 512, F 512, 32 experts, K 4: one token 20.8 / 14.0, five 29.8 / 23.0;
 // H 1024, F 1024, 64 experts, K 8: 36.1 / 24.9, 65.5 / 59.7; Qwen-like: 42.5 / 30.9, 84.2 / 73.1; H 256, F 256: 19.8 / 14.0.
 constexpr long long kFewDownBytes = 64ll << 20;
-constexpr int kFewAssign = kFewMaxTokens * 32;  // most assignments (token, k)
 
 struct FewLayerParams {
   const __nv_bfloat16* x;  // [T, H]
@@ -273,7 +290,7 @@ struct FewPicks {
 
 // Every thread of the CTA calls; returns the number of used experts.
 __device__ __forceinline__ int few_picks(const FewLayerParams& p, FewPicks& s) {
-  static_assert(kMaxExperts == kFewThreads, "a thread per expert");
+  static_assert(kMaxExperts == kFewThreads && kFewAssign <= kFewThreads, "a thread per expert, a thread per assignment");
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   s.mark[tid] = 0;
   __syncthreads();
@@ -316,8 +333,9 @@ __device__ __forceinline__ int few_rows(const FewLayerParams& p, const FewPicks&
   return min(n, kFewMaxTokens);
 }
 
+// The columns of one tile, for the `rows` (at most R) assignments listed, its rows from r0 on.
 template <int R>
-__device__ __forceinline__ void few_gate_up(const FewLayerParams& p, size_t base, int tile, const int* list, int rows) {
+__device__ __forceinline__ void few_gate_up(const FewLayerParams& p, size_t base, int tile, int r0, const int* list, int rows) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   int off[R];
 #pragma unroll
@@ -325,7 +343,7 @@ __device__ __forceinline__ void few_gate_up(const FewLayerParams& p, size_t base
   for (int n = blockIdx.x * kFewWarps + warp; n < p.F; n += gridDim.x * kFewWarps) {
     const size_t at = base + (size_t)n * p.ldb;
     const float mine = few_dots<R, true>(p.w1 + at, p.w2 + at, p.x, off, p.H);
-    if (lane < rows) p.inter[((size_t)tile * kTileRows + lane) * p.F + n] = __float2bfloat16_rn(mine);
+    if (lane < rows) p.inter[((size_t)tile * kTileRows + r0 + lane) * p.F + n] = __float2bfloat16_rn(mine);
   }
 }
 
@@ -343,7 +361,7 @@ few_gate_up_kernel(const FewLayerParams p) {
   const int warp = threadIdx.x / 32;
   const int e = s.used[u], tile = p.tile_step > 0 ? e * p.tile_step : u;
   const int* list = s_list[warp];
-  const int rows = min(few_rows(p, s, e, s_list[warp]), R);
+  const int rows = few_rows(p, s, e, s_list[warp]);
   if (blockIdx.x == gridDim.x - 1) {  // this tile's rows and table entries, for whoever looks at them after the layer
     const int vec = p.H / 8;
     for (int i = threadIdx.x; i < rows * vec; i += kFewThreads) {
@@ -371,10 +389,14 @@ few_gate_up_kernel(const FewLayerParams p) {
       }
   }
   const size_t base = (size_t)(e / p.tp) * p.expert_stride + (size_t)(e % p.tp) * p.shard_offset;
-  if (rows == 1) few_gate_up<1>(p, base, tile, list, rows);
-  else if (R >= 2 && rows == 2) few_gate_up<(R < 2 ? R : 2)>(p, base, tile, list, rows);
-  else if (R >= 4 && rows <= 4) few_gate_up<(R < 4 ? R : 4)>(p, base, tile, list, rows);
-  else few_gate_up<R>(p, base, tile, list, rows);
+  for (int r0 = 0; r0 < rows; r0 += R) {
+    const int n = min(R, rows - r0);
+    if (n == 1) few_gate_up<1>(p, base, tile, r0, list + r0, n);
+    else if (R >= 2 && n == 2) few_gate_up<(R < 2 ? R : 2)>(p, base, tile, r0, list + r0, n);
+    else if (R >= 4 && n <= 4) few_gate_up<(R < 4 ? R : 4)>(p, base, tile, r0, list + r0, n);
+    else few_gate_up<R>(p, base, tile, r0, list + r0, n);
+    if (R < 8) break;  // as many rows as tokens at most
+  }
 }
 
 // The first 4 KB of a weight row on their way into L2.
@@ -384,11 +406,11 @@ __device__ __forceinline__ void few_prefetch(const __nv_bfloat16* w, int Kd) {
 }
 
 template <int R>
-__device__ __forceinline__ float few_down(const FewLayerParams& p, const __nv_bfloat16* w, int tile, int rows) {
+__device__ __forceinline__ float few_down(const FewLayerParams& p, const __nv_bfloat16* w, int row0, int rows) {
   int off[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) off[r] = (r < rows ? r : 0) * p.F;
-  return few_dots<R, false>(w, nullptr, p.inter + (size_t)tile * kTileRows * p.F, off, p.F);
+  return few_dots<R, false>(w, nullptr, p.inter + (size_t)row0 * p.F, off, p.F);
 }
 
 // A CTA holds kFewWarps / S columns, a column's used tiles being dealt to S warps; the CTA then adds up each token's K
@@ -415,23 +437,28 @@ few_down_kernel(const FewLayerParams p) {
       if (s.idx[a] < 0) s_val[c][a] = 0.0f;
     for (int u = part; u < n_used && n < p.H; u += S) {
       const int e = s.used[u], tile = p.tile_step > 0 ? e * p.tile_step : u;
-      const int rows = min(few_rows(p, s, e, s_list[warp]), R);
+      const int rows = few_rows(p, s, e, s_list[warp]);
       if (u + S < n_used) few_prefetch(weights(s.used[u + S], n), p.F);
       else if (n + (int)gridDim.x * C < p.H) few_prefetch(weights(s.used[part], n + gridDim.x * C), p.F);
       const __nv_bfloat16* w = weights(e, n);
-      float v;
-      if (rows == 1) v = few_down<1>(p, w, tile, rows);
-      else if (R >= 2 && rows == 2) v = few_down<(R < 2 ? R : 2)>(p, w, tile, rows);
-      else if (R >= 4 && rows <= 4) v = few_down<(R < 4 ? R : 4)>(p, w, tile, rows);
-      else v = few_down<R>(p, w, tile, rows);
-      if (lane < rows) {
-        const int a = s_list[warp][lane];
-        const __nv_bfloat16 b = __float2bfloat16_rn(v);
-        p.out[(p.push ? (size_t)a : (size_t)tile * kTileRows + lane) * p.H + n] = b;
-        s_val[c][a] = __bfloat162float(b);
+      for (int r0 = 0; r0 < rows; r0 += R) {
+        const int m = min(R, rows - r0), row0 = tile * kTileRows + r0;
+        float v;
+        if (m == 1) v = few_down<1>(p, w, row0, m);
+        else if (R >= 2 && m == 2) v = few_down<(R < 2 ? R : 2)>(p, w, row0, m);
+        else if (R >= 4 && m <= 4) v = few_down<(R < 4 ? R : 4)>(p, w, row0, m);
+        else v = few_down<R>(p, w, row0, m);
+        if (lane < m) {
+          const int a = s_list[warp][r0 + lane];
+          const __nv_bfloat16 b = __float2bfloat16_rn(v);
+          p.out[(size_t)(p.push ? a : row0 + lane) * p.H + n] = b;
+          s_val[c][a] = __bfloat162float(b);
+        }
+        if (R < 8) break;
       }
     }
     __syncthreads();
+    static_assert(kFewMaxTokens * C <= kFewThreads, "a thread per token and column");
     if ((int)threadIdx.x < p.T * C) {
       const int t = threadIdx.x / C, cc = threadIdx.x % C;
       if (n0 + cc < p.H) {
@@ -458,11 +485,11 @@ template <int R>
 static int launch_few_layer(moe_plan* p, FewLayerParams q, const void* wd, cudaStream_t st) {
   const moe_config_t& c = p->cfg;
   static SmemAttrOnce once;
+  const int tiles = min(c.T * c.K, c.E);  // at most this many are used
   few_prefer_l1(few_gate_up_kernel<R>, p->device, once);
-  if (launch_pdl(few_gate_up_kernel<R>, few_grid(p, c.F), dim3(kFewThreads), 0, st, q) != cudaSuccess) return MOE_ERR_CUDA;
+  if (launch_pdl(few_gate_up_kernel<R>, few_grid(p, tiles, c.F), dim3(kFewThreads), 0, st, q) != cudaSuccess) return MOE_ERR_CUDA;
   p->launches += 1;
   mark(p, 4, st);
-  const int tiles = few_tiles(p);
   // The combined form for one token, and for more while the down matrices are small: its warps wait for the slowest
   // tile of their column, which costs more than a launch when experts have unequal row counts and long columns.  Measured,
   // down (+ 5 us for the combine launch) / combined, us, by the down matrices' bytes: one token 23 MB 14.3 / 14.3, 235 MB
@@ -540,7 +567,8 @@ int launch_few_layer(moe_plan* p, const void* x, const void* wg, const void* wu,
   if (c.T <= 1) return launch_few_layer<1>(p, q, wd, st);
   if (c.T <= 2) return launch_few_layer<2>(p, q, wd, st);
   if (c.T <= 4) return launch_few_layer<4>(p, q, wd, st);
-  return launch_few_layer<kFewMaxTokens>(p, q, wd, st);
+  if (c.T <= 5) return launch_few_layer<5>(p, q, wd, st);
+  return launch_few_layer<8>(p, q, wd, st);
 }
 
 }  // namespace moehub

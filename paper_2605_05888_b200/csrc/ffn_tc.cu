@@ -608,10 +608,8 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   const bool pairs = c.ffn_kernel == 2 || (c.ffn_kernel == 0 && (long long)c.T * c.K > (long long)kTileRows * c.E && c.H >= 1536 &&
                                            c.F >= 1024 && overlap_x == nullptr && c.ffn_hot_min_tiles <= 0 &&
                                            c.ffn_thin_tiles >= 0 && !p->trace);
-  // Up to five tokens: plain FMAs on every SM (ffn_few.cu).  Measured, layer time tensor cores / few: one token 1.23 (256
-  // experts of 88 MB) to 1.81 (32 of 6 MB), five 1.03-1.21, six 0.93-1.22, eight 0.92-1.11 (an expert's rows share a
-  // weight's load but not its FMAs); H 256, F 256 1.6 for one to five.  Calls without row counts and the options that only
-  // the tensor-core kernel has keep it.
+  // A handful of tokens, or some tens in a small layer: plain FMAs on every SM (the rule is in ffn_few.cu).  Calls without
+  // row counts and the options that only the tensor-core kernel has keep it.
   const bool few = few_applies(p) && tile_count != nullptr && overlap_x == nullptr;
   if (p->P > kMaxListTiles) return MOE_ERR_UNSUPPORTED;  // the work list lives in the kernel's shared memory
   if ((long long)p->P * (NB1 + NB2) >= (1ll << kThinShift)) return MOE_ERR_UNSUPPORTED;  // item index field of the ring

@@ -418,7 +418,7 @@ int launch_ffn_pair(moe_plan* p, const void* recv, const void* wg, const void* w
                     cudaStream_t st);
 
 // A handful of tokens: plain FMAs, every SM streams weights (ffn_few.cu).
-constexpr int kFewMaxTokens = 5;
+constexpr int kFewMaxTokens = 32;  // (beyond five: small layers only)
 bool few_applies(const moe_plan* p);
 int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
                    const int* push_src, cudaStream_t st);

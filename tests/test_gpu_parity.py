@@ -345,7 +345,7 @@ def test_router_filter_chain_numbering(T, case):
     Hh.check_route(idx, tw, ridx, rw)
 
 
-# The kernel for a handful of tokens: one to five tokens (an expert with one to five rows; six go to the tensor cores),
+# The kernel for a handful of tokens: one to five tokens (an expert with one to five rows; six of this size go to the tensor cores),
 # H and F that end inside a lane's vectors and a warp's columns, few and many experts (more tiles than the table's first
 # 256 entries), TP shards, the push epilogue, and a call whose rows never become available.
 FEW = [
@@ -353,6 +353,8 @@ FEW = [
     (1, 1032, 8, 2, 520, 1, 0), (2, 1288, 4, 4, 776, 1, 0), (3, 1024, 2, 2, 512, 1, 1), (4, 1544, 6, 3, 1056, 2, 0),
     (5, 1032, 5, 5, 520, 1, 1), (5, 1024, 256, 8, 512, 1, 0), (5, 1032, 128, 16, 1040, 2, 1), (6, 1032, 8, 2, 520, 1, 0), (1, 256, 8, 2, 256, 1, 0),
     (4, 264, 40, 6, 264, 1, 1), (3, 4096, 4, 2, 2064, 1, 0), (2, 2048, 24, 4, 2064, 1, 1), (1, 2048, 16, 16, 1040, 1, 0),
+    # small layers of more tokens: experts of up to 32 rows (groups of eight), the largest of the range, one past it
+    (32, 256, 4, 2, 264, 1, 0), (31, 264, 2, 2, 256, 1, 1), (9, 512, 16, 3, 528, 2, 0), (16, 512, 100, 4, 256, 1, 0), (33, 256, 4, 2, 256, 1, 0),
 ]
 
 
@@ -375,7 +377,7 @@ def test_few_tokens_kernel(case, mode):
 # Up to five tokens the layer resolves the addresses and combines inside the two expert kernels: the tables it leaves are
 # a dispatch's, and the result is, byte for byte, that of the steps called one after the other.
 @pytest.mark.parametrize("mode", MODES)
-@pytest.mark.parametrize("case", [c for c in FEW if c[0] <= 5], ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}_push{c[6]}")
+@pytest.mark.parametrize("case", [c for c in FEW if c[0] not in (6, 33)], ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}_push{c[6]}")
 def test_few_tokens_layer_equals_its_steps(case, mode):
     T, H, E, K, F, tp, combine = case
     w = inputs.Workload("few", T=T, H=H, E=E, R=1, K=K, F=F, dtype=BF16, zipf_s=1.2, seed=32)
@@ -425,6 +427,30 @@ def test_few_tokens_kernel_wait_runs_out_and_reports_it():
     torch.cuda.synchronize()
     assert plan.moe_last_status()[0] == -6       # MOE_ERR_TIMEOUT; the context stays usable
     assert torch.count_nonzero(out) == 0
+
+
+def test_few_tokens_kernel_expert_named_twice():
+    """A caller's own routing may name an expert more than once for a token: more rows than tokens in a tile."""
+    w = inputs.Workload("few_twice", T=3, H=520, E=4, R=1, K=4, F=264, dtype=BF16, seed=33)
+    x, _, _, wg, wu, wd = Hh.oracle_inputs(w)
+    idx = np.array([[2, 2, 2, 2], [2, 2, 2, 1], [2, 2, 2, 2]], np.int32)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    rows = plan.P * 128
+    recv, out = (torch.zeros((rows, w.H), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    cnt, te, src = (torch.empty(n, dtype=torch.int32, device="cuda") for n in (w.E, plan.P, rows))
+    slot, tiles, done = (torch.empty(n, dtype=torch.int32, device="cuda") for n in ((w.T, w.K), (plan.P,), (1,)))
+    plan.moe_dispatch(Hh.to_dev(x), Hh.to_dev(idx), recv, cnt, te, src, slot, tiles, done)
+    dw = [Hh.to_dev(a) for a in (wg, wu, wd)]
+    plan.moe_expert_ffn(recv, te, *dw, out, tiles, done)
+    whole = torch.zeros_like(out)
+    plan.moe_expert_ffn(recv, te, *dw, whole)     # without row counts: the tensor-core kernel, every tile whole
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0) and cnt.cpu().tolist() == [0, 1, 11, 0]
+    used = slot.flatten().long()
+    a, b = out[used].float(), whole[used].float()
+    # both round an fp32 sum of F products to bf16 after an intermediate rounded to bf16: two units in the last place of the
+    # largest output cover the order of additions
+    assert float((a - b).abs().max()) <= 2 * 2.0 ** -8 * float(b.abs().max())
 
 
 # ------------------------------------------------------------------ dispatch edge cases

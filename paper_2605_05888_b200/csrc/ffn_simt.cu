@@ -90,9 +90,9 @@ ffn_simt_kernel(const XT* __restrict__ A, int lda, const int* __restrict__ tile_
 }
 
 // ---- dtype fp32 ----------------------------------------------------------------------------------------
-// Bound by fp32 FMA issue (128 per clock and SM).  A CTA computes 8 TM rows of a tile x 16 TN columns (GEMM1: half of
-// them gate, half up columns of the same f); a warp has 2 TM rows, a lane TM x TN results.  Operands stay in their
-// natural K-major rows: TMA brings 128 bytes (32 k) of every row per stage (128-byte swizzle), a lane reads 16 bytes
+// Bound by fp32 FMA issue (128 per clock and SM).  A CTA computes 2 TM WR rows of a tile x 64 TN / WR columns (GEMM1:
+// half of them gate, half up columns of the same f); a warp has 2 TM rows and 16 TN columns, a lane TM x TN results.
+// Operands stay in their natural K-major rows: TMA brings 128 bytes (32 k) of every row per stage (128-byte swizzle), a lane reads 16 bytes
 // (4 k) of its TM rows and TN columns - two pipe cycles each, lanes of a warp being 2 row groups x 16 column groups -
 // for TM x TN x 2 packed FMAs (fma.rn.f32x2 on pairs of neighbouring k: a result is the sum of its even and its odd k).
 // With scalar FMAs half of them found their accumulator in the register bank of the operand that changes (the four k of
@@ -101,21 +101,21 @@ ffn_simt_kernel(const XT* __restrict__ A, int lda, const int* __restrict__ tile_
 // registers); the warps wait per stage on its mbarrier.  A warp whose rows a partly filled tile does not have leaves at
 // once.
 // Measured against the plain 128 x 64 kernel above on fp32 data: T 1000, H 1024, 16 experts, top-2,
-// F 2048: whole layer 1311 -> 735 us (801 with scalar FMAs); T 256, H 128, 8 experts, top-2, F 256: 96 -> 35 us.
+// F 2048: whole layer 1311 -> 735 us (801 with scalar FMAs); T 256, H 128, 8 experts, top-2, F 256: 96 -> 33 us.
 constexpr int kF32Warps = 4;
 constexpr int kF32Threads = 32 * kF32Warps;
 constexpr int kF32K = 32;  // k per stage
 // stages and CTAs per SM: 8 x 8 results fill the registers with two CTAs, smaller tiles fit three
-template <int TM, int TN> constexpr int kF32Stages = TM * TN == 32 ? 3 : 4;
-template <int TM, int TN> constexpr int kF32Ctas = TM * TN == 64 ? 2 : 3;
-template <int TM, int TN> constexpr int kF32StageBytes = (kF32Warps * 2 * TM + 16 * TN) * kF32K * 4;
+template <int TM, int TN, int WR> constexpr int kF32Stages = TM * TN == 32 || WR == 1 ? 3 : 4;
+template <int TM, int TN, int WR> constexpr int kF32Ctas = TM * TN == 64 || WR == 1 ? 2 : 3;
+template <int TM, int TN, int WR> constexpr int kF32StageBytes = (WR * 2 * TM + kF32Warps / WR * 16 * TN) * kF32K * 4;
 
 struct Fp32Params {
   const int* tile_expert;  // [P]
   const int* tile_count;   // [P] rows per tile, or nullptr
   const int* rows_done;
   int total_rows;
-  int E, tp, N, Kd;        // experts (TP shards counted), columns of the result, length of the sums
+  int P, E, tp, N, Kd;     // tiles, experts (TP shards counted), columns of the result, length of the sums
   float* C;                // [P * 128, N]
   unsigned long long wait_ns;
   int* status;
@@ -131,41 +131,76 @@ __device__ __forceinline__ float sum_x2(unsigned long long v) {
   return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
 }
 
-template <int TM, int TN, bool SWIGLU>
-__global__ void __launch_bounds__(kF32Threads, kF32Ctas<TM, TN>)
+// WR: how many of the four warps stand along the rows (the others beside them, along the columns).
+template <int TM, int TN, int WR, bool SWIGLU>
+__global__ void __launch_bounds__(kF32Threads, (kF32Ctas<TM, TN, WR>))
 ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b1,
                 const __grid_constant__ CUtensorMap map_b2, const Fp32Params p) {
-  constexpr int BM = kF32Warps * 2 * TM, BN = 16 * TN;  // rows and columns of B per CTA
+  constexpr int WN = kF32Warps / WR, BM = WR * 2 * TM, BN = WN * 16 * TN;  // rows and columns of B per CTA
   constexpr int NOUT = SWIGLU ? BN / 2 : BN;             // columns of the result per CTA
-  constexpr int kA = BM * kF32K * 4, kStage = kF32StageBytes<TM, TN>;
-  constexpr int kStages = kF32Stages<TM, TN>;
+  constexpr int kA = BM * kF32K * 4, kStage = kF32StageBytes<TM, TN, WR>;
+  constexpr int kStages = kF32Stages<TM, TN, WR>;
   constexpr int kParts = kTileRows / BM;
   __shared__ unsigned long long s_full[kStages], s_empty[kStages];
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_block[4];
   extern __shared__ uint8_t f32_dyn[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(f32_dyn) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int tile = blockIdx.x / kParts, part = blockIdx.x % kParts;
-  const int n0 = blockIdx.y * NOUT;
   pdl_wait();
   pdl_trigger();
+  // This CTA's block of rows and columns: the blocks that have rows come first, one column of blocks after the other, so
+  // they spread over all SMs.  (With a CTA for every block a tile could have, the empty ones leave at once but the others
+  // stand at every fourth place: 37 of the 148 SMs had work.  T 64, H 1024, 32 experts,
+  // top-4, F 2048: layer 329 -> 252 us; T 100, H 512, 8 experts, top-2, F 512: 80 -> 69.)
+  if (warp == 0) {
+    const bool counted = p.tile_count != nullptr && *p.rows_done >= p.total_rows;
+    auto blocks_of = [&](int t) {  // a tile without an owner, or owned by no expert at all (a caller's own table), has none
+      const int e = t < p.P ? p.tile_expert[t] : -1;
+      return e < 0 || e >= p.E ? 0 : counted ? (min(kTileRows, p.tile_count[t]) + BM - 1) / BM : kParts;
+    };
+    int total = 0;
+    for (int t = lane; t < p.P; t += 32) total += blocks_of(t);
+    total = __reduce_add_sync(0xffffffffu, total);
+    int col = -1, block = 0;
+    if (total > 0) {
+      col = blockIdx.x / total;
+      block = blockIdx.x - col * total;
+    }
+    if (col >= (p.N + NOUT - 1) / NOUT) col = -1;
+    if (lane == 0) s_block[0] = col;
+    for (int t = lane, before = 0; col >= 0 && before <= block; t += 32) {
+      const int mine = blocks_of(t);
+      int incl = mine;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
+      }
+      const int first = before + incl - mine;
+      if (block >= first && block < first + mine) {
+        s_block[1] = t;
+        s_block[2] = block - first;
+        s_block[3] = counted ? min(kTileRows, p.tile_count[t]) : kTileRows;
+      }
+      before += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  __syncthreads();
+  if (s_block[0] < 0) return;
+  const int n0 = s_block[0] * NOUT, tile = s_block[1], part = s_block[2], rows = min(s_block[3] - part * BM, BM);
   const int e = p.tile_expert[tile];
-  if (e < 0 || e >= p.E) return;  // no owner, or no expert at all (a caller's own table): nothing of the weights is read
-  int rows = kTileRows;
-  if (p.tile_count != nullptr && *p.rows_done >= p.total_rows) rows = p.tile_count[tile];
-  rows = min(rows - part * BM, BM);
-  if (rows <= 0) return;
-  const int live_warps = (rows + 2 * TM - 1) / (2 * TM);
+  const int rw = warp % WR, cw = warp / WR;
+  const int live_rows = (rows + 2 * TM - 1) / (2 * TM);
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&s_full[s]), 1);
-      mbar_init(smem_u32(&s_empty[s]), live_warps);
+      mbar_init(smem_u32(&s_empty[s]), min(live_rows, WR) * WN);
     }
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (warp >= live_warps) return;
+  if (rw >= live_rows) return;
   volatile int* abort_flag = &s_abort;
   const int nk = (p.Kd + kF32K - 1) / kF32K;
   const size_t row0 = (size_t)tile * kTileRows + part * BM;
@@ -192,7 +227,9 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0ull;
-  const int r0 = warp * 2 * TM + lane % 2, c0 = lane / 2;  // rows r0 + 2 i, columns of B c0 + 16 j
+  // rows r0 + 2 i; columns of B c0 + 16 j (GEMM1: the first half of the j gate, the others the same columns' up rows)
+  constexpr int kCols = SWIGLU ? TN / 2 : TN;
+  const int r0 = rw * 2 * TM + lane % 2, c0 = cw * 16 * kCols + lane / 2;
   // the swizzle's row bits: a lane's rows r0 + 2 i take four values of (row % 8), its columns c0 + 16 j only one
   uint32_t aoff[4];
 #pragma unroll
@@ -218,7 +255,7 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const uint32_t u = (uint32_t)(half * (kF32K / 8) + uu) << 4;
         unsigned long long bl[TN], bh[TN];
 #pragma unroll
-        for (int j = 0; j < TN; ++j) lds_k4(b_base + (boff ^ u) + (uint32_t)j * 16u * 128u, bl[j], bh[j]);
+        for (int j = 0; j < TN; ++j) lds_k4(b_base + (boff ^ u) + (uint32_t)(j < kCols ? 16 * j : BN / 2 + 16 * (j - kCols)) * 128u, bl[j], bh[j]);
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
           unsigned long long al, ah;
@@ -251,11 +288,11 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     if (r0 + 2 * i >= rows) continue;
     float* crow = p.C + (row0 + r0 + 2 * i) * p.N;
 #pragma unroll
-    for (int j = 0; j < (SWIGLU ? TN / 2 : TN); ++j) {
+    for (int j = 0; j < kCols; ++j) {
       const int n = n0 + c0 + 16 * j;
       if (n >= p.N) continue;
       float v = sum_x2(acc[i][j]);
-      if (SWIGLU) v = v / (1.0f + expf(-v)) * sum_x2(acc[i][SWIGLU ? TN / 2 + j : j]);
+      if (SWIGLU) v = v / (1.0f + expf(-v)) * sum_x2(acc[i][SWIGLU ? kCols + j : j]);
       crow[n] = v;
     }
   }
@@ -271,10 +308,10 @@ static int make_map_f32(EncodeTiledFn enc, CUtensorMap* m, const void* base, int
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
 }
 
-template <int TM, int TN, bool SWIGLU>
+template <int TM, int TN, int WR, bool SWIGLU>
 static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
                             const Fp32Params& q, cudaStream_t st) {
-  constexpr int BM = kF32Warps * 2 * TM, BN = 16 * TN, NOUT = SWIGLU ? BN / 2 : BN;
+  constexpr int BM = WR * 2 * TM, BN = kF32Warps / WR * 16 * TN, NOUT = SWIGLU ? BN / 2 : BN;
   const cuuint64_t E = (cuuint64_t)p->cfg.E, K = (cuuint64_t)q.Kd, N = (cuuint64_t)q.N, tp = (cuuint64_t)p->tp;
   CUtensorMap ma, mb1, mb2;
   int rc;
@@ -289,11 +326,15 @@ static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const
     if ((rc = make_map_f32(enc, &mb1, b1, 4, dims, str, BN)) != MOE_OK) return rc;
     mb2 = mb1;
   }
-  auto kern = ffn_fp32_kernel<TM, TN, SWIGLU>;
-  constexpr size_t smem = 1024 + (size_t)kF32Stages<TM, TN> * kF32StageBytes<TM, TN>;
+  auto kern = ffn_fp32_kernel<TM, TN, WR, SWIGLU>;
+  constexpr size_t smem = 1024 + (size_t)kF32Stages<TM, TN, WR> * kF32StageBytes<TM, TN, WR>;
   static SmemAttrOnce once;
   if (ensure_dynamic_smem(kern, smem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
-  const dim3 grid((unsigned)(p->P * (kTileRows / BM)), (unsigned)((q.N + NOUT - 1) / NOUT));
+  // As many blocks of rows as there can be: inside moe_layer the counts add up to T * K, so besides full blocks there is at
+  // most one per tile; a caller's counters may be incomplete, and its tiles are whole then.
+  const long long row_blocks = q.tile_count == p->s.tile_count ? min((long long)p->P * (kTileRows / BM), (long long)q.total_rows / BM + p->P)
+                                                       : (long long)p->P * (kTileRows / BM);
+  const dim3 grid((unsigned)(row_blocks * ((q.N + NOUT - 1) / NOUT)));
   p->launches += 1;
   return launch_pdl(kern, grid, dim3(kF32Threads), smem, st, ma, mb1, mb2, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
 }
@@ -310,6 +351,7 @@ static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, co
   q.tile_count = tile_count;
   q.rows_done = rows_done;
   q.total_rows = c.T * c.K;
+  q.P = (int)p->P;
   q.E = c.E;
   q.tp = p->tp;
   q.wait_ns = kDefaultWaitNs;  // the waits are on this CTA's own copies: nothing a caller's limit is meant for
@@ -321,22 +363,38 @@ static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, co
   // 37 rows 470 / 409 / 365.
   const long long rows = (long long)c.T * c.K, blocks = rows / 64 + c.E;  // 64-row blocks, about
   const int shape = rows >= 192ll * c.E ? 2 : rows >= 96ll * c.E ? 1 : 0;
+  // 4 x 4: how many warps stand along the rows.  An expert's last block of rows leaves warps without rows, and a warp
+  // that leaves leaves its scheduler idle, so blocks of eight rows (all warps along the columns) up to 48 rows per expert,
+  // of 16 up to 96.  With fewer than eight rows there is one block either way, and the smaller CTAs of 32 rows let GEMM2's
+  // start beside GEMM1's.  Measured, whole layer, us, 4 / 2 / 1 warps along the rows, by rows per expert: 4 (H 1024, F 1024)
+  // 86 / 109 / 109, 4 (H 512, F 1024) 83 / 85 / 72; 8 (H 1024, F 2048) 252 / 259 / 217; 19 (H 512, F 512) 97 / 83 / 80; 25 (H
+  // 512, F 512) 69 / 62 / 56; 33 (H 512, F 256) 102 / 99 / 90; 64 (H 128, F 256) 35 / 33 / 31; 67 (H 512, F 1024) 436 / 429 /
+  // 484; 450 (H 256, F 512) 72 / 74 / 80.
+  auto along = [&](int n, int cols) {  // cols: the columns of a CTA with all warps along them
+    int wr = rows < 8ll * c.E || rows >= 96ll * c.E ? 4 : rows < 48ll * c.E ? 1 : 2;
+    while (wr < 4 && cols / wr > n) wr *= 2;
+    return wr;
+  };
   mark(p, 3, st);
   q.N = c.F;
   q.Kd = c.H;
   q.C = (float*)p->s.inter;
   const bool enough1 = blocks * ((c.F + 63) / 64) >= 2 * sms, enough2 = blocks * ((c.H + 127) / 128) >= 3 * sms / 2;
-  if (shape == 2 && enough1) rc = launch_fp32_gemm<8, 8, true>(p, enc, recv, wg, wu, q, st);
-  else if (shape == 1 && enough1) rc = launch_fp32_gemm<4, 8, true>(p, enc, recv, wg, wu, q, st);
-  else rc = launch_fp32_gemm<4, 4, true>(p, enc, recv, wg, wu, q, st);
+  if (shape == 2 && enough1) rc = launch_fp32_gemm<8, 8, 4, true>(p, enc, recv, wg, wu, q, st);
+  else if (shape == 1 && enough1) rc = launch_fp32_gemm<4, 8, 4, true>(p, enc, recv, wg, wu, q, st);
+  else if (along(c.F, 128) == 1) rc = launch_fp32_gemm<4, 4, 1, true>(p, enc, recv, wg, wu, q, st);
+  else if (along(c.F, 128) == 2) rc = launch_fp32_gemm<4, 4, 2, true>(p, enc, recv, wg, wu, q, st);
+  else rc = launch_fp32_gemm<4, 4, 4, true>(p, enc, recv, wg, wu, q, st);
   if (rc != 0) return rc;
   mark(p, 4, st);
   q.N = c.H;
   q.Kd = c.F;
   q.C = (float*)out_rows;
-  if (shape == 2 && enough2) return launch_fp32_gemm<8, 8, false>(p, enc, p->s.inter, wd, nullptr, q, st);
-  if (shape == 1 && enough2) return launch_fp32_gemm<4, 8, false>(p, enc, p->s.inter, wd, nullptr, q, st);
-  return launch_fp32_gemm<4, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (shape == 2 && enough2) return launch_fp32_gemm<8, 8, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (shape == 1 && enough2) return launch_fp32_gemm<4, 8, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (along(c.H, 256) == 1) return launch_fp32_gemm<4, 4, 1, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (along(c.H, 256) == 2) return launch_fp32_gemm<4, 4, 2, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  return launch_fp32_gemm<4, 4, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
 }
 
 template <typename XT>

@@ -246,6 +246,8 @@ FP32_FFN = [
     # (T, H, E, K, F, tp, zipf_s)
     (1, 4, 2, 1, 4, 1, 0.0), (40, 36, 4, 2, 68, 1, 1.2), (300, 132, 3, 2, 100, 1, 1.2), (1200, 260, 8, 2, 1284, 1, 1.2),
     (700, 516, 16, 3, 1028, 1, 1.0), (1300, 2052, 8, 2, 260, 1, 1.0), (900, 1284, 16, 2, 1284, 1, 1.0), (129, 100, 6, 2, 264, 2, 1.0),
+    # blocks of 8 and of 16 rows (warps side by side), columns that end inside a warp's, TP shards of 68 columns
+    (200, 260, 16, 2, 1028, 1, 1.2), (500, 1028, 12, 2, 516, 1, 1.0), (100, 260, 16, 2, 136, 2, 0.0), (64, 516, 16, 2, 260, 1, 0.0),
 ]
 
 

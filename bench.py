@@ -531,7 +531,7 @@ def run_cuda(args, w: inputs.Workload) -> None:
         sustained = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
         long_run = ms_total >= 1000.0
         peak = sustained if long_run else peaks["bf16_tflops"]
-        roofline = {"kernel": "ffn_tc_kernel (expert GEMM1 + SwiGLU + GEMM2, tcgen05)", "bound": "tensor",
+        roofline = {"kernel": "expert kernel (GEMM1 + SwiGLU + GEMM2, tcgen05: ffn_pair_kernel, or ffn_tc_kernel where experts have a tile of rows at most)", "bound": "tensor",
                     "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                     "traffic": ncu_traffic_bytes(w.name),
                     "peak_source": f"{peak_kind} " + ("bf16_tflops_sustained (timed region of %.1f s)" % (ms_total / 1e3) if long_run else

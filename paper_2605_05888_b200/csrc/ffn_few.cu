@@ -112,35 +112,37 @@ __device__ __forceinline__ void few_columns(const FewParams& p, size_t base, int
   }
 }
 
-template <int R, bool SWIGLU>
-__global__ void __launch_bounds__(kFewThreads)
-ffn_few_kernel(const FewParams p) {
-  __shared__ int s_used[kFewWarps];
-  __shared__ int s_tile, s_rows;
+struct FewTile {  // shared memory
+  int used[kFewWarps];
+  int tile, rows, owned;
+};
+
+// The tile that is number `ordinal` among the owned ones (-1: there are not so many).  The whole CTA calls.
+__device__ __forceinline__ int few_find_tile(const FewParams& p, FewTile& s, int ordinal) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (threadIdx.x == 0) s_tile = -1;
-  __syncthreads();
-  pdl_wait();
-  pdl_trigger();
-  // this CTA's tile: number blockIdx.y among the used ones
-  const int ordinal = blockIdx.y;
-  for (int base = 0, seen = 0; base < p.P && seen <= ordinal; base += kFewThreads) {
+  int seen = 0;
+  for (int base = 0; base < p.P; base += kFewThreads) {
     const int t = base + threadIdx.x;
     const int e = t < p.P ? p.tile_expert[t] : -1;
     const unsigned used = __ballot_sync(0xffffffffu, e >= 0 && e < p.E);
-    if (lane == 0) s_used[warp] = __popc(used);
+    if (lane == 0) s.used[warp] = __popc(used);
     __syncthreads();
     int before = seen;
     for (int w = 0; w < kFewWarps; ++w) {
-      if (w < warp) before += s_used[w];
-      seen += s_used[w];
+      if (w < warp) before += s.used[w];
+      seen += s.used[w];
     }
-    if (((used >> lane) & 1u) && before + __popc(used & ((1u << lane) - 1u)) == ordinal) s_tile = t;
+    if (((used >> lane) & 1u) && before + __popc(used & ((1u << lane) - 1u)) == ordinal) s.tile = t;
     __syncthreads();
   }
-  const int tile = s_tile;
-  if (tile < 0) return;
-  if (threadIdx.x == 0) {  // availability of the tile's rows (Section IV-D): as in the tensor-core kernels, bounded
+  if (threadIdx.x == 0) s.owned = seen;
+  return s.tile;
+}
+
+// How many rows the tile holds, once they are available (Section IV-D; as in the tensor-core kernels, bounded: -1 when the
+// wait ran out).  The whole CTA calls.
+__device__ __forceinline__ int few_tile_rows(const FewParams& p, FewTile& s, int tile) {
+  if (threadIdx.x == 0) {
     const unsigned long long t0 = globaltimer();
     bool ready = true;
     while (ld_acquire(&p.tile_count[tile]) < kTileRows && ld_acquire(p.rows_done) < p.total_rows) {
@@ -151,23 +153,73 @@ ffn_few_kernel(const FewParams p) {
       }
       __nanosleep(64);
     }
-    s_rows = ready ? min(kTileRows, p.tile_count[tile]) : 0;
+    s.rows = ready ? min(kTileRows, p.tile_count[tile]) : -1;
   }
   __syncthreads();
-  const int rows = s_rows;
-  if (rows <= 0) return;
+  return s.rows;
+}
+
+__device__ __forceinline__ size_t few_weights(const FewParams& p, int tile) {
   const int e = p.tile_expert[tile];
-  const size_t base = (size_t)(e / p.tp) * p.expert_stride + (size_t)(e % p.tp) * p.shard_offset;
-  if (rows == 1) few_columns<1, SWIGLU>(p, base, tile, 0, rows);
-  else if (R >= 2 && rows == 2) few_columns<(R < 2 ? R : 2), SWIGLU>(p, base, tile, 0, rows);
-  else if (R >= 4 && rows <= 4) few_columns<(R < 4 ? R : 4), SWIGLU>(p, base, tile, 0, rows);
-  else few_columns<R, SWIGLU>(p, base, tile, 0, min(rows, R));
-  for (int r0 = R; r0 < rows;) {  // more rows than tokens: a caller's routing that names an expert twice for a token
-    const int n = R < 8 || rows - r0 < 8 ? 1 : 8;  // (or more than 8 tokens)
-    if (n == 1) few_columns<1, SWIGLU>(p, base, tile, r0, 1);
-    else few_columns<(R < 8 ? 1 : 8), SWIGLU>(p, base, tile, r0, 8);
-    r0 += n;
+  return (size_t)(e / p.tp) * p.expert_stride + (size_t)(e % p.tp) * p.shard_offset;
+}
+
+// The owned tiles beyond the first gridDim.y: what a dispatch leaves owns at most T * K tiles, one per blockIdx.y, but a
+// caller's own table may name an owner for every tile of its regions.  Row by row and not inlined, so that the kernel's body
+// keeps its registers.  Measured on moe_expert_ffn, one to five tokens, four shapes, against the kernel that looks at the first
+// gridDim.y only: 0.90 to 1.07 of its time, mean 1.01; moe_layer, whose table is a dispatch's, has that kernel.
+template <bool SWIGLU>
+__device__ __noinline__ void few_more_tiles(const FewParams& p, FewTile& s) {
+  for (int ordinal = blockIdx.y + gridDim.y;; ordinal += gridDim.y) {
+    __syncthreads();
+    if (threadIdx.x == 0) s.tile = -1;
+    __syncthreads();
+    const int tile = few_find_tile(p, s, ordinal);
+    if (tile < 0) return;
+    const int rows = few_tile_rows(p, s, tile);
+    if (rows < 0) return;
+    const size_t base = few_weights(p, tile);
+    for (int r0 = 0; r0 < rows; ++r0) few_columns<1, SWIGLU>(p, base, tile, r0, 1);
   }
+}
+
+// ANY: the table may be any caller's (false: a dispatch's).
+template <int R, bool SWIGLU, bool ANY>
+__device__ __forceinline__ void few_tiles(const FewParams& p) {
+  __shared__ FewTile s;
+  if (threadIdx.x == 0) s.tile = -1;
+  __syncthreads();
+  pdl_wait();
+  pdl_trigger();
+  const int tile = few_find_tile(p, s, blockIdx.y);
+  if (tile < 0) return;
+  const int rows = few_tile_rows(p, s, tile);
+  if (rows < 0 || (!ANY && rows == 0)) return;
+  if (!ANY || rows > 0) {
+    const size_t base = few_weights(p, tile);
+    if (rows == 1) few_columns<1, SWIGLU>(p, base, tile, 0, rows);
+    else if (R >= 2 && rows == 2) few_columns<(R < 2 ? R : 2), SWIGLU>(p, base, tile, 0, rows);
+    else if (R >= 4 && rows <= 4) few_columns<(R < 4 ? R : 4), SWIGLU>(p, base, tile, 0, rows);
+    else few_columns<R, SWIGLU>(p, base, tile, 0, min(rows, R));
+    for (int r0 = R; r0 < rows;) {  // more rows than tokens: a caller's routing that names an expert twice for a token
+      const int n = R < 8 || rows - r0 < 8 ? 1 : 8;  // (or more than 8 tokens)
+      if (n == 1) few_columns<1, SWIGLU>(p, base, tile, r0, 1);
+      else few_columns<(R < 8 ? 1 : 8), SWIGLU>(p, base, tile, r0, 8);
+      r0 += n;
+    }
+  }
+  if (ANY && (int)(blockIdx.y + gridDim.y) < s.owned) few_more_tiles<SWIGLU>(p, s);
+}
+
+template <int R, bool SWIGLU>
+__global__ void __launch_bounds__(kFewThreads)
+ffn_few_kernel(const FewParams p) {
+  few_tiles<R, SWIGLU, false>(p);
+}
+template <int R, bool SWIGLU>
+__global__ void __launch_bounds__(kFewThreads)
+ffn_few_any_kernel(const __grid_constant__ FewParams p) {
+  few_tiles<R, SWIGLU, true>(p);
 }
 
 static dim3 few_grid(const moe_plan* p, int tiles, int columns) {  // CTAs per tile: up to eight per SM in all
@@ -191,7 +243,7 @@ bool few_applies(const moe_plan* p) {
          c.ffn_split == 0 && !p->trace;
 }
 
-template <int R>
+template <int R, bool ANY>
 static int launch_few_gate_up(moe_plan* p, FewParams q, const void* recv, const void* wg, const void* wu, cudaStream_t st) {
   const moe_config_t& c = p->cfg;
   q.expert_stride = (size_t)c.F * p->tp * c.H;
@@ -204,10 +256,10 @@ static int launch_few_gate_up(moe_plan* p, FewParams q, const void* recv, const 
   q.Kd = c.H;
   q.C = (__nv_bfloat16*)p->s.inter;
   p->launches += 1;
-  return launch_pdl(ffn_few_kernel<R, true>, few_grid(p, (int)min((long long)c.T * c.K, (long long)p->P), c.F), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+  return launch_pdl(ANY ? ffn_few_any_kernel<R, true> : ffn_few_kernel<R, true>, few_grid(p, (int)min((long long)c.T * c.K, (long long)p->P), c.F), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
 }
 
-template <int R>
+template <int R, bool ANY>
 static int launch_few_down(moe_plan* p, FewParams q, const void* wd, void* out, const int* push_src, cudaStream_t st) {
   const moe_config_t& c = p->cfg;
   q.expert_stride = (size_t)c.F * p->tp * c.H;
@@ -220,16 +272,16 @@ static int launch_few_down(moe_plan* p, FewParams q, const void* wd, void* out, 
   q.C = (__nv_bfloat16*)out;
   q.push_src = push_src;
   p->launches += 1;
-  return launch_pdl(ffn_few_kernel<R, false>, few_grid(p, (int)min((long long)c.T * c.K, (long long)p->P), c.H), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+  return launch_pdl(ANY ? ffn_few_any_kernel<R, false> : ffn_few_kernel<R, false>, few_grid(p, (int)min((long long)c.T * c.K, (long long)p->P), c.H), dim3(kFewThreads), 0, st, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
 }
 
-template <int R>
+template <int R, bool ANY>
 static int launch_few(moe_plan* p, const FewParams& q, const void* recv, const void* wg, const void* wu, const void* wd, void* out,
                       const int* push_src, cudaStream_t st) {
-  int rc = launch_few_gate_up<R>(p, q, recv, wg, wu, st);
+  int rc = launch_few_gate_up<R, ANY>(p, q, recv, wg, wu, st);
   if (rc != 0) return rc;
   mark(p, 4, st);
-  return launch_few_down<R>(p, q, wd, out, push_src, st);
+  return launch_few_down<R, ANY>(p, q, wd, out, push_src, st);
 }
 
 int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
@@ -245,11 +297,14 @@ int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu
   q.wait_ns = prm.wait_ns;
   q.status = prm.status;
   const int T = p->cfg.T;
-  if (T <= 1) return launch_few<1>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
-  if (T <= 2) return launch_few<2>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
-  if (T <= 4) return launch_few<4>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
-  if (T <= 5) return launch_few<5>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
-  return launch_few<8>(p, q, recv, wg, wu, wd, prm.out, push_src, st);
+  const bool any = prm.tile_count != p->s.tile_count;  // inside moe_layer the table is the dispatch's own
+#define MOEHUB_FEW(R) (any ? launch_few<R, true>(p, q, recv, wg, wu, wd, prm.out, push_src, st) : launch_few<R, false>(p, q, recv, wg, wu, wd, prm.out, push_src, st))
+  if (T <= 1) return MOEHUB_FEW(1);
+  if (T <= 2) return MOEHUB_FEW(2);
+  if (T <= 4) return MOEHUB_FEW(4);
+  if (T <= 5) return MOEHUB_FEW(5);
+  return MOEHUB_FEW(8);
+#undef MOEHUB_FEW
 }
 
 // ---- the whole layer behind the router ----------------------------------------------------------------
@@ -505,7 +560,7 @@ static int launch_few_layer(moe_plan* p, FewLayerParams q, const void* wd, cudaS
     d.total_rows = c.T * c.K;
     d.wait_ns = kDefaultWaitNs;
     d.status = q.status;
-    int rc = launch_few_down<R>(p, d, wd, q.out, q.push ? q.src_info : nullptr, st);
+    int rc = launch_few_down<R, false>(p, d, wd, q.out, q.push ? q.src_info : nullptr, st);
     if (rc != 0) return rc;
     mark(p, 5, st);
     return launch_combine(p, q.out, q.slot_of, q.topk_w, q.y, st, q.push) ? MOE_ERR_CUDA : 0;

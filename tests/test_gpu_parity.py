@@ -455,6 +455,43 @@ def test_few_tokens_kernel_expert_named_twice():
     assert float((a - b).abs().max()) <= 2 * 2.0 ** -8 * float(b.abs().max())
 
 
+@pytest.mark.parametrize("push", [0, 1])
+@pytest.mark.parametrize("case", [(1, 8, 2), (3, 5, 1), (1, 256, 1)], ids=lambda c: f"T{c[0]}_E{c[1]}_K{c[2]}")
+def test_few_tokens_kernel_walks_every_owned_tile(case, push):
+    """A caller's own table may name an owner for every tile of its static regions, also where no row is: more owned tiles
+    than the batch has assignments, rows only in the last regions."""
+    T, E, K = case
+    w = inputs.Workload("few_owned", T=T, H=520, E=E, R=1, K=K, F=264, dtype=BF16, seed=34)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_STATIC)
+    assert plan.P == E
+    g = torch.Generator(device="cuda").manual_seed(34)
+    wg, wu, wd = (torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.05, generator=g)
+                  for s in ((E, w.F, w.H), (E, w.F, w.H), (E, w.H, w.F)))
+    recv = torch.empty((E * 128, w.H), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    te = torch.arange(E, dtype=torch.int32, device="cuda")
+    counts, done = torch.zeros(E, dtype=torch.int32, device="cuda"), torch.full((1,), T * K, dtype=torch.int32, device="cuda")
+    slots = [(E - 1) * 128 + i for i in range(T * K - T * K // 2)] + [(E - 2) * 128 + i for i in range(T * K // 2)]
+    for s in slots:
+        counts[s // 128] += 1
+    src = torch.full((E * 128,), -1, dtype=torch.int32, device="cuda")
+    src[slots] = torch.arange(T * K, dtype=torch.int32, device="cuda")
+    whole = torch.zeros_like(recv)
+    plan.moe_expert_ffn(recv, te, wg, wu, wd, whole)     # without row counts: the tensor-core kernel, every tile whole
+    if push:
+        out = torch.zeros((T * K, w.H), dtype=torch.bfloat16, device="cuda")
+        plan.moe_expert_ffn_push(recv, te, src, wg, wu, wd, out, counts, done)
+        got = out
+    else:
+        out = torch.zeros_like(recv)
+        plan.moe_expert_ffn(recv, te, wg, wu, wd, out, counts, done)
+        got = out[slots]
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    a, b = got.float(), whole[slots].float()
+    # (the bound of test_few_tokens_kernel_expert_named_twice)
+    assert float(b.abs().max()) > 0 and float((a - b).abs().max()) <= 2 * 2.0 ** -8 * float(b.abs().max())
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

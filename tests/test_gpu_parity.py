@@ -492,6 +492,26 @@ def test_few_tokens_kernel_walks_every_owned_tile(case, push):
     assert float(b.abs().max()) > 0 and float((a - b).abs().max()) <= 2 * 2.0 ** -8 * float(b.abs().max())
 
 
+def test_static_regions_of_more_rows_than_the_batch_keep_the_tensor_cores():
+    """A decode-size plan may hold static regions that other callers fill (capacity_rows above the batch): whole tiles of
+    rows belong on the tensor cores, with the same bytes as without row counts."""
+    E, H, F, cap = 3, 520, 264, 256
+    w = inputs.Workload("few_regions", T=1, H=H, E=E, R=1, K=1, F=F, dtype=BF16, seed=35)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_STATIC, capacity_rows=cap)
+    g = torch.Generator(device="cuda").manual_seed(35)
+    wg, wu, wd = (torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.05, generator=g)
+                  for s in ((E, F, H), (E, F, H), (E, H, F)))
+    recv = torch.empty((E * cap, H), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    te = torch.arange(plan.P, dtype=torch.int32, device="cuda") // (cap // 128)
+    counts, done = torch.full((plan.P,), 128, dtype=torch.int32, device="cuda"), torch.full((1,), E * cap, dtype=torch.int32, device="cuda")
+    out, whole = torch.zeros_like(recv), torch.ones_like(recv)
+    plan.moe_expert_ffn(recv, te, wg, wu, wd, out, counts, done)
+    assert plan.moe_last_launch_count() == 1     # (the kernels for few tokens are two launches)
+    plan.moe_expert_ffn(recv, te, wg, wu, wd, whole)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0) and torch.equal(out, whole)
+
+
 # ------------------------------------------------------------------ dispatch edge cases
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_all_tokens_to_one_expert_and_empty_experts(mode):

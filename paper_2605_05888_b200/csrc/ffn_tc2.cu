@@ -494,6 +494,7 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
         const int row = (first ? rows.t[0] : rows.t[1]) * kTileRows + r0 + (lane >> 2);  // this lane's rows: row, row + 8
         const bool last = unit + kPairEpiWarps / 4 >= units;
         uint32_t w[8];
+        __syncwarp();  // (the loads below want the whole warp; the last unit's stores left it by columns)
         if (it.type == 0) {
           uint32_t g[16], u[16];
           tc_ld_frag(base + c, g);
@@ -522,17 +523,18 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
         __syncwarp();
         const uint4 lo = lds128(ld_addr), hi = lds128(ld_addr + 8u * kPairPitch);
         const int col = col0 + (b ? 256 : 0);
-        if (col >= ld) continue;
-        if (it.type == 0 || prm.push_src == nullptr) {
-          if ((lane >> 2) < nrow) *reinterpret_cast<uint4*>(dst + (size_t)row * ld + col) = lo;
-          if ((lane >> 2) + 8 < nrow) *reinterpret_cast<uint4*>(dst + (size_t)(row + 8) * ld + col) = hi;
-        } else {
-          // push-style combine: a row goes to its token's position (anything beyond those is none: a stale word after a
-          // dispatch that gave up)
-          const int s0 = (lane >> 2) < nrow ? __ldcg(prm.push_src + row) : -1;
-          const int s1 = (lane >> 2) + 8 < nrow ? __ldcg(prm.push_src + row + 8) : -1;
-          if (s0 >= 0 && s0 < prm.total_rows) *reinterpret_cast<uint4*>(dst + (size_t)s0 * ld + col) = lo;
-          if (s1 >= 0 && s1 < prm.total_rows) *reinterpret_cast<uint4*>(dst + (size_t)s1 * ld + col) = hi;
+        if (col < ld) {
+          if (it.type == 0 || prm.push_src == nullptr) {
+            if ((lane >> 2) < nrow) *reinterpret_cast<uint4*>(dst + (size_t)row * ld + col) = lo;
+            if ((lane >> 2) + 8 < nrow) *reinterpret_cast<uint4*>(dst + (size_t)(row + 8) * ld + col) = hi;
+          } else {
+            // push-style combine: a row goes to its token's position (anything beyond those is none: a stale word after a
+            // dispatch that gave up)
+            const int s0 = (lane >> 2) < nrow ? __ldcg(prm.push_src + row) : -1;
+            const int s1 = (lane >> 2) + 8 < nrow ? __ldcg(prm.push_src + row + 8) : -1;
+            if (s0 >= 0 && s0 < prm.total_rows) *reinterpret_cast<uint4*>(dst + (size_t)s0 * ld + col) = lo;
+            if (s1 >= 0 && s1 < prm.total_rows) *reinterpret_cast<uint4*>(dst + (size_t)s1 * ld + col) = hi;
+          }
         }
       }
       __syncwarp();

@@ -322,6 +322,26 @@ def test_pair_expert_kernel_by_default(tp, combine):
     assert torch.equal(ys[0], ys[1])
 
 
+# H and F that end inside the 32 columns of an epilogue warp (at 8, 16 and 24 of them): some lanes of the warp store and
+# others do not, several units of rows long, with and without the push epilogue.
+@pytest.mark.parametrize("combine", [0, 1])
+@pytest.mark.parametrize("extra", [8, 16, 24])
+def test_pair_expert_kernel_columns_end_inside_a_warp(extra, combine):
+    w = inputs.Workload("pair_cols", T=700, H=1536 + extra, E=4, R=1, K=2, F=1056 - extra, dtype=BF16, zipf_s=0.7, seed=24)
+    args = [Hh.to_dev(a) for a in Hh.oracle_inputs(w)]
+    ys = []
+    for thin in (0, -1):        # pairs by default; one CTA per tile
+        plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, combine_mode=combine, ffn_thin_tiles=thin)
+        y = torch.empty((w.T, w.H), dtype=torch.bfloat16, device="cuda")
+        for i in (2, 7):
+            plan.layer_tensor(i).fill_(float("nan"))
+        plan.moe_layer(*args, y)
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == (0, 0)
+        ys.append(y)
+    assert torch.equal(ys[0], ys[1]) and bool(torch.isfinite(ys[0]).all())
+
+
 # The refine kernel's numbering of the chains: token counts that give its CTAs 12 to 64 tokens (a whole wave on 148 SMs),
 # with every token's candidates in ONE class of experts modulo eight (its bucket overflows into the others' free slots),
 # with two classes, and with more candidates than a CTA has threads (every expert the same: all 256 are candidates).

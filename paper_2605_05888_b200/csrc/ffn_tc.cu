@@ -441,6 +441,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
               for (int i = 0; i < 16; ++i)
                 inter[(row0 + c + i) * F + f] = __float2bfloat16_rn(silu_mul(__uint_as_float(g[i]), __uint_as_float(u[i])));
             }
+            __syncwarp();  // (some lanes stored, others did not; the next loads want the whole warp)
           }
         } else {
 #pragma unroll 1
@@ -462,6 +463,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
                   if (orow >= 0) out[(size_t)orow * H + h] = __float2bfloat16_rn(__uint_as_float(v[i]));
                 }
               }
+              __syncwarp();
             }
           }
         }
@@ -480,13 +482,15 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
             const float gv = __uint_as_float(g[i]);
             s[i] = silu_mul(gv, __uint_as_float(u[i]));
           }
-          if (!row_live) continue;
-          if (wide1 && c + 16 <= ncols) {
-            st_global_32B(dst + c, Vec16<__nv_bfloat16>::pack(s), Vec16<__nv_bfloat16>::pack(s + 8));
-          } else {
-            if (c + 8 <= ncols) *reinterpret_cast<uint4*>(dst + c) = Vec16<__nv_bfloat16>::pack(s);
-            if (c + 16 <= ncols) *reinterpret_cast<uint4*>(dst + c + 8) = Vec16<__nv_bfloat16>::pack(s + 8);
+          if (row_live) {
+            if (wide1 && c + 16 <= ncols) {
+              st_global_32B(dst + c, Vec16<__nv_bfloat16>::pack(s), Vec16<__nv_bfloat16>::pack(s + 8));
+            } else {
+              if (c + 8 <= ncols) *reinterpret_cast<uint4*>(dst + c) = Vec16<__nv_bfloat16>::pack(s);
+              if (c + 16 <= ncols) *reinterpret_cast<uint4*>(dst + c + 8) = Vec16<__nv_bfloat16>::pack(s + 8);
+            }
           }
+          __syncwarp();  // (some lanes stored, others did not; the next loads want the whole warp)
         }
       } else {
         // Push-style combine (paper Section IV-B, all-to-all combine): the expert reads the row's source
@@ -507,15 +511,17 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
           float f[32];
 #pragma unroll
           for (int i = 0; i < 16; ++i) { f[i] = __uint_as_float(r0[i]); f[16 + i] = __uint_as_float(r1[i]); }
-          if (!row_live) continue;
-          if (wide2 && c + 32 <= ncols) {
-            st_global_32B(dst + c, Vec16<__nv_bfloat16>::pack(f), Vec16<__nv_bfloat16>::pack(f + 8));
-            st_global_32B(dst + c + 16, Vec16<__nv_bfloat16>::pack(f + 16), Vec16<__nv_bfloat16>::pack(f + 24));
-          } else {
+          if (row_live) {
+            if (wide2 && c + 32 <= ncols) {
+              st_global_32B(dst + c, Vec16<__nv_bfloat16>::pack(f), Vec16<__nv_bfloat16>::pack(f + 8));
+              st_global_32B(dst + c + 16, Vec16<__nv_bfloat16>::pack(f + 16), Vec16<__nv_bfloat16>::pack(f + 24));
+            } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (c + 8 * q + 8 <= ncols) *reinterpret_cast<uint4*>(dst + c + 8 * q) = Vec16<__nv_bfloat16>::pack(f + 8 * q);
+              for (int q = 0; q < 4; ++q)
+                if (c + 8 * q + 8 <= ncols) *reinterpret_cast<uint4*>(dst + c + 8 * q) = Vec16<__nv_bfloat16>::pack(f + 8 * q);
+            }
           }
+          __syncwarp();
         }
       }
       tc_fence_before();

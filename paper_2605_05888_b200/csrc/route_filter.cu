@@ -187,6 +187,7 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 #pragma unroll
           for (int q = 0; q < 16; q += 4) *reinterpret_cast<float4*>(dst + c + q) = make_float4(f[q], f[q + 1], f[q + 2], f[q + 3]);
         }
+        __syncwarp();  // (the last tokens' lanes stored, those past T did not; the next loads want the whole warp)
       }
     }
     if (fail_site) sh->abort_flag = 1;

@@ -686,6 +686,34 @@ def test_expert_kernel_can_be_called_again_without_a_dispatch_in_between(split, 
         Hh.assert_output_close(Hh.to_host_f64(y), want["y"], w.dtype)
 
 
+@pytest.mark.parametrize("push", [0, 1])
+@pytest.mark.parametrize("rows", [(5, 40, 64), (129, 190, 7), (128, 200, 256)], ids=lambda r: "_".join(map(str, r)))
+def test_tensor_core_epilogue_lanes_that_do_not_store(rows, push):
+    """The one-CTA kernel's three epilogues (narrow form, M = 64 form, whole tiles) where some lanes of a warp store and
+    others do not: columns that end inside a warp's 32, rows without a source (push), the M = 64 form's unused lanes.  Every
+    row against the same call without row counts (whole tiles only)."""
+    E, H, F = len(rows), 328, 200
+    w = inputs.Workload("epi_lanes", T=sum(rows), H=H, E=E, R=1, K=1, F=F, dtype=BF16, seed=36)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    g = torch.Generator(device="cuda").manual_seed(36)
+    W = [torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.05, generator=g) for s in ((E, F, H), (E, F, H), (E, H, F))]
+    x = torch.empty((w.T, H), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    idx = torch.repeat_interleave(torch.arange(E, dtype=torch.int32), torch.tensor(rows)).reshape(-1, 1).cuda()
+    b = _dispatch_with_counters(w, plan, x, idx)
+    whole = torch.zeros_like(b["recv"])
+    plan.moe_expert_ffn(b["recv"], b["te"], *W, whole)
+    want = whole[b["slot"].flatten().long()]
+    if push:
+        got = torch.full((w.T, H), 7.0, dtype=torch.bfloat16, device="cuda")
+        plan.moe_expert_ffn_push(b["recv"], b["te"], b["src"], *W, got, b["tile_count"], b["rows_done"])
+    else:
+        out = torch.full_like(whole, 7.0)
+        plan.moe_expert_ffn(b["recv"], b["te"], *W, out, b["tile_count"], b["rows_done"])
+        got = out[b["slot"].flatten().long()]
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0) and torch.equal(got, want)
+
+
 @pytest.mark.parametrize("mode", MODES)
 def test_expert_id_outside_the_range_is_reported_and_dropped(mode):
     """A caller-supplied topk_idx with an id that is no expert: the status word says bad argument and names

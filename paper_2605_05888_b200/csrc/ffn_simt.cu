@@ -238,15 +238,14 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   int b = 0;
   uint32_t phase = 0;
   for (int k = 0; k < nk; ++k) {
-    if (!mbar_wait(smem_u32(&s_full[b]), phase, abort_flag, p.wait_ns)) {
-      failed = true;
-      break;
-    }
+    // (After a wait that ran out the stage is computed all the same, on whatever it holds: the vote behind it has the warp
+    // leave together.)
+    failed = !mbar_wait(smem_u32(&s_full[b]), phase, abort_flag, p.wait_ns);
     const uint32_t a_base = smem_u32(ring) + (uint32_t)(b * kStage) + (uint32_t)r0 * 128u;
     const uint32_t b_base = smem_u32(ring) + (uint32_t)(b * kStage + kA) + (uint32_t)c0 * 128u;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
-      if (half == 1 && issued > 0 && issued < nk) {  // the first thread: refill the stage used up in the last iteration
+      if (half == 1 && issued > 0 && issued < nk && !failed) {  // the first thread: refill the stage used up in the last iteration
         if (k > 0 && !mbar_wait(smem_u32(&s_empty[fill]), (uint32_t)((k - 1) / kStages) & 1u, abort_flag, p.wait_ns)) failed = true;
         else issue();
       }

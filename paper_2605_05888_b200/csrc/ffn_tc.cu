@@ -405,14 +405,14 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
     const int row_in_tile = quarter * 32 + lane;
     for (int local_item = 0; !fail_site; ++local_item) {
       const int slot = local_item & (kItemRing - 1);
-      if (!mbar_wait(smem_u32(&sh->item_bar[slot]), (uint32_t)(local_item / kItemRing) & 1u, abort_flag, wait_ns)) { fail_site = kWaitItem; break; }
+      if (!warp_agrees(mbar_wait(smem_u32(&sh->item_bar[slot]), (uint32_t)(local_item / kItemRing) & 1u, abort_flag, wait_ns))) { fail_site = kWaitItem; break; }
       const int entry = item_ring[slot];
       if (entry < 0) break;
       const int item = entry & ((1 << kThinShift) - 1), n16 = entry >> kThinShift;
       const Item it = decode(item);
       const int acc = local_item & 1;
       const uint32_t acc_phase = (uint32_t)(local_item >> 1) & 1u;
-      if (!mbar_wait(smem_u32(&sh->tmem_full[acc]), acc_phase, abort_flag, wait_ns, 500)) { fail_site = kWaitMbarEpi; break; }
+      if (!warp_agrees(mbar_wait(smem_u32(&sh->tmem_full[acc]), acc_phase, abort_flag, wait_ns, 500))) { fail_site = kWaitMbarEpi; break; }
       tc_fence_after();
       if (prm.item_ns && warp == 2 && lane == 0) prm.item_ns[4 * (size_t)item + 1] = globaltimer();  // MMAs complete
       const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kUmmaN);

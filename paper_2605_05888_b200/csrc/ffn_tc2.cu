@@ -454,7 +454,7 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
     int acc = 0;
     for (int local_item = 0; !fail_site; ++local_item) {
       const int slot = local_item & (kPairRing - 1);
-      if (!mbar_wait_cluster(smem_u32(&sh->item_bar[slot]), (uint32_t)(local_item / kPairRing) & 1u, abort_flag, wait_ns)) { fail_site = kWaitItem; break; }
+      if (!warp_agrees(mbar_wait_cluster(smem_u32(&sh->item_bar[slot]), (uint32_t)(local_item / kPairRing) & 1u, abort_flag, wait_ns))) { fail_site = kWaitItem; break; }
       const int item = item_ring[slot][0];
       if (item < 0) break;
       PairRows rows;
@@ -463,7 +463,7 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
       const bool wide = rows.n > 128;
       const uint32_t halves = wide ? 3u : 1u << acc;
       for (int a = 0; a < 2 && !fail_site; ++a)
-        if (((halves >> a) & 1u) && !mbar_wait(smem_u32(&sh->tmem_full[a]), (acc_phase >> a) & 1u, abort_flag, wait_ns)) fail_site = kWaitMbarEpi;
+        if (((halves >> a) & 1u) && !warp_agrees(mbar_wait(smem_u32(&sh->tmem_full[a]), (acc_phase >> a) & 1u, abort_flag, wait_ns))) fail_site = kWaitMbarEpi;
       if (fail_site) break;
       acc_phase ^= halves;
       tc_fence_after();

@@ -171,11 +171,8 @@ route_chains_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     int ring_stage = 0;
     uint32_t ring_phase = 0;
     for (int box0 = 0; box0 < nbox; box0 += p.boxes) {
-      if (!mbar_wait(smem_u32(&s_full[ring_stage]), ring_phase, abort_flag, p.wait_ns)) {
-        failed = true;
-        s_abort = 1;
-        break;
-      }
+      // A lane whose wait ran out stays with its warp (the others' may not have) and computes on whatever the stage holds.
+      failed |= !mbar_wait(smem_u32(&s_full[ring_stage]), ring_phase, abort_flag, p.wait_ns);
       const int boxes = min(p.boxes, nbox - box0);
       const uint32_t base = ring0 + (uint32_t)(ring_stage * stage_bytes);
       uint32_t xa[TM], wa[TN];
@@ -208,6 +205,7 @@ route_chains_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
       if (lane == 0) mbar_arrive(smem_u32(&s_empty[ring_stage]));
       if (++ring_stage == p.stages) { ring_stage = 0; ring_phase ^= 1u; }
     }
+    if (failed) s_abort = 1;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int t = tl + GT * i;

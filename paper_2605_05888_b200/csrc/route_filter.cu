@@ -163,7 +163,7 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     }
     // epilogue: the accumulator row of token t0 + 32 * (warp % 4) + lane, 16 experts at a time
     const int quarter = warp & 3;
-    if (!mbar_wait(smem_u32(&sh->acc_full), 0u, abort_flag, wait_ns, 200)) {
+    if (!warp_agrees(mbar_wait(smem_u32(&sh->acc_full), 0u, abort_flag, wait_ns, 200))) {
       fail_site = kWaitMbarEpi;
     } else {
       tc_fence_after();

@@ -117,6 +117,9 @@ __device__ __forceinline__ void tc2_commit_both(uint32_t bar) {  // arrives on `
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
       ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
+__device__ __forceinline__ void tc2_commit(uint32_t bar) {  // on `bar` of this CTA
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void tc2_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t accumulate) {
   asm volatile(
@@ -153,10 +156,11 @@ struct PairShared {
   unsigned long long tmem_full[2];        // used in each CTA
   unsigned long long tmem_empty[2];       // used in the leader
   unsigned long long item_bar[kPairRing];
-  unsigned long long drain;               // the MMA thread's last commit when it gives up
+  unsigned long long drain;               // the MMA thread's last commit after an abort
   int item_ring[kPairRing][2];            // item (-1: no more); rows of its two tiles, low and high half-word
+  int fills[2];                           // in the leader: the stages' fills that each CTA's producer has issued
   uint32_t tmem_base;
-  int abort_flag;
+  int abort_flag;                         // set in both CTAs or in neither
   int last_cta;
 };
 static_assert(sizeof(PairShared) <= 1024, "the epilogue's staging tiles follow");
@@ -269,7 +273,7 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
     if (lane == 0) {
       int stage = 0;
       uint32_t phase_bit = 0;
-      bool issued = false;
+      int fills = 0;
       int item = item_begin + first_claim;
       const uint64_t pol_once = l2_policy_evict_first(), pol_keep = l2_policy_evict_normal();
       for (int local_item = 0; !fail_site; ++local_item) {
@@ -369,17 +373,12 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
           };
           if (len0 > 0) load_rows(row0, len0);
           if (len1 > 0) load_rows(row1, len1);
-          issued = true;
+          ++fills;
           if (++stage == kPairStages) { stage = 0; phase_bit ^= 1u; }
         }
       }
-      if (fail_site || *abort_flag) {
-        abort_pair();
-        if (issued) {  // give copies in flight time to land before this CTA's shared memory goes away
-          const unsigned long long t0 = globaltimer();
-          while (globaltimer() - t0 < 200000ull) __nanosleep(1000);
-        }
-      }
+      if (fail_site) abort_pair();
+      st_cluster(map_to_cta(smem_u32(&sh->fills[rank]), 0), fills);
     }
   } else if (warp == 1) {
     // ===================== MMA issuer (leader CTA only) =====================
@@ -428,13 +427,6 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
           if ((halves >> a) & 1u) tc2_commit_both(smem_u32(&sh->tmem_full[a]));
       }
       if (fail_site) abort_pair();
-      if (fail_site || *abort_flag) {
-        // Giving up with MMAs possibly still running: wait (bounded) for all of them before tensor memory is freed.
-        tc2_commit_both(smem_u32(&sh->drain));
-        const unsigned long long t0 = globaltimer();
-        while (!mbar_try(smem_u32(&sh->drain), 0u))
-          if (globaltimer() - t0 > wait_ns + 1000000ull) break;
-      }
     }
   } else {
     // ===================== epilogue (both CTAs: their own 128 rows of each weight block) =====================
@@ -558,6 +550,29 @@ ffn_pair_kernel(const __grid_constant__ PairMaps maps, const FfnParams prm) {
   __syncthreads();
   cluster_sync_all();  // neither CTA leaves while its partner may still touch its shared memory or TMEM
   tc_fence_after();
+  if (sh->abort_flag) {  // (of both CTAs: the barrier above is behind every abort_pair)
+    // Whichever role gave up, copies and MMAs that others had issued may still be in flight: all of them have to end before
+    // the shared memory and the tensor memory are given up.  The MMAs: the issuing thread's commit comes after them.  The
+    // copies: a fill that only one CTA has issued lacks the other one's arrival; with that its phase completes when its bytes
+    // are there.  Both waits are bounded.
+    if (leader && warp == 1 && lane == 0) {
+      tc2_commit(smem_u32(&sh->drain));
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_try(smem_u32(&sh->drain), 0u))
+        if (globaltimer() - t0 > wait_ns + 1000000ull) break;
+    }
+    if (leader && threadIdx.x == 0) {
+      const int all = max(sh->fills[0], sh->fills[1]);
+      for (int g = min(sh->fills[0], sh->fills[1]); g < all; ++g) mbar_arrive(smem_u32(&sh->full[g % kPairStages]));
+      for (int g = max(0, all - kPairStages); g < all; ++g) {
+        const unsigned long long t0 = globaltimer();
+        while (!mbar_try(smem_u32(&sh->full[g % kPairStages]), (uint32_t)(g / kPairStages) & 1u))
+          if (globaltimer() - t0 > wait_ns + 1000000ull) break;
+      }
+    }
+    __syncthreads();
+    cluster_sync_all();
+  }
   pdl_trigger();
   probe.finish();
   if (threadIdx.x == 0) {  // the last CTA to leave puts the counters back to zero (see ffn_tc_kernel)

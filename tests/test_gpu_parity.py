@@ -773,6 +773,51 @@ def test_consumer_wait_runs_out_and_reports_it(kernel):
     Hh.assert_output_close(Hh.to_host_f64(y), ref["y"], w.dtype)
 
 
+@pytest.mark.parametrize("split", [1, 2])
+@pytest.mark.parametrize("kernel", [0, 2])
+def test_consumer_wait_runs_out_with_other_tiles_in_flight(kernel, split):
+    """Some tiles are ready and computed while others never become so: the wait (20 ms) runs out with loads and MMAs of the
+    ready tiles in flight.  The kernel lands them, reports the timeout and returns; the layer then gives its bytes again."""
+    w = inputs.Workload("wait_busy", T=1000, H=1544, E=4, R=1, K=2, F=1040, dtype=BF16, zipf_s=0.7, seed=25)
+    args = [Hh.to_dev(a) for a in Hh.oracle_inputs(w)]
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, ffn_kernel=kernel, ffn_split=split, wait_limit_ns=20_000_000)
+    y, y2 = (torch.empty((w.T, w.H), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    plan.moe_layer(*args, y)
+    b = _dispatch_with_counters(w, plan, args[0], plan.layer_tensor(0))
+    owned = (b["te"] >= 0).nonzero().flatten()
+    for ready in (1, int(owned.numel()) // 2, int(owned.numel()) - 1):
+        counts = torch.zeros_like(b["tile_count"])
+        counts[owned[:ready]] = 128
+        plan.moe_expert_ffn(b["recv"], b["te"], *args[3:], torch.zeros_like(b["recv"]), counts, torch.zeros_like(b["rows_done"]))
+        assert plan.moe_last_status()[0] == -6       # MOE_ERR_TIMEOUT
+        plan.moe_layer(*args, y2)
+        assert plan.moe_last_status() == (0, 0) and torch.equal(y, y2)
+
+
+@pytest.mark.parametrize("split", [1, 2])
+@pytest.mark.parametrize("kernel", [2])
+def test_expert_kernel_with_a_tiny_wait_limit_reports_or_computes(kernel, split):
+    """Limits shorter than a load, an MMA or an item take: any role may give up first, with what the others have issued still
+    in flight.  Every call either reports the timeout or has computed its bytes, and the next plan's layer is untouched."""
+    w = inputs.Workload("wait_tiny", T=1000, H=1544, E=4, R=1, K=2, F=1040, dtype=BF16, zipf_s=0.7, seed=26)
+    args = [Hh.to_dev(a) for a in Hh.oracle_inputs(w)]
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, ffn_kernel=kernel, ffn_split=split)
+    y, y2 = (torch.empty((w.T, w.H), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    plan.moe_layer(*args, y)
+    b = _dispatch_with_counters(w, plan, args[0], plan.layer_tensor(0))
+    want = torch.zeros_like(b["recv"])
+    plan.moe_expert_ffn(b["recv"], b["te"], *args[3:], want, b["tile_count"], b["rows_done"])
+    used = b["slot"].flatten().long()
+    for limit in (1, 500, 2_000, 5_000, 20_000, 100_000):
+        tiny = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, ffn_kernel=kernel, ffn_split=split, wait_limit_ns=limit)
+        out = torch.zeros_like(want)
+        tiny.moe_expert_ffn(b["recv"], b["te"], *args[3:], out, b["tile_count"], b["rows_done"])
+        code = tiny.moe_last_status()[0]
+        assert code in (0, -6) and (code != 0 or torch.equal(out[used], want[used]))
+        plan.moe_layer(*args, y2)
+        assert plan.moe_last_status() == (0, 0) and torch.equal(y, y2)
+
+
 # ------------------------------------------------------------------ dispatch and experts in one launch
 OVERLAP_CASES = [SMALL[3], SMALL[4], SMALL[5], SMALL[7],
                  inputs.Workload("three_tiles", T=700, H=320, E=4, R=2, K=2, F=392, dtype=BF16),

@@ -62,8 +62,9 @@ struct TcShared {
   unsigned long long tmem_full[2];
   unsigned long long tmem_empty[2];
   unsigned long long item_bar[kItemRing];
-  unsigned long long drain;  // the MMA thread's last commit when it gives up: nothing of its own is in flight after it
+  unsigned long long drain;  // the MMA thread's last commit after an abort: nothing of its own is in flight behind it
   int item_ring[kItemRing];
+  int fills;                 // fills of the stages that the producer has issued
   uint32_t tmem_base;
   int abort_flag;
   int last_cta;
@@ -199,9 +200,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
     if (lane == 0) {
       int stage = 0;
       uint32_t phase_bit = 0;
-      int armed[kStages];
-#pragma unroll
-      for (int s = 0; s < kStages; ++s) armed[s] = 0;
+      int fills = 0;
       int item = item_begin + first_claim;
       const uint64_t pol_stream = l2_policy_evict_first();
       for (int local_item = 0; !fail_site; ++local_item) {
@@ -319,26 +318,14 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
           } else {
             tma_load_4d(b_dst, &map_bd, full, kb * kBK, it.nb * 256, it.e % prm.tp, it.e / prm.tp);
           }
-#pragma unroll
-          for (int s = 0; s < kStages; ++s)
-            if (s == stage) armed[s] += 1;
+          ++fills;
           if (++stage == kStages) { stage = 0; phase_bit ^= 1u; }
         }
         if (trace) trace[3] = globaltimer();  // every load of the item issued
         item = next_item;
       }
-      if (fail_site || *abort_flag) {
-        // Leave no copy in flight: wait (bounded) for the last fill of every stage.
-        sh->abort_flag = 1;
-#pragma unroll
-        for (int s = 0; s < kStages; ++s) {
-          if (armed[s] == 0) continue;
-          const uint32_t par = (uint32_t)((armed[s] - 1) & 1);
-          const unsigned long long t0 = globaltimer();
-          while (!mbar_try(smem_u32(&sh->full[s]), par))
-            if (globaltimer() - t0 > wait_ns) break;
-        }
-      }
+      if (fail_site) sh->abort_flag = 1;
+      sh->fills = fills;
     }
   } else if (warp == 1) {
     // ===================== MMA issuer =====================
@@ -387,14 +374,6 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
         tc_commit(smem_u32(&sh->tmem_full[acc]));  // accumulator complete
       }
       if (fail_site) sh->abort_flag = 1;
-      if (fail_site || *abort_flag) {
-        // Giving up with MMAs possibly still running: they read the stages and write tensor memory, so wait
-        // (bounded) for all of them before the CTA frees either.
-        tc_commit(smem_u32(&sh->drain));
-        const unsigned long long t0 = globaltimer();
-        while (!mbar_try(smem_u32(&sh->drain), 0u))
-          if (globaltimer() - t0 > wait_ns + 1000000ull) break;
-      }
     }
   } else {
     // ===================== epilogue =====================
@@ -544,6 +523,24 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (sh->abort_flag) {
+    // Whichever role gave up, what the others had issued may still be in flight: the MMAs read the stages and write tensor
+    // memory, the copies write the stages.  All of them end (both waits are bounded) before the CTA frees either.
+    if (warp == 1 && lane == 0) {
+      tc_commit(smem_u32(&sh->drain));
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_try(smem_u32(&sh->drain), 0u))
+        if (globaltimer() - t0 > wait_ns + 1000000ull) break;
+    }
+    if (threadIdx.x == 0) {
+      for (int g = max(0, sh->fills - kStages); g < sh->fills; ++g) {
+        const unsigned long long t0 = globaltimer();
+        while (!mbar_try(smem_u32(&sh->full[g % kStages]), (uint32_t)(g / kStages) & 1u))
+          if (globaltimer() - t0 > wait_ns + 1000000ull) break;
+      }
+    }
+    __syncthreads();
+  }
   pdl_trigger();
   probe.finish();
   if (threadIdx.x == 0) {

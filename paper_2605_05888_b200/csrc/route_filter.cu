@@ -52,6 +52,7 @@ struct RfShared {
   unsigned long long empty[kStages];
   unsigned long long acc_full;
   unsigned long long drain;
+  int fills;  // stages that the producer has filled
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -93,10 +94,8 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 
   if (warp == 0) {
     if (lane == 0) {  // TMA producer: the tokens' x tile and all experts' Wr block, 64 columns of h per stage
-      int stage = 0, armed[kStages];
+      int stage = 0, fills = 0;
       uint32_t phase_bit = 0;
-#pragma unroll
-      for (int s = 0; s < kStages; ++s) armed[s] = 0;
       for (int kb = 0; kb < KB; ++kb) {
         if (!mbar_wait(smem_u32(&sh->empty[stage]), phase_bit ^ 1u, abort_flag, wait_ns)) { fail_site = kWaitMbarTma; break; }
         const uint32_t full = smem_u32(&sh->full[stage]);
@@ -104,21 +103,11 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         mbar_expect_tx(full, (uint32_t)(kABytes + kBBytes / 2));
         tma_load_2d(a_dst, &map_x, full, kb * kBK, t0);   // rows past T and columns past H arrive as zeros
         tma_load_2d(a_dst + kABytes, &map_w, full, kb * kBK, e0);  // 128 experts' rows
-#pragma unroll
-        for (int s = 0; s < kStages; ++s)
-          if (s == stage) armed[s] += 1;
+        ++fills;
         if (++stage == kStages) { stage = 0; phase_bit ^= 1u; }
       }
-      if (fail_site || *abort_flag) {  // leave no copy in flight
-        sh->abort_flag = 1;
-#pragma unroll
-        for (int s = 0; s < kStages; ++s) {
-          if (armed[s] == 0) continue;
-          const unsigned long long ts = globaltimer();
-          while (!mbar_try(smem_u32(&sh->full[s]), (uint32_t)((armed[s] - 1) & 1)))
-            if (globaltimer() - ts > wait_ns + 1000000ull) break;
-        }
-      }
+      if (fail_site) sh->abort_flag = 1;
+      sh->fills = fills;
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer: D[128 tokens, 256 experts] += x tile * Wr block^T
@@ -139,12 +128,6 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
       }
       if (!fail_site) tc_commit(smem_u32(&sh->acc_full));
       if (fail_site) sh->abort_flag = 1;
-      if (fail_site || *abort_flag) {  // nothing of this thread's may still run when the CTA frees tensor memory
-        tc_commit(smem_u32(&sh->drain));
-        const unsigned long long ts = globaltimer();
-        while (!mbar_try(smem_u32(&sh->drain), 0u))
-          if (globaltimer() - ts > wait_ns + 1000000ull) break;
-      }
     }
   } else {
     // While the main loop runs: |w_e|^2 for this CTA's share of the experts (the refine kernel's error bound).
@@ -196,6 +179,22 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (sh->abort_flag) {  // whichever role gave up: MMAs and copies in flight end (bounded) before their memory is freed
+    if (warp == 1 && lane == 0) {
+      tc_commit(smem_u32(&sh->drain));
+      const unsigned long long ts = globaltimer();
+      while (!mbar_try(smem_u32(&sh->drain), 0u))
+        if (globaltimer() - ts > wait_ns + 1000000ull) break;
+    }
+    if (threadIdx.x == 0) {
+      for (int g = max(0, sh->fills - kStages); g < sh->fills; ++g) {
+        const unsigned long long ts = globaltimer();
+        while (!mbar_try(smem_u32(&sh->full[g % kStages]), (uint32_t)(g / kStages) & 1u))
+          if (globaltimer() - ts > wait_ns + 1000000ull) break;
+      }
+    }
+    __syncthreads();
+  }
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
 }

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/moehub.h"
+#include "smem_attr.h"
 
 namespace moehub {
 
@@ -132,20 +133,6 @@ template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args&&... args) {
   return launch_maybe_pdl(true, kern, grid, block, smem, st, static_cast<Args&&>(args)...);
-}
-
-// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) applies to the CURRENT device only, so the "already
-// set" flag of a kernel is kept per device (a process may hold plans on several GPUs).  Setting it twice
-// is harmless, so concurrent first calls need no lock.
-struct SmemAttrOnce {
-  size_t set[64] = {};  // bytes the attribute was last set to, per device
-};
-template <typename Kern>
-inline cudaError_t ensure_dynamic_smem(Kern kern, size_t bytes, int device, SmemAttrOnce& once) {
-  if (device >= 0 && device < 64 && once.set[device] >= bytes) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess && device >= 0 && device < 64) once.set[device] = bytes;
-  return e;
 }
 
 // ---- launchers (defined in the other .cu files); each returns a cudaError_t as int ------------

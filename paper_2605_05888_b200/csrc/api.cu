@@ -254,10 +254,10 @@ int moe_dispatch(moe_plan_t* p, const void* d_x, const int32_t* d_topk_idx, void
 
 static int ffn_dispatch(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu,
                         const void* wd, void* out_rows, const int* tile_count, const int* rows_done,
-                        cudaStream_t st) {
+                        cudaStream_t st, bool own) {
   if (p->cfg.dtype == MOE_DTYPE_BF16 && p->cfg.ffn_kernel != 1)
-    return launch_ffn_tc(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
-  return launch_ffn_simt(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
+    return launch_ffn_tc(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st, own);
+  return launch_ffn_simt(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st, own);
 }
 
 int moe_expert_ffn(moe_plan_t* p, const void* d_recv, const int32_t* d_tile_expert, const void* d_wg,
@@ -270,7 +270,7 @@ int moe_expert_ffn(moe_plan_t* p, const void* d_recv, const int32_t* d_tile_expe
   p->launches = 0;
   if ((d_tile_count == nullptr) != (d_rows_done == nullptr)) return MOE_ERR_ARG;
   int rc = ffn_dispatch(p, d_recv, d_tile_expert, d_wg, d_wu, d_wd, d_out_rows, d_tile_count, d_rows_done,
-                        (cudaStream_t)stream);
+                        (cudaStream_t)stream, false);
   return rc == 0 ? MOE_OK : (rc < 0 ? rc : MOE_ERR_CUDA);
 }
 
@@ -285,7 +285,7 @@ int moe_expert_ffn_push(moe_plan_t* p, const void* d_recv, const int32_t* d_tile
   if ((d_tile_count == nullptr) != (d_rows_done == nullptr)) return MOE_ERR_ARG;
   p->launches = 0;
   int rc = launch_ffn_tc(p, d_recv, d_tile_expert, d_wg, d_wu, d_wd, d_staged, d_tile_count, d_rows_done,
-                         (cudaStream_t)stream, nullptr, nullptr, d_src_info);
+                         (cudaStream_t)stream, false, nullptr, nullptr, d_src_info);
   return rc == 0 ? MOE_OK : (rc < 0 ? rc : MOE_ERR_CUDA);
 }
 
@@ -348,11 +348,11 @@ int moe_layer(moe_plan_t* p, const void* d_x, const void* d_wr, const float* d_b
   mark(p, 2, st);
   const bool push = c.combine_mode == 1;  // the expert kernel returns every row to its token's position itself
   if (overlap || push) {
-    int rc = launch_ffn_tc(p, s.recv, s.tile_expert, d_wg, d_wu, d_wd, s.out_rows, s.tile_count, s.rows_done, st,
+    int rc = launch_ffn_tc(p, s.recv, s.tile_expert, d_wg, d_wu, d_wd, s.out_rows, s.tile_count, s.rows_done, st, true,
                            overlap ? d_x : nullptr, overlap ? s.topk_idx : nullptr, push ? s.src_info : nullptr);
     if (rc != 0) return rc < 0 && rc != MOE_ERR_CUDA ? rc : cuda_failed(3);
   } else if (!p->cfg.identity_experts) {
-    int rc = ffn_dispatch(p, s.recv, s.tile_expert, d_wg, d_wu, d_wd, s.out_rows, s.tile_count, s.rows_done, st);
+    int rc = ffn_dispatch(p, s.recv, s.tile_expert, d_wg, d_wu, d_wd, s.out_rows, s.tile_count, s.rows_done, st, true);
     if (rc != 0) return rc < 0 && rc != MOE_ERR_CUDA ? rc : cuda_failed(3);
   } else {
     mark(p, 3, st);

@@ -156,15 +156,16 @@ PrepArgs make_prep(moe_plan* p, int* expert_count, int* tile_expert, int* src_in
 // staged: rows holds assignment (t, k) at row t*K+k (push-style combine); slot_of then only tells dropped assignments.
 int launch_combine(moe_plan* p, const void* rows, const int* slot_of, const float* topk_w, void* y,
                    cudaStream_t st, bool staged = false);
-// tile_count / rows_done: how many rows each tile holds (nullptr: every tile is computed whole).
+// tile_count / rows_done: how many rows each tile holds (nullptr: every tile is computed whole).  own: table and counters are
+// what this plan's dispatch leaves inside moe_layer; a caller's may own any tiles, and its counters may be incomplete.
 int launch_ffn_simt(moe_plan* p, const void* recv, const int* tile_expert, const void* wg,
                     const void* wu, const void* wd, void* out_rows, const int* tile_count, const int* rows_done,
-                    cudaStream_t st);
+                    cudaStream_t st, bool own);
 // tile_count / rows_done: availability counters the GEMM1 producer waits on before it reads a tile
 // (nullptr: the rows are complete when the kernel starts).
 int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const void* wg,
                   const void* wu, const void* wd, void* out_rows, const int* tile_count,
-                  const int* rows_done, cudaStream_t st, const void* overlap_x = nullptr,
+                  const int* rows_done, cudaStream_t st, bool own, const void* overlap_x = nullptr,
                   const int* overlap_idx = nullptr, const int* push_src = nullptr);
 // A handful of tokens: everything of the layer that follows the router, dispatch and combine included (ffn_few.cu).
 bool few_layer_applies(const moe_plan* p);

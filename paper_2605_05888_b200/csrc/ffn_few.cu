@@ -285,7 +285,7 @@ static int launch_few(moe_plan* p, const FewParams& q, const void* recv, const v
 }
 
 int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
-                   const int* push_src, cudaStream_t st) {
+                   const int* push_src, cudaStream_t st, bool own) {
   FewParams q = {};
   q.tp = p->tp;
   q.tile_expert = prm.tile_expert;
@@ -297,8 +297,7 @@ int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu
   q.wait_ns = prm.wait_ns;
   q.status = prm.status;
   const int T = p->cfg.T;
-  const bool any = prm.tile_count != p->s.tile_count;  // inside moe_layer the table is the dispatch's own
-#define MOEHUB_FEW(R) (any ? launch_few<R, true>(p, q, recv, wg, wu, wd, prm.out, push_src, st) : launch_few<R, false>(p, q, recv, wg, wu, wd, prm.out, push_src, st))
+#define MOEHUB_FEW(R) (own ? launch_few<R, false>(p, q, recv, wg, wu, wd, prm.out, push_src, st) : launch_few<R, true>(p, q, recv, wg, wu, wd, prm.out, push_src, st))
   if (T <= 1) return MOEHUB_FEW(1);
   if (T <= 2) return MOEHUB_FEW(2);
   if (T <= 4) return MOEHUB_FEW(4);

@@ -131,82 +131,84 @@ __device__ __forceinline__ float sum_x2(unsigned long long v) {
   return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
 }
 
-// WR: how many of the four warps stand along the rows (the others beside them, along the columns).
+struct Fp32Shared {
+  unsigned long long full[4], empty[4];
+  int abort;
+  int col, tile, part, tile_rows;  // the block (col < 0: none)
+  int next;                        // the CTA's next block, -1: there is none
+};
+
+// Block number id in the order described below: where it lies.  Warp 0 calls; the others see it behind a barrier.
+template <int BM, int NOUT>
+__device__ __forceinline__ void fp32_find_block(const Fp32Params& p, Fp32Shared& s, int id) {
+  constexpr int kParts = kTileRows / BM;
+  const int lane = threadIdx.x % 32;
+  const bool counted = p.tile_count != nullptr && *p.rows_done >= p.total_rows;
+  auto blocks_of = [&](int t) {  // a tile without an owner, or owned by no expert at all (a caller's own table), has none
+    const int e = t < p.P ? p.tile_expert[t] : -1;
+    return e < 0 || e >= p.E ? 0 : counted ? (min(kTileRows, p.tile_count[t]) + BM - 1) / BM : kParts;
+  };
+  int total = 0;
+  for (int t = lane; t < p.P; t += 32) total += blocks_of(t);
+  total = __reduce_add_sync(0xffffffffu, total);
+  int col = -1, block = 0;
+  if (total > 0) {
+    col = id / total;
+    block = id - col * total;
+  }
+  const int cols = (p.N + NOUT - 1) / NOUT;
+  if (col >= cols) col = -1;
+  if (lane == 0) {
+    s.col = col;
+    s.next = (long long)id + gridDim.x < (long long)total * cols ? id + (int)gridDim.x : -1;
+  }
+  for (int t = lane, before = 0; col >= 0 && before <= block; t += 32) {
+    const int mine = blocks_of(t);
+    int incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    const int first = before + incl - mine;
+    if (block >= first && block < first + mine) {
+      s.tile = t;
+      s.part = block - first;
+      s.tile_rows = counted ? min(kTileRows, p.tile_count[t]) : kTileRows;
+    }
+    before += __shfl_sync(0xffffffffu, incl, 31);
+  }
+}
+
+// The block in s.  Warps without rows leave at once; a wait that ran out is left in s.abort.
 template <int TM, int TN, int WR, bool SWIGLU>
-__global__ void __launch_bounds__(kF32Threads, (kF32Ctas<TM, TN, WR>))
-ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b1,
-                const __grid_constant__ CUtensorMap map_b2, const Fp32Params p) {
+__device__ __forceinline__ void fp32_block(const CUtensorMap& map_a, const CUtensorMap& map_b1, const CUtensorMap& map_b2,
+                                           const Fp32Params& p, Fp32Shared& s, uint8_t* ring) {
   constexpr int WN = kF32Warps / WR, BM = WR * 2 * TM, BN = WN * 16 * TN;  // rows and columns of B per CTA
   constexpr int NOUT = SWIGLU ? BN / 2 : BN;             // columns of the result per CTA
   constexpr int kA = BM * kF32K * 4, kStage = kF32StageBytes<TM, TN, WR>;
   constexpr int kStages = kF32Stages<TM, TN, WR>;
-  constexpr int kParts = kTileRows / BM;
-  __shared__ unsigned long long s_full[kStages], s_empty[kStages];
-  __shared__ int s_abort, s_block[4];
-  extern __shared__ uint8_t f32_dyn[];
-  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(f32_dyn) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  pdl_wait();
-  pdl_trigger();
-  // This CTA's block of rows and columns: the blocks that have rows come first, one column of blocks after the other, so
-  // they spread over all SMs.  (With a CTA for every block a tile could have, the empty ones leave at once but the others
-  // stand at every fourth place: 37 of the 148 SMs had work.  T 64, H 1024, 32 experts,
-  // top-4, F 2048: layer 329 -> 252 us; T 100, H 512, 8 experts, top-2, F 512: 80 -> 69.)
-  if (warp == 0) {
-    const bool counted = p.tile_count != nullptr && *p.rows_done >= p.total_rows;
-    auto blocks_of = [&](int t) {  // a tile without an owner, or owned by no expert at all (a caller's own table), has none
-      const int e = t < p.P ? p.tile_expert[t] : -1;
-      return e < 0 || e >= p.E ? 0 : counted ? (min(kTileRows, p.tile_count[t]) + BM - 1) / BM : kParts;
-    };
-    int total = 0;
-    for (int t = lane; t < p.P; t += 32) total += blocks_of(t);
-    total = __reduce_add_sync(0xffffffffu, total);
-    int col = -1, block = 0;
-    if (total > 0) {
-      col = blockIdx.x / total;
-      block = blockIdx.x - col * total;
-    }
-    if (col >= (p.N + NOUT - 1) / NOUT) col = -1;
-    if (lane == 0) s_block[0] = col;
-    for (int t = lane, before = 0; col >= 0 && before <= block; t += 32) {
-      const int mine = blocks_of(t);
-      int incl = mine;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-      }
-      const int first = before + incl - mine;
-      if (block >= first && block < first + mine) {
-        s_block[1] = t;
-        s_block[2] = block - first;
-        s_block[3] = counted ? min(kTileRows, p.tile_count[t]) : kTileRows;
-      }
-      before += __shfl_sync(0xffffffffu, incl, 31);
-    }
-  }
-  __syncthreads();
-  if (s_block[0] < 0) return;
-  const int n0 = s_block[0] * NOUT, tile = s_block[1], part = s_block[2], rows = min(s_block[3] - part * BM, BM);
+  const int n0 = s.col * NOUT, tile = s.tile, part = s.part, rows = min(s.tile_rows - part * BM, BM);
   const int e = p.tile_expert[tile];
   const int rw = warp % WR, cw = warp / WR;
   const int live_rows = (rows + 2 * TM - 1) / (2 * TM);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(smem_u32(&s_full[s]), 1);
-      mbar_init(smem_u32(&s_empty[s]), min(live_rows, WR) * WN);
+    for (int i = 0; i < kStages; ++i) {
+      mbar_init(smem_u32(&s.full[i]), 1);
+      mbar_init(smem_u32(&s.empty[i]), min(live_rows, WR) * WN);
     }
-    s_abort = 0;
+    s.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   if (rw >= live_rows) return;
-  volatile int* abort_flag = &s_abort;
+  volatile int* abort_flag = &s.abort;
   const int nk = (p.Kd + kF32K - 1) / kF32K;
   const size_t row0 = (size_t)tile * kTileRows + part * BM;
   int issued = 0, fill = 0;  // copies issued so far (by the first thread), the stage the next one goes to
   auto issue = [&]() {
-    const uint32_t bar = smem_u32(&s_full[fill]), dst = smem_u32(ring) + (uint32_t)(fill * kStage);
+    const uint32_t bar = smem_u32(&s.full[fill]), dst = smem_u32(ring) + (uint32_t)(fill * kStage);
     const int kc = issued * kF32K;
     mbar_expect_tx(bar, (uint32_t)kStage);  // rows and columns outside a matrix arrive as zeros
     tma_load_2d(dst, &map_a, bar, kc, (int)row0);
@@ -240,13 +242,13 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   for (int k = 0; k < nk; ++k) {
     // (After a wait that ran out the stage is computed all the same, on whatever it holds: the vote behind it has the warp
     // leave together.)
-    failed = !mbar_wait(smem_u32(&s_full[b]), phase, abort_flag, p.wait_ns);
+    failed = !mbar_wait(smem_u32(&s.full[b]), phase, abort_flag, p.wait_ns);
     const uint32_t a_base = smem_u32(ring) + (uint32_t)(b * kStage) + (uint32_t)r0 * 128u;
     const uint32_t b_base = smem_u32(ring) + (uint32_t)(b * kStage + kA) + (uint32_t)c0 * 128u;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
       if (half == 1 && issued > 0 && issued < nk && !failed) {  // the first thread: refill the stage used up in the last iteration
-        if (k > 0 && !mbar_wait(smem_u32(&s_empty[fill]), (uint32_t)((k - 1) / kStages) & 1u, abort_flag, p.wait_ns)) failed = true;
+        if (k > 0 && !mbar_wait(smem_u32(&s.empty[fill]), (uint32_t)((k - 1) / kStages) & 1u, abort_flag, p.wait_ns)) failed = true;
         else issue();
       }
 #pragma unroll
@@ -268,16 +270,16 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
     failed = __any_sync(0xffffffffu, failed);
     if (failed) break;
-    if (lane == 0) mbar_arrive(smem_u32(&s_empty[b]));
+    if (lane == 0) mbar_arrive(smem_u32(&s.empty[b]));
     if (++b == kStages) { b = 0; phase ^= 1u; }
   }
   if (failed) {
-    s_abort = 1;
+    s.abort = 1;
     set_status(p.status, MOE_ERR_TIMEOUT, kWaitMbarTma);
     // no copy may still be landing when the CTA's shared memory goes away (only the first thread has issued any)
     for (int g = max(0, issued - kStages); g < issued; ++g) {
       const unsigned long long ts = globaltimer();
-      while (!mbar_try(smem_u32(&s_full[g % kStages]), (uint32_t)(g / kStages) & 1u))
+      while (!mbar_try(smem_u32(&s.full[g % kStages]), (uint32_t)(g / kStages) & 1u))
         if (globaltimer() - ts > p.wait_ns + 1000000ull) break;
     }
     return;
@@ -297,6 +299,47 @@ ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   }
 }
 
+// A CTA computes one block of rows and columns, and with ANY goes on to the next ones a grid apart while there are any (a grid
+// that holds every block a caller's table could ask for would be mostly empty: see launch_fp32_gemm).  The blocks that have
+// rows come first, one column of blocks after the other, so they spread over all SMs.  (With a CTA for every block a tile could
+// have, the empty ones leave at once but the others stand at every fourth place: 37 of the 148 SMs had work.  T 64, H 1024,
+// 32 experts, top-4, F 2048: layer 329 -> 252 us; T 100, H 512, 8 experts, top-2, F 512: 80 -> 69.)
+// WR: how many of the four warps stand along the rows (the others beside them, along the columns).
+template <int TM, int TN, int WR, bool SWIGLU, bool ANY>
+__global__ void __launch_bounds__(kF32Threads, (kF32Ctas<TM, TN, WR>))
+ffn_fp32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b1,
+                const __grid_constant__ CUtensorMap map_b2, const Fp32Params p) {
+  constexpr int BM = WR * 2 * TM, BN = kF32Warps / WR * 16 * TN, NOUT = SWIGLU ? BN / 2 : BN;
+  constexpr int kStages = kF32Stages<TM, TN, WR>;
+  static_assert(kStages <= 4, "barriers in Fp32Shared");
+  __shared__ Fp32Shared s;
+  extern __shared__ uint8_t f32_dyn[];
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(f32_dyn) + 1023) & ~(uintptr_t)1023);
+  pdl_wait();
+  pdl_trigger();
+  if (threadIdx.x < 32) fp32_find_block<BM, NOUT>(p, s, blockIdx.x);
+  __syncthreads();
+  if (s.col < 0) return;
+  for (;;) {
+    fp32_block<TM, TN, WR, SWIGLU>(map_a, map_b1, map_b2, p, s, ring);
+    if (!ANY || s.next < 0) return;
+    __syncthreads();
+    if (s.abort) return;
+    if (threadIdx.x == 0) {  // (every copy has been waited for, every arrival made)
+      for (int i = 0; i < kStages; ++i) {
+        mbar_inval(smem_u32(&s.full[i]));
+        mbar_inval(smem_u32(&s.empty[i]));
+      }
+    }
+    if (threadIdx.x < 32) {
+      const int id = s.next;
+      __syncwarp();  // (the search writes the next one)
+      fp32_find_block<BM, NOUT>(p, s, id);
+    }
+    __syncthreads();
+  }
+}
+
 // fp32 tensor, innermost dimension first, rows of 32 elements by box_rows, 128-byte swizzle.
 static int make_map_f32(EncodeTiledFn enc, CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims,
                         const cuuint64_t* strides, int box_rows) {
@@ -307,8 +350,8 @@ static int make_map_f32(EncodeTiledFn enc, CUtensorMap* m, const void* base, int
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
 }
 
-template <int TM, int TN, int WR, bool SWIGLU>
-static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
+template <int TM, int TN, int WR, bool SWIGLU, bool ANY>
+static int launch_fp32_grid(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
                             const Fp32Params& q, cudaStream_t st) {
   constexpr int BM = WR * 2 * TM, BN = kF32Warps / WR * 16 * TN, NOUT = SWIGLU ? BN / 2 : BN;
   const cuuint64_t E = (cuuint64_t)p->cfg.E, K = (cuuint64_t)q.Kd, N = (cuuint64_t)q.N, tp = (cuuint64_t)p->tp;
@@ -325,22 +368,32 @@ static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const
     if ((rc = make_map_f32(enc, &mb1, b1, 4, dims, str, BN)) != MOE_OK) return rc;
     mb2 = mb1;
   }
-  auto kern = ffn_fp32_kernel<TM, TN, WR, SWIGLU>;
+  auto kern = ffn_fp32_kernel<TM, TN, WR, SWIGLU, ANY>;
   constexpr size_t smem = 1024 + (size_t)kF32Stages<TM, TN, WR> * kF32StageBytes<TM, TN, WR>;
   static SmemAttrOnce once;
   if (ensure_dynamic_smem(kern, smem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
-  // As many blocks of rows as there can be: inside moe_layer the counts add up to T * K, so besides full blocks there is at
-  // most one per tile; a caller's counters may be incomplete, and its tiles are whole then.
-  const long long row_blocks = q.tile_count == p->s.tile_count ? min((long long)p->P * (kTileRows / BM), (long long)q.total_rows / BM + p->P)
-                                                       : (long long)p->P * (kTileRows / BM);
-  const dim3 grid((unsigned)(row_blocks * ((q.N + NOUT - 1) / NOUT)));
+  // Inside moe_layer a CTA per block that there can be: the counts add up to T * K, so besides full blocks there is at most
+  // one per tile.  A caller's table may have any number of whole tiles or of empty ones, and each CTA walks the table: not
+  // more than 16 CTAs per SM then, five times what is resident.  Measured, moe_expert_ffn with counters, us, a CTA per block
+  // there could be / this: 1024 tiles of static regions, 500 tokens, H 256, F 512 193 / 83; 12 tiles, T 256, H 128, F 256 23.6 /
+  // 25.6; 31 tiles, T 1000, H 1024, F 2048 722 / 708; 81 tiles, T 700, H 512, F 512 189 / 196; 32 and 64 per SM: 83 and 95 on the first.
+  const long long cols = (q.N + NOUT - 1) / NOUT, all = (long long)p->P * (kTileRows / BM) * cols;
+  const int sms = p->sm_count > 0 ? p->sm_count : 148;
+  const dim3 grid((unsigned)min(all, ANY ? 16ll * sms : ((long long)q.total_rows / BM + p->P) * cols));
   p->launches += 1;
   return launch_pdl(kern, grid, dim3(kF32Threads), smem, st, ma, mb1, mb2, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
 }
 
+template <int TM, int TN, int WR, bool SWIGLU>
+static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
+                            const Fp32Params& q, cudaStream_t st, bool own) {
+  return own ? launch_fp32_grid<TM, TN, WR, SWIGLU, false>(p, enc, A, b1, b2, q, st)
+             : launch_fp32_grid<TM, TN, WR, SWIGLU, true>(p, enc, A, b1, b2, q, st);
+}
+
 // Both GEMMs of an fp32 plan.
 static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu, const void* wd,
-                       void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st) {
+                       void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st, bool own) {
   const moe_config_t& c = p->cfg;
   EncodeTiledFn enc;
   int rc = get_encoder(p, &enc);
@@ -379,21 +432,21 @@ static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, co
   q.Kd = c.H;
   q.C = (float*)p->s.inter;
   const bool enough1 = blocks * ((c.F + 63) / 64) >= 2 * sms, enough2 = blocks * ((c.H + 127) / 128) >= 3 * sms / 2;
-  if (shape == 2 && enough1) rc = launch_fp32_gemm<8, 8, 4, true>(p, enc, recv, wg, wu, q, st);
-  else if (shape == 1 && enough1) rc = launch_fp32_gemm<4, 8, 4, true>(p, enc, recv, wg, wu, q, st);
-  else if (along(c.F, 128) == 1) rc = launch_fp32_gemm<4, 4, 1, true>(p, enc, recv, wg, wu, q, st);
-  else if (along(c.F, 128) == 2) rc = launch_fp32_gemm<4, 4, 2, true>(p, enc, recv, wg, wu, q, st);
-  else rc = launch_fp32_gemm<4, 4, 4, true>(p, enc, recv, wg, wu, q, st);
+  if (shape == 2 && enough1) rc = launch_fp32_gemm<8, 8, 4, true>(p, enc, recv, wg, wu, q, st, own);
+  else if (shape == 1 && enough1) rc = launch_fp32_gemm<4, 8, 4, true>(p, enc, recv, wg, wu, q, st, own);
+  else if (along(c.F, 128) == 1) rc = launch_fp32_gemm<4, 4, 1, true>(p, enc, recv, wg, wu, q, st, own);
+  else if (along(c.F, 128) == 2) rc = launch_fp32_gemm<4, 4, 2, true>(p, enc, recv, wg, wu, q, st, own);
+  else rc = launch_fp32_gemm<4, 4, 4, true>(p, enc, recv, wg, wu, q, st, own);
   if (rc != 0) return rc;
   mark(p, 4, st);
   q.N = c.H;
   q.Kd = c.F;
   q.C = (float*)out_rows;
-  if (shape == 2 && enough2) return launch_fp32_gemm<8, 8, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
-  if (shape == 1 && enough2) return launch_fp32_gemm<4, 8, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
-  if (along(c.H, 256) == 1) return launch_fp32_gemm<4, 4, 1, false>(p, enc, p->s.inter, wd, nullptr, q, st);
-  if (along(c.H, 256) == 2) return launch_fp32_gemm<4, 4, 2, false>(p, enc, p->s.inter, wd, nullptr, q, st);
-  return launch_fp32_gemm<4, 4, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st);
+  if (shape == 2 && enough2) return launch_fp32_gemm<8, 8, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st, own);
+  if (shape == 1 && enough2) return launch_fp32_gemm<4, 8, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st, own);
+  if (along(c.H, 256) == 1) return launch_fp32_gemm<4, 4, 1, false>(p, enc, p->s.inter, wd, nullptr, q, st, own);
+  if (along(c.H, 256) == 2) return launch_fp32_gemm<4, 4, 2, false>(p, enc, p->s.inter, wd, nullptr, q, st, own);
+  return launch_fp32_gemm<4, 4, 4, false>(p, enc, p->s.inter, wd, nullptr, q, st, own);
 }
 
 template <typename XT>
@@ -417,11 +470,11 @@ static int launch_typed(moe_plan* p, const void* recv, const int* tile_expert, c
 }
 
 int launch_ffn_simt(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu,
-                    const void* wd, void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st) {
+                    const void* wd, void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st, bool own) {
   if (p->P == 0 || p->cfg.T == 0) return 0;
   if (p->cfg.dtype == MOE_DTYPE_BF16)
     return launch_typed<__nv_bfloat16>(p, recv, tile_expert, wg, wu, wd, out_rows, st);
-  return launch_fp32(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
+  return launch_fp32(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st, own);
 }
 
 }  // namespace moehub

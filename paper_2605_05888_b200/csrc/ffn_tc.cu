@@ -576,7 +576,7 @@ OrderedParams make_ordered_params(moe_plan* p, const void* x, const int* topk_id
 // overlap_x / overlap_idx != nullptr: the overlapped form - the launch that runs the GEMM1 items also
 // dispatches x (ordered scheme, into recv and the plan's own dispatch outputs) on its first CTAs.
 int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu,
-                  const void* wd, void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st,
+                  const void* wd, void* out_rows, const int* tile_count, const int* rows_done, cudaStream_t st, bool own,
                   const void* overlap_x, const int* overlap_idx, const int* push_src) {
   const moe_config_t& c = p->cfg;
   if (p->P == 0 || c.T == 0) return 0;
@@ -616,7 +616,7 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   // rows than such a batch fills (rows from elsewhere: expert e's region of an expert-parallel rank, say).  Measured there, one
   // token, 8 regions of 1024 rows, H 2048, F 1408: 0.14 ms with tensor cores; the FMAs take 0.53 ms for the first 128 rows.
   const bool few = few_applies(p) && tile_count != nullptr && overlap_x == nullptr &&
-                   (tile_count == p->s.tile_count || p->cap_rows <= kTileRows);
+                   (own || p->cap_rows <= kTileRows);
   if (p->P > kMaxListTiles) return MOE_ERR_UNSUPPORTED;  // the work list lives in the kernel's shared memory
   if ((long long)p->P * (NB1 + NB2) >= (1ll << kThinShift)) return MOE_ERR_UNSUPPORTED;  // item index field of the ring
   // The kernels put their counters back to zero themselves; a call without counters may come before any dispatch.
@@ -655,7 +655,7 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   prm.band = 0;
   prm.push_src = push_src;
   if (few) {
-    rc = launch_ffn_few(p, recv, wg, wu, wd, prm, push_src, st);
+    rc = launch_ffn_few(p, recv, wg, wu, wd, prm, push_src, st, own);
     if (rc != 0) return rc;
     return cudaGetLastError() == cudaSuccess ? 0 : MOE_ERR_CUDA;
   }

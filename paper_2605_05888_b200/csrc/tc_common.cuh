@@ -26,6 +26,7 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint32_t bar) { asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
@@ -424,7 +425,7 @@ int launch_ffn_pair(moe_plan* p, const void* recv, const void* wg, const void* w
 constexpr int kFewMaxTokens = 32;  // (beyond five: small layers only)
 bool few_applies(const moe_plan* p);
 int launch_ffn_few(moe_plan* p, const void* recv, const void* wg, const void* wu, const void* wd, const FfnParams& prm,
-                   const int* push_src, cudaStream_t st);
+                   const int* push_src, cudaStream_t st, bool own);
 
 // ---- tensor maps (host side) ---------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,

@@ -272,6 +272,35 @@ def test_fp32_expert_kernel_edges(case):
     assert torch.equal(rows[used], plan.layer_tensor(7)[used])
 
 
+# A caller's own tables in fp32: more blocks than the grid has CTAs (each goes on to further blocks, a barrier set per block),
+# tiles of 0 to 128 rows; counters that are complete, incomplete (tiles whole) and absent (whole).
+@pytest.mark.parametrize("case", [(1, 8, 1024, 132, 260), (40, 4, 2048, 260, 1284), (900, 3, 2048, 516, 516)], ids=lambda c: f"T{c[0]}_E{c[1]}_cap{c[2]}")
+def test_fp32_expert_kernel_more_blocks_than_ctas(case):
+    T, E, cap, H, F = case
+    w = inputs.Workload("fp32_blocks", T=T, H=H, E=E, R=1, K=1, F=F, dtype=FP32, seed=18)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_STATIC, capacity_rows=cap)
+    g = torch.Generator(device="cuda").manual_seed(18)
+    wg, wu, wd = (torch.empty(s, device="cuda").normal_(0.0, 0.05, generator=g) for s in ((E, F, H), (E, F, H), (E, H, F)))
+    recv = torch.empty((E * cap, H), device="cuda").normal_(generator=g)
+    te = torch.arange(plan.P, dtype=torch.int32, device="cuda") // (cap // 128)
+    te[1::5] = -1
+    x = recv.double().view(E, cap, H)
+    h = x @ wg.double().transpose(1, 2)
+    want = ((h / (1 + torch.exp(-h)) * (x @ wu.double().transpose(1, 2))) @ wd.double().transpose(1, 2)).view(E * cap, H)
+    rows_of = torch.randint(0, 129, (plan.P,), dtype=torch.int32, device="cuda", generator=g)
+    owned = (te >= 0).repeat_interleave(128)
+    stored = owned & (torch.arange(128, device="cuda").repeat(plan.P) < rows_of.repeat_interleave(128))
+    for counts, done, rows in ((rows_of, T, stored), (rows_of, T - 1, owned), (None, None, owned)):
+        out = torch.zeros_like(recv)
+        rd = None if done is None else torch.full((1,), done, dtype=torch.int32, device="cuda")
+        plan.moe_expert_ffn(recv, te, wg, wu, wd, out, counts, rd)
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == (0, 0)
+        Hh.assert_output_close(Hh.to_host_f64(out[rows]), want[rows].cpu().numpy(), FP32)
+        assert torch.count_nonzero(out[~rows]) == 0 or counts is not None     # (a block's rows that are not there hold anything)
+        assert torch.count_nonzero(out[~owned]) == 0
+
+
 # The CTA-pair expert kernel where its items end: an expert's rows around 16, 32, 128 (one tile), 129, 256 (a pair of
 # tiles) and 257, all experts the same so that every count is met; in the paged layout (tiles of an expert apart) and
 # the ordered one; H and F that end inside its 512- and 256-column blocks and inside a k-block; one and two launches.

@@ -120,9 +120,10 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   t.gemm1_done = (int*)take(sizeof(int) * (size_t)((g.P > 0 ? g.P : 1) + 4));  // + the expert kernel's item and exit counters
   const size_t pool_rows = (size_t)g.P * kTileRows;
   if (!c.identity_experts) t.inter = take(pool_rows * c.F * g.eb);
-  const bool wide = c.E / g.tp > 64;  // (c.E counts every TP shard)
-  const bool filter = wide && c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
-  t.route_logits = wide ? (float*)take(sizeof(float) * (size_t)(c.T > 0 ? c.T : 1) * 256) : nullptr;
+  const int experts = c.E / g.tp;  // (c.E counts every TP shard)
+  const bool chains = route_chains_apply(experts, c.T);
+  const bool filter = !chains && c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
+  t.route_logits = filter || (chains && experts > 64) ? (float*)take(sizeof(float) * (size_t)(c.T > 0 ? c.T : 1) * 256) : nullptr;
   t.route_wnorm2 = filter ? (float*)take(sizeof(float) * 256) : nullptr;
   t.topk_idx = (int*)take(sizeof(int) * (size_t)c.T * c.K);
   t.topk_w = (float*)take(sizeof(float) * (size_t)c.T * c.K);

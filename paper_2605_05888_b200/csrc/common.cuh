@@ -40,8 +40,8 @@ struct Scratch {          // device pointers carved out of the caller's workspac
   unsigned long long* item_ns;   // [4 * P * (NB1 + NB2)] work-item timeline of the tensor-core expert kernel (measurement)
   int* gemm1_done;        // [P+4]  per-tile status counter: GEMM1 blocks finished (x4 epilogue warps); [P..P+1] item counters, [P+2..P+3] exit counters of the expert kernel's launches
   void* inter;            // [P*128, F] SwiGLU intermediate
-  float* route_logits;    // [T, 256] router logits, more than 64 experts (the tensor-core filter's: approximate)
-  float* route_wnorm2;    // [256]    squared norms of the router's weight rows, recomputed by every call
+  float* route_logits;    // [T, 256] router logits, more than 64 experts: the chain kernel's, or the tensor-core filter's approximate ones
+  float* route_wnorm2;    // [256]    squared norms of the router's weight rows, recomputed by every call (filter)
   // moe_layer's internal buffers
   int* topk_idx;
   float* topk_w;
@@ -140,7 +140,8 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 int launch_route(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx,
                  float* topk_w, const PrepArgs* prep, cudaStream_t st);
 // every chain, few enough of them to run at the chain's own speed (route_chains.cu)
-bool route_chains_apply(const moe_plan* p);
+constexpr int kRcMaxWideTokens = 1024;  // with more than 64 experts: up to this many tokens
+inline bool route_chains_apply(int experts, int tokens) { return experts <= 64 || tokens <= kRcMaxWideTokens; }
 int launch_route_chains(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,
                         const PrepArgs& prep, cudaStream_t st);
 // the tensor-core filter in front of the exact chains (many experts, bf16): see route_filter.cu

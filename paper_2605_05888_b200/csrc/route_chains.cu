@@ -28,7 +28,6 @@ constexpr int kRcBox = 128;                 // bytes of a row per TMA box
 constexpr int kRcMaxBoxes = 4;              // most boxes per stage
 constexpr int kRcMaxStages = 8;
 constexpr int kRcRingBytes = 160 * 1024;    // most shared memory for the ring
-constexpr int kRcMaxWideTokens = 1024;      // with more than 64 experts: up to this many tokens
 constexpr int kRcMaxWarps = 24;             // most compute warps per CTA (one CTA per SM, 80 registers a thread)
 
 // One 16-byte unit of TM tokens' rows against one of TN experts' rows.
@@ -345,11 +344,6 @@ static int launch_chains_typed(moe_plan* p, const void* x, const void* wr, const
   if (chains <= 1536ll * sms) return MOEHUB_CHAINS(true, 1, 2, 2, (E + 63) / 64);
   return MOEHUB_CHAINS(true, 4, 2, 2, (E + 63) / 64);
 #undef MOEHUB_CHAINS
-}
-
-bool route_chains_apply(const moe_plan* p) {
-  if (p->route_E <= 64) return true;
-  return p->cfg.T <= kRcMaxWideTokens;
 }
 
 int launch_route_chains(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,

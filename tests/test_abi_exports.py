@@ -84,3 +84,18 @@ def test_host_side_checks_without_gpu(lib):
     h = ctypes.c_void_p()
     assert lib.moe_plan_create(ctypes.byref(ok), None, 0, ctypes.byref(h)) == -1   # null workspace
     assert lib.moe_route(None, None, None, None, None, None, None) == -1
+
+
+def test_workspace_holds_the_wide_router_logits_only_where_a_kernel_reads_them(lib):
+    """[T, 256] fp32 (and 256 squared norms) for the tensor-core filter; nothing for routers of many tokens without it."""
+    T, H, E = 2048, 256, 256
+
+    def need(dtype, route_filter=0, tokens=T):
+        return B.moe_workspace_bytes(B.make_config(tokens, H, E, 1, 8, 0, dtype, identity_experts=1, route_filter=route_filter))
+
+    plain = need(B.DTYPE_BF16, -1)
+    assert need(B.DTYPE_BF16) == plain + T * 1024 + 1024
+    rows = B.moe_pool_tiles(B.make_config(T, H, E, 1, 8, 0, B.DTYPE_FP32, identity_experts=1)) * 128
+    assert need(B.DTYPE_FP32) == plain + 2 * H * (rows + 4 * T)      # fp32 rows and staging buffers, no logits
+    # a batch that the chain kernel takes keeps its logits, whatever route_filter says
+    assert need(B.DTYPE_BF16, 0, 512) == need(B.DTYPE_BF16, -1, 512)

@@ -20,6 +20,7 @@
 //   T 512, H 2048, 60 experts 18.6 -> 12.0; T 2777 65.7 -> 28.8; T 8192 170 -> 66; T 24, H 4096, 8 experts 30.9 -> 16.6;
 //   T 4096 32.9 -> 20.7; T 1023, H 4096, 16 experts 41.9 -> 18.7; H 7168, 256 experts: T 64 151 -> 27, T 256 123 -> 43.
 #include "route_common.cuh"
+#include "route_shape.h"
 #include "tc_common.cuh"
 
 namespace moehub {
@@ -272,15 +273,8 @@ static int launch_chains(moe_plan* p, const void* x, const void* wr, const float
   constexpr int GT = (SWAP ? 2 : 16) * TM, EPC = EW * (SWAP ? 16 : 2) * TN;
   constexpr int kMaxTw = kRcMaxWarps / EW;
   const moe_config_t& c = p->cfg;
-  // Token warps per CTA: the fewest that fit the batch on the SMs in one wave, so that every SM scheduler has as few
-  // chains as possible; past that, the count that leaves the least to do (ties: fewer waves).
   const int sms = p->sm_count > 0 ? p->sm_count : 148;
-  int tw = 1, best = 1 << 30;
-  for (int i = 1; i <= kMaxTw; ++i) {
-    const int waves = (int)(((long long)((c.T + GT * i - 1) / (GT * i)) * split + sms - 1) / sms);
-    if (waves * i <= best) { best = waves * i; tw = i; }
-    if (waves == 1) break;
-  }
+  const int tw = route_token_warps(c.T, c.H, GT, split, EW, TM * TN, kMaxTw, sms);
   ChainParams q;
   q.bias = bias;
   q.T = c.T;
@@ -341,7 +335,8 @@ static int launch_chains_typed(moe_plan* p, const void* x, const void* wr, const
   if (E <= 8) return MOEHUB_CHAINS(false, 1, 2, 2, 1);
   if (E <= 16) return MOEHUB_CHAINS(false, 1, 2, 4, 1);
   if (E <= 32) return MOEHUB_CHAINS(true, 1, 2, 1, 1);
-  if (chains <= 1536ll * sms) return MOEHUB_CHAINS(true, 1, 2, 2, (E + 63) / 64);
+  const long long slots = (long long)T * ((E + 63) / 64) * 64;  // (a CTA has 64 experts' chains whether or not they exist)
+  if (slots <= 1536ll * sms) return MOEHUB_CHAINS(true, 1, 2, 2, (E + 63) / 64);
   return MOEHUB_CHAINS(true, 4, 2, 2, (E + 63) / 64);
 #undef MOEHUB_CHAINS
 }

@@ -221,6 +221,8 @@ CHAIN_SHAPES = [
     (3, 584, 33, 4, BF16), (1, 2056, 64, 8, BF16), (601, 584, 31, 5, BF16), (4700, 72, 61, 4, BF16), (4700, 36, 64, 4, FP32),
     (1, 584, 256, 8, BF16), (9, 292, 193, 32, FP32), (129, 136, 128, 6, BF16), (768, 136, 192, 8, BF16),
     (769, 136, 192, 8, BF16), (768, 68, 256, 8, FP32), (769, 68, 256, 8, FP32),
+    # just past what one wave of CTAs holds (two waves of fewer tokens each)
+    (985, 72, 160, 4, BF16), (890, 72, 224, 8, BF16), (7200, 40, 32, 2, BF16), (14300, 36, 12, 2, FP32),
 ]
 
 

@@ -121,8 +121,8 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   const size_t pool_rows = (size_t)g.P * kTileRows;
   if (!c.identity_experts) t.inter = take(pool_rows * c.F * g.eb);
   const int experts = c.E / g.tp;  // (c.E counts every TP shard)
-  const bool chains = route_chains_apply(experts, c.T);
-  const bool filter = !chains && c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
+  const bool may_filter = c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
+  const bool chains = route_chains_apply(experts, c.T, c.H, may_filter), filter = may_filter && !chains;
   t.route_logits = filter || (chains && experts > 64) ? (float*)take(sizeof(float) * (size_t)(c.T > 0 ? c.T : 1) * 256) : nullptr;
   t.route_wnorm2 = filter ? (float*)take(sizeof(float) * 256) : nullptr;
   t.topk_idx = (int*)take(sizeof(int) * (size_t)c.T * c.K);

@@ -140,8 +140,14 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 int launch_route(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx,
                  float* topk_w, const PrepArgs* prep, cudaStream_t st);
 // every chain, few enough of them to run at the chain's own speed (route_chains.cu)
-constexpr int kRcMaxWideTokens = 1024;  // with more than 64 experts: up to this many tokens
-inline bool route_chains_apply(int experts, int tokens) { return experts <= 64 || tokens <= kRcMaxWideTokens; }
+// With more than 64 experts: up to 1024 tokens; up to 864 where the tensor-core filter is there to take over and the chains
+// are long and in four CTAs per block of tokens.  Measured, router call on bf16 data, us, every chain / filter: 256 experts, H 7168:
+// T 256 46 / 120, T 512 75 / 110, T 768 103 / 108, T 864 107 / 108, T 896 122 / 109, T 1024 122 / 108; H 5120: T 864 81 / 85,
+// T 896 91 / 85; H 4096: T 896 74 / 74, T 1024 75 / 75; H 2048: T 1024 44 / 50; 192 experts, H 7168: T 1024 105 / 110; 128, H
+// 4096: 46 / 75; 96, H 2048: 30 / 50.  fp32, every chain / route_wide_kernel: 256 experts, H 7168, T 1024 142 / 523.
+inline bool route_chains_apply(int experts, int tokens, int H, bool filter) {
+  return experts <= 64 || tokens <= (filter && experts > 192 && H > 4096 ? 864 : 1024);
+}
 int launch_route_chains(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,
                         const PrepArgs& prep, cudaStream_t st);
 // the tensor-core filter in front of the exact chains (many experts, bf16): see route_filter.cu

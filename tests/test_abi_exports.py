@@ -99,3 +99,14 @@ def test_workspace_holds_the_wide_router_logits_only_where_a_kernel_reads_them(l
     assert need(B.DTYPE_FP32) == plain + 2 * H * (rows + 4 * T)      # fp32 rows and staging buffers, no logits
     # a batch that the chain kernel takes keeps its logits, whatever route_filter says
     assert need(B.DTYPE_BF16, 0, 512) == need(B.DTYPE_BF16, -1, 512)
+
+
+def test_wide_router_hands_over_to_the_filter_where_the_chains_get_slower(lib):
+    """256 experts and long rows: from 865 tokens on the filter (its squared norms are in the workspace); shorter rows: 1025."""
+    def norms(tokens, H, E=256):
+        a, b = (B.moe_workspace_bytes(B.make_config(tokens, H, E, 1, 8, 0, B.DTYPE_BF16, identity_experts=1, route_filter=f)) for f in (0, -1))
+        return a - b - (tokens * 1024 if tokens > 1024 else 0)
+
+    assert [norms(t, 7168) for t in (864, 865, 1024, 1025)] == [0, 1024, 1024, 1024]
+    assert [norms(t, 4096) for t in (864, 865, 1024, 1025)] == [0, 0, 0, 1024]
+    assert [norms(t, 7168, 192) for t in (865, 1024, 1025)] == [0, 0, 1024]

@@ -214,13 +214,16 @@ def test_router_every_kernel_shape(shape):
 
 # The chain kernel where its shapes end: expert counts at the edges of its lane grids and clusters (8 / 16 / 32 / 64 /
 # 128 / 192 / 256), one token, token counts around its blocks, one, two and eight chains per thread, an h range shorter
-# than a box and one that ends inside a box and inside a stage; and the filter just past its first batch size.
+# than a box and one that ends inside a box and inside a stage; and both sides of the switches to the filter (bf16) and to
+# the register-tiled kernel (fp32).
 CHAIN_SHAPES = [
     # (T, H, E, K, dtype)
     (1, 8, 8, 8, BF16), (1, 4, 1, 1, FP32), (17, 72, 9, 2, BF16), (5000, 72, 8, 2, BF16), (5000, 36, 16, 3, FP32),
     (3, 584, 33, 4, BF16), (1, 2056, 64, 8, BF16), (601, 584, 31, 5, BF16), (4700, 72, 61, 4, BF16), (4700, 36, 64, 4, FP32),
     (1, 584, 256, 8, BF16), (9, 292, 193, 32, FP32), (129, 136, 128, 6, BF16), (768, 136, 192, 8, BF16),
     (769, 136, 192, 8, BF16), (768, 68, 256, 8, FP32), (769, 68, 256, 8, FP32),
+    (1024, 136, 256, 8, BF16), (1025, 136, 256, 8, BF16), (864, 4104, 193, 8, BF16), (865, 4104, 193, 8, BF16),
+    (1024, 68, 65, 8, FP32), (1025, 68, 65, 8, FP32), (1024, 136, 65, 8, BF16), (1025, 136, 65, 8, BF16),
     # just past what one wave of CTAs holds (two waves of fewer tokens each)
     (985, 72, 160, 4, BF16), (890, 72, 224, 8, BF16), (7200, 40, 32, 2, BF16), (14300, 36, 12, 2, FP32),
 ]

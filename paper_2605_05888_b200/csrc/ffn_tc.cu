@@ -580,22 +580,6 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
                   const void* overlap_x, const int* overlap_idx, const int* push_src) {
   const moe_config_t& c = p->cfg;
   if (p->P == 0 || c.T == 0) return 0;
-  EncodeTiledFn enc;
-  int rc = get_encoder(p, &enc);
-  if (rc != MOE_OK) return rc;
-  const uint64_t pool_rows = (uint64_t)p->P * kTileRows;
-  CUtensorMap a1, bg, bu, a2, bd;
-  if ((rc = make_map_2d(enc, &a1, recv, pool_rows, c.H, kTileRows)) != MOE_OK) return rc;
-  if ((rc = make_map_3d(enc, &bg, wg, c.E, c.F, c.H, 128)) != MOE_OK) return rc;
-  if ((rc = make_map_3d(enc, &bu, wu, c.E, c.F, c.H, 128)) != MOE_OK) return rc;
-  if ((rc = make_map_2d(enc, &a2, p->s.inter, pool_rows, c.F, kTileRows)) != MOE_OK) return rc;
-  if ((rc = make_map_wd(enc, &bd, wd, c.E / p->tp, p->tp, c.H, c.F, 256)) != MOE_OK) return rc;
-  CUtensorMap a1t, a2t;  // the first kThinRows rows of a tile, for tiles computed the other way round
-  if ((rc = make_map_2d(enc, &a1t, recv, pool_rows, c.H, kThinRows)) != MOE_OK) return rc;
-  if ((rc = make_map_2d(enc, &a2t, p->s.inter, pool_rows, c.F, kThinRows)) != MOE_OK) return rc;
-
-  static SmemAttrOnce once;
-  if (ensure_dynamic_smem(ffn_tc_kernel, kTcSmem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
   const int grid = p->sm_count;
   const int NB1 = (c.F + 127) / 128, NB2 = (c.H + 255) / 256;
   // One launch for both GEMMs, or one per GEMM.  With many small experts (E = 256 under Zipf routing)
@@ -623,7 +607,6 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   if (tile_count == nullptr &&
       cudaMemsetAsync(p->s.gemm1_done, 0, sizeof(int) * (size_t)(p->P + 4), st) != cudaSuccess)
     return MOE_ERR_CUDA;
-  mark(p, 3, st);
   FfnParams prm;
   prm.tile_expert = tile_expert;
   prm.P = (int)p->P;
@@ -654,16 +637,35 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
   prm.hot_first = 0;
   prm.band = 0;
   prm.push_src = push_src;
+  int rc;
   if (few) {
+    mark(p, 3, st);
     rc = launch_ffn_few(p, recv, wg, wu, wd, prm, push_src, st, own);
     if (rc != 0) return rc;
     return cudaGetLastError() == cudaSuccess ? 0 : MOE_ERR_CUDA;
   }
   if (pairs) {
+    mark(p, 3, st);
     rc = launch_ffn_pair(p, recv, wg, wu, wd, prm, st);
     if (rc != 0) return rc;
     return cudaGetLastError() == cudaSuccess ? 0 : MOE_ERR_CUDA;
   }
+  EncodeTiledFn enc;
+  if ((rc = get_encoder(p, &enc)) != MOE_OK) return rc;
+  const uint64_t pool_rows = (uint64_t)p->P * kTileRows;
+  CUtensorMap a1, bg, bu, a2, bd;
+  if ((rc = make_map_2d(enc, &a1, recv, pool_rows, c.H, kTileRows)) != MOE_OK) return rc;
+  if ((rc = make_map_3d(enc, &bg, wg, c.E, c.F, c.H, 128)) != MOE_OK) return rc;
+  if ((rc = make_map_3d(enc, &bu, wu, c.E, c.F, c.H, 128)) != MOE_OK) return rc;
+  if ((rc = make_map_2d(enc, &a2, p->s.inter, pool_rows, c.F, kTileRows)) != MOE_OK) return rc;
+  if ((rc = make_map_wd(enc, &bd, wd, c.E / p->tp, p->tp, c.H, c.F, 256)) != MOE_OK) return rc;
+  CUtensorMap a1t, a2t;  // the first kThinRows rows of a tile, for tiles computed the other way round
+  if ((rc = make_map_2d(enc, &a1t, recv, pool_rows, c.H, kThinRows)) != MOE_OK) return rc;
+  if ((rc = make_map_2d(enc, &a2t, p->s.inter, pool_rows, c.F, kThinRows)) != MOE_OK) return rc;
+
+  static SmemAttrOnce once;
+  if (ensure_dynamic_smem(ffn_tc_kernel, kTcSmem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
+  mark(p, 3, st);
   OverlapParams ov = {};
   const bool overlap = overlap_x != nullptr;
   if (overlap) {

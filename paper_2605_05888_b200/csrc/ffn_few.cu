@@ -583,7 +583,8 @@ static int launch_few_layer(moe_plan* p, FewLayerParams q, const void* wd, cudaS
 // and five tokens: 230 and 219).
 bool few_layer_applies(const moe_plan* p) {
   const moe_config_t& c = p->cfg;
-  return c.T > 0 && (c.T <= 3 || c.F <= 8192) && c.dtype == MOE_DTYPE_BF16 && !c.identity_experts && c.overlap == 0 && few_applies(p);
+  return c.T > 0 && (c.T <= 3 || c.F <= 8192) && c.dtype == MOE_DTYPE_BF16 && !c.identity_experts && c.overlap == 0 &&
+         p->P <= kMaxListTiles /* the expert call's limit, whatever the batch */ && few_applies(p);
 }
 
 int launch_few_layer(moe_plan* p, const void* x, const void* wg, const void* wu, const void* wd, void* y, cudaStream_t st) {

@@ -485,6 +485,22 @@ def test_few_tokens_kernel_wait_runs_out_and_reports_it():
     assert torch.count_nonzero(out) == 0
 
 
+@pytest.mark.parametrize("T", [2, 6])
+def test_layer_refuses_a_pool_beyond_the_work_list_whatever_the_batch(T):
+    """More than 4608 tiles are outside what the bf16 expert kernels take: also for the few tokens that need no work list."""
+    w = inputs.Workload("few_refused", T=T, H=256, E=8, R=1, K=2, F=256, dtype=BF16, seed=37)
+    args = [Hh.to_dev(a) for a in Hh.oracle_inputs(w)]
+    y = torch.empty((T, w.H), dtype=torch.bfloat16, device="cuda")
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_STATIC, capacity_rows=128 * 577)
+    assert plan.P == 4616
+    with pytest.raises(B.MoeError) as err:
+        plan.moe_layer(*args, y)
+    assert err.value.code == -3      # MOE_ERR_UNSUPPORTED
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_STATIC, capacity_rows=128 * 576)
+    plan.moe_layer(*args, y)
+    assert plan.moe_last_status() == (0, 0)
+
+
 def test_few_tokens_kernel_expert_named_twice():
     """A caller's own routing may name an expert more than once for a token: more rows than tokens in a tile."""
     w = inputs.Workload("few_twice", T=3, H=520, E=4, R=1, K=4, F=264, dtype=BF16, seed=33)

@@ -82,12 +82,23 @@ typedef struct {
   int32_t ffn_kernel;           /* 0: tensor-core (tcgen05) kernel for bf16 - one CTA per tile, or
                                    CTA pairs (cta_group::2, two tiles of an expert per item)
                                    where experts have more than one tile of rows on average, or
-                                   plain FMAs for up to five tokens (small layers: 32) - and the fp32-FMA kernel for fp32; 1: plain SIMT fp32-FMA
-                                   kernel for bf16 (check path); 2: always CTA pairs (bf16)   */
+                                   plain FMAs for up to five tokens (small layers: 32; only with
+                                   row counts and with ffn_split, ffn_thin_tiles and
+                                   ffn_hot_min_tiles left at 0) - and the fp32-FMA kernel for
+                                   fp32; 1: plain SIMT fp32-FMA kernel for bf16 (check path);
+                                   2: always CTA pairs (bf16).
+                                   The tensor-core forms add up every result in the same order,
+                                   so a row's bytes do not depend on which of them computes it,
+                                   nor on how many other rows there are.  The plain-FMA kernel
+                                   for few tokens adds in another order (fp32 as well): with 0, a
+                                   token's y may differ in the last bits of bf16 between a batch
+                                   of 5 and one of 6, and moe_expert_ffn's rows between calls with
+                                   and without row counts.  Naming ffn_split (1 or 2) keeps the
+                                   tensor-core forms, and a token's bytes, at every batch size */
   int32_t ffn_split;            /* 1: one launch per expert GEMM; 2: both GEMMs in one persistent
                                    launch (per-tile status counters gate GEMM2); 0: choose
                                    (one launch when E <= 64; with more, smaller experts two
-                                   launches measure faster)                                   */
+                                   launches measure faster; few tokens: see ffn_kernel)        */
   int32_t ffn_hot_min_tiles;    /* two-launch form of the tensor-core kernel: > 0 = experts with at
                                    least this many tiles count as tensor-bound, the others as
                                    bound by streaming their weights, and the kernel walks the two
@@ -124,7 +135,13 @@ typedef struct {
   int32_t route_filter;         /* router with more than 64 experts on bf16 data: 0 = tensor-core filter
                                    (approximate logits by tcgen05 MMAs, then the exact fp32 chain only
                                    for the experts that can still be among the K largest: the picks
-                                   are the exact ones, bit for bit); -1 = every chain computed        */
+                                   are the exact ones, bit for bit) for batches of more than 1024
+                                   tokens (more than 192 experts and H above 4096: 864), every chain
+                                   for smaller ones; -1 = every chain computed.  In the filter's
+                                   softmax weights the experts that were ruled out enter the
+                                   denominator with their approximate logits: measured up to 2.4e-6
+                                   relative from the weights of the chains, which -1 gives at every
+                                   batch size (1e-5 is the bound that is tested)                      */
   int64_t capacity_rows;        /* mode 1: rows per expert region, multiple of 128, 0 = T
                                    rounded up (overflow-free); modes 0/2: ignored            */
   uint64_t spin_limit;          /* bound (iterations) on the dispatch kernels' waits, 0 = 1<<22 */
@@ -149,7 +166,7 @@ int moe_plan_destroy(moe_plan_t* plan);
 
 /* Step 1 (Section II-A, routing): logits l[t,e] = sum_h x[t,h]*Wr[e,h] (+bias[e]) as one
  * ascending fp32 FMA chain, softmax over the E experts, the K largest logits (lowest index
- * wins ties), in descending order.  (With more than 64 experts on bf16 data the chain is evaluated only for
+ * wins ties), in descending order.  (For large batches with more than 64 experts on bf16 data the chain is evaluated only for
  * the experts that a tensor-core pass and an error bound derived from the data leave in question; the picks are
  * those of the chains of all experts, bit for bit - see route_filter in moe_config_t.)
  * d_x [T,H], d_wr [E,H] (dtype); d_bias [E] fp32 or NULL;
@@ -188,10 +205,11 @@ int moe_dispatch(moe_plan_t* plan, const void* d_x, const int32_t* d_topk_idx, v
  *     neither.  When given, the tensor-core kernel waits before it reads a tile until
  *     tile_count[p] >= 128 or rows_done >= T*K (bounded by wait_limit_ns; on expiry the status
  *     word reads MOE_ERR_TIMEOUT and the kernel returns).  NULL: the rows are complete when the
- *     call is reached in stream order.  The SIMT kernel ignores them (stream order).  The
- *     counters also tell the kernel how many rows a tile holds: with them, an expert whose only
- *     tile holds at most 64 rows is computed in a narrower form (same result, less work);
- *     without them every tile is computed as 128 rows.
+ *     call is reached in stream order.  The SIMT check kernel (ffn_kernel 1) ignores them; the fp32
+ *     kernel waits for nothing (stream order) but, when rows_done >= T*K, computes only the
+ *     tile_count rows of each tile.  The counters also tell the tensor-core kernel how many rows a
+ *     tile holds: with them, an expert whose only tile holds at most 64 rows is computed in a
+ *     narrower form (same result, less work); without them every tile is computed as 128 rows.
  * out: d_out_rows [P*128,H] (dtype); rows of empty slots hold unspecified values.
  * The tensor-core kernels keep their work list in shared memory: P <= 4608 tiles (T*K <= 557 056 rows at
  * E = 256), MOE_ERR_UNSUPPORTED beyond. */

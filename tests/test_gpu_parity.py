@@ -376,6 +376,23 @@ def test_pair_expert_kernel_columns_end_inside_a_warp(extra, combine):
     assert torch.equal(ys[0], ys[1]) and bool(torch.isfinite(ys[0]).all())
 
 
+def test_named_split_keeps_a_tokens_bytes_whatever_the_batch():
+    """The tensor-core kernels add up each result in one order, in every form (narrow, M = 64, whole tiles, CTA pairs).  A plan
+    that names ffn_split never takes the plain-FMA kernels for few tokens, so a token's bytes do not depend on its batch."""
+    T, H, E, K, F = 300, 1536, 4, 2, 1024
+    w = inputs.Workload("batch_bytes", T=T, H=H, E=E, R=1, K=K, F=F, dtype=BF16, seed=38)
+    x, wr, _, wg, wu, wd = (Hh.to_dev(a) for a in Hh.oracle_inputs(w))
+    for split in (1, 2):
+        ys = {}
+        for n in (1, 3, 5, 6, 16, 17, 70, 140, T):      # 300: more than a tile of rows per expert, CTA pairs
+            plan = B.Plan(B.make_config(n, H, E, 1, K, F, BF16, ffn_split=split))
+            ys[n] = torch.empty((n, H), dtype=torch.bfloat16, device="cuda")
+            plan.moe_layer(x[:n], wr, None, wg, wu, wd, ys[n])
+            assert plan.moe_last_status() == (0, 0)
+        for n, y in ys.items():
+            assert torch.equal(y, ys[T][:n]), (split, n)
+
+
 # The refine kernel's numbering of the chains: token counts that give its CTAs 12 to 64 tokens (a whole wave on 148 SMs),
 # with every token's candidates in ONE class of experts modulo eight (its bucket overflows into the others' free slots),
 # with two classes, and with more candidates than a CTA has threads (every expert the same: all 256 are candidates).

@@ -139,9 +139,10 @@ typedef struct {
                                    tokens (more than 192 experts and H above 4096: 864), every chain
                                    for smaller ones; -1 = every chain computed.  In the filter's
                                    softmax weights the experts that were ruled out enter the
-                                   denominator with their approximate logits: measured up to 2.4e-6
-                                   relative from the weights of the chains, which -1 gives at every
-                                   batch size (1e-5 is the bound that is tested)                      */
+                                   denominator with their approximate logits: up to 2.7e-6 relative
+                                   from the weights of the chains (1e-5 is tested; rows of one sign,
+                                   whose logits are in the hundreds, 4e-4: the chains' own rounding
+                                   there), which -1 gives at every batch size                         */
   int64_t capacity_rows;        /* mode 1: rows per expert region, multiple of 128, 0 = T
                                    rounded up (overflow-free); modes 0/2: ignored            */
   uint64_t spin_limit;          /* bound (iterations) on the dispatch kernels' waits, 0 = 1<<22 */

@@ -21,7 +21,9 @@
 // the data of the call.  The K experts with the largest l~ have l >= kth~ - eps
 // and every expert below the threshold kth~ - 2 eps has l < kth~ - eps, so none of those can be among the K
 // largest l, ties included.  The kernel checks the model on every candidate (both values are at hand) and
-// reports MOE_ERR_INTERNAL if |l~ - l| ever exceeded eps.
+// reports MOE_ERR_INTERNAL if |l~ - l| ever exceeded eps.  Largest |l~ - l| / eps over EVERY expert of 1100 tokens, H 64 to
+// 7168: 0.16 on constant rows of one sign (where S is all of |x| |w| and every rounding goes the same way), 0.04 on rows
+// that fall off over twenty binades, at most 0.03 on normal, parallel, one-sign, cancelling, spiked and wide-ranged ones.
 //
 // The softmax weights use the exact logits of the candidates and the approximate ones of the rest: the rest
 // only enters the denominator.  What the accumulation's rounding adds up to grows with the number of additions
@@ -214,7 +216,8 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 // What bounds it: shared memory (ncu, T 8192, H 7168, 256 experts: its pipe 65 % busy with 5.4 wavefronts per 16-byte load
 // and another 11 % with the TMA writes; issue slots 48 %).  Whole router call, us, before / after the numbering by e % 8,
 // CTAs of any even token count (T 8192: 147 CTAs of 56 tokens instead of 128 of 64) and x asked for ahead / with the
-// error bound counted per MMA (before: H * 2^-23 * S for the approximate logit too, half a candidate more per token): T 2048
+// error bound counted per MMA (before: H * 2^-23 * S for the approximate logit too, half a candidate more per token), all
+// experts equally popular (with Zipf 1.2 at T 16384 the call takes 492 instead of 431: popular classes overflow): T 2048
 // 113 / 108 / 107, T 4096 147 / 131 / 130, T 6000 262 / 176 / 169, T 8192 258 / 225 / 213, T 16384 508 / 438 / 414.
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT * 16, 1)

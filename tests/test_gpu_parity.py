@@ -166,10 +166,11 @@ def test_router_tie_patterns_exhaustive():
             Hh.check_route(idx, tw, ridx, rw)
 
 
-@pytest.mark.parametrize("E", [60, 160])   # the narrow router; the tensor-core filter of the wide one
+# every chain: up to 64 experts, and more of them with few tokens; the tensor-core filter, from one k-block per accumulator on
+@pytest.mark.parametrize("E,T,H", [(60, 200, 512), (160, 200, 512), (160, 1100, 512), (256, 1030, 1032)])
 @pytest.mark.parametrize("renorm", [0, 1])
-def test_router_renormalize_and_bias(renorm, E):
-    w = inputs.Workload("renorm", T=200, H=512, E=E, R=4, K=4, F=8, dtype=BF16, zipf_s=1.0, seed=3)
+def test_router_renormalize_and_bias(renorm, E, T, H):
+    w = inputs.Workload("renorm", T=T, H=H, E=E, R=4, K=4, F=8, dtype=BF16, zipf_s=1.0, seed=3)
     x, wr, bias, *_ = Hh.oracle_inputs(w, with_experts=False)
     cfg = B.make_config(w.T, w.H, w.E, w.R, w.K, w.F, w.dtype, renormalize=renorm)
     plan = B.Plan(cfg)
@@ -180,10 +181,11 @@ def test_router_renormalize_and_bias(renorm, E):
     Hh.check_route(idx, tw, ridx, rw)
 
 
-# Every shape of the two router kernels: the narrow kernel's four lane layouts (E <= 8, 16, 32, 64), each
-# with a block boundary inside T and an h range that ends inside a chunk, in both dtypes; the wide kernel
-# with every register-tile height it picks (4 to 8 tokens per thread follows from T on a 148-SM part:
-# T <= 4736 -> 4, <= 5920 -> 5, <= 7104 -> 6, <= 8288 -> 7, <= 9472 -> 8) and E below and at 256.
+# Every router kernel: the chain kernel's lane layouts (E <= 8, 16, 32, 64 and several CTAs per block of tokens), each
+# with a block boundary inside T and an h range that ends inside a chunk, in both dtypes; above 1024 tokens and 64 experts
+# the filter and the register-tiled kernel, with every tile height it picks (4 to 8 tokens per thread follows from T on a
+# 148-SM part: T <= 4736 -> 4, <= 5920 -> 5, <= 7104 -> 6, <= 8288 -> 7, <= 9472 -> 8) and E below and at 256; the filter
+# with h ranges that use its four accumulators unevenly.
 ROUTER_SHAPES = [
     # (T, H, E, K, dtype, zipf_s)
     (77, 264, 7, 2, BF16, 0.0), (1100, 520, 8, 3, BF16, 1.0), (45, 132, 5, 5, FP32, 0.0),
@@ -193,6 +195,7 @@ ROUTER_SHAPES = [
     (200, 72, 65, 8, BF16, 0.0), (4000, 40, 256, 8, BF16, 1.0), (5000, 40, 200, 4, BF16, 0.0),
     (6500, 40, 256, 8, BF16, 1.0), (8000, 40, 129, 2, BF16, 0.0), (9000, 40, 256, 8, BF16, 1.0),
     (300, 36, 100, 5, FP32, 1.0), (5100, 20, 256, 3, FP32, 0.0),
+    (1100, 1032, 200, 8, BF16, 1.0), (1300, 2120, 129, 4, BF16, 0.0), (1025, 264, 65, 6, BF16, 1.0),
 ]
 
 
@@ -203,7 +206,7 @@ def test_router_every_kernel_shape(shape):
                         identity_experts=True)
     x, wr, bias, *_ = Hh.oracle_inputs(w, with_experts=False)
     ridx, rw, _ = oracle.route(x, wr, bias, K, dtype)
-    for route_filter in ((0, -1) if (dtype == BF16 and E > 64) else (0,)):   # -1: the all-chains kernel for many experts
+    for route_filter in ((0, -1) if (dtype == BF16 and E > 64) else (0,)):   # -1: every chain, also above 1024 tokens
         plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, route_filter=route_filter)
         idx = torch.empty((T, K), dtype=torch.int32, device="cuda")
         tw = torch.empty((T, K), dtype=torch.float32, device="cuda")
@@ -911,7 +914,7 @@ def test_overlapped_dispatch_and_experts_match_oracle(w, split):
         plan.moe_layer(*args, y)
         torch.cuda.synchronize()
         assert plan.moe_last_status() == (0, 0)
-        router = 2 if (w.dtype == BF16 and w.E > 64) else 1                     # many experts on bf16: filter + refine
+        router = 2 if (w.dtype == BF16 and w.E > 64) else 1                     # many experts: chains + select, or filter + refine
         assert plan.moe_last_launch_count() == router + 1 + (2 if split == 1 else 1)   # router, expert launch(es) carrying the dispatch, combine
         Hh.check_route(plan.layer_tensor(0), plan.layer_tensor(1), ref["topk_idx"], ref["topk_w"])
         Hh.check_dispatch(w, plan.P, x, ref["topk_idx"], ref, plan.layer_tensor(2), plan.layer_tensor(3),
@@ -1040,7 +1043,8 @@ def test_push_combine_is_refused_where_it_is_not_built():
 TP_CASES = [(inputs.Workload("tp_bf16", T=333, H=264, E=12, R=3, K=3, F=400, dtype=BF16), 2),
             (inputs.Workload("tp_bf16_4", T=700, H=320, E=4, R=2, K=2, F=1024, dtype=BF16, zipf_s=1.0), 4),
             (inputs.Workload("tp_many", T=300, H=256, E=64, R=8, K=8, F=256, dtype=BF16, zipf_s=1.0), 4),
-            (inputs.Workload("tp_filtered_router", T=260, H=512, E=128, R=8, K=4, F=256, dtype=BF16, zipf_s=1.0), 2),  # 128 experts: the router's filter path
+            (inputs.Workload("tp_filtered_router", T=260, H=512, E=128, R=8, K=4, F=256, dtype=BF16, zipf_s=1.0), 2),  # 128 experts, few tokens: every chain
+            (inputs.Workload("tp_filter", T=1100, H=512, E=96, R=8, K=4, F=128, dtype=BF16, zipf_s=1.0), 2),  # the router's filter path
             (inputs.Workload("tp_fp32", T=130, H=128, E=8, R=2, K=2, F=192, dtype=FP32), 3)]
 
 
@@ -1283,26 +1287,42 @@ def _route_only(w, x, wr, bias, **kw):
     return plan, idx, tw
 
 
-@pytest.mark.parametrize("case", ["zero_rows", "equal_experts", "near_ties"])
-def test_router_filter_degenerate_rows(case):
+@pytest.mark.parametrize("T,H", [(150, 512), (1100, 512), (1030, 1032), (1100, 4104)])   # (150 tokens: every chain; then the filter)
+@pytest.mark.parametrize("case", ["zero_rows", "equal_experts", "near_ties", "one_sign"])
+def test_router_filter_degenerate_rows(case, T, H):
     """The tensor-core filter of the wide router where its candidate sets are as large as they get: tokens that are
     all zero (every logit equal: all 256 experts are candidates, the picks are experts 0..K-1), experts with identical
-    weight rows (exact ties decided by index), and logits a few ulps apart."""
-    w = inputs.Workload("filter_" + case, T=150, H=512, E=256, R=8, K=8, F=8, dtype=BF16, identity_experts=True, seed=4)
+    weight rows (exact ties decided by index), logits a few ulps apart, and rows of one sign (every addition rounds the same
+    way, and the magnitudes add up to what the error bound allows for).  Several k-blocks in each of its four accumulators."""
+    w = inputs.Workload("filter_" + case, T=T, H=H, E=256, R=8, K=8, F=8, dtype=BF16, identity_experts=True, seed=4)
     x, wr, bias, *_ = Hh.oracle_inputs(w, with_experts=False)
     x, wr = x.copy(), wr.copy()
     if case == "zero_rows":
         x[::3] = 0
     elif case == "equal_experts":
         wr[1::2] = wr[0::2]                 # experts 2i and 2i+1 are the same row: every logit comes twice
+    elif case == "one_sign":
+        x, wr = x & 0x7FFF, wr & 0x7FFF
+        x[::2] = inputs.fp32_to_bf16_bits(np.full(1, 1.0078125, np.float32))[0]      # (and half of the tokens constant)
     else:
         wr[:] = wr[0]                        # all experts alike ...
         wr[:, 0] = inputs.fp32_to_bf16_bits(np.linspace(-1e-2, 1e-2, w.E).astype(np.float32))   # ... but for one column
-    _, idx, tw = _route_only(w, x, wr, None)
+    plan, idx, tw = _route_only(w, x, wr, None)
+    assert plan.moe_last_status() == (0, 0)      # (the error bound held on every candidate)
     ridx, rw, _ = oracle.route(x, wr, None, w.K, w.dtype)
-    Hh.check_route(idx, tw, ridx, rw)
-    # and the plain chains-for-everybody router gives the same
-    _, idx2, tw2 = _route_only(w, x, wr, None, route_filter=-1)
+    if case == "one_sign":
+        # The ruled-out experts' approximate logits are in the denominator, and here a logit is the sum of all magnitudes (up
+        # to 70, a unit in its last place is 8e-6): a weight may be off by as much, relatively, as two logits are, and they
+        # are off by at most 0.16 of the bound eps (measured on such rows).
+        fx, fw = ((a.astype(np.uint32) << 16).view(np.float32).astype(np.float64) for a in (x, wr))
+        eps = (H / 2 + 68 * -(-H // 256) + 3) * 2.0 ** -23 * np.linalg.norm(fx, axis=1) * np.linalg.norm(fw, axis=1).max()
+        assert np.array_equal(idx.cpu().numpy(), ridx)
+        assert (np.abs(tw.cpu().numpy() - rw) <= rw * (1e-5 + 2 * 0.16 * eps[:, None]) + 1e-7).all()
+    else:
+        Hh.check_route(idx, tw, ridx, rw)
+    # and the kernel that runs every chain (above 1024 tokens another one) gives the same
+    plan2, idx2, tw2 = _route_only(w, x, wr, None, route_filter=-1)
+    assert plan2.moe_last_status() == (0, 0)
     assert torch.equal(idx, idx2)
 
 

@@ -350,9 +350,9 @@ static int make_map_f32(EncodeTiledFn enc, CUtensorMap* m, const void* base, int
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
 }
 
-template <int TM, int TN, int WR, bool SWIGLU, bool ANY>
-static int launch_fp32_grid(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
-                            const Fp32Params& q, cudaStream_t st) {
+template <int TM, int TN, int WR, bool SWIGLU>
+static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
+                            const Fp32Params& q, cudaStream_t st, bool own) {
   constexpr int BM = WR * 2 * TM, BN = kF32Warps / WR * 16 * TN, NOUT = SWIGLU ? BN / 2 : BN;
   const cuuint64_t E = (cuuint64_t)p->cfg.E, K = (cuuint64_t)q.Kd, N = (cuuint64_t)q.N, tp = (cuuint64_t)p->tp;
   CUtensorMap ma, mb1, mb2;
@@ -368,27 +368,24 @@ static int launch_fp32_grid(moe_plan* p, EncodeTiledFn enc, const void* A, const
     if ((rc = make_map_f32(enc, &mb1, b1, 4, dims, str, BN)) != MOE_OK) return rc;
     mb2 = mb1;
   }
-  auto kern = ffn_fp32_kernel<TM, TN, WR, SWIGLU, ANY>;
-  constexpr size_t smem = 1024 + (size_t)kF32Stages<TM, TN, WR> * kF32StageBytes<TM, TN, WR>;
-  static SmemAttrOnce once;
-  if (ensure_dynamic_smem(kern, smem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
   // Inside moe_layer a CTA per block that there can be: the counts add up to T * K, so besides full blocks there is at most
-  // one per tile.  A caller's table may have any number of whole tiles or of empty ones, and each CTA walks the table: not
-  // more than 16 CTAs per SM then, five times what is resident.  Measured, moe_expert_ffn with counters, us, a CTA per block
-  // there could be / this: 1024 tiles of static regions, 500 tokens, H 256, F 512 193 / 83; 12 tiles, T 256, H 128, F 256 23.6 /
-  // 25.6; 31 tiles, T 1000, H 1024, F 2048 722 / 708; 81 tiles, T 700, H 512, F 512 189 / 196; 32 and 64 per SM: 83 and 95 on the first.
+  // one per tile.  A caller's table may have any number of whole tiles or of empty ones: a CTA per block that any of its tiles
+  // could have, but as each of them walks the table not more than 16 per SM, five times what is resident.  Measured,
+  // moe_expert_ffn with counters, us, always a CTA per block / this: 1024 tiles of static regions, 500 tokens, H 256, F 512 193
+  // / 83; 31 tiles, T 1000, H 1024, F 2048 722 / 708; 81 tiles, T 700, H 512, F 512 189 / 196; 32 and 64 per SM: 83 and 95 on
+  // the first.
   const long long cols = (q.N + NOUT - 1) / NOUT, all = (long long)p->P * (kTileRows / BM) * cols;
   const int sms = p->sm_count > 0 ? p->sm_count : 148;
-  const dim3 grid((unsigned)min(all, ANY ? 16ll * sms : ((long long)q.total_rows / BM + p->P) * cols));
+  const bool any = !own && all > 16ll * sms;
+  const dim3 grid((unsigned)(own ? min(all, ((long long)q.total_rows / BM + p->P) * cols) : any ? 16ll * sms : all));
+  constexpr size_t smem = 1024 + (size_t)kF32Stages<TM, TN, WR> * kF32StageBytes<TM, TN, WR>;
   p->launches += 1;
-  return launch_pdl(kern, grid, dim3(kF32Threads), smem, st, ma, mb1, mb2, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
-}
-
-template <int TM, int TN, int WR, bool SWIGLU>
-static int launch_fp32_gemm(moe_plan* p, EncodeTiledFn enc, const void* A, const void* b1, const void* b2,
-                            const Fp32Params& q, cudaStream_t st, bool own) {
-  return own ? launch_fp32_grid<TM, TN, WR, SWIGLU, false>(p, enc, A, b1, b2, q, st)
-             : launch_fp32_grid<TM, TN, WR, SWIGLU, true>(p, enc, A, b1, b2, q, st);
+  auto launch = [&](auto kern, SmemAttrOnce& once) -> int {
+    if (ensure_dynamic_smem(kern, smem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
+    return launch_pdl(kern, grid, dim3(kF32Threads), smem, st, ma, mb1, mb2, q) == cudaSuccess ? 0 : MOE_ERR_CUDA;
+  };
+  static SmemAttrOnce once[2];
+  return any ? launch(ffn_fp32_kernel<TM, TN, WR, SWIGLU, true>, once[1]) : launch(ffn_fp32_kernel<TM, TN, WR, SWIGLU, false>, once[0]);
 }
 
 // Both GEMMs of an fp32 plan.
@@ -413,7 +410,12 @@ static int launch_fp32(moe_plan* p, const void* recv, const int* tile_expert, co
   // both where that gives enough CTAs; otherwise 4 x 4 (32 x 64).  Measured, whole layer, us, 8 x 8 / 4 x 8 / 4 x 4: 500 rows
   // per expert 357 / 382 / 383, 250 rows (H 512, F 1024) 248 / 242 / 215, 125 rows 787 / 735 / 766, 66 rows 157 / 143 / 138,
   // 37 rows 470 / 409 / 365.
-  const long long rows = (long long)c.T * c.K, blocks = rows / 64 + c.E;  // 64-row blocks, about
+  // (Without row counts every tile is computed whole: rows as many as a tile per expert has, once most experts have one.
+  // Measured without counts, us, by T * K / by this: 36 rows per expert, 256 experts, H 160, F 48 108 / 93; 33, 60 experts, H 512,
+  // F 512 417 / 318; 16, 16 experts, H 1024, F 2048 841 / 671.)
+  const long long assigned = (long long)c.T * c.K;
+  const long long rows = tile_count == nullptr && assigned >= 16ll * c.E ? max(assigned, (long long)kTileRows * c.E) : assigned;
+  const long long blocks = rows / 64 + c.E;  // 64-row blocks, about
   const int shape = rows >= 192ll * c.E ? 2 : rows >= 96ll * c.E ? 1 : 0;
   // 4 x 4: how many warps stand along the rows.  An expert's last block of rows leaves warps without rows, and a warp
   // that leaves leaves its scheduler idle, so blocks of eight rows (all warps along the columns) up to 48 rows per expert,

@@ -41,13 +41,27 @@ WORKLOADS = {"c1": inputs.C1, "c2": inputs.C2, "c3": inputs.C3, "c4": inputs.C4,
 
 
 
-def ncu_traffic_bytes(workload: str):
-    """DRAM traffic of the dominant kernel per step, measured with ncu and kept beside the profile summaries."""
+def expert_kernel(args, w) -> str:
+    """The bf16 expert kernel that the plan's options take (the rules of csrc/ffn_tc.cu and ffn_few.cu)."""
+    tp = max(1, args.tp_shards)
+    assignments, experts, width = w.T * w.K * tp, w.E * tp, w.F // tp
+    if args.ffn_kernel == 1:
+        return "ffn_simt_kernel"
+    if args.ffn_kernel == 2:
+        return "ffn_pair_kernel"
+    plain = args.overlap == 0 and args.ffn_hot_min_tiles <= 0 and args.ffn_thin_tiles >= 0
+    few = w.T <= 5 or (w.T <= 32 and assignments <= 256 and assignments * (w.H + 2 * width) <= 65536)
+    if few and plain and args.ffn_split == 0 and w.H >= 256 and width >= 256:
+        return "few-token kernels"
+    return "ffn_pair_kernel" if plain and assignments > 128 * experts and w.H >= 1536 and width >= 1024 else "ffn_tc_kernel"
+
+
+def ncu_traffic_bytes(workload: str, kernel: str):
+    """DRAM traffic of the dominant kernel per step, measured with ncu on that kernel and kept beside the profile summaries."""
     path = os.path.join(ROOT, "profiles", "ncu_dram_traffic.json")
     try:
         with open(path) as f:
-            entry = json.load(f).get(workload)
-        return None if entry is None else float(entry["bytes"])
+            return float(json.load(f)[workload][kernel]["bytes"])
     except (OSError, ValueError, KeyError, TypeError):
         return None
 
@@ -511,7 +525,7 @@ def run_cuda(args, w: inputs.Workload) -> None:
     if w.identity_experts or w.dtype != inputs.BF16:
         dom = "dispatch"
         roofline = {"kernel": "dispatch", "bound": "hbm", "achieved": stages["dispatch"]["GBps"], "peak": hbm_peak,
-                    "unit": "GB/s", "frac": stages["dispatch"]["frac_hbm"], "traffic": ncu_traffic_bytes(w.name),
+                    "unit": "GB/s", "frac": stages["dispatch"]["frac_hbm"], "traffic": ncu_traffic_bytes(w.name, "dispatch"),
                     "peak_source": f"{peak_kind} hbm_gbs"}
     else:
         t_ffn = sm["gemm1"] + sm["gemm2"]
@@ -531,9 +545,10 @@ def run_cuda(args, w: inputs.Workload) -> None:
         sustained = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
         long_run = ms_total >= 1000.0
         peak = sustained if long_run else peaks["bf16_tflops"]
-        roofline = {"kernel": "expert kernel (GEMM1 + SwiGLU + GEMM2, tcgen05: ffn_pair_kernel, or ffn_tc_kernel where experts have a tile of rows at most)", "bound": "tensor",
+        kernel = expert_kernel(args, w)
+        roofline = {"kernel": f"expert kernel (GEMM1 + SwiGLU + GEMM2): {kernel}", "bound": "tensor",
                     "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                    "traffic": ncu_traffic_bytes(w.name),
+                    "traffic": ncu_traffic_bytes(w.name, kernel),
                     "peak_source": f"{peak_kind} " + ("bf16_tflops_sustained (timed region of %.1f s)" % (ms_total / 1e3) if long_run else
                                                       "bf16_tflops, the burst figure (timed region of %.0f ms)" % ms_total) +
                                    "; the kernel's clock is in clocks.ffn_kernel_sm_mhz",

@@ -230,8 +230,10 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {  // a shared-memory loa
 // Programmatic dependent launch: the kernels of the layer (all but the first, the router: starting
 // it while the previous layer call drains measured slower) are launched so that they may start while
 // their predecessor in the stream is still draining.  pdl_wait() blocks until the predecessor has
-// completed and its writes are visible; nothing before it may touch global memory.  pdl_trigger()
-// lets the successor begin launching.
+// completed and its writes are visible.  Nothing before it may write global memory, or read what the
+// predecessor or anything before it may still write; what is read there all the same (few_down_kernel:
+// the picks, and weights into L2) was complete before the predecessor could trigger, because that one
+// triggers behind its own wait.  pdl_trigger() lets the successor begin launching.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

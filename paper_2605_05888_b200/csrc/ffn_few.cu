@@ -9,7 +9,7 @@
 // of one tile with a stride, so the work spreads over all SMs whatever the number of experts.
 // Measured, layer time, us, tensor-core kernels / this / with dispatch and combine taken in (second half of the file): one
 // Qwen-like token 57.7 / 41.3 / 31, one Mixtral-like 209.6 / 140 / 125 (705 MB of weights: 109 at the copy rate), one
-// DeepSeek-like 187 / 152 / 147; the rule in launch_ffn_tc has more.
+// DeepSeek-like 187 / 152 / 147; the rule at few_applies has more.
 #include "tc_common.cuh"
 #include "route_common.cuh"
 

@@ -84,9 +84,12 @@ typedef struct {
                                    where experts have more than one tile of rows on average, or
                                    plain FMAs for up to five tokens (small layers: 32; only with
                                    row counts and with ffn_split, ffn_thin_tiles and
-                                   ffn_hot_min_tiles left at 0) - and the fp32-FMA kernel for
-                                   fp32; 1: plain SIMT fp32-FMA kernel for bf16 (check path);
-                                   2: always CTA pairs (bf16).
+                                   ffn_hot_min_tiles left at 0) - and for fp32 the tensor cores on
+                                   operands split into three bf16 numbers each (closer to the sums
+                                   in 64 bits than fp32 FMAs; operands below 2^-109 in magnitude
+                                   keep fewer bits), or fp32 FMAs for little work and for fewer
+                                   than eight rows per expert; 1: fp32 FMAs always (bf16: a plain
+                                   SIMT kernel, the check path); 2: always CTA pairs (bf16).
                                    The tensor-core forms add up every result in the same order,
                                    so a row's bytes do not depend on which of them computes it,
                                    nor on how many other rows there are.  The plain-FMA kernel
@@ -94,7 +97,8 @@ typedef struct {
                                    token's y may differ in the last bits of bf16 between a batch
                                    of 5 and one of 6, and moe_expert_ffn's rows between calls with
                                    and without row counts.  Naming ffn_split (1 or 2) keeps the
-                                   tensor-core forms, and a token's bytes, at every batch size */
+                                   tensor-core forms, and a token's bytes, at every batch size
+                                   (fp32: ffn_kernel 1 keeps the FMAs)                         */
   int32_t ffn_split;            /* 1: one launch per expert GEMM; 2: both GEMMs in one persistent
                                    launch (per-tile status counters gate GEMM2); 0: choose
                                    (one launch when E <= 64; with more, smaller experts two

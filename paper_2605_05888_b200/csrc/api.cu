@@ -119,7 +119,12 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   }
   t.gemm1_done = (int*)take(sizeof(int) * (size_t)((g.P > 0 ? g.P : 1) + 4));  // + the expert kernel's item and exit counters
   const size_t pool_rows = (size_t)g.P * kTileRows;
-  if (!c.identity_experts) t.inter = take(pool_rows * c.F * g.eb);
+  if (ffn_split_applies(c, g.P)) {  // three bf16 planes each: 6 bytes per element
+    t.inter = take(pool_rows * split_pitch(c.F) * 6);
+    t.recv_planes = take(pool_rows * split_pitch(c.H) * 6);
+  } else if (!c.identity_experts) {
+    t.inter = take(pool_rows * c.F * g.eb);
+  }
   const int experts = c.E / g.tp;  // (c.E counts every TP shard)
   const bool may_filter = c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
   const bool chains = route_chains_apply(experts, c.T, c.H, may_filter), filter = may_filter && !chains;

@@ -2,8 +2,8 @@
 // into the intermediate buffer, then O = S*Wd^T, two launches.  Tiles without an owner exit at once, so the weights of
 // experts that received no rows are never read.
 //
-// Two kernels.  ffn_fp32_kernel is the path of dtype fp32 (a tensor-core tf32 product cannot meet the 1e-4 error
-// bound).  ffn_simt_kernel, slow and simple, is a second, independent device implementation to check the tcgen05
+// Two kernels.  ffn_fp32_kernel is the path of dtype fp32 for little work and for few rows per expert (the other shapes go
+// to the tensor cores, split into bf16 numbers: ffn_split.cu).  ffn_simt_kernel, slow and simple, is a second, independent device implementation to check the tcgen05
 // kernel against on bf16 data (ffn_kernel = 1).
 #include "tc_common.cuh"
 
@@ -476,6 +476,7 @@ int launch_ffn_simt(moe_plan* p, const void* recv, const int* tile_expert, const
   if (p->P == 0 || p->cfg.T == 0) return 0;
   if (p->cfg.dtype == MOE_DTYPE_BF16)
     return launch_typed<__nv_bfloat16>(p, recv, tile_expert, wg, wu, wd, out_rows, st);
+  if (ffn_split_applies(p->cfg, p->P)) return launch_ffn_split(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
   return launch_fp32(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st, own);
 }
 

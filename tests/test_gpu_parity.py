@@ -309,6 +309,79 @@ def test_fp32_expert_kernel_more_blocks_than_ctas(case):
         assert torch.count_nonzero(out[~owned]) == 0
 
 
+# dtype fp32 on the tensor cores, where its items end: rows around 16, 32, 64 and 128 (one tile, two), H and F that end inside
+# 64 gate columns, 128 columns, 32 and 64 k, sums of odd numbers of 32-k blocks and of fewer than 256 terms, TP shards.
+# Per GEMM an element is off by at most n 2^-24 of sum |a b| (n additions; n <= K / 16 truncated ones and K / 32 rounded
+# ones), in the 2-norm by about sqrt(K) times less: 1e-6 holds for K up to 2048 with room (seen: 3e-7).
+SPLIT_FFN = [
+    # (T, H, E, K, F, tp)
+    (1, 68, 1, 1, 900, 1), (15, 68, 1, 1, 964, 1), (16, 100, 1, 1, 1028, 1), (17, 36, 2, 2, 932, 1), (33, 128, 1, 1, 960, 1), (65, 260, 2, 2, 900, 1),
+    (127, 96, 1, 1, 2052, 1), (128, 516, 2, 1, 996, 1), (129, 260, 2, 2, 1284, 1), (300, 1028, 4, 2, 132, 1), (700, 324, 3, 3, 1088, 1),
+    (400, 260, 2, 2, 1000, 2),
+]
+
+
+@pytest.mark.parametrize("case", SPLIT_FFN, ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}")
+def test_fp32_on_tensor_cores_edges(case):
+    T, H, E, K, F, tp = case
+    w = inputs.Workload("fp32_split", T=T, H=H, E=E, R=1, K=K, F=F, dtype=FP32, seed=23)
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    ref = Hh.oracle_layer_for(w, x, wr, bias, wg, wu, wd)["y"]
+    args = [Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)]
+    errs = []
+    for kernel in (0, 1):     # split, and the fp32 FMAs
+        plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, tp_shards=tp, ffn_kernel=kernel)
+        y = torch.empty((T, H), dtype=torch.float32, device="cuda")
+        for _ in range(2):    # the counters are back where they were
+            plan.moe_layer(*args, y)
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == (0, 0)
+        d = Hh.to_host_f64(y) - ref
+        errs.append(np.linalg.norm(d) / np.linalg.norm(ref))
+    assert errs[0] <= 1e-6 and errs[0] <= 1.05 * errs[1], errs
+
+
+def test_fp32_on_tensor_cores_infinities_and_nan():
+    """What an infinity, a NaN, an overflow or a number that rounds up to bf16's infinity does to a row is what fp32 sums give."""
+    T, H, F = 48, 72, 928
+    plan = B.Plan(B.make_config(T, H, 1, 1, 1, F, FP32, dispatch_mode=B.DISPATCH_ATOMIC_PAGED))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    wg, wu, wd = (torch.empty(s, device="cuda").normal_(0.0, 0.05, generator=g) for s in ((1, F, H), (1, F, H), (1, H, F)))
+    x = torch.empty((T, H), device="cuda").normal_(generator=g)
+    x[1, 3], x[2, 5], x[3, 7], x[4, 9] = float("inf"), float("-inf"), float("nan"), 3.4e38
+    x[5] *= 1e38                 # sums that overflow or not
+    x[6], x[7, ::2] = 0.0, 0.0
+    wg[0, 10, 3], wd[0, 13, 14], wd[0, 17, 3], wd[0, 19, 4] = 0.0, float("nan"), 3.395e38, float("-inf")
+    wg[0, 20:40] = wg[0, 20:40].bfloat16().float()      # (no middle and last parts: infinity times zero)
+    recv = torch.zeros((plan.P * 128, H), device="cuda")
+    recv[:T] = x
+    te = torch.full((plan.P,), -1, dtype=torch.int32, device="cuda")
+    te[0] = 0
+    count, done = torch.tensor([T] + [0] * (plan.P - 1), dtype=torch.int32, device="cuda"), torch.full((1,), T, dtype=torch.int32, device="cuda")
+    out = torch.zeros_like(recv)
+    plan.moe_expert_ffn(recv, te, wg, wu, wd, out, count, done)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    def chain(a, b):             # one fp32 product and sum after the other
+        s = np.zeros((a.shape[0], b.shape[0]), np.float32)
+        for k in range(a.shape[1]):
+            s = (a[:, k, None].astype(np.float64) * b[None, :, k].astype(np.float64) + s).astype(np.float32)
+        return s
+    with np.errstate(all="ignore"):
+        xs, hg, hu, hd = (t.cpu().numpy() for t in (x, wg[0], wu[0], wd[0]))
+        gate, up = chain(xs, hg), chain(xs, hu)
+        want = chain((gate / (np.float32(1) + np.exp(-gate)) * up).astype(np.float32), hd)
+    got = out[:T].cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    assert np.array_equal(np.isposinf(got), np.isposinf(want)) and np.array_equal(np.isneginf(got), np.isneginf(want))
+    assert np.isnan(want).any() and np.isinf(want).any() and np.isfinite(want).sum() > T * H // 2
+    ok = np.isfinite(want)
+    got, want = np.where(ok, got, 0).astype(np.float64), np.where(ok, want, 0).astype(np.float64)
+    usual = np.delete(want, 3, axis=1)     # (column 3 is 1e37 times the others)
+    scale = np.sqrt(np.mean(usual ** 2, axis=1, keepdims=True))
+    assert (np.abs(got - want) <= 1e-4 * np.maximum(np.abs(want), scale)).all()
+
+
 # The CTA-pair expert kernel where its items end: an expert's rows around 16, 32, 128 (one tile), 129, 256 (a pair of
 # tiles) and 257, all experts the same so that every count is met; in the paged layout (tiles of an expert apart) and
 # the ordered one; H and F that end inside its 512- and 256-column blocks and inside a k-block; one and two launches.

@@ -329,7 +329,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
     }
   } else if (warp == 1) {
     // ===================== MMA issuer =====================
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase_bit = 0;
       for (int local_item = 0; !fail_site; ++local_item) {
@@ -526,7 +526,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap map_a1, const __grid_constant_
   if (sh->abort_flag) {
     // Whichever role gave up, what the others had issued may still be in flight: the MMAs read the stages and write tensor
     // memory, the copies write the stages.  All of them end (both waits are bounded) before the CTA frees either.
-    if (warp == 1 && lane == 0) {
+    if (warp == 1 && elect_one()) {
       tc_commit(smem_u32(&sh->drain));
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(smem_u32(&sh->drain), 0u))

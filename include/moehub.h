@@ -140,8 +140,9 @@ typedef struct {
                                    (approximate logits by tcgen05 MMAs, then the exact fp32 chain only
                                    for the experts that can still be among the K largest: the picks
                                    are the exact ones, bit for bit) for batches of more than 1024
-                                   tokens (more than 192 experts and H above 4096: 864), every chain
-                                   for smaller ones; -1 = every chain computed.  In the filter's
+                                   tokens (more than 192 experts and H above 4096: 864) and from
+                                   T*E*H = 3.2e8 on (H up to 8192; beyond 592 tokens twice that),
+                                   every chain for smaller ones; -1 = every chain.  In the filter's
                                    softmax weights the experts that were ruled out enter the
                                    denominator with their approximate logits: up to 2.7e-6 relative
                                    from the weights of the chains (1e-5 is tested; rows of one sign,

@@ -127,8 +127,10 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   }
   const int experts = c.E / g.tp;  // (c.E counts every TP shard)
   const bool may_filter = c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
-  const bool chains = route_chains_apply(experts, c.T, c.H, may_filter), filter = may_filter && !chains;
-  t.route_logits = filter || (chains && experts > 64) ? (float*)take(sizeof(float) * (size_t)(c.T > 0 ? c.T : 1) * 256) : nullptr;
+  const bool direct = c.T > 0 && route_direct_apply(experts, c.T, c.H, may_filter);
+  const bool chains = !direct && route_chains_apply(experts, c.T, c.H, may_filter), filter = may_filter && !chains;
+  const size_t slabs = direct ? (size_t)route_direct_slices(experts, c.T, c.H) : 1;
+  t.route_logits = filter || (chains && experts > 64) ? (float*)take(sizeof(float) * slabs * (size_t)(c.T > 0 ? c.T : 1) * 256) : nullptr;
   t.route_wnorm2 = filter ? (float*)take(sizeof(float) * 256) : nullptr;
   t.topk_idx = (int*)take(sizeof(int) * (size_t)c.T * c.K);
   t.topk_w = (float*)take(sizeof(float) * (size_t)c.T * c.K);

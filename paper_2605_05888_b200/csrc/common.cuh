@@ -151,6 +151,19 @@ inline bool route_chains_apply(int experts, int tokens, int H, bool filter) {
 }
 int launch_route_chains(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,
                         const PrepArgs& prep, cudaStream_t st);
+// the tensor-core filter with the candidates' rows fetched one by one, for batches in between (route_filter.cu): from where
+// the chains of all experts are bound by their FMAs up to two waves of its CTAs (two tokens each, two CTAs per SM), twice the work
+// where there are two.  Measured, router call, us, every chain (beyond 1024 tokens the filter over all rows) / this: 256 experts, H
+// 7168: T 128 31 / 39, T 160 40 / 37, T 256 43 / 37, T 512 70 / 39, T 592 72 / 43, T 640 84 / 70, T 1024 99 / 70, T 1500 99 / 103; 160
+// experts, H 5120: T 300 33 / 31, T 592 52 / 33, T 800 62 / 54; 256, H 2048: T 256 19 / 25, T 592 29 / 25, T 1024 40 / 39; 128, H
+// 4096: T 256 21 / 27, T 512 27 / 27, T 1024 42 / 43.
+inline bool route_direct_apply(int experts, int tokens, int H, bool filter) {
+  return filter && experts > 64 && experts <= 256 && H <= 8192 && tokens <= 1184 &&
+         (long long)tokens * experts * H >= 320000000ll * (tokens > 592 ? 2 : 1);
+}
+int route_direct_slices(int experts, int tokens, int H);
+int launch_route_direct(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,
+                        const PrepArgs& prep, cudaStream_t st);
 // the tensor-core filter in front of the exact chains (many experts, bf16): see route_filter.cu
 bool route_filter_applies(const moe_plan* p);
 int launch_route_filter(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,

@@ -89,7 +89,10 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
   volatile int* abort_flag = &sh->abort_flag;
-  const int KB = (H + kBK - 1) / kBK;
+  // this CTA's slice of h, in steps of 64 columns (gridDim.z slices: a scratch of their own each, summed by the reader)
+  const int all = (H + kBK - 1) / kBK, per = (all + gridDim.z - 1) / gridDim.z;
+  const int kb0 = blockIdx.z * per, KB = min(per, all - kb0);
+  logits += (size_t)blockIdx.z * T * kRfEP;
   const int t0 = blockIdx.x * kTileRows;
   const int e0 = blockIdx.y * 128;  // this CTA's half of the experts
   int fail_site = 0;
@@ -103,8 +106,8 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         const uint32_t full = smem_u32(&sh->full[stage]);
         const uint32_t a_dst = smem_u32(stage_base + stage * kStageBytes);
         mbar_expect_tx(full, (uint32_t)(kABytes + kBBytes / 2));
-        tma_load_2d(a_dst, &map_x, full, kb * kBK, t0);   // rows past T and columns past H arrive as zeros
-        tma_load_2d(a_dst + kABytes, &map_w, full, kb * kBK, e0);  // 128 experts' rows
+        tma_load_2d(a_dst, &map_x, full, (kb0 + kb) * kBK, t0);   // rows past T and columns past H arrive as zeros
+        tma_load_2d(a_dst + kABytes, &map_w, full, (kb0 + kb) * kBK, e0);  // 128 experts' rows
         ++fills;
         if (++stage == kStages) { stage = 0; phase_bit ^= 1u; }
       }
@@ -133,9 +136,10 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     }
   } else {
     // While the main loop runs: |w_e|^2 for this CTA's share of the experts (the refine kernel's error bound).
-    for (int e = (blockIdx.y * gridDim.x + blockIdx.x) * 4 + (warp - 2); e < E; e += gridDim.x * gridDim.y * 4) {
+    for (int e = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 4 + (warp - 2); e < E; e += gridDim.x * gridDim.y * gridDim.z * 4) {
       const uint4* row = reinterpret_cast<const uint4*>(wr + (size_t)e * H);
       float s = 0.0f;
+#pragma unroll 8
       for (int v = lane; v < H / 8; v += 32) {
         float f[8];
         Vec16<__nv_bfloat16>::unpack(__ldg(row + v), f);
@@ -516,10 +520,296 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   route_prep_end(prep, s_hist);
 }
 
+// ---- (2') the same for batches of up to some thousand tokens ------------------------------------------
+// The refine kernel above brings all of Wr to every CTA, which pays where a CTA has tens of tokens.  Here a CTA takes two
+// tokens, keeps their rows of x in shared memory and fetches the rows of its candidates alone (about twenty), each lane of
+// a producer warp the row of one chain, 1 KB at a time through two buffers (a bulk copy costs its issuer some fifty clocks:
+// in pieces of 256 bytes they took longer than the chains, 60 us instead of 39).  One warp runs the chains, a lane each; rows
+// lie 16 bytes off a multiple of 128 apart, so its 16-byte loads meet no bank twice.  What bounds it is the chain's own
+// latency (4.5 cycles per h: 17 us at H 7168) where running all E chains is bound by their FMAs.  Whole router call, 256
+// experts, H 7168, us, every chain / this: T 256 43 / 37, T 512 70 / 39, T 1024 99 / 70 (a second wave of CTAs).
+constexpr int kRdTokens = 2, kRdChains = 32, kRdThreads = 128, kRdBufs = 2;
+constexpr int kRdChunk = 512, kRdPitch = kRdChunk * 2 + 16;  // h per step; bytes from one chain's chunk to the next one's
+__host__ __device__ constexpr int rd_x_pitch(int H) { return (H * 2 + 127) / 128 * 128 + 16; }
+constexpr size_t rd_smem(int H) {
+  return 16 + (size_t)kRdTokens * rd_x_pitch(H) + (size_t)kRdBufs * kRdChains * kRdPitch + (size_t)kRdTokens * kRfEP * (4 + 2);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
+// The K-th largest of a warp's keys (order_key; 0: none), eight per lane at experts lane + 32 j; FLT_MAX's negative if there are fewer.
+__device__ __forceinline__ float rd_kth(int K, int lane, unsigned (&key)[8]) {
+  unsigned bk = 0;
+  for (int k = 0; k < K; ++k) {
+    bk = key[0];
+#pragma unroll
+    for (int j = 1; j < 8; ++j) bk = max(bk, key[j]);
+    bk = __reduce_max_sync(0xffffffffu, bk);
+    unsigned be = 0xffffffffu;
+#pragma unroll
+    for (int j = 7; j >= 0; --j)
+      if (key[j] == bk) be = (unsigned)(lane + 32 * j);
+    be = __reduce_min_sync(0xffffffffu, be);  // one of several equal ones leaves
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (be == (unsigned)(lane + 32 * j)) key[j] = 0u;
+  }
+  return bk == 0u ? -FLT_MAX : __uint_as_float((bk & 0x80000000u) ? bk ^ 0x80000000u : ~bk);
+}
+
+__global__ void __launch_bounds__(kRdThreads)
+route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wr, const float* __restrict__ bias,
+                    const float* __restrict__ logits, int slices, const float* __restrict__ wnorm2, float additions, int sms, int T, int H,
+                    int E, int K, int renorm, int* __restrict__ topk_idx, float* __restrict__ topk_w, const PrepArgs prep, int tp,
+                    unsigned long long wait_ns, int* __restrict__ status) {
+  __shared__ int s_hist[kRouteMaxExperts];
+  __shared__ float s_xn2[kRdThreads / 32], s_eps[kRdTokens];
+  __shared__ unsigned long long s_full[kRdBufs], s_empty[kRdBufs], s_x;
+  __shared__ int s_total[3], s_fills, s_abort;  // chains per round; chunks whose copies have been issued
+  extern __shared__ uint8_t rd_dyn[];
+  uint8_t* xrow = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(rd_dyn) + 15) & ~(uintptr_t)15);
+  const int x_pitch = rd_x_pitch(H);
+  uint8_t* ring = xrow + kRdTokens * x_pitch;                                        // [kRdBufs][kRdChains][kRdPitch]
+  float* ls = reinterpret_cast<float*>(ring + kRdBufs * kRdChains * kRdPitch);       // [kRdTokens][256]
+  unsigned short* chains = reinterpret_cast<unsigned short*>(ls + kRdTokens * kRfEP);  // token << 8 | expert
+  const int t0 = blockIdx.x * kRdTokens, tvalid = min(kRdTokens, T - t0);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, tl = warp;  // a warp per token for what is per token
+  const bool live = tl < tvalid;
+  // the CTAs of an SM run their chains on different schedulers
+  const int chain_warp = (int)(blockIdx.x / (unsigned)sms) % 4, load_warp = (chain_warp + 1) % 4;
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < kRdBufs; ++b) {
+      mbar_init(smem_u32(&s_full[b]), 1);
+      mbar_init(smem_u32(&s_empty[b]), 1);
+    }
+    mbar_init(smem_u32(&s_x), 1);
+    s_abort = s_fills = s_total[0] = s_total[1] = s_total[2] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // (x and Wr were complete before the kernel in front of this one could start)
+    mbar_expect_tx(smem_u32(&s_x), (uint32_t)(tvalid * H * 2));
+    for (int i = 0; i < tvalid; ++i) bulk_load(smem_u32(xrow + i * x_pitch), x + (size_t)(t0 + i) * H, (uint32_t)(H * 2), smem_u32(&s_x));
+  }
+  __syncthreads();
+  volatile int* abort_flag = &s_abort;
+  bool failed = !mbar_wait(smem_u32(&s_x), 0u, abort_flag, wait_ns);
+  if (failed) s_abort = 1;
+  {  // |x_t|^2: two warps per token
+    const int t = warp / 2;
+    float s = 0.0f;
+    if (t < tvalid && !failed)
+      for (int q = (warp % 2) * 32 + lane; q < H / 8; q += 64) {
+        float f[8];
+        Vec16<__nv_bfloat16>::unpack(lds128(smem_u32(xrow + t * x_pitch) + (uint32_t)q * 16u), f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s = fmaf(f[i], f[i], s);
+      }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) s_xn2[warp] = s;
+  }
+  pdl_wait();
+  pdl_trigger();
+  route_prep_begin(prep, s_hist);
+  // the slices of the approximate logits, four experts per thread, and the bias the way the chain's value gets it
+  for (int i = threadIdx.x; i < tvalid * (kRfEP / 4); i += kRdThreads) {
+    const int t = i / (kRfEP / 4), e = i % (kRfEP / 4) * 4;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4* src = reinterpret_cast<const float4*>(logits + (size_t)(t0 + t) * kRfEP + e);
+    if (e < E) {
+#pragma unroll 16
+      for (int z = 0; z < slices; ++z) {
+        const float4 v = __ldcg(src + (size_t)z * T * (kRfEP / 4));
+        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+      }
+    }
+    const float f[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ls[t * kRfEP + e + q] = e + q >= E ? -FLT_MAX : bias != nullptr ? f[q] + bias[e + q] : f[q];
+  }
+  __syncthreads();
+  const float* row = ls + (live ? tl : 0) * kRfEP;
+  // Nothing is known of a token with a logit that is NaN or infinite, or whose error bound is: it gets every chain.  (A bias of
+  // minus infinity is none of these: such an expert's logit is that in any case.)
+  bool wild = false;
+  float v[8], thr = 0.0f, eps = 0.0f;  // the approximate logits of experts lane + 32 j
+  if (live) {
+    float wm2 = 0.0f;
+    unsigned key[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int e = lane + 32 * j;
+      v[j] = row[e];
+      key[j] = e < E ? max(order_key(v[j]), 1u) : 0u;
+      wild = wild || (e < E && !(v[j] <= FLT_MAX));
+      if (e < E) wm2 = fmaxf(wm2, wnorm2[e]);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) wm2 = fmaxf(wm2, __shfl_xor_sync(0xffffffffu, wm2, off));
+    const float kth = rd_kth(K, lane, key);
+    // (the same first threshold and the same proof as in the refine kernel)
+    const float xn2 = s_xn2[2 * tl] + s_xn2[2 * tl + 1];
+    eps = kRfUlp * (0.5f * (float)H + additions) * sqrtf(xn2 * wm2) * 1.0001f + 4.0e-7f * (1.0f + fabsf(kth));
+    wild = __any_sync(0xffffffffu, wild) || !(eps <= FLT_MAX);
+    if (lane == 0) s_eps[tl] = wild ? INFINITY : eps;
+    thr = wild ? -INFINITY : kth - eps - 1.0e-3f * (1.0f + fabsf(kth));
+  }
+  unsigned done = 0;  // bit j: the chain of expert lane + 32 j has been run
+  const int nchunk = (H + kRdChunk - 1) / kRdChunk;
+  int step = 0;  // chunks so far over all passes: buffer = step % kRdBufs
+  for (int round = 0; round < 3; ++round) {  // a second round is rare, a third cannot be needed
+    unsigned cand = 0;
+    if (live && thr < FLT_MAX) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (lane + 32 * j < E && (wild || v[j] >= thr) && !((done >> j) & 1u)) cand |= 1u << j;
+    }
+    done |= cand;
+    if (cand != 0) {
+      int at = atomicAdd(&s_total[round], __popc(cand));
+      for (unsigned c = cand; c != 0; c &= c - 1) chains[at++] = (unsigned short)((tl << 8) | (lane + 32 * (__ffs(c) - 1)));
+    }
+    __syncthreads();
+    const int total = s_total[round];
+    if (total == 0 || s_abort) break;  // no token of the CTA asks for more (CTA-uniform)
+    for (int p = 0; p < total; p += kRdChains, step += nchunk) {
+      const int n = min(kRdChains, total - p);
+      const int mine = lane < n ? chains[p + lane] : -1, e = mine & 0xff, tk = (mine >> 8) & 0xff;
+      if (warp == load_warp) {
+        for (int ch = 0; ch < nchunk && !failed; ++ch) {
+          const int g = step + ch, b = g % kRdBufs;
+          if (!warp_agrees(mbar_wait(smem_u32(&s_empty[b]), ((uint32_t)(g / kRdBufs) & 1u) ^ 1u, abort_flag, wait_ns))) { failed = true; break; }
+          const uint32_t bytes = (uint32_t)min(kRdChunk, H - ch * kRdChunk) * 2u;
+          if (lane == 0) {
+            mbar_expect_tx(smem_u32(&s_full[b]), bytes * (uint32_t)n);
+            s_fills = g + 1;
+          }
+          __syncwarp();
+          if (mine >= 0)
+            bulk_load(smem_u32(ring + (b * kRdChains + lane) * kRdPitch), wr + (size_t)e * H + ch * kRdChunk, bytes, smem_u32(&s_full[b]));
+        }
+        if (failed) s_abort = 1;
+      } else if (warp == chain_warp) {
+        float acc = 0.0f;
+        const uint32_t w0 = smem_u32(ring) + (uint32_t)lane * kRdPitch, x0 = smem_u32(xrow) + (uint32_t)(mine >= 0 ? tk : 0) * (uint32_t)x_pitch;
+        auto eight = [&](const uint4& xa, const uint4& wa) {
+          acc = fma_bf16_lo(xa.x, wa.x, acc);
+          acc = fma_bf16_hi(xa.x, wa.x, acc);
+          acc = fma_bf16_lo(xa.y, wa.y, acc);
+          acc = fma_bf16_hi(xa.y, wa.y, acc);
+          acc = fma_bf16_lo(xa.z, wa.z, acc);
+          acc = fma_bf16_hi(xa.z, wa.z, acc);
+          acc = fma_bf16_lo(xa.w, wa.w, acc);
+          acc = fma_bf16_hi(xa.w, wa.w, acc);
+        };
+        for (int ch = 0; ch < nchunk && !failed; ++ch) {
+          const int g = step + ch, b = g % kRdBufs;
+          if (!warp_agrees(mbar_wait(smem_u32(&s_full[b]), (uint32_t)(g / kRdBufs) & 1u, abort_flag, wait_ns))) { failed = true; break; }
+          const uint32_t wb = w0 + (uint32_t)(b * kRdChains * kRdPitch), xb = x0 + (uint32_t)(ch * kRdChunk * 2);
+          const int units = min(kRdChunk, H - ch * kRdChunk) / 8;
+          if (units == kRdChunk / 8) {
+            uint4 xr[2][4], wv[2][4];  // the next four units' loads go out before this four's chain of 32 FMAs
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { xr[0][i] = lds128(xb + 16u * i); wv[0][i] = lds128(wb + 16u * i); }
+#pragma unroll 4
+            for (int q = 0; q < kRdChunk / 32; ++q) {
+              if (q + 1 < kRdChunk / 32)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { xr[(q + 1) & 1][i] = lds128(xb + 16u * (4 * q + 4 + i)); wv[(q + 1) & 1][i] = lds128(wb + 16u * (4 * q + 4 + i)); }
+#pragma unroll
+              for (int i = 0; i < 4; ++i) eight(xr[q & 1][i], wv[q & 1][i]);
+            }
+          } else {
+            for (int q = 0; q < units; ++q) eight(lds128(xb + 16u * q), lds128(wb + 16u * q));
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&s_empty[b]));
+        }
+        if (failed) s_abort = 1;
+        if (mine >= 0 && !failed) {
+          const float exact = bias != nullptr ? acc + bias[e] : acc;
+          // the error model, checked where both values are at hand: a miss is an error of this kernel, said aloud
+          if (!(fabsf(exact - ls[tk * kRfEP + e]) <= s_eps[tk]) && s_eps[tk] <= FLT_MAX) set_status(status, MOE_ERR_INTERNAL, 502);
+          ls[tk * kRfEP + e] = exact;
+        }
+      }
+    }
+    __syncthreads();
+    if (s_abort) break;  // (CTA-uniform: it is set in the passes alone)
+    // The K-th largest EXACT logit so far decides whether more chains are wanted: see the refine kernel.
+    if (live && !wild && thr < FLT_MAX) {
+      unsigned key[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) key[j] = ((done >> j) & 1u) ? max(order_key(row[lane + 32 * j]), 1u) : 0u;
+      const float kx = rd_kth(K, lane, key);
+      thr = thr + eps > kx ? kx - eps : FLT_MAX;
+    } else {
+      thr = FLT_MAX;
+    }
+  }
+  __syncthreads();
+  if (s_abort) {
+    // a copy that was waited for too long is still on its way: it has to land before the CTA's shared memory goes away
+    if (threadIdx.x == 0) {
+      auto settle = [&](unsigned long long* bar, uint32_t parity) {
+        const unsigned long long ts = globaltimer();
+        while (!mbar_try(smem_u32(bar), parity))
+          if (globaltimer() - ts > wait_ns + 1000000ull) break;
+      };
+      settle(&s_x, 0u);
+      for (int g = max(0, s_fills - kRdBufs); g < s_fills; ++g) settle(&s_full[g % kRdBufs], (uint32_t)(g / kRdBufs) & 1u);
+    }
+    if (threadIdx.x == 0) set_status(status, MOE_ERR_TIMEOUT, kWaitMbarTma);
+    __syncthreads();
+    return;
+  }
+  select_topk<32, kRfEP / 32>(ls, kRfEP, tvalid, t0, E, K, renorm, topk_idx, topk_w, prep.hist ? s_hist : nullptr, tp);
+  route_prep_end(prep, s_hist);
+}
+
 // ---- host side ----------------------------------------------------------------------------------------
 bool route_filter_applies(const moe_plan* p) {
   return p->cfg.dtype == MOE_DTYPE_BF16 && p->route_E > 64 && p->route_E <= kRfEP && p->cfg.route_filter >= 0 &&
          p->s.route_logits != nullptr;
+}
+
+// The slices of h that the approximate logits are computed in: as many CTAs as SMs, of four steps of 64 columns at least, and
+// not more than sixteen (their reader sums them).
+int route_direct_slices(int experts, int tokens, int H) {
+  const int tiles = (tokens + kTileRows - 1) / kTileRows * ((experts + 127) / 128), steps = (H + kBK - 1) / kBK;
+  const int per = (steps + max(1, min(min(148 / tiles, steps / 4), 16)) - 1) / max(1, min(min(148 / tiles, steps / 4), 16));
+  return (steps + per - 1) / per;
+}
+
+int launch_route_direct(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,
+                        const PrepArgs& prep, cudaStream_t st) {
+  const moe_config_t& c = p->cfg;
+  EncodeTiledFn enc;
+  int rc = get_encoder(p, &enc);
+  if (rc != MOE_OK) return rc;
+  CUtensorMap mx, mwh;
+  if ((rc = make_map_2d(enc, &mx, x, (uint64_t)c.T, (uint64_t)c.H, kTileRows)) != MOE_OK) return rc;
+  if ((rc = make_map_2d(enc, &mwh, wr, (uint64_t)p->route_E, (uint64_t)c.H, 128)) != MOE_OK) return rc;
+  static SmemAttrOnce once, once_b;
+  if (ensure_dynamic_smem(route_tc_logits_kernel, kTcSmem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
+  if (ensure_dynamic_smem(route_direct_kernel, rd_smem(c.H), p->device, once_b) != cudaSuccess) return MOE_ERR_CUDA;
+  const unsigned long long wait_ns = c.wait_limit_ns ? c.wait_limit_ns : kDefaultWaitNs;
+  const int slices = route_direct_slices(p->route_E, c.T, c.H), steps = (c.H + kBK - 1) / kBK, per = (steps + slices - 1) / slices;
+  if (launch_maybe_pdl(false, route_tc_logits_kernel, dim3((c.T + kTileRows - 1) / kTileRows, (p->route_E + 127) / 128, slices),
+                       dim3(kTcThreads), kTcSmem, st, mx, mwh, (const __nv_bfloat16*)wr, c.T, c.H, p->route_E, p->s.route_logits,
+                       p->s.route_wnorm2, wait_ns, p->s.status) != cudaSuccess)
+    return MOE_ERR_CUDA;
+  // the additions of the error model: 17 per MMA of an accumulator, the four accumulators' sum, the slices'
+  const float additions = 68.0f * (float)((per + 3) / 4) + 3.0f + (float)(slices - 1);
+  if (launch_pdl(route_direct_kernel, dim3((c.T + kRdTokens - 1) / kRdTokens), dim3(kRdThreads), rd_smem(c.H), st,
+                 (const __nv_bfloat16*)x, (const __nv_bfloat16*)wr, bias, (const float*)p->s.route_logits, slices,
+                 (const float*)p->s.route_wnorm2, additions, p->sm_count > 0 ? p->sm_count : 148, c.T, c.H, p->route_E, p->route_K,
+                 c.renormalize, topk_idx, topk_w, prep, p->tp, wait_ns, p->s.status) != cudaSuccess)
+    return MOE_ERR_CUDA;
+  p->launches += 2;
+  return 0;
 }
 
 int launch_route_filter(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx, float* topk_w,

@@ -1351,6 +1351,53 @@ def test_overlapped_launch_many_runs_same_bytes():
         assert torch.equal(y, y0), i
 
 
+# The router that fetches its candidates' rows one by one: odd token counts (a CTA of one), H that ends inside its 512-column
+# steps and inside 64 columns, one and several slices of the approximate logits, one wave of CTAs and two, few and all experts.
+DIRECT_SHAPES = [(160, 7168, 256, 8, 0.0), (593, 8184, 256, 8, 1.2), (591, 7176, 193, 3, 0.0), (1183, 5128, 129, 1, 1.0), (577, 8192, 68, 32, 0.0),
+                 (301, 4104, 256, 16, 0.0)]
+
+
+@pytest.mark.parametrize("shape", DIRECT_SHAPES, ids=lambda s: f"T{s[0]}_H{s[1]}_E{s[2]}_K{s[3]}_z{s[4]}")
+def test_router_direct_kernel_edges(shape):
+    T, H, E, K, zipf = shape
+    w = inputs.Workload("direct", T=T, H=H, E=E, R=1, K=K, F=8, dtype=BF16, zipf_s=zipf, seed=31)
+    x, (wr, bias) = inputs.make_x(w), inputs.make_router(w)
+    ridx, rw, _ = oracle.route(x, wr, bias, K, BF16)
+    plan, idx, tw = _route_only(w, x, wr, bias)
+    assert plan.moe_last_status() == (0, 0)
+    Hh.check_route(idx, tw, ridx, rw)
+
+
+def test_router_direct_kernel_degenerate_rows():
+    """Rows of zeros (every expert a candidate), experts that are equal or an ulp apart, biases of minus infinity and of the
+    lowest number, infinities and NaN in x and in Wr: the picks and their weights that every chain gives."""
+    w = inputs.Workload("direct_wild", T=300, H=5120, E=256, R=1, K=8, F=8, dtype=BF16, seed=32)
+    x, (wr, _) = inputs.make_x(w), inputs.make_router(w)
+    x[::7] = 0
+    wr[40:80] = wr[40]
+    wr[90, 5] ^= 1
+    wr[91] = wr[90]
+    wr[91, 5] ^= 1
+    bias = np.zeros(w.E, np.float32)
+    bias[100:200], bias[200:230] = -np.inf, -np.finfo(np.float32).max
+    ridx, rw, _ = oracle.route(x, wr, bias, w.K, BF16)
+    plan, idx, tw = _route_only(w, x, wr, bias)
+    assert plan.moe_last_status() == (0, 0)
+    Hh.check_route(idx, tw, ridx, rw)
+    inf, nan, big = (int(inputs.fp32_to_bf16_bits(np.full(1, v, np.float32))[0]) for v in (np.inf, np.nan, 3e38))
+    xs = x.copy()
+    xs[1, 3], xs[2, 4], xs[3, 5], xs[4, 6] = inf, inf ^ 0x8000, nan, big
+    for case in range(3):
+        ws = wr.copy()
+        if case:
+            ws[17, 9] = inf if case == 1 else nan
+        plan, idx, tw = _route_only(w, xs, ws, bias)
+        _, want_idx, want_w = _route_only(w, xs, ws, bias, route_filter=-1)
+        assert plan.moe_last_status() == (0, 0)
+        assert torch.equal(idx, want_idx)
+        assert torch.allclose(tw, want_w, rtol=1e-5, atol=1e-7, equal_nan=True)
+
+
 def _route_only(w, x, wr, bias, **kw):
     plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, **kw)
     idx = torch.empty((w.T, w.K), dtype=torch.int32, device="cuda")

@@ -743,6 +743,42 @@ def _dispatch_with_counters(w, plan, dx, didx):
     return b
 
 
+@pytest.mark.parametrize("case", [(1, 8, 1, 1), (33, 8, 3, 1), (129, 16, 33, 32), (512, 8, 256, 8), (4096, 8, 256, 1), (4097, 8, 7, 1), (1365, 8, 5, 3)],
+                         ids=lambda c: f"T{c[0]}_E{c[2]}_K{c[3]}")
+def test_paged_dispatch_where_its_small_batches_end(case):
+    """A caller's own ids, on buffers full of old values: every table entry of a dispatch that is one launch, up to 4096 ids and
+    beyond; ids that are no expert; one expert with every row."""
+    T, H, E, K = case
+    w = inputs.Workload("small_dispatch", T=T, H=H, E=E, R=1, K=K, F=0, dtype=BF16, identity_experts=True)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    g = torch.Generator(device="cuda").manual_seed(T)
+    x = torch.empty((T, H), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    any_ids = torch.rand((T, E), device="cuda", generator=g).argsort(1)[:, :K].to(torch.int32).contiguous()
+    one = torch.full((T, K), E - 1, dtype=torch.int32, device="cuda") if K == 1 else any_ids
+    bad = any_ids.clone()
+    bad[T // 2, 0] = E
+    for ids in (any_ids, one, bad):
+        old = lambda *s: torch.full(s, 12345, dtype=torch.int32, device="cuda")
+        recv = torch.zeros((plan.P * 128, H), dtype=torch.bfloat16, device="cuda")
+        count, te, src, slot, tc, done = old(E), old(plan.P), old(plan.P * 128), old(T, K), old(plan.P), old(1)
+        for _ in range(2):
+            plan.moe_dispatch(x, ids, recv, count, te, src, slot, tc, done)
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == ((0, 0) if ids is not bad else (-1, T // 2))
+        flat, good = slot.flatten().long(), (ids.flatten() < E)
+        assert (flat[~good] == -1).all() and done.item() == T * K
+        want = torch.bincount(ids.flatten()[good].long(), minlength=E)
+        assert torch.equal(count.long(), want)
+        rows = flat[good]
+        assert rows.unique().numel() == rows.numel() and torch.equal(te[rows // 128], ids.flatten()[good])
+        source = torch.full((plan.P * 128,), -1, dtype=torch.int64, device="cuda")
+        source[rows] = torch.arange(T * K, device="cuda")[good]
+        assert torch.equal(src.long(), source)
+        assert torch.equal(tc.long(), torch.bincount(rows // 128, minlength=plan.P))
+        assert torch.equal(te >= 0, tc > 0) and torch.equal(torch.bincount(te[te >= 0].long(), minlength=E), (want + 127) // 128)
+        assert torch.equal(recv[rows], x.repeat_interleave(K, 0)[good])
+
+
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_availability_counters_and_gated_consumer(mode):
     """Section IV-D in software: after dispatch every tile's status counter equals the rows stored in it

@@ -141,6 +141,7 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 int launch_route(moe_plan* p, const void* x, const void* wr, const float* bias, int* topk_idx,
                  float* topk_w, const PrepArgs* prep, cudaStream_t st);
 // every chain, few enough of them to run at the chain's own speed (route_chains.cu)
+// (Asked after route_direct_apply, below: on bf16 data what is left of the long rows here are small batches, and any batch beyond H 8192.)
 // With more than 64 experts: up to 1024 tokens; up to 864 where the tensor-core filter is there to take over and the chains
 // are long and in four CTAs per block of tokens.  Measured, router call on bf16 data, us, every chain / filter: 256 experts, H 7168:
 // T 256 46 / 120, T 512 75 / 110, T 768 103 / 108, T 864 107 / 108, T 896 122 / 109, T 1024 122 / 108; H 5120: T 864 81 / 85,

@@ -102,11 +102,32 @@ def test_workspace_holds_the_wide_router_logits_only_where_a_kernel_reads_them(l
 
 
 def test_wide_router_hands_over_to_the_filter_where_the_chains_get_slower(lib):
-    """256 experts and long rows: from 865 tokens on the filter (its squared norms are in the workspace); shorter rows: 1025."""
+    """256 experts and long rows: from 865 tokens on the filter (its squared norms are in the workspace); shorter rows: 1025.
+    (H 8200, and 2400 with 256 experts, are where the form that fetches its candidates' rows one by one never applies.)"""
     def norms(tokens, H, E=256):
         a, b = (B.moe_workspace_bytes(B.make_config(tokens, H, E, 1, 8, 0, B.DTYPE_BF16, identity_experts=1, route_filter=f)) for f in (0, -1))
         return a - b - (tokens * 1024 if tokens > 1024 else 0)
 
-    assert [norms(t, 7168) for t in (864, 865, 1024, 1025)] == [0, 1024, 1024, 1024]
-    assert [norms(t, 4096) for t in (864, 865, 1024, 1025)] == [0, 0, 0, 1024]
-    assert [norms(t, 7168, 192) for t in (865, 1024, 1025)] == [0, 0, 1024]
+    assert [norms(t, 8200) for t in (864, 865, 1024, 1025)] == [0, 1024, 1024, 1024]
+    assert [norms(t, 2400) for t in (864, 865, 1024, 1025)] == [0, 0, 0, 1024]
+    assert [norms(t, 8200, 192) for t in (865, 1024, 1025)] == [0, 0, 1024]
+
+
+def test_router_that_fetches_its_candidates_holds_one_set_of_logits_per_slice(lib):
+    """From T*E*H = 3.2e8 on (beyond 592 tokens twice that), up to 1184 tokens and H 8192: [slices, T, 256] fp32 and the squared
+    norms; outside, what the chains (one set of logits) or the filter (one set and the norms) need."""
+    def extra(tokens, H, E):
+        a, b = (B.moe_workspace_bytes(B.make_config(tokens, H, E, 1, 4, 0, B.DTYPE_BF16, identity_experts=1, route_filter=f)) for f in (0, -1))
+        return a - b + (tokens * 1024 if tokens <= 1024 else 0)      # (-1: the chains' logits up to 1024 tokens)
+
+    def slices(tokens, H, E):      # as many CTAs of 128 tokens x 128 experts as SMs, at most 16 slices, of 4 steps of 64 columns at least
+        tiles, steps = -(-tokens // 128) * -(-E // 128), -(-H // 64)
+        return -(-steps // -(-steps // max(1, min(148 // tiles, steps // 4, 16))))
+
+    for tokens, H, E in ((175, 7168, 256), (592, 2112, 256), (593, 4224, 256), (864, 7168, 256), (1025, 7168, 256), (1184, 7168, 256), (300, 8192, 160),
+                         (1000, 8192, 80)):
+        assert extra(tokens, H, E) == slices(tokens, H, E) * tokens * 1024 + 1024, (tokens, H, E)
+    for tokens, H, E in ((174, 7168, 256), (592, 2104, 256), (593, 4208, 256), (300, 8200, 160), (1000, 8192, 64)):      # the chains
+        assert extra(tokens, H, E) == tokens * 1024, (tokens, H, E)
+    for tokens, H, E in ((1185, 7168, 256), (865, 8200, 256), (1184, 2048, 256)):                                        # the filter over all rows
+        assert extra(tokens, H, E) == tokens * 1024 + 1024, (tokens, H, E)

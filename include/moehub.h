@@ -194,9 +194,11 @@ int moe_route(moe_plan_t* plan, const void* d_x, const void* d_wr, const float* 
  *      indexed with such an id and the assignment's row is not stored);
  *      availability counters (Section IV-D, data availability manager), both or neither,
  *      NULL = kept in the plan's workspace: d_tile_count [P] rows stored so far in each tile,
- *      d_rows_done [1] assignments whose rows are stored; both raised with release semantics
- *      after the rows they count are written, so a consumer that reads tile_count[p] >= 128
- *      or rows_done == T*K with acquire semantics may read the tile. */
+ *      d_rows_done [1] assignments whose rows are stored; the call sets them to zero and raises
+ *      both with release semantics after the rows they count are written, so a consumer that reads
+ *      tile_count[p] >= 128 or rows_done == T*K with acquire semantics may read the tile (a
+ *      consumer that may look before the call has begun finds what the caller left there).  Mode 2
+ *      raises all of them at once, behind the last row, where T*K <= 4096. */
 int moe_dispatch(moe_plan_t* plan, const void* d_x, const int32_t* d_topk_idx, void* d_recv,
                  int32_t* d_expert_count, int32_t* d_tile_expert, int32_t* d_src_info,
                  int32_t* d_slot_of, int32_t* d_tile_count, int32_t* d_rows_done, void* stream);

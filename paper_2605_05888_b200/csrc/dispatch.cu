@@ -345,12 +345,16 @@ dispatch_atomic_kernel(const uint4* __restrict__ x, const int* __restrict__ topk
 // reads all of the batch's expert ids - a few KB, from L2 - and counts for itself how many rows each expert gets in all and from
 // the tokens before its own, so it knows every address, and the tables besides, without asking anyone: one tile after the
 // other, expert by expert, rows in token-block order (the paged scheme leaves tiles and rows in any order).  The tables are
-// plain stores, each by one CTA: whoever reads them is behind the end of this kernel.
+// plain stores, each by one CTA: whoever reads them is behind the end of this kernel.  So are the counters inside moe_layer
+// (ticket nullptr); a caller's may be watched from elsewhere while this runs, so there they are zero until every CTA has
+// stored its rows, and the last CTA to say so raises them (the tiles' first: rows_done == T*K says that all of them are final).
 // reset: also the per-call start state that the kernel in front of a prepared dispatch has left (see make_prep), so that a
 // dispatch called on its own is one launch.
 // Measured against dispatch_atomic_kernel, us, the call alone / a layer of identity experts: T 24, H 4096, 8 experts, top-2 15.9 ->
 // 11.2 / 23.0 -> 21.6; T 512, H 2048, 60 experts, top-4 11.4 -> 9.0 / 23.4 -> 20.7; T 256, H 7168, 256 experts, top-8 12.4 -> 9.2; 500
-// tokens there (4000 ids, 65 MB of rows) 17.8 -> 17.7, where the line is drawn.
+// tokens there (4000 ids, 65 MB of rows) 17.8 -> 17.7, where the line is drawn (all without the ticket).
+// The ticket and what follows it add 1.4 to 2.1 us (back to back, without / with a caller's counters: 3.8 / 5.1, 5.3 / 7.3, 8.1 / 9.9,
+// 15.8 / 17.9).
 constexpr int kSmallAssign = 4096;
 struct SmallParams {
   const uint4* x;
@@ -361,12 +365,15 @@ struct SmallParams {
   int* status;
   int reset;
   int *own_rows_done, *gemm1_done;  // with reset: the plan's own counters
+  int* ticket;                   // zero; back to zero when the kernel ends.  nullptr: the counters are read in stream order alone
+  unsigned long long* avail_ns;  // with a ticket: the availability trace (see signal_rows), or nullptr
 };
 __global__ void __launch_bounds__(kDispThreads)
 dispatch_small_kernel(const SmallParams q) {
   __shared__ int s_total[kMaxExperts], s_next[kMaxExperts], s_tile[kMaxExperts + 1];  // rows; next row of this CTA; first tile
   __shared__ int s_slot[kMaxAssign], s_error[2];
   __shared__ unsigned short s_owner[kSmallAssign / kTileRows + kMaxExperts];  // (as many tiles as the pool has at most)
+  __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid % 32, E = q.E, n = q.T * q.K;
   const int t0 = blockIdx.x * q.tok_per_blk, ntok = min(q.tok_per_blk, q.T - t0), a0 = t0 * q.K, na = ntok * q.K;
   s_total[tid] = s_next[tid] = 0;
@@ -374,6 +381,7 @@ dispatch_small_kernel(const SmallParams q) {
   __syncthreads();
   pdl_wait();
   pdl_trigger();
+  if (q.avail_ns != nullptr && tid == 0) atomicMin(q.avail_ns, now_ns());
   constexpr int kPer = 8;  // ids fetched at once
   for (int b = 0; b < n; b += kPer * kDispThreads) {
     int e[kPer];
@@ -446,7 +454,7 @@ dispatch_small_kernel(const SmallParams q) {
     q.expert_count[e] = rows;
     for (int t = first; t < last; ++t) {
       q.tile_expert[t] = e;
-      if (q.tile_count != nullptr) q.tile_count[t] = min(kTileRows, rows - (t - first) * kTileRows);
+      q.tile_count[t] = q.ticket != nullptr ? 0 : min(kTileRows, rows - (t - first) * kTileRows);
     }
   }
   if (q.reset) {
@@ -459,7 +467,7 @@ dispatch_small_kernel(const SmallParams q) {
     }
     for (int t = used + gtid; t < q.P; t += gthreads) {
       q.tile_expert[t] = -1;
-      if (q.tile_count != nullptr) q.tile_count[t] = 0;
+      q.tile_count[t] = 0;
     }
     for (int r = used * kTileRows + gtid; r < q.P * kTileRows; r += gthreads) q.src_info[r] = -1;
     for (int t = gtid; t < q.P + 4; t += gthreads) q.gemm1_done[t] = 0;
@@ -471,12 +479,36 @@ dispatch_small_kernel(const SmallParams q) {
     } else if (s_error[0] != 0) {
       set_status(q.status, s_error[0], s_error[1]);
     }
-    if (q.rows_done != nullptr) *q.rows_done = n;
-    if (q.reset) *q.own_rows_done = n;
+    if (q.reset) *q.own_rows_done = 0;
+    *q.rows_done = q.ticket != nullptr ? 0 : n;
   }
   __syncthreads();
   copy_rows<4>(q.x, q.recv, s_slot, t0, ntok, q.K, q.vec_per_row);
   asm volatile("fence.proxy.async.global;" ::: "memory");  // the rows are read through TMA
+  if (q.ticket == nullptr) return;
+  __syncthreads();  // (what the CTA stored before a barrier, one thread's release behind it covers)
+  if (tid == 0) {
+    int before;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(q.ticket) : "memory");
+    s_last = before == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int e = tid; e < E; e += kDispThreads) {
+    const int rows = s_total[e], first = s_tile[e], last = min(s_tile[e + 1], q.P);
+    for (int t = first; t < last; ++t) {
+      const int here = min(kTileRows, rows - (t - first) * kTileRows);
+      asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(q.tile_count + t), "r"(here) : "memory");  // (a release with the fence above)
+      if (q.avail_ns != nullptr && here == kTileRows) q.avail_ns[2 + t] = now_ns();
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    *q.ticket = 0;
+    st_release(q.rows_done, n);
+    if (q.avail_ns != nullptr) q.avail_ns[1] = now_ns();
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -599,16 +631,19 @@ int launch_dispatch(moe_plan* p, const void* x, const int* topk_idx, void* recv,
   const moe_config_t& c = p->cfg;
   const int eb = c.dtype == MOE_DTYPE_BF16 ? 2 : 4;
   const int vec_per_row = c.H * eb / 16;
-  // Small batches in the paged scheme: up to where the rows bound both (measured above).
-  const bool small = c.dispatch_mode == MOE_DISPATCH_ATOMIC_PAGED && c.T > 0 && (long long)c.T * c.K <= kSmallAssign && !p->trace;
-  if (small) {
+  // Small batches in the paged scheme: up to where the rows bound both (measured above).  (With the trace on its start state
+  // comes from the launch in front.)
+  const bool small = c.dispatch_mode == MOE_DISPATCH_ATOMIC_PAGED && c.T > 0 && (long long)c.T * c.K <= kSmallAssign;
+  auto launch_small = [&](bool reset) {
+    const bool watched = tile_count != p->s.tile_count || p->trace;
     SmallParams q = {(const uint4*)x, topk_idx, c.T, c.E, c.K, p->dispatch_tokens, vec_per_row, (int)p->P, p->tiles_per_expert,
-                     (uint4*)recv, expert_count, tile_expert, src_info, slot_of, tile_count, rows_done, p->s.status, prepared ? 0 : 1,
-                     p->s.rows_done, p->s.gemm1_done};
+                     (uint4*)recv, expert_count, tile_expert, src_info, slot_of, tile_count, rows_done, p->s.status, reset ? 1 : 0,
+                     p->s.rows_done, p->s.gemm1_done, watched ? p->s.scan_ticket : nullptr, p->trace ? p->s.avail_ns : nullptr};
     launch_pdl(dispatch_small_kernel, dim3(p->nblk), dim3(kDispThreads), 0, st, q);
     p->launches += 1;
     return (int)cudaGetLastError();
-  }
+  };
+  if (small && !p->trace) return launch_small(!prepared);
   // Per-call start state (and, for the ordered scheme, the rows per expert): done by the kernel before this
   // call when `prepared`, else by one small launch here.
   if (!prepared) {
@@ -620,6 +655,7 @@ int launch_dispatch(moe_plan* p, const void* x, const int* topk_idx, void* recv,
     p->launches += 1;
   }
   if (c.T == 0) return 0;
+  if (small) return launch_small(false);
   if (c.dispatch_mode == MOE_DISPATCH_ATOMIC_ORDERED)
     return launch_dispatch_ordered(p, x, topk_idx, recv, expert_count, tile_expert, src_info, slot_of, tile_count,
                                    rows_done, st);

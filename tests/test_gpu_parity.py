@@ -779,6 +779,47 @@ def test_paged_dispatch_where_its_small_batches_end(case):
         assert torch.equal(recv[rows], x.repeat_interleave(K, 0)[good])
 
 
+@pytest.mark.parametrize("case", [(1, 64, 1), (37, 64, 32), (511, 256, 8), (4096, 8, 1)], ids=lambda c: f"T{c[0]}_E{c[1]}_K{c[2]}")
+def test_paged_dispatch_counters_seen_from_another_stream_follow_the_rows(case):
+    """Whoever looks while a small dispatch runs: copies of the counters, each followed by a copy of a piece of every row, on a
+    second stream beside the dispatch (they wait for nothing).  Where the counters say so, the rows are there."""
+    T, E, K = case
+    H = 8192
+    w = inputs.Workload("watched", T=T, H=H, E=E, R=1, K=K, F=0, dtype=BF16, identity_experts=True)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    g = torch.Generator(device="cuda").manual_seed(T)
+    x = torch.empty((T, H), dtype=torch.bfloat16, device="cuda").uniform_(1.0, 2.0, generator=g)
+    ids = torch.rand((T, E), device="cuda", generator=g).argsort(1)[:, :K].to(torch.int32).contiguous()
+    ints = lambda *n: torch.zeros(n, dtype=torch.int32, device="cuda")
+    recv = torch.zeros((plan.P * 128, H), dtype=torch.bfloat16, device="cuda")
+    count, te, src, slot, counters = ints(E), ints(plan.P), ints(plan.P * 128), ints(T, K), ints(plan.P + 1)
+    looks = 40
+    seen, rows = ints(looks, plan.P + 1), torch.zeros((looks, plan.P * 128, 8), dtype=torch.bfloat16, device="cuda")
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        for i in range(looks):
+            seen[i].copy_(counters)
+            rows[i].copy_(recv[:, -8:])
+    early = late = 0
+    for _ in range(20):
+        recv.zero_()
+        counters.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            graph.replay()
+        plan.moe_dispatch(x, ids, recv, count, te, src, slot, counters[:plan.P], counters[plan.P:])
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == (0, 0) and counters[-1].item() == T * K
+        flat, want = slot.flatten().long(), x[:, -8:].repeat_interleave(K, 0)
+        there = (rows[:, flat] == want).all(2)                                   # [looks, T*K]
+        tile_said = seen[:, :-1].gather(1, (flat // 128).expand(looks, -1)) >= 128
+        said = tile_said | (seen[:, -1:] >= T * K)
+        assert (there | ~said).all()
+        assert ((seen[:, :-1] == counters[:-1]).all(1) | (seen[:, -1] < T * K)).all()
+        early, late = early + (~said).any().item(), late + said.any().item()
+    assert early and late
+
+
 @pytest.mark.parametrize("mode", MODES)
 def test_dispatch_availability_counters_and_gated_consumer(mode):
     """Section IV-D in software: after dispatch every tile's status counter equals the rows stored in it

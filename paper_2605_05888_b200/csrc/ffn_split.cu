@@ -158,7 +158,8 @@ __device__ __noinline__ float fp32_chain(const float* __restrict__ a, const floa
   for (int k = 0; k < n; ++k) s = __fmaf_rn(a[k], b[k], s);
   return s;
 }
-__device__ __noinline__ float fp32_chain_planes(const __nv_bfloat16* __restrict__ a, size_t plane, const float* __restrict__ b, int n) {
+// (a: written by other CTAs of this launch, so neither const __restrict__ nor any other way to the non-coherent loads)
+__device__ __noinline__ float fp32_chain_planes(const __nv_bfloat16* a, size_t plane, const float* b, int n) {
   float s = 0.0f;
   for (int k = 0; k < n; ++k) {
     const float hi = __bfloat162float(a[k]), mid = __bfloat162float(a[plane + k]), lo = __bfloat162float(a[2 * plane + k]);
@@ -574,6 +575,7 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
             }
           }
         }
+        if (bad != 0) ld_acquire(&prm.gemm1_done[it.tile]);  // (complete, or the MMAs would not have had it: these loads come behind it too)
         for (; bad != 0; bad &= bad - 1) {
           const int at = __ffs(bad) - 1, r = (4 * (at >> 4) + h) * 16 + (at & 15);
           dst[(size_t)r * H] = fp32_chain_planes(prm.inter + (row0 + r) * prm.inter_pitch, plane,

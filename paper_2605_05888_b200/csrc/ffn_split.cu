@@ -699,7 +699,7 @@ int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, cons
   q.out = (float*)out_rows;
   q.gemm1_done = p->s.gemm1_done;
   q.work_counter = p->s.gemm1_done + p->P;
-  q.wait_ns = kDefaultWaitNs;
+  q.wait_ns = c.wait_limit_ns ? c.wait_limit_ns : kDefaultWaitNs;
   q.status = p->s.status;
   const int grid = p->sm_count;
   q.lag = grid;

@@ -1038,6 +1038,30 @@ def test_expert_kernel_with_a_tiny_wait_limit_reports_or_computes(kernel, split)
         assert plan.moe_last_status() == (0, 0) and torch.equal(y, y2)
 
 
+def test_fp32_expert_kernel_with_a_tiny_wait_limit_reports_or_computes():
+    """The same for dtype fp32 on the tensor cores: the limit bounds its waits (with 1 ns GEMM2's wait for the intermediate of
+    another CTA runs out).  Every call either reports the timeout or has computed its bytes."""
+    w = inputs.Workload("wait_fp32", T=1000, H=516, E=4, R=1, K=2, F=1028, dtype=FP32, zipf_s=0.7, seed=27)
+    args = [Hh.to_dev(a) for a in Hh.oracle_inputs(w)]
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    y, y2 = (torch.empty((w.T, w.H), dtype=torch.float32, device="cuda") for _ in range(2))
+    plan.moe_layer(*args, y)
+    b = _dispatch_with_counters(w, plan, args[0], plan.layer_tensor(0))
+    want = torch.zeros_like(b["recv"])
+    plan.moe_expert_ffn(b["recv"], b["te"], *args[3:], want, b["tile_count"], b["rows_done"])
+    used = b["slot"].flatten().long()
+    codes = []
+    for limit in (1, 500, 2_000, 5_000, 20_000, 100_000):
+        tiny = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, wait_limit_ns=limit)
+        out = torch.zeros_like(want)
+        tiny.moe_expert_ffn(b["recv"], b["te"], *args[3:], out, b["tile_count"], b["rows_done"])
+        codes.append(tiny.moe_last_status()[0])
+        assert codes[-1] in (0, -6) and (codes[-1] != 0 or torch.equal(out[used], want[used]))
+        plan.moe_layer(*args, y2)
+        assert plan.moe_last_status() == (0, 0) and torch.equal(y, y2)
+    assert codes[0] == -6
+
+
 # ------------------------------------------------------------------ dispatch and experts in one launch
 OVERLAP_CASES = [SMALL[3], SMALL[4], SMALL[5], SMALL[7],
                  inputs.Workload("three_tiles", T=700, H=320, E=4, R=2, K=2, F=392, dtype=BF16),

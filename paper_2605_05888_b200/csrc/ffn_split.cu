@@ -19,8 +19,11 @@
 // of 128 rows instead of 40 (six MMAs read A and B, 48 KB; split, 12 KB written), and that is the bound.  The rows are
 // split once, by split_rows_kernel in front.
 //
-// A value that is not finite (an infinity or NaN in an operand, an overflow, an hi that rounded up to infinity) is
-// recomputed as a chain of fp32 FMAs by the lane that holds it: inf * 0 in the split products is not what fp32 gives.
+// What infinities and NaN in the operands make of a sum, the hi*hi products say: hi of an infinity is one, hi of a number is zero
+// only if the number is (down to 2^-134), and their signs are the numbers' own; the other five (inf * mid has any sign, inf * 0 none)
+// are clamped to finite numbers before they are added, which changes nothing where hi*hi is infinite or NaN.  Where a value that is not
+// finite has no infinity or NaN behind it, or also large numbers (an overflow, an hi that rounded up to infinity: explained
+// below), the lane that holds it recomputes it as a chain of fp32 FMAs.
 //
 // Roles (864 threads): warp 0 claims and publishes the items and loads weights, warp 1 MMA issuer and TMEM owner, warps 2-9
 // split weights (two sets of four, two A stages each), warps 10-25 drain accumulators and write results, warp 26 loads the
@@ -51,8 +54,9 @@ struct SplitParams {
   int total_rows;
   int P, E, F, H, tp, lag;
   const float *recv, *wg, *wu, *wd;
-  __nv_bfloat16* inter;    // [3][P * 128][inter_pitch]
-  int inter_pitch;
+  const __nv_bfloat16* recv_planes;  // [3][P * 128][recv_pitch]
+  __nv_bfloat16* inter;              // [3][P * 128][inter_pitch]
+  int recv_pitch, inter_pitch;
   float* out;              // [P * 128, H]
   int* gemm1_done;
   int* work_counter;
@@ -152,6 +156,78 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict
   }
 }
 
+// Which of a warp's values that are not finite (bits of todo: rows h * 16 + 0...15 of the tile, and from bit 16 on the sixteen
+// that lie 64 rows on) are what their operands' infinities and NaN make of them: the row's, and those of this lane's weight row and,
+// in GEMM1, of the one 16 lanes on.  Returns the others.  All 32 lanes.  Large numbers are those whose products may add up to an overflow.
+// Measured, layer, T 1000, H 1024, 16 experts, top-2, F 2048 (215 us as a rule), us, FMAs / every such value recomputed / this: one
+// row with a NaN 737 / 465 / 217, one infinity in one Wg 741 / 24589 / 352, in every Wg 737 / 48854 / 546, every row NaN 698 / 66874 / 289,
+// infinite 698 / - / 549, every Wg NaN 743 / - / 600.
+struct Explain {
+  const __nv_bfloat16* rows;    // hi plane
+  const float* w;
+  int pitch, K;
+  bool paired;                  // GEMM1
+};
+constexpr float kLarge = 1.0e18f;
+__device__ __noinline__ uint32_t unexplained(const Explain& q, uint32_t todo) {
+  const int lane = threadIdx.x % 32;
+  constexpr uint32_t all = 0xffffffffu;
+  uint32_t row_inf = 0, row_large = 0;
+  for (uint32_t m = __reduce_or_sync(all, todo); m != 0; m &= m - 1) {
+    const uint32_t bit = m & (0u - m);
+    const int b = __ffs(m) - 1;
+    const uint2* at = reinterpret_cast<const uint2*>(q.rows + (size_t)((b >> 4) * 64 + (b & 15)) * q.pitch);
+    for (int k0 = 0; k0 < q.K; k0 += 512) {
+      bool nan = false;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int k = k0 + i * 128 + lane * 4;
+        const uint2 v = k < q.K ? at[k / 4] : make_uint2(0u, 0u);
+        const uint32_t f[4] = {v.x << 16 & 0x7fff0000u, v.x & 0x7fff0000u, v.y << 16 & 0x7fff0000u, v.y & 0x7fff0000u};  // magnitudes' bits
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          nan = nan || f[j] > 0x7f800000u;
+          if (f[j] == 0x7f800000u) row_inf |= bit;
+          else if (f[j] > __float_as_uint(kLarge)) row_large |= bit;
+        }
+      }
+      if (__any_sync(all, nan)) {
+        todo &= ~bit;
+        break;
+      }
+    }
+  }
+  row_inf = __reduce_or_sync(all, row_inf);
+  row_large = __reduce_or_sync(all, row_large);
+  const uint32_t here = todo;
+  if (q.paired) todo |= __shfl_xor_sync(all, todo, 16);
+  uint32_t flags = 0;  // of this lane's weight row: 1 NaN (then looked at no further), 2 an infinity, 4 a large number
+  for (uint32_t m = __ballot_sync(all, todo != 0); m != 0; m &= m - 1) {
+    const int from = __ffs(m) - 1;
+    const float* w = reinterpret_cast<const float*>(__shfl_sync(all, reinterpret_cast<unsigned long long>(q.w), from));
+    uint32_t seen = 0;
+    for (int k0 = 0; k0 < q.K; k0 += 512) {
+      uint32_t now = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int k = k0 + i * 128 + lane * 4;
+        const float4 v = k < q.K ? *reinterpret_cast<const float4*>(w + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (!(fabsf(f[j]) <= kLarge)) now |= isnan(f[j]) ? 1u : isinf(f[j]) ? 2u : 4u;
+      }
+      seen |= __reduce_or_sync(all, now);
+      if (seen & 1u) break;
+    }
+    if (lane == from) flags = seen;
+  }
+  const uint32_t others = __shfl_xor_sync(all, flags, 16);
+  if (q.paired) flags |= others;
+  if (flags & 1u) return 0u;
+  if (!(flags & 4u)) todo &= ~((flags & 2u ? all : row_inf) & ~row_large);
+  return todo & here;
+}
 // The recomputation of a value that is not finite.
 __device__ __noinline__ float fp32_chain(const float* __restrict__ a, const float* __restrict__ b, int n) {
   float s = 0.0f;
@@ -163,12 +239,12 @@ __device__ __noinline__ float fp32_chain_planes(const __nv_bfloat16* a, size_t p
   float s = 0.0f;
   for (int k = 0; k < n; ++k) {
     const float hi = __bfloat162float(a[k]), mid = __bfloat162float(a[plane + k]), lo = __bfloat162float(a[2 * plane + k]);
-    s = __fmaf_rn(hi + (mid + lo), b[k], s);
+    s = __fmaf_rn(fabsf(hi) <= FLT_MAX ? hi + (mid + lo) : hi, b[k], s);
   }
   return s;
 }
 constexpr float kNearTop = 3.38e38f;  // (bf16's largest finite number is 3.39e38: beyond that a number may round to infinity)
-__device__ __forceinline__ bool is_finite(float v) { return fabsf(v) <= FLT_MAX; }
+__device__ __forceinline__ bool is_finite(float v) { return fabsf(v) < FLT_MAX; }  // (or the largest, which a clamped number leaves)
 
 __global__ void __launch_bounds__(kSpThreads, 1)
 ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) {
@@ -479,12 +555,17 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
       for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 8; ++j) sum[i][j] = 0ull;
-      auto add = [&](uint32_t from) {
+      auto add = [&](uint32_t from, auto rest) {
         if (h >= n16) return;
         uint32_t r[2][16];  // (the second unit whether or not it has rows: a condition on one load has the compiler spill; the
         tc_ld16(lanes + from + (uint32_t)h * 16u, r[0]);        // columns exist, and the sums are not used)
         tc_ld16(lanes + from + (uint32_t)(h + 4) * 16u, r[1]);
         tc_wait_ld();
+        if (decltype(rest)::value != 0)
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[i][j] = __float_as_uint(fminf(fmaxf(__uint_as_float(r[i][j]), -FLT_MAX), FLT_MAX));
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -495,7 +576,7 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
         if (!warp_agrees(mbar_wait(smem_u32(&sh->hh_full[half]), (h_ph >> half) & 1u, abort_flag, wait_ns))) { fail_site = kWaitMbarEpi; break; }
         h_ph ^= 1u << half;
         tc_fence_after();
-        add(half * 128u);
+        add(half * 128u, Const<0>());
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sh->hh_empty[half]));
@@ -503,13 +584,14 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
       if (fail_site) break;
       if (!warp_agrees(mbar_wait(smem_u32(&sh->rest_full), (uint32_t)local_item & 1u, abort_flag, wait_ns))) { fail_site = kWaitMbarEpi; break; }
       tc_fence_after();
-      add(kSpRest);
+      add(kSpRest, Const<1>());
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&sh->rest_empty));
       const size_t row0 = (size_t)it.tile * kTileRows;
       auto acc = [&](int i, int j) { return __uint_as_float((uint32_t)(sum[i][j >> 1] >> (32 * (j & 1)))); };
       uint32_t bad = 0;  // results that are not finite
+      auto exist = [&]() { return ((1u << min(max(rows - h * 16, 0), 16)) - 1u) | ((1u << min(max(rows - (h + 4) * 16, 0), 16)) - 1u) << 16; };
       if (it.type == 0) {
         const bool up = lane >= 16, odd = (lane & 1) != 0;
         const int f = it.nb * 64 + q * 16 + (lane & 15);
@@ -528,7 +610,7 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
               const float got = __shfl_xor_sync(0xffffffffu, up ? acc(i, j + n) : acc(i, j + n + 8), 16);
               const float g = up ? got : acc(i, j + n), u = up ? acc(i, j + n + 8) : got;
               v[n] = g / (1.0f + expf(-g)) * u;
-              if (!is_finite(g) || !is_finite(u) || fabsf(v[n]) > kNearTop) bad |= 1u << (8 * i + j + n);
+              if (!is_finite(g) || !is_finite(u) || (fabsf(v[n]) > kNearTop && is_finite(v[n]))) bad |= 1u << (16 * i + j + n);
             }
             uint32_t part[3];
             split_pair(v[0], v[1], part[0], part[1], part[2]);
@@ -541,9 +623,13 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
           }
         }
         __syncwarp();
+        if (__any_sync(0xffffffffu, bad != 0)) {
+          const float* w = (up ? prm.wu : prm.wg) + ((size_t)it.e * F + min(f, F - 1)) * H;
+          bad = f < F ? (up ? bad << 8 : bad) & exist() : 0u;
+          bad = unexplained(Explain{prm.recv_planes + (row0 + h * 16) * prm.recv_pitch, w, prm.recv_pitch, H, true}, bad);
+        }
         for (; bad != 0; bad &= bad - 1) {
-          const int at = __ffs(bad) - 1, r = (4 * (at >> 3) + h) * 16 + (at & 7) + (up ? 8 : 0);
-          if (f >= F || r >= rows) continue;
+          const int at = __ffs(bad) - 1, r = (4 * (at >> 4) + h) * 16 + (at & 15);
           const float* a = prm.recv + (row0 + r) * H;
           const size_t w = ((size_t)it.e * F + f) * H;
           const float g = fp32_chain(a, prm.wg + w, H), u = fp32_chain(a, prm.wu + w, H);
@@ -575,7 +661,11 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
             }
           }
         }
-        if (bad != 0) ld_acquire(&prm.gemm1_done[it.tile]);  // (complete, or the MMAs would not have had it: these loads come behind it too)
+        if (__any_sync(0xffffffffu, bad != 0)) {
+          ld_acquire(&prm.gemm1_done[it.tile]);  // (complete, or the MMAs would not have had it: these loads come behind it too)
+          const float* w = prm.wd + ((size_t)(it.e / prm.tp) * H + min(hc, H - 1)) * F * prm.tp + (size_t)(it.e % prm.tp) * F;
+          bad = unexplained(Explain{prm.inter + (row0 + h * 16) * prm.inter_pitch, w, prm.inter_pitch, F, false}, bad);
+        }
         for (; bad != 0; bad &= bad - 1) {
           const int at = __ffs(bad) - 1, r = (4 * (at >> 4) + h) * 16 + (at & 15);
           dst[(size_t)r * H] = fp32_chain_planes(prm.inter + (row0 + r) * prm.inter_pitch, plane,
@@ -691,6 +781,8 @@ int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, cons
   q.H = c.H;
   q.tp = p->tp;
   q.recv = (const float*)recv;
+  q.recv_planes = (const __nv_bfloat16*)p->s.recv_planes;
+  q.recv_pitch = (int)hp;
   q.wg = (const float*)wg;
   q.wu = (const float*)wu;
   q.wd = (const float*)wd;

@@ -382,6 +382,84 @@ def test_fp32_on_tensor_cores_infinities_and_nan():
     assert (np.abs(got - want) <= 1e-4 * np.maximum(np.abs(want), scale)).all()
 
 
+def _fp32_experts(T, H, E, K, F, spoil=None, **kw):
+    plan = B.Plan(B.make_config(T, H, E, 1, K, F, FP32, dispatch_mode=B.DISPATCH_ATOMIC_PAGED, **kw))
+    g = torch.Generator(device="cuda").manual_seed(11)
+    normal = lambda *s, std=1.0: torch.empty(s, device="cuda").normal_(0.0, std, generator=g)
+    a = dict(x=normal(T, H), wr=normal(E, H, std=0.02), wg=normal(E, F, H, std=0.02), wu=normal(E, F, H, std=0.02), wd=normal(E, H, F, std=0.02))
+    if spoil is not None:
+        spoil(a)
+    y = torch.empty((T, H), device="cuda")
+
+    def layer():
+        plan.moe_layer(a["x"], a["wr"], None, a["wg"], a["wu"], a["wd"], y)
+        return y
+    return plan, a, layer
+
+
+def _spoil(name, value, *at):
+    def spoil(a):
+        a[name][at] = value
+    return spoil
+
+
+def _times(name, factor, *at):
+    def spoil(a):
+        a[name][at] *= factor
+    return spoil
+
+
+NOT_FINITE = {"nan_row": _spoil("x", float("nan"), 17, 3), "inf_row": _spoil("x", float("-inf"), 17), "wg_inf": _spoil("wg", float("inf"), slice(None), 10, 3),
+              "wg_nan": _spoil("wg", float("nan")), "wd_inf": _spoil("wd", float("inf"), 2, 10, 3), "large_row": _times("x", 1e37, 17),
+              "all_nan": _spoil("x", float("nan")), "all_inf": _spoil("x", float("inf"))}
+
+
+@pytest.mark.parametrize("what", NOT_FINITE)
+def test_fp32_values_that_are_not_finite_take_no_longer_than_the_fmas(what):
+    """(A tenth more is let pass as noise.)  And the same elements are NaN, infinite and finite as with the FMAs, which round elsewhere;
+    tokens that nothing was done to keep their bytes."""
+    shape = (1000, 1024, 16, 2, 2048)
+    took, ys = [], []
+    for kernel in (0, 1):
+        plan, a, layer = _fp32_experts(*shape, spoil=NOT_FINITE[what], ffn_kernel=kernel)
+        layer()
+        best = 1e9
+        for _ in range(3):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            ys.append(layer().clone())
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        assert plan.moe_last_status() == (0, 0)
+        took.append(best)
+    assert took[0] <= 1.1 * took[1], took
+    got, want = ys[0], ys[-1]
+    assert torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isposinf(), want.isposinf()) and torch.equal(got.isneginf(), want.isneginf())
+    if what in ("nan_row", "inf_row", "large_row"):
+        clean = _fp32_experts(*shape)[2]()
+        others = torch.arange(shape[0], device="cuda") != 17
+        assert torch.equal(got[others], clean[others]) and torch.isfinite(got[others]).all()
+
+
+def test_fp32_experts_without_row_counts_on_a_pool_of_nan():
+    """Rows that nobody wrote to hold NaN: the others are the bytes that a call with row counts gives."""
+    plan, a, layer = _fp32_experts(700, 260, 6, 2, 1032)
+    layer()
+    w = inputs.Workload("nan_pool", T=700, H=260, E=6, R=1, K=2, F=1032, dtype=FP32)
+    b = _dispatch_with_counters(w, plan, a["x"], plan.layer_tensor(0))
+    used = b["slot"].flatten().long()
+    pool = torch.full_like(b["recv"], float("nan"))
+    pool[used] = b["recv"][used]
+    outs = []
+    for counts in ((), (b["tile_count"], b["rows_done"])):
+        outs.append(torch.zeros_like(pool))
+        plan.moe_expert_ffn(pool, b["te"], a["wg"], a["wu"], a["wd"], outs[-1], *counts)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    assert torch.equal(outs[0][used], outs[1][used]) and torch.isfinite(outs[0][used]).all()
+
+
 # The CTA-pair expert kernel where its items end: an expert's rows around 16, 32, 128 (one tile), 129, 256 (a pair of
 # tiles) and 257, all experts the same so that every count is met; in the paged layout (tiles of an expert apart) and
 # the ordered one; H and F that end inside its 512- and 256-column blocks and inside a k-block; one and two launches.

@@ -87,8 +87,9 @@ typedef struct {
                                    ffn_hot_min_tiles left at 0) - and for fp32 the tensor cores on
                                    operands split into three bf16 numbers each (closer to the sums
                                    in 64 bits than fp32 FMAs; operands below 2^-109 in magnitude
-                                   keep fewer bits), or fp32 FMAs for little work and for fewer
-                                   than eight rows per expert; 1: fp32 FMAs always (bf16: a plain
+                                   keep fewer bits), or fp32 FMAs for little work, for fewer
+                                   than eight rows per expert and for static regions of more tiles
+                                   than the batch can fill; 1: fp32 FMAs always (bf16: a plain
                                    SIMT kernel, the check path); 2: always CTA pairs (bf16).
                                    The tensor-core forms add up every result in the same order,
                                    so a row's bytes do not depend on which of them computes it,
@@ -160,13 +161,16 @@ typedef struct {
 int moe_pool_tiles(const moe_config_t* cfg, int64_t* out_tiles);
 
 /* Bytes of device workspace moe_plan_create needs (scratch counters, tile tables, the SwiGLU
- * intermediate, and the internal buffers moe_layer uses between its stages). */
+ * intermediate, and the internal buffers moe_layer uses between its stages).  dtype fp32 with ffn_kernel
+ * 0: where the experts run on the tensor cores this holds the operands' three bf16 parts, 6 bytes per
+ * element of the receive pool and of the intermediate instead of the intermediate's 4. */
 int moe_workspace_bytes(const moe_config_t* cfg, size_t* out_bytes);
 
 /* Analogue of the paper's rowspMalloc (Section IV-A, runtime API): registers the receive
  * regions (base, row size, tile pool) once.  d_workspace: device memory, 256-byte aligned,
  * at least moe_workspace_bytes() long, owned by the caller, must outlive the plan's queued
- * work.  Runs on the current CUDA device.  *out is freed by moe_plan_destroy. */
+ * work.  (dtype fp32: as long as the same configuration needs with ffn_kernel 1 is enough; below
+ * moe_workspace_bytes() the plan's experts are computed as with ffn_kernel 1.)  Runs on the current CUDA device.  *out is freed by moe_plan_destroy. */
 int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, moe_plan_t** out);
 int moe_plan_destroy(moe_plan_t* plan);
 

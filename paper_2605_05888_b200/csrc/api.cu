@@ -87,8 +87,9 @@ int check_config(const moe_config_t* user, Geometry* g) {
   return MOE_OK;
 }
 
-// Lays the scratch out in the workspace; with base == nullptr only measures it.
-size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, size_t* counters_bytes) {
+// Lays the scratch out in the workspace; with base == nullptr only measures it.  planes: with what the fp32 experts on tensor cores
+// need, where they are used (dtype fp32; without, the plan's experts are fp32 FMAs).
+size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, size_t* counters_bytes, bool planes = true) {
   size_t off = 0;
   auto take = [&](size_t bytes) -> char* {
     char* ptr = base ? base + off : nullptr;
@@ -119,7 +120,7 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   }
   t.gemm1_done = (int*)take(sizeof(int) * (size_t)((g.P > 0 ? g.P : 1) + 4));  // + the expert kernel's item and exit counters
   const size_t pool_rows = (size_t)g.P * kTileRows;
-  if (ffn_split_applies(c, g.P)) {  // three bf16 planes each: 6 bytes per element
+  if (planes && ffn_split_applies(c, g.P)) {  // three bf16 planes each: 6 bytes per element
     t.inter = take(pool_rows * split_pitch(c.F) * 6);
     t.recv_planes = take(pool_rows * split_pitch(c.H) * 6);
   } else if (!c.identity_experts) {
@@ -180,7 +181,8 @@ int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, mo
   if (rc != MOE_OK) return rc;
   if (!d_workspace) return MOE_ERR_ARG;
   if (reinterpret_cast<uintptr_t>(d_workspace) % kAlign != 0) return MOE_ERR_WORKSPACE;
-  if (bytes < carve(g.eff, g, nullptr, nullptr, nullptr)) return MOE_ERR_WORKSPACE;
+  const bool planes = bytes >= carve(g.eff, g, nullptr, nullptr, nullptr);
+  if (!planes && bytes < carve(g.eff, g, nullptr, nullptr, nullptr, false)) return MOE_ERR_WORKSPACE;
   moe_plan* p = new (std::nothrow) moe_plan();
   if (!p) return MOE_ERR_ARG;
   p->cfg = g.eff;
@@ -203,7 +205,7 @@ int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, mo
   p->copy_in = p->copy_out = nullptr;
   p->submitted = 0;
   for (int b = 0; b < 2; ++b) p->ev_in[b] = p->ev_done[b] = p->ev_out[b] = nullptr;
-  carve(g.eff, g, (char*)d_workspace, &p->s, &p->counters_bytes);
+  carve(g.eff, g, (char*)d_workspace, &p->s, &p->counters_bytes, planes);
   if (cudaGetDevice(&p->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
     delete p;

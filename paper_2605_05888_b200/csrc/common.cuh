@@ -39,8 +39,8 @@ struct Scratch {          // device pointers carved out of the caller's workspac
   unsigned long long* avail_ns;  // [P+2] availability trace (measurement): dispatch start, all-ready time, per-tile ready time
   unsigned long long* item_ns;   // [4 * P * (NB1 + NB2)] work-item timeline of the tensor-core expert kernel (measurement)
   int* gemm1_done;        // [P+4]  per-tile status counter: GEMM1 blocks finished (x4 epilogue warps); [P..P+1] item counters, [P+2..P+3] exit counters of the expert kernel's launches
-  void* inter;            // [P*128, F] SwiGLU intermediate (ffn_split_kernel: three bf16 planes of it)
-  void* recv_planes;      // dtype fp32: the receive pool as three bf16 planes (ffn_split.cu)
+  void* inter;            // [P*128, F] SwiGLU intermediate (with recv_planes: three bf16 planes of it)
+  void* recv_planes;      // the receive pool as three bf16 planes, where the fp32 experts run on tensor cores (ffn_split.cu); else nullptr
   float* route_logits;    // [T, 256] router logits, more than 64 experts: the chain kernel's, or the tensor-core filter's approximate ones
   float* route_wnorm2;    // [256]    squared norms of the router's weight rows, recomputed by every call (filter)
   // moe_layer's internal buffers
@@ -189,7 +189,7 @@ int launch_ffn_tc(moe_plan* p, const void* recv, const int* tile_expert, const v
                   const void* wu, const void* wd, void* out_rows, const int* tile_count,
                   const int* rows_done, cudaStream_t st, bool own, const void* overlap_x = nullptr,
                   const int* overlap_idx = nullptr, const int* push_src = nullptr);
-// dtype fp32 on the tensor cores, every operand as three bf16 numbers (ffn_split.cu)
+// dtype fp32 on the tensor cores, every operand as three bf16 numbers (ffn_split.cu): whether a plan of P tiles wants them, given the workspace
 bool ffn_split_applies(const moe_config_t& c, int64_t P);
 int split_pitch(int n);  // elements per row of a plane
 int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu, const void* wd,

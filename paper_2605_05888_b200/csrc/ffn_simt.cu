@@ -476,7 +476,7 @@ int launch_ffn_simt(moe_plan* p, const void* recv, const int* tile_expert, const
   if (p->P == 0 || p->cfg.T == 0) return 0;
   if (p->cfg.dtype == MOE_DTYPE_BF16)
     return launch_typed<__nv_bfloat16>(p, recv, tile_expert, wg, wu, wd, out_rows, st);
-  if (ffn_split_applies(p->cfg, p->P)) return launch_ffn_split(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
+  if (p->s.recv_planes != nullptr) return launch_ffn_split(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st);
   return launch_fp32(p, recv, tile_expert, wg, wu, wd, out_rows, tile_count, rows_done, st, own);
 }
 

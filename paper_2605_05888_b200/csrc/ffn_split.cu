@@ -738,11 +738,15 @@ int split_pitch(int n) { return (n + 7) / 8 * 8; }  // of a plane's rows: 16 byt
 // experts) 117 / 69, 1677 M (444 x 1568) 425 / 136, 4194 M (T 1000, 1024 x 2048, 16 experts) 737 / 206.  Long sums: 22 M (92 x 1216) 88
 // / 50, 8 M (148 x 1432) 62 / 50.  Few rows per expert, where both stream weights: 7 rows (60 experts, 448 x 200) 51 / 69, 6
 // (308 x 1124) 118 / 126, 8 (32 experts, 1024 x 2048) 213 / 217.
+// The planes take 6 bytes per element of the pool and of the intermediate, which alone takes 4 with the FMAs: T 8192, H 4096, 8 experts,
+// top-2, F 14336 3.0 GB of workspace instead of 2.1.  Static regions, whose pool is not bounded by the rows, keep the FMAs (T 4096, H
+// 4096, 64 experts, top-2, F 2048 would hold 18.5 GB instead of 11.0).
 // (Calls with and without row counts go the same way, so their rows are the same bytes.)
 bool ffn_split_applies(const moe_config_t& c, int64_t P) {
   const long long rows = (long long)c.T * c.K, items = (long long)P * ((c.F + 63) / 64 + (c.H + 127) / 128);
   if (c.dtype != MOE_DTYPE_FP32 || c.identity_experts || c.ffn_kernel == 1) return false;
   if (P > kMaxListTiles || items >= (1ll << kSpRowShift)) return false;  // the work list, the item ring's fields
+  if (P > rows / kTileRows + c.E) return false;  // static regions of more tiles than the batch's rows fill: planes of all of them
   return rows >= 8ll * c.E && (rows * c.H * c.F >= 24000000ll || c.F >= 900);
 }
 

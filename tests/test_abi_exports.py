@@ -101,6 +101,20 @@ def test_workspace_holds_the_wide_router_logits_only_where_a_kernel_reads_them(l
     assert need(B.DTYPE_BF16, 0, 512) == need(B.DTYPE_BF16, -1, 512)
 
 
+def test_fp32_workspace_holds_the_operands_parts_only_where_tensor_cores_read_them(lib):
+    def need(T, H, E, K, F, kernel, mode=B.DISPATCH_ATOMIC_PAGED, **kw):
+        return B.moe_workspace_bytes(B.make_config(T, H, E, 1, K, F, B.DTYPE_FP32, dispatch_mode=mode, ffn_kernel=kernel, **kw))
+
+    paged = (8192, 4096, 8, 2, 14336)
+    rows = (8192 * 2 // 128 + 8) * 128
+    assert need(*paged, 0) == need(*paged, 1) + rows * (6 * 4096 + 2 * 14336)
+    static = (4096, 4096, 64, 2, 2048)                # a region of every expert for every token: 32 times the rows there are
+    assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC) == need(*static, 1, B.DISPATCH_ATOMIC_STATIC) < 11.1e9
+    assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC, capacity_rows=256) > need(*static, 1, B.DISPATCH_ATOMIC_STATIC, capacity_rows=256)
+    assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC, capacity_rows=384) == need(*static, 1, B.DISPATCH_ATOMIC_STATIC, capacity_rows=384)
+    assert need(16, 256, 8, 2, 256, 0) == need(16, 256, 8, 2, 256, 1)      # (little work: FMAs)
+
+
 def test_wide_router_hands_over_to_the_filter_where_the_chains_get_slower(lib):
     """256 experts and long rows: from 865 tokens on the filter (its squared norms are in the workspace); shorter rows: 1025.
     (H 8200, and 2400 with 256 experts, are where the form that fetches its candidates' rows one by one never applies.)"""

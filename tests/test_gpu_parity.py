@@ -3,6 +3,7 @@ the same seeded inputs.  Routing indices and dispatch contents bit-exact (rows i
 compared after sorting by source id: arrival order is free, Section IV-B of the paper), routing
 weights within 1e-5 relative, combined output within 1e-4 (fp32, element-wise with an rms floor) /
 2e-2 (bf16, per-token normwise) of the oracle: see parity_helpers.assert_output_close."""
+import ctypes
 import itertools
 
 import numpy as np
@@ -440,6 +441,29 @@ def test_fp32_values_that_are_not_finite_take_no_longer_than_the_fmas(what):
         clean = _fp32_experts(*shape)[2]()
         others = torch.arange(shape[0], device="cuda") != 17
         assert torch.equal(got[others], clean[others]) and torch.isfinite(got[others]).all()
+
+
+def test_fp32_plan_on_a_workspace_without_room_for_the_parts():
+    """A workspace as large as the FMAs need is taken, and they are used; a byte less than they need is refused."""
+    shape = (300, 260, 4, 2, 1028)
+    plan, a, layer = _fp32_experts(*shape, ffn_kernel=1)
+    want = layer().clone()
+    cfg = B.make_config(*shape[:3], 1, *shape[3:], FP32, dispatch_mode=B.DISPATCH_ATOMIC_PAGED)
+    full, lean = B.moe_workspace_bytes(cfg), B.moe_workspace_bytes(plan.cfg)
+    assert full > lean
+    room = torch.empty(full, dtype=torch.uint8, device="cuda")
+    for nbytes, same in ((lean, True), (full - 1, True), (full, False)):
+        small = B.Plan(cfg)
+        small.close()
+        room.fill_(0xff)
+        small.handle, small.workspace = ctypes.c_void_p(), room
+        assert B.lib().moe_plan_create(ctypes.byref(cfg), room.data_ptr(), nbytes, ctypes.byref(small.handle)) == 0
+        y = torch.empty_like(want)
+        small.moe_layer(a["x"], a["wr"], None, a["wg"], a["wu"], a["wd"], y)
+        torch.cuda.synchronize()
+        assert small.moe_last_status() == (0, 0) and torch.equal(y, want) == same
+        assert (room[nbytes:] == 0xff).all()
+    assert B.lib().moe_plan_create(ctypes.byref(cfg), room.data_ptr(), lean - 1, ctypes.byref(ctypes.c_void_p())) == -7
 
 
 def test_fp32_experts_without_row_counts_on_a_pool_of_nan():

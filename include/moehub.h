@@ -170,7 +170,9 @@ int moe_workspace_bytes(const moe_config_t* cfg, size_t* out_bytes);
  * regions (base, row size, tile pool) once.  d_workspace: device memory, 256-byte aligned,
  * at least moe_workspace_bytes() long, owned by the caller, must outlive the plan's queued
  * work.  (dtype fp32: as long as the same configuration needs with ffn_kernel 1 is enough; below
- * moe_workspace_bytes() the plan's experts are computed as with ffn_kernel 1.)  Runs on the current CUDA device.  *out is freed by moe_plan_destroy. */
+ * moe_workspace_bytes() the plan's experts are computed as with ffn_kernel 1.  Likewise for a router
+ * that holds several sets of logits, from T*E*H = 3.2e8 on: with room for one set, and 1 KB, it
+ * computes every chain, or filters all rows: see route_filter.)  Runs on the current CUDA device.  *out is freed by moe_plan_destroy. */
 int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, moe_plan_t** out);
 int moe_plan_destroy(moe_plan_t* plan);
 

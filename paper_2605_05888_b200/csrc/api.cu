@@ -87,9 +87,10 @@ int check_config(const moe_config_t* user, Geometry* g) {
   return MOE_OK;
 }
 
-// Lays the scratch out in the workspace; with base == nullptr only measures it.  planes: with what the fp32 experts on tensor cores
-// need, where they are used (dtype fp32; without, the plan's experts are fp32 FMAs).
-size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, size_t* counters_bytes, bool planes = true) {
+// Lays the scratch out in the workspace; with base == nullptr only measures it.  roomy: with what the fp32 experts on tensor cores
+// and the router that fetches its candidates' rows take for themselves, where they are used (a plan without has the kernels that
+// want no more than before them: FMAs, and the chains or the filter over all rows).
+size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, size_t* counters_bytes, bool roomy = true) {
   size_t off = 0;
   auto take = [&](size_t bytes) -> char* {
     char* ptr = base ? base + off : nullptr;
@@ -120,7 +121,7 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   }
   t.gemm1_done = (int*)take(sizeof(int) * (size_t)((g.P > 0 ? g.P : 1) + 4));  // + the expert kernel's item and exit counters
   const size_t pool_rows = (size_t)g.P * kTileRows;
-  if (planes && ffn_split_applies(c, g.P)) {  // three bf16 planes each: 6 bytes per element
+  if (roomy && ffn_split_applies(c, g.P)) {  // three bf16 planes each: 6 bytes per element
     t.inter = take(pool_rows * split_pitch(c.F) * 6);
     t.recv_planes = take(pool_rows * split_pitch(c.H) * 6);
   } else if (!c.identity_experts) {
@@ -128,9 +129,10 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   }
   const int experts = c.E / g.tp;  // (c.E counts every TP shard)
   const bool may_filter = c.dtype == MOE_DTYPE_BF16 && c.route_filter >= 0;
-  const bool direct = c.T > 0 && route_direct_apply(experts, c.T, c.H, may_filter);
+  const bool direct = roomy && c.T > 0 && route_direct_apply(experts, c.T, c.H, may_filter);
   const bool chains = !direct && route_chains_apply(experts, c.T, c.H, may_filter), filter = may_filter && !chains;
-  const size_t slabs = direct ? (size_t)route_direct_slices(experts, c.T, c.H) : 1;
+  t.route_slices = direct ? route_direct_slices(experts, c.T, c.H) : 0;
+  const size_t slabs = direct ? (size_t)t.route_slices : 1;
   t.route_logits = filter || (chains && experts > 64) ? (float*)take(sizeof(float) * slabs * (size_t)(c.T > 0 ? c.T : 1) * 256) : nullptr;
   t.route_wnorm2 = filter ? (float*)take(sizeof(float) * 256) : nullptr;
   t.topk_idx = (int*)take(sizeof(int) * (size_t)c.T * c.K);
@@ -181,8 +183,8 @@ int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, mo
   if (rc != MOE_OK) return rc;
   if (!d_workspace) return MOE_ERR_ARG;
   if (reinterpret_cast<uintptr_t>(d_workspace) % kAlign != 0) return MOE_ERR_WORKSPACE;
-  const bool planes = bytes >= carve(g.eff, g, nullptr, nullptr, nullptr);
-  if (!planes && bytes < carve(g.eff, g, nullptr, nullptr, nullptr, false)) return MOE_ERR_WORKSPACE;
+  const bool roomy = bytes >= carve(g.eff, g, nullptr, nullptr, nullptr);
+  if (!roomy && bytes < carve(g.eff, g, nullptr, nullptr, nullptr, false)) return MOE_ERR_WORKSPACE;
   moe_plan* p = new (std::nothrow) moe_plan();
   if (!p) return MOE_ERR_ARG;
   p->cfg = g.eff;
@@ -205,7 +207,7 @@ int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, mo
   p->copy_in = p->copy_out = nullptr;
   p->submitted = 0;
   for (int b = 0; b < 2; ++b) p->ev_in[b] = p->ev_done[b] = p->ev_out[b] = nullptr;
-  carve(g.eff, g, (char*)d_workspace, &p->s, &p->counters_bytes, planes);
+  carve(g.eff, g, (char*)d_workspace, &p->s, &p->counters_bytes, roomy);
   if (cudaGetDevice(&p->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
     delete p;

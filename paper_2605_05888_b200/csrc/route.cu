@@ -222,7 +222,7 @@ int launch_route(moe_plan* p, const void* x, const void* wr, const float* bias, 
   if (p->cfg.T == 0) return 0;
   PrepArgs prep = {};
   if (prep_or_null != nullptr) prep = *prep_or_null;
-  if (route_direct_apply(p->route_E, p->cfg.T, p->cfg.H, p->cfg.dtype == MOE_DTYPE_BF16 && p->cfg.route_filter >= 0)) return launch_route_direct(p, x, wr, bias, topk_idx, topk_w, prep, st);
+  if (p->s.route_slices > 0) return launch_route_direct(p, x, wr, bias, topk_idx, topk_w, prep, st);
   if (route_chains_apply(p->route_E, p->cfg.T, p->cfg.H, p->cfg.dtype == MOE_DTYPE_BF16 && p->cfg.route_filter >= 0)) return launch_route_chains(p, x, wr, bias, topk_idx, topk_w, prep, st);
   if (route_filter_applies(p)) return launch_route_filter(p, x, wr, bias, topk_idx, topk_w, prep, st);
   if (p->cfg.dtype == MOE_DTYPE_BF16)

@@ -796,7 +796,7 @@ int launch_route_direct(moe_plan* p, const void* x, const void* wr, const float*
   if (ensure_dynamic_smem(route_tc_logits_kernel, kTcSmem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
   if (ensure_dynamic_smem(route_direct_kernel, rd_smem(c.H), p->device, once_b) != cudaSuccess) return MOE_ERR_CUDA;
   const unsigned long long wait_ns = c.wait_limit_ns ? c.wait_limit_ns : kDefaultWaitNs;
-  const int slices = route_direct_slices(p->route_E, c.T, c.H), steps = (c.H + kBK - 1) / kBK, per = (steps + slices - 1) / slices;
+  const int slices = p->s.route_slices, steps = (c.H + kBK - 1) / kBK, per = (steps + slices - 1) / slices;
   if (launch_maybe_pdl(false, route_tc_logits_kernel, dim3((c.T + kTileRows - 1) / kTileRows, (p->route_E + 127) / 128, slices),
                        dim3(kTcThreads), kTcSmem, st, mx, mwh, (const __nv_bfloat16*)wr, c.T, c.H, p->route_E, p->s.route_logits,
                        p->s.route_wnorm2, wait_ns, p->s.status) != cudaSuccess)

@@ -1571,6 +1571,30 @@ def test_router_direct_kernel_edges(shape):
     Hh.check_route(idx, tw, ridx, rw)
 
 
+@pytest.mark.parametrize("tokens", [300, 900])
+def test_router_on_a_workspace_without_room_for_the_slices(tokens):
+    """One set of logits and the norms: the picks and the weights (the chains' at 300 tokens, the filter's at 900) all the same."""
+    w = inputs.Workload("direct_lean", T=tokens, H=4608, E=256, R=1, K=8, F=8, dtype=BF16, seed=33, identity_experts=True)
+    x, wr, bias, *_ = Hh.oracle_inputs(w, with_experts=False)
+    ridx, rw, _ = oracle.route(x, wr, bias, w.K, BF16)
+    plan, idx, tw = _route_only(w, x, wr, bias)
+    full, chains = B.moe_workspace_bytes(plan.cfg), B.moe_workspace_bytes(B.make_config(w.T, w.H, w.E, 1, w.K, 0, BF16, identity_experts=1, route_filter=-1,
+                                                                                        dispatch_mode=plan.cfg.dispatch_mode))
+    lean = chains + (1024 if tokens > 864 else 0)
+    assert lean < full and plan.moe_last_launch_count() == 2
+    plan.close()
+    plan.handle = ctypes.c_void_p()
+    plan.workspace.fill_(0xff)
+    base = (plan.workspace.data_ptr() + 255) // 256 * 256
+    assert B.lib().moe_plan_create(ctypes.byref(plan.cfg), base, lean - 1, ctypes.byref(ctypes.c_void_p())) == -7
+    assert B.lib().moe_plan_create(ctypes.byref(plan.cfg), base, lean, ctypes.byref(plan.handle)) == 0
+    plan.moe_route(Hh.to_dev(x), Hh.to_dev(wr), Hh.to_dev(bias), idx, tw)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0) and plan.moe_last_launch_count() == 2
+    Hh.check_route(idx, tw, ridx, rw)
+    assert (plan.workspace[base - plan.workspace.data_ptr() + lean:] == 0xff).all()
+
+
 def test_router_direct_kernel_degenerate_rows():
     """Rows of zeros (every expert a candidate), experts that are equal or an ulp apart, biases of minus infinity and of the
     lowest number, infinities and NaN in x and in Wr: the picks and their weights that every chain gives."""

@@ -139,16 +139,20 @@ route_tc_logits_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     for (int e = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 4 + (warp - 2); e < E; e += gridDim.x * gridDim.y * gridDim.z * 4) {
       const uint4* row = reinterpret_cast<const uint4*>(wr + (size_t)e * H);
       float s = 0.0f;
+      uint32_t bits = 0;
 #pragma unroll 8
       for (int v = lane; v < H / 8; v += 32) {
         float f[8];
-        Vec16<__nv_bfloat16>::unpack(__ldg(row + v), f);
+        const uint4 u = __ldg(row + v);
+        bits |= u.x | u.y | u.z | u.w;
+        Vec16<__nv_bfloat16>::unpack(u, f);
 #pragma unroll
         for (int q = 0; q < 8; ++q) s = fmaf(f[q], f[q], s);
       }
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (lane == 0) wnorm2[e] = s;
+      const bool zeros = __all_sync(0xffffffffu, (bits & 0x7fff7fffu) == 0u);
+      if (lane == 0) wnorm2[e] = zeros ? 0.0f : fmaxf(s, FLT_MIN);  // (zero: a row of zeros; fmaxf keeps s unless it underflowed or is NaN)
     }
     // epilogue: the accumulator row of token t0 + 32 * (warp % 4) + lane, 16 experts at a time
     const int quarter = warp & 3;
@@ -528,7 +532,14 @@ route_refine_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
 // lie 16 bytes off a multiple of 128 apart, so its 16-byte loads meet no bank twice.  What bounds it is the chain's own
 // latency (4.5 cycles per h: 17 us at H 7168) where running all E chains is bound by their FMAs.  Whole router call, 256
 // experts, H 7168, us, every chain / this: T 256 43 / 37, T 512 70 / 39, T 1024 99 / 70 (a second wave of CTAs).
+// A CTA with more than two warps' worth of candidates (logits that differ by less than their bound, large numbers in x) brings 64
+// columns of all of Wr at a time, and each of its threads runs the chains of two experts for both tokens.  The call at H 7168,
+// 256 experts, us, candidates' passes alone / so / every chain in its kernel: one such CTA, T 256 and 512 183 / 83 / 48 and 75, T
+// 1024 189 / 87 / 124; every CTA, T 512 324 / 107 / 75, T 1024 624 / 204 / 124.  A token of zeros, a router of zeros and a token
+// with a NaN or an infinity have no need of chains: T 512 42 us (324 for zeros before), where every row is zero 22.
 constexpr int kRdTokens = 2, kRdChains = 32, kRdThreads = 128, kRdBufs = 2;
+constexpr int kRdMany = 2 * kRdChains;  // more candidates than this: all of Wr
+constexpr int kRdWideBufs = 2, kRdWideChunk = kRfChunk, kRdWideBytes = kRfWBytes;  // boxes of 64 h of every expert's row
 constexpr int kRdChunk = 512, kRdPitch = kRdChunk * 2 + 16;  // h per step; bytes from one chain's chunk to the next one's
 __host__ __device__ constexpr int rd_x_pitch(int H) { return (H * 2 + 127) / 128 * 128 + 16; }
 constexpr size_t rd_smem(int H) {
@@ -560,19 +571,150 @@ __device__ __forceinline__ float rd_kth(int K, int lane, unsigned (&key)[8]) {
   return bk == 0u ? -FLT_MAX : __uint_as_float((bk & 0x80000000u) ? bk ^ 0x80000000u : ~bk);
 }
 
+// A token with a logit that is NaN or infinite, or without a bound, or with a bound of zero.  Three kinds need no chains (thr: FLT_MAX).
+// x or Wr zero: every chain is zero, and what the tensor cores made of it.  A NaN in x makes one of every chain.  An infinity in x
+// makes of every chain what the tensor cores made of the sum, unless large numbers beside it may overflow.  Of the others an
+// expert whose logit or whose weights' norm is not finite is a candidate, whatever its logit, and so is every expert where that
+// leaves no bound.  checked: infinity where chains are run whose values the bound says nothing of, else eps.  A warp.
+struct RdUnusual { unsigned must; float eps, thr, checked; };
+__device__ __noinline__ RdUnusual rd_unusual(float* l, uint32_t x, const float* wnorm2, int H, int E, float xn2, float kth, float slope, float floor) {
+  constexpr uint32_t warp = 0xffffffffu;
+  const int lane = threadIdx.x % 32;
+  RdUnusual r = {0u, INFINITY, FLT_MAX, INFINITY};
+  float wm2 = 0.0f;
+  bool finite = false;  // a logit that is
+  for (int e = lane, j = 0; e < E; e += 32, ++j) {
+    const float n2 = wnorm2[e], v = l[e];
+    if (!(n2 <= FLT_MAX) || !(v <= FLT_MAX)) r.must |= 1u << j;
+    if (n2 <= FLT_MAX) wm2 = fmaxf(wm2, n2);
+    finite = finite || fabsf(v) <= FLT_MAX;
+  }
+  for (int off = 16; off > 0; off >>= 1) wm2 = fmaxf(wm2, __shfl_xor_sync(warp, wm2, off));
+  const bool any_must = __any_sync(warp, r.must != 0u);
+  if (!any_must && xn2 <= FLT_MAX && (xn2 == 0.0f || wm2 == 0.0f)) return r;
+  if (!(xn2 <= FLT_MAX)) {
+    const bool nan = isnan(xn2);
+    bool large = finite || !(wm2 <= 1.0e36f);
+    for (int q = lane; q < H / 8; q += 32) {
+      float f[8];
+      Vec16<__nv_bfloat16>::unpack(lds128(x + (uint32_t)q * 16u), f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) large = large || (fabsf(f[i]) > 1.0e18f && !isinf(f[i]));
+    }
+    large = __any_sync(warp, large);
+    if (nan || !large) {
+      for (int e = lane; e < E; e += 32)
+        if (nan || isnan(l[e])) l[e] = __int_as_float(0x7fffffff);
+      r.must = 0u;
+      return r;
+    }
+  }
+  r.eps = slope * sqrtf(xn2 * wm2) + floor;
+  r.thr = kth - r.eps - fminf(r.eps, 1.0e-3f * (1.0f + fabsf(kth)));
+  if (!(r.eps <= FLT_MAX) || !(fabsf(r.thr) <= FLT_MAX)) {
+    r.must = 0xffu;
+    r.thr = -INFINITY;
+  } else if (!any_must) {
+    r.checked = r.eps;
+  }
+  return r;
+}
+
+// The chains of all experts for both tokens, by all threads: experts threadIdx.x and threadIdx.x + 128, 64 h of every expert's row at
+// a time (62 us at H 7168 for one CTA, what an SM fetches in boxes of 128-byte rows; boxes of 128 experts or of 32 h take 85 to 108).
+// Eight lanes' 16-byte loads meet different units of the swizzled rows, and the four chains of a thread take turns, FMA by FMA, or
+// each would wait for itself.  Only candidates' values are used, so that what a token gets does not depend on the other.  false, for
+// all threads: a wait ran out.  (Apart from the kernel, which is 3 us slower with this in it.)
+struct RdEvery {
+  const CUtensorMap* map_w;
+  const float* bias;
+  float* ls;
+  uint32_t xrow, ring, bars;
+  const uint32_t* cand;
+  const float* eps;
+  int* fills;
+  volatile int* abort_flag;
+  unsigned long long wait_ns;
+  int* status;
+  int x_pitch, H, tvalid, step;  // step: boxes so far: buffer = step % kRdWideBufs
+};
+__device__ __noinline__ bool rd_every_chain(const RdEvery& q) {
+  const uint32_t wide = (q.ring + 1023u) & ~1023u, swizzle = (uint32_t)(threadIdx.x & 7) << 4;
+  const int n = (q.H + kRdWideChunk - 1) / kRdWideChunk;
+  auto fill = [&](int i) {  // (one thread; the buffer is free)
+    const int b = (q.step + i) % kRdWideBufs;
+    mbar_expect_tx(q.bars + 8 * b, kRdWideBytes);
+    tma_load_2d(wide + b * kRdWideBytes, q.map_w, q.bars + 8 * b, i * kRdWideChunk, 0);
+    *q.fills = q.step + i + 1;
+  };
+  if (threadIdx.x == 0)
+    for (int i = 0; i < min(kRdWideBufs, n); ++i) fill(i);
+  float acc[2][kRdTokens] = {};
+  for (int ch = 0; ch < n; ++ch) {
+    const int g = q.step + ch, b = g % kRdWideBufs;
+    const bool late = !mbar_wait(q.bars + 8 * b, (uint32_t)(g / kRdWideBufs) & 1u, q.abort_flag, q.wait_ns);
+    if (!late) {
+      const uint32_t w0 = wide + b * kRdWideBytes + threadIdx.x * 128u, x0 = q.xrow + (uint32_t)(ch * kRdWideChunk) * 2u;
+      auto eight = [&](int u) {
+        uint32_t wv[2][4], xv[kRdTokens][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const uint4 w = lds128(w0 + i * (kRdWideBytes / 2) + ((uint32_t)(u << 4) ^ swizzle));
+          wv[i][0] = w.x, wv[i][1] = w.y, wv[i][2] = w.z, wv[i][3] = w.w;
+        }
+#pragma unroll
+        for (int t = 0; t < kRdTokens; ++t) {
+          const uint4 x = lds128(x0 + (uint32_t)(t * q.x_pitch + u * 16));
+          xv[t][0] = x.x, xv[t][1] = x.y, xv[t][2] = x.z, xv[t][3] = x.w;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+          for (int c = 0; c < 2 * kRdTokens; ++c) acc[c & 1][c >> 1] = fma_bf16_lo(xv[c >> 1][j], wv[c & 1][j], acc[c & 1][c >> 1]);
+#pragma unroll
+          for (int c = 0; c < 2 * kRdTokens; ++c) acc[c & 1][c >> 1] = fma_bf16_hi(xv[c >> 1][j], wv[c & 1][j], acc[c & 1][c >> 1]);
+        }
+      };
+      const int units = min(kRdWideChunk, q.H - ch * kRdWideChunk) / 8;
+      if (units == kRdWideChunk / 8) {
+#pragma unroll
+        for (int u = 0; u < kRdWideChunk / 8; ++u) eight(u);
+      } else {
+        for (int u = 0; u < units; ++u) eight(u);
+      }
+    }
+    if (__syncthreads_or(late)) return false;
+    if (threadIdx.x == 0 && ch + kRdWideBufs < n) fill(ch + kRdWideBufs);
+  }
+#pragma unroll
+  for (int t = 0; t < kRdTokens; ++t)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = (int)threadIdx.x + 128 * i;
+      if (t >= q.tvalid || !((q.cand[t * (kRfEP / 32) + e / 32] >> (e % 32)) & 1u)) continue;
+      const float exact = q.bias != nullptr ? acc[i][t] + q.bias[e] : acc[i][t];
+      float& l = q.ls[t * kRfEP + e];
+      if (!(fabsf(exact - l) <= q.eps[t]) && q.eps[t] <= FLT_MAX) set_status(q.status, MOE_ERR_INTERNAL, 502);  // (the error model, as below)
+      l = exact;
+    }
+  return true;
+}
+
 __global__ void __launch_bounds__(kRdThreads)
-route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wr, const float* __restrict__ bias,
+route_direct_kernel(const __grid_constant__ CUtensorMap map_w, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wr, const float* __restrict__ bias,
                     const float* __restrict__ logits, int slices, const float* __restrict__ wnorm2, float additions, int sms, int T, int H,
                     int E, int K, int renorm, int* __restrict__ topk_idx, float* __restrict__ topk_w, const PrepArgs prep, int tp,
                     unsigned long long wait_ns, int* __restrict__ status) {
   __shared__ int s_hist[kRouteMaxExperts];
   __shared__ float s_xn2[kRdThreads / 32], s_eps[kRdTokens];
-  __shared__ unsigned long long s_full[kRdBufs], s_empty[kRdBufs], s_x;
-  __shared__ int s_total[3], s_fills, s_abort;  // chains per round; chunks whose copies have been issued
+  __shared__ uint32_t s_cand[kRdTokens][kRfEP / 32];  // the tokens' candidates, where there are many
+  __shared__ unsigned long long s_full[kRdBufs], s_empty[kRdBufs], s_wide[kRdWideBufs], s_x;
+  __shared__ int s_total[3], s_fills, s_wide_fills, s_abort;  // chains per round; chunks and boxes whose copies have been issued
   extern __shared__ uint8_t rd_dyn[];
   uint8_t* xrow = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(rd_dyn) + 15) & ~(uintptr_t)15);
   const int x_pitch = rd_x_pitch(H);
   uint8_t* ring = xrow + kRdTokens * x_pitch;                                        // [kRdBufs][kRdChains][kRdPitch]
+  static_assert(kRdBufs * kRdChains * kRdPitch >= kRdWideBufs * kRdWideBytes + 1008, "or, on 1024 bytes, [kRdWideBufs][256 experts][128 bytes]");
   float* ls = reinterpret_cast<float*>(ring + kRdBufs * kRdChains * kRdPitch);       // [kRdTokens][256]
   unsigned short* chains = reinterpret_cast<unsigned short*>(ls + kRdTokens * kRfEP);  // token << 8 | expert
   const int t0 = blockIdx.x * kRdTokens, tvalid = min(kRdTokens, T - t0);
@@ -585,8 +727,9 @@ route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
       mbar_init(smem_u32(&s_full[b]), 1);
       mbar_init(smem_u32(&s_empty[b]), 1);
     }
+    for (int b = 0; b < kRdWideBufs; ++b) mbar_init(smem_u32(&s_wide[b]), 1);
     mbar_init(smem_u32(&s_x), 1);
-    s_abort = s_fills = s_total[0] = s_total[1] = s_total[2] = 0;
+    s_abort = s_fills = s_wide_fills = s_total[0] = s_total[1] = s_total[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // (x and Wr were complete before the kernel in front of this one could start)
     mbar_expect_tx(smem_u32(&s_x), (uint32_t)(tvalid * H * 2));
@@ -599,16 +742,20 @@ route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
   {  // |x_t|^2: two warps per token
     const int t = warp / 2;
     float s = 0.0f;
+    uint32_t bits = 0;
     if (t < tvalid && !failed)
       for (int q = (warp % 2) * 32 + lane; q < H / 8; q += 64) {
         float f[8];
-        Vec16<__nv_bfloat16>::unpack(lds128(smem_u32(xrow + t * x_pitch) + (uint32_t)q * 16u), f);
+        const uint4 u = lds128(smem_u32(xrow + t * x_pitch) + (uint32_t)q * 16u);
+        bits |= u.x | u.y | u.z | u.w;
+        Vec16<__nv_bfloat16>::unpack(u, f);
 #pragma unroll
         for (int i = 0; i < 8; ++i) s = fmaf(f[i], f[i], s);
       }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) s_xn2[warp] = s;
+    const bool zeros = __all_sync(0xffffffffu, (bits & 0x7fff7fffu) == 0u);
+    if (lane == 0) s_xn2[warp] = s == 0.0f && !zeros ? FLT_MIN : s;  // (zero: a row of zeros)
   }
   pdl_wait();
   pdl_trigger();
@@ -631,40 +778,49 @@ route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
   }
   __syncthreads();
   const float* row = ls + (live ? tl : 0) * kRfEP;
-  // Nothing is known of a token with a logit that is NaN or infinite, or whose error bound is: it gets every chain.  (A bias of
-  // minus infinity is none of these: such an expert's logit is that in any case.)
-  bool wild = false;
+  unsigned must = 0;                   // bit j: expert lane + 32 j is a candidate whatever its logit
   float v[8], thr = 0.0f, eps = 0.0f;  // the approximate logits of experts lane + 32 j
   if (live) {
     float wm2 = 0.0f;
     unsigned key[8];
+    bool unusual = false;  // a logit that is NaN or infinite.  (A bias of minus infinity makes none: such an expert's logit is that in any case.)
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int e = lane + 32 * j;
       v[j] = row[e];
       key[j] = e < E ? max(order_key(v[j]), 1u) : 0u;
-      wild = wild || (e < E && !(v[j] <= FLT_MAX));
+      unusual = unusual || (e < E && !(v[j] <= FLT_MAX));
       if (e < E) wm2 = fmaxf(wm2, wnorm2[e]);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) wm2 = fmaxf(wm2, __shfl_xor_sync(0xffffffffu, wm2, off));
     const float kth = rd_kth(K, lane, key);
     // (the same first threshold and the same proof as in the refine kernel)
-    const float xn2 = s_xn2[2 * tl] + s_xn2[2 * tl + 1];
-    eps = kRfUlp * (0.5f * (float)H + additions) * sqrtf(xn2 * wm2) * 1.0001f + 4.0e-7f * (1.0f + fabsf(kth));
-    wild = __any_sync(0xffffffffu, wild) || !(eps <= FLT_MAX);
-    if (lane == 0) s_eps[tl] = wild ? INFINITY : eps;
-    thr = wild ? -INFINITY : kth - eps - 1.0e-3f * (1.0f + fabsf(kth));
+    const float xn2 = s_xn2[2 * tl] + s_xn2[2 * tl + 1], norms = xn2 * wm2;
+    const float slope = kRfUlp * (0.5f * (float)H + additions) * 1.0001f, floor = 4.0e-7f * (1.0f + fabsf(kth));
+    eps = slope * sqrtf(norms) + floor;
+    float checked = eps;
+    // (below the bound a sliver, so that the candidates' exact values settle the matter in one round; the bound itself is enough for that)
+    thr = kth - eps - fminf(eps, 1.0e-3f * (1.0f + fabsf(kth)));
+    unusual = __any_sync(0xffffffffu, unusual);
+    if (unusual || !(eps <= FLT_MAX) || !(norms > 0.0f)) {  // (the same for all lanes)
+      const RdUnusual u = rd_unusual(ls + tl * kRfEP, smem_u32(xrow) + (uint32_t)(tl * x_pitch), wnorm2, H, E, xn2, kth, slope, floor);
+      must = u.must;
+      eps = u.eps;
+      thr = u.thr;
+      checked = u.checked;
+    }
+    if (lane == 0) s_eps[tl] = checked;
   }
   unsigned done = 0;  // bit j: the chain of expert lane + 32 j has been run
   const int nchunk = (H + kRdChunk - 1) / kRdChunk;
-  int step = 0;  // chunks so far over all passes: buffer = step % kRdBufs
+  int step = 0, wide_step = 0;  // chunks, boxes so far over all passes: buffer = step % kRdBufs, wide_step % kRdWideBufs
   for (int round = 0; round < 3; ++round) {  // a second round is rare, a third cannot be needed
     unsigned cand = 0;
     if (live && thr < FLT_MAX) {
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (lane + 32 * j < E && (wild || v[j] >= thr) && !((done >> j) & 1u)) cand |= 1u << j;
+        if (lane + 32 * j < E && (((must >> j) & 1u) || v[j] >= thr) && !((done >> j) & 1u)) cand |= 1u << j;
     }
     done |= cand;
     if (cand != 0) {
@@ -674,6 +830,18 @@ route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
     __syncthreads();
     const int total = s_total[round];
     if (total == 0 || s_abort) break;  // no token of the CTA asks for more (CTA-uniform)
+    if (total > kRdMany) {
+      if (live)
+        for (int j = 0; j < kRfEP / 32; ++j) {
+          const uint32_t word = __ballot_sync(0xffffffffu, (cand >> j) & 1u);
+          if (lane == 0) s_cand[tl][j] = word;
+        }
+      __syncthreads();
+      failed = !rd_every_chain(RdEvery{&map_w, bias, ls, smem_u32(xrow), smem_u32(ring), smem_u32(s_wide), &s_cand[0][0], s_eps, &s_wide_fills, abort_flag,
+                                       wait_ns, status, x_pitch, H, tvalid, wide_step});
+      wide_step += (H + kRdWideChunk - 1) / kRdWideChunk;
+      if (failed) s_abort = 1;
+    } else
     for (int p = 0; p < total; p += kRdChains, step += nchunk) {
       const int n = min(kRdChains, total - p);
       const int mine = lane < n ? chains[p + lane] : -1, e = mine & 0xff, tk = (mine >> 8) & 0xff;
@@ -739,7 +907,7 @@ route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
     __syncthreads();
     if (s_abort) break;  // (CTA-uniform: it is set in the passes alone)
     // The K-th largest EXACT logit so far decides whether more chains are wanted: see the refine kernel.
-    if (live && !wild && thr < FLT_MAX) {
+    if (live && thr < FLT_MAX) {
       unsigned key[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) key[j] = ((done >> j) & 1u) ? max(order_key(row[lane + 32 * j]), 1u) : 0u;
@@ -760,6 +928,7 @@ route_direct_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __
       };
       settle(&s_x, 0u);
       for (int g = max(0, s_fills - kRdBufs); g < s_fills; ++g) settle(&s_full[g % kRdBufs], (uint32_t)(g / kRdBufs) & 1u);
+      for (int g = max(0, s_wide_fills - kRdWideBufs); g < s_wide_fills; ++g) settle(&s_wide[g % kRdWideBufs], (uint32_t)(g / kRdWideBufs) & 1u);
     }
     if (threadIdx.x == 0) set_status(status, MOE_ERR_TIMEOUT, kWaitMbarTma);
     __syncthreads();
@@ -789,9 +958,10 @@ int launch_route_direct(moe_plan* p, const void* x, const void* wr, const float*
   EncodeTiledFn enc;
   int rc = get_encoder(p, &enc);
   if (rc != MOE_OK) return rc;
-  CUtensorMap mx, mwh;
+  CUtensorMap mx, mwh, mwide;
   if ((rc = make_map_2d(enc, &mx, x, (uint64_t)c.T, (uint64_t)c.H, kTileRows)) != MOE_OK) return rc;
   if ((rc = make_map_2d(enc, &mwh, wr, (uint64_t)p->route_E, (uint64_t)c.H, 128)) != MOE_OK) return rc;
+  if ((rc = make_map_2d(enc, &mwide, wr, (uint64_t)p->route_E, (uint64_t)c.H, kRfEP)) != MOE_OK) return rc;
   static SmemAttrOnce once, once_b;
   if (ensure_dynamic_smem(route_tc_logits_kernel, kTcSmem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;
   if (ensure_dynamic_smem(route_direct_kernel, rd_smem(c.H), p->device, once_b) != cudaSuccess) return MOE_ERR_CUDA;
@@ -803,7 +973,7 @@ int launch_route_direct(moe_plan* p, const void* x, const void* wr, const float*
     return MOE_ERR_CUDA;
   // the additions of the error model: 17 per MMA of an accumulator, the four accumulators' sum, the slices'
   const float additions = 68.0f * (float)((per + 3) / 4) + 3.0f + (float)(slices - 1);
-  if (launch_pdl(route_direct_kernel, dim3((c.T + kRdTokens - 1) / kRdTokens), dim3(kRdThreads), rd_smem(c.H), st,
+  if (launch_pdl(route_direct_kernel, dim3((c.T + kRdTokens - 1) / kRdTokens), dim3(kRdThreads), rd_smem(c.H), st, mwide,
                  (const __nv_bfloat16*)x, (const __nv_bfloat16*)wr, bias, (const float*)p->s.route_logits, slices,
                  (const float*)p->s.route_wnorm2, additions, p->sm_count > 0 ? p->sm_count : 148, c.T, c.H, p->route_E, p->route_K,
                  c.renormalize, topk_idx, topk_w, prep, p->tp, wait_ns, p->s.status) != cudaSuccess)

@@ -1625,6 +1625,81 @@ def test_router_direct_kernel_degenerate_rows():
         assert torch.allclose(tw, want_w, rtol=1e-5, atol=1e-7, equal_nan=True)
 
 
+def _zero_tokens(step):
+    def spoil(x, wr):
+        x[::step] = 0
+    return spoil
+
+
+def _put(name, at, value):
+    def spoil(x, wr):
+        (x if name == "x" else wr)[at] = value
+    return spoil
+
+
+def _small_router(x, wr):
+    wr.mul_(5e-4)
+
+
+ROUTER_DATA = {"one_zero": _put("x", 7, 0), "zeros_12_percent": _zero_tokens(8), "all_zero": _zero_tokens(1), "one_nan": _put("x", (7, 100), float("nan")),
+               "nans_12_percent": _put("x", slice(None, None, 8), float("nan")), "infs_12_percent": _put("x", (slice(None, None, 8), 3), float("-inf")),
+               "one_nan_weight": _put("wr", (3, 5), float("nan")), "one_inf_weight": _put("wr", (3, 5), float("inf")), "zero_router": _put("wr", slice(None), 0), "small_router": _small_router}
+
+
+@pytest.mark.parametrize("tokens", [256, 512])
+@pytest.mark.parametrize("what", ROUTER_DATA)
+def test_router_direct_kernel_takes_no_longer_than_every_chain(what, tokens):
+    """Whatever padding or a new router's weights hold; and the chains' picks and weights.  (A twentieth more is let pass as noise.)"""
+    H, E, K = 7168, 256, 8
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.empty((tokens, H), device="cuda").normal_(generator=g).bfloat16()
+    wr = torch.empty((E, H), device="cuda").normal_(0.0, 0.02, generator=g).bfloat16()
+    ROUTER_DATA[what](x, wr)
+    got, took = [], []
+    for route_filter in (0, -1):
+        plan = B.Plan(B.make_config(tokens, H, E, 1, K, 0, BF16, dispatch_mode=B.DISPATCH_ATOMIC_PAGED, identity_experts=1, route_filter=route_filter))
+        idx, tw = torch.empty((tokens, K), dtype=torch.int32, device="cuda"), torch.empty((tokens, K), device="cuda")
+        best = 1e9
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(100000)      # (the launches are in the queue by the time the first one starts)
+            t0.record()
+            for _ in range(8):
+                plan.moe_route(x, wr, None, idx, tw)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        assert plan.moe_last_status() == (0, 0)
+        got.append((idx, tw))
+        took.append(best)
+    assert torch.equal(got[0][0], got[1][0]) and torch.allclose(got[0][1], got[1][1], rtol=1e-5, atol=1e-8, equal_nan=True)
+    assert took[0] <= 1.05 * took[1], took
+
+
+def test_router_direct_kernel_many_candidates():
+    """More than 64 candidates in a CTA of two tokens, from one of them or both: infinities, ties and near ties across 70 to 256
+    experts, beside tokens that have few; E below and above 128, an odd number of tokens, H that ends inside 64 columns."""
+    for T, H, E in ((251, 7176, 256), (601, 8184, 136), (1001, 7168, 100)):
+        w = inputs.Workload("many", T=T, H=H, E=E, R=1, K=8, F=8, dtype=BF16, seed=35)
+        x, (wr, _) = inputs.make_x(w), inputs.make_router(w)
+        inf = int(inputs.fp32_to_bf16_bits(np.full(1, np.inf, np.float32))[0])
+        wr[10:80] = wr[10]
+        wr[20:75, 3] ^= 1                                    # an ulp apart in one column
+        bias = np.zeros(E, np.float32)
+        bias[10:80] = 100.0                                  # those 70 are every token's best: ties are candidates of all
+        for b in (bias, None):
+            ridx, rw, _ = oracle.route(x, wr, b, w.K, BF16)
+            plan, idx, tw = _route_only(w, x, wr, b)
+            assert plan.moe_last_status() == (0, 0)
+            Hh.check_route(idx, tw, ridx, rw)
+        xs = x.copy()
+        xs[::9, 5], xs[T - 1, 0] = inf, inf ^ 0x8000
+        plan, idx, tw = _route_only(w, xs, wr, None)
+        _, want_idx, want_w = _route_only(w, xs, wr, None, route_filter=-1)
+        assert plan.moe_last_status() == (0, 0) and torch.equal(idx, want_idx)
+        assert torch.allclose(tw, want_w, rtol=1e-5, atol=1e-7, equal_nan=True)
+
+
 def _route_only(w, x, wr, bias, **kw):
     plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, **kw)
     idx = torch.empty((w.T, w.K), dtype=torch.int32, device="cuda")

@@ -87,9 +87,10 @@ typedef struct {
                                    ffn_hot_min_tiles left at 0) - and for fp32 the tensor cores on
                                    operands split into three bf16 numbers each (closer to the sums
                                    in 64 bits than fp32 FMAs; operands below 2^-109 in magnitude
-                                   keep fewer bits), or fp32 FMAs for little work, for fewer
-                                   than eight rows per expert and for static regions of more tiles
-                                   than the batch can fill; 1: fp32 FMAs always (bf16: a plain
+                                   keep fewer bits), or fp32 FMAs for little work, for few
+                                   rows per expert (on average fewer than 8, with more than 16
+                                   experts 16, with more than 64 and H below 384 32) and for static
+                                   regions of more tiles than the batch can fill; 1: fp32 FMAs always (bf16: a plain
                                    SIMT kernel, the check path); 2: always CTA pairs (bf16).
                                    The tensor-core forms add up every result in the same order,
                                    so a row's bytes do not depend on which of them computes it,

@@ -736,8 +736,11 @@ int split_pitch(int n) { return (n + 7) / 8 * 8; }  // of a plane's rows: 16 byt
 // their GEMM2.  Measured, whole layer, us, FMAs / this: rows x H x F of 6 to 22 M 34 / 38 (mean of twelve shapes, none faster by
 // more than 5 %), 30 M (132 x 128, 4 experts) 39.5 / 39.5, 26 M (912 x 624) 70 / 58, 77 M (284 x 536) 62 / 51, 375 M (412 x 508, 32
 // experts) 117 / 69, 1677 M (444 x 1568) 425 / 136, 4194 M (T 1000, 1024 x 2048, 16 experts) 737 / 206.  Long sums: 22 M (92 x 1216) 88
-// / 50, 8 M (148 x 1432) 62 / 50.  Few rows per expert, where both stream weights: 7 rows (60 experts, 448 x 200) 51 / 69, 6
-// (308 x 1124) 118 / 126, 8 (32 experts, 1024 x 2048) 213 / 217.
+// / 50, 8 M (148 x 1432) 62 / 50.  Few rows per expert, where both stream weights and this splits all of them, the more experts the
+// worse.  This over FMAs at 8 / 12 / 16 / 24 rows per expert, six shapes each (512 x 1024, 1024 x 2048, 448 x 400, 928 x 556, 1024 x
+// 512; last 256 x 2048, whose short sums have the most items for their work): 8 and 16 experts 0.65-0.92 / 0.67-0.91 / 0.60-0.85 / 0.59-0.93;
+// 32 experts 0.92-1.11 / 0.86-1.12 / 0.68-0.88, 0.74; 64 1.09-1.28 / 0.83-1.15 / 0.75-0.92, 0.85; 128 1.17-1.42 / 0.95-1.18 / 0.79-0.99, 1.12
+// / 0.62-0.86, 0.96; 256 1.26-1.58 / 0.97-1.19 / 0.83-1.04, 1.58 / 0.60-0.77, 1.17, at 32 rows 0.49-0.63, 0.93.
 // The planes take 6 bytes per element of the pool and of the intermediate, which alone takes 4 with the FMAs: T 8192, H 4096, 8 experts,
 // top-2, F 14336 3.0 GB of workspace instead of 2.1.  Static regions, whose pool is not bounded by the rows, keep the FMAs (T 4096, H
 // 4096, 64 experts, top-2, F 2048 would hold 18.5 GB instead of 11.0).
@@ -747,7 +750,8 @@ bool ffn_split_applies(const moe_config_t& c, int64_t P) {
   if (c.dtype != MOE_DTYPE_FP32 || c.identity_experts || c.ffn_kernel == 1) return false;
   if (P > kMaxListTiles || items >= (1ll << kSpRowShift)) return false;  // the work list, the item ring's fields
   if (P > rows / kTileRows + c.E) return false;  // static regions of more tiles than the batch's rows fill: planes of all of them
-  return rows >= 8ll * c.E && (rows * c.H * c.F >= 24000000ll || c.F >= 900);
+  const int few = c.E <= 16 ? 8 : c.E > 64 && c.H < 384 ? 32 : 16;  // rows per expert from which on the tensor cores are the faster ones
+  return rows >= (long long)few * c.E && (rows * c.H * c.F >= 24000000ll || c.F >= 900);
 }
 
 int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu, const void* wd,

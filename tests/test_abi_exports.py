@@ -113,6 +113,10 @@ def test_fp32_workspace_holds_the_operands_parts_only_where_tensor_cores_read_th
     assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC, capacity_rows=256) > need(*static, 1, B.DISPATCH_ATOMIC_STATIC, capacity_rows=256)
     assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC, capacity_rows=384) == need(*static, 1, B.DISPATCH_ATOMIC_STATIC, capacity_rows=384)
     assert need(16, 256, 8, 2, 256, 0) == need(16, 256, 8, 2, 256, 1)      # (little work: FMAs)
+    for E, H, rows_per_expert in ((8, 512, 8), (16, 512, 8), (17, 512, 16), (64, 256, 16), (65, 384, 16), (65, 380, 32), (256, 256, 32)):
+        at, below = rows_per_expert * E, rows_per_expert * E - 1           # (few rows per expert: FMAs, the more experts the longer)
+        assert need(at, H, E, 1, 1024, 0) > need(at, H, E, 1, 1024, 1), (E, H)
+        assert need(below, H, E, 1, 1024, 0) == need(below, H, E, 1, 1024, 1), (E, H)
 
 
 def test_wide_router_hands_over_to_the_filter_where_the_chains_get_slower(lib):

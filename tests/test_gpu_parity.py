@@ -281,6 +281,24 @@ def test_fp32_expert_kernel_edges(case):
     assert torch.equal(rows[used], plan.layer_tensor(7)[used])
 
 
+@pytest.mark.parametrize("case", [c for c in FP32_FFN if c[0] >= 8], ids=lambda c: f"T{c[0]}_H{c[1]}_E{c[2]}_K{c[3]}_F{c[4]}_tp{c[5]}")
+def test_fp32_fma_kernel_edges(case):
+    """The same with ffn_kernel 1: the FMAs where the tensor cores would take over, every register tile of theirs among them."""
+    T, H, E, K, F, tp, zipf = case
+    w = inputs.Workload("fp32_edges", T=T, H=H, E=E, R=1, K=K, F=F, dtype=FP32, zipf_s=zipf, seed=17)
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    ref = Hh.oracle_layer_for(w, x, wr, bias, wg, wu, wd)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED, tp_shards=tp, ffn_kernel=1)
+    y = torch.empty((T, H), dtype=torch.float32, device="cuda")
+    args = [Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)]
+    plan.moe_layer(*args, y)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0) and plan.moe_last_launch_count() == 5
+    Hh.assert_output_close(Hh.to_host_f64(y), ref["y"], FP32)
+    # (1e-6: the bound of the tensor-core form's test, below, holds for sums that round every addition as well)
+    assert np.linalg.norm(Hh.to_host_f64(y) - ref["y"]) <= 1e-6 * np.linalg.norm(ref["y"])
+
+
 # A caller's own tables in fp32: more blocks than the grid has CTAs (each goes on to further blocks, a barrier set per block),
 # tiles of 0 to 128 rows; counters that are complete, incomplete (tiles whole) and absent (whole).
 @pytest.mark.parametrize("case", [(1, 8, 1024, 132, 260), (40, 4, 2048, 260, 1284), (900, 3, 2048, 516, 516)], ids=lambda c: f"T{c[0]}_E{c[1]}_cap{c[2]}")
@@ -340,6 +358,44 @@ def test_fp32_on_tensor_cores_edges(case):
         d = Hh.to_host_f64(y) - ref
         errs.append(np.linalg.norm(d) / np.linalg.norm(ref))
     assert errs[0] <= 1e-6 and errs[0] <= 1.05 * errs[1], errs
+
+
+@pytest.mark.parametrize("mode", [B.DISPATCH_SCAN, B.DISPATCH_ATOMIC_STATIC, B.DISPATCH_ATOMIC_PAGED, B.DISPATCH_ATOMIC_ORDERED])
+def test_fp32_on_tensor_cores_in_every_dispatch_mode(mode):
+    """(Static regions too, where they are no larger than the batch can fill.)"""
+    w = inputs.Workload("split_modes", T=256, H=132, E=2, R=1, K=1, F=1028, dtype=FP32, seed=29)
+    x, wr, bias, wg, wu, wd = Hh.oracle_inputs(w)
+    ref = Hh.oracle_layer_for(w, x, wr, bias, wg, wu, wd)
+    plan = Hh.make_plan(w, mode)
+    assert B.moe_workspace_bytes(plan.cfg) > B.moe_workspace_bytes(Hh.make_plan(w, mode, ffn_kernel=1).cfg)
+    y = torch.empty((w.T, w.H), dtype=torch.float32, device="cuda")
+    plan.moe_layer(*[Hh.to_dev(a) for a in (x, wr, bias, wg, wu, wd)], y)
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    assert np.linalg.norm(Hh.to_host_f64(y) - ref["y"]) <= 1e-6 * np.linalg.norm(ref["y"])
+
+
+@pytest.mark.parametrize("rows", [1, 2, 15, 16, 17, 33, 127])
+def test_fp32_on_tensor_cores_tiles_of_few_rows(rows):
+    """A caller's own table: a full tile and one of few rows of the same expert, one of few rows alone."""
+    T, H, E, F = 300, 100, 2, 932
+    plan = B.Plan(B.make_config(T, H, E, 1, 1, F, FP32, dispatch_mode=B.DISPATCH_ATOMIC_PAGED))
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    wg, wu, wd = (torch.empty(s, device="cuda").normal_(0.0, 0.05, generator=g) for s in ((E, F, H), (E, F, H), (E, H, F)))
+    recv = torch.empty((plan.P * 128, H), device="cuda").normal_(generator=g)
+    ints = lambda v: torch.tensor(v, dtype=torch.int32, device="cuda")
+    te, count = ints([0, -1, 0, 1]), ints([128, 0, rows, rows])
+    out = torch.zeros_like(recv)
+    plan.moe_expert_ffn(recv, te, wg, wu, wd, out, count, ints([T]))
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    for tile in (0, 2, 3):
+        e, n = int(te[tile]), int(count[tile])
+        x = recv[tile * 128:tile * 128 + n].double()
+        gate = x @ wg[e].double().T
+        want = (gate * torch.sigmoid(gate) * (x @ wu[e].double().T)) @ wd[e].double().T
+        assert (out[tile * 128:tile * 128 + n].double() - want).norm() <= 1e-6 * want.norm(), tile
+    assert torch.count_nonzero(out[128:256]) == 0
 
 
 def test_fp32_on_tensor_cores_infinities_and_nan():
@@ -1764,3 +1820,22 @@ def test_router_filter_with_a_tiny_wait_limit_reports_or_routes():
     plan2, idx2, tw2 = _route_only(w, x, wr, bias)
     assert plan2.moe_last_status() == (0, 0)
     Hh.check_route(idx2, tw2, ridx, rw)
+
+
+@pytest.mark.parametrize("ties", [0, 200])
+def test_router_direct_kernel_with_a_tiny_wait_limit_reports_or_routes(ties):
+    """The same for the kernel that fetches its candidates' rows, few of them and, with equal experts, all of Wr."""
+    w = inputs.Workload("direct_timeout", T=300, H=5120, E=256, R=8, K=8, F=8, dtype=BF16, identity_experts=True)
+    x, wr, bias, *_ = Hh.oracle_inputs(w, with_experts=False)
+    wr[:ties] = wr[0]
+    ridx, rw, _ = oracle.route(x, wr, bias, w.K, w.dtype)
+    for limit in (1, 1_000, 20_000):
+        plan, idx, tw = _route_only(w, x, wr, bias, wait_limit_ns=limit)
+        code, detail = plan.moe_last_status()
+        if code == 0:
+            Hh.check_route(idx, tw, ridx, rw)
+        else:
+            assert code == -6 and detail in (3, 4, 5), (code, detail)
+        plan2, idx2, tw2 = _route_only(w, x, wr, bias)
+        assert plan2.moe_last_status() == (0, 0)
+        Hh.check_route(idx2, tw2, ridx, rw)

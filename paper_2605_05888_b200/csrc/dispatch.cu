@@ -488,8 +488,8 @@ dispatch_small_kernel(const SmallParams q) {
   if (q.ticket == nullptr) return;
   __syncthreads();  // (what the CTA stored before a barrier, one thread's release behind it covers)
   if (tid == 0) {
-    int before;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(q.ticket) : "memory");
+    int before = 0;
+    if (gridDim.x > 1) asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(q.ticket) : "memory");
     s_last = before == (int)gridDim.x - 1;
   }
   __syncthreads();

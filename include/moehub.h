@@ -86,8 +86,8 @@ typedef struct {
                                    row counts and with ffn_split, ffn_thin_tiles and
                                    ffn_hot_min_tiles left at 0) - and for fp32 the tensor cores on
                                    operands split into three bf16 numbers each (closer to the sums
-                                   in 64 bits than fp32 FMAs; operands below 2^-109 in magnitude
-                                   keep fewer bits), or fp32 FMAs for little work, for few
+                                   in 64 bits than fp32 FMAs, over the whole range of exponents), or
+                                   fp32 FMAs for little work, for few
                                    rows per expert (on average fewer than 8, with more than 16
                                    experts 16, with more than 64 and H below 384 32) and for static
                                    regions of more tiles than the batch can fill; 1: fp32 FMAs always (bf16: a plain

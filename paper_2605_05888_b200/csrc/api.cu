@@ -124,6 +124,7 @@ size_t carve(const moe_config_t& c, const Geometry& g, char* base, Scratch* s, s
   if (roomy && ffn_split_applies(c, g.P)) {  // three bf16 planes each: 6 bytes per element
     t.inter = take(pool_rows * split_pitch(c.F) * 6);
     t.recv_planes = take(pool_rows * split_pitch(c.H) * 6);
+    t.group_large = (unsigned char*)take(pool_rows / 16);
   } else if (!c.identity_experts) {
     t.inter = take(pool_rows * c.F * g.eb);
   }

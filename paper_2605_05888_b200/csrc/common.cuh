@@ -41,6 +41,7 @@ struct Scratch {          // device pointers carved out of the caller's workspac
   int* gemm1_done;        // [P+4]  per-tile status counter: GEMM1 blocks finished (x4 epilogue warps); [P..P+1] item counters, [P+2..P+3] exit counters of the expert kernel's launches
   void* inter;            // [P*128, F] SwiGLU intermediate (with recv_planes: three bf16 planes of it)
   void* recv_planes;      // the receive pool as three bf16 planes, where the fp32 experts run on tensor cores (ffn_split.cu); else nullptr
+  unsigned char* group_large;  // [P*8] with recv_planes: which groups of 16 rows hold large numbers
   float* route_logits;    // [T, 256] router logits, more than 64 experts: the chain kernel's, or the tensor-core filter's approximate ones
   int route_slices;       // the slices of h that they are in (route_direct_kernel's: [route_slices, T, 256]); 0: another router
   float* route_wnorm2;    // [256]    squared norms of the router's weight rows, recomputed by every call (filter)

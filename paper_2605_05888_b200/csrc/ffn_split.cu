@@ -20,7 +20,7 @@
 // split once, by split_rows_kernel in front.
 //
 // What infinities and NaN in the operands make of a sum, the hi*hi products say: hi of an infinity is one, hi of a number is zero
-// only if the number is (down to 2^-134), and their signs are the numbers' own; the other five (inf * mid has any sign, inf * 0 none)
+// only if the number is (below 2^-118 also in a group of large rows), and their signs are the numbers' own; the other five (inf * mid has any sign, inf * 0 none)
 // are clamped to finite numbers before they are added, which changes nothing where hi*hi is infinite or NaN.  Where a value that is not
 // finite has no infinity or NaN behind it, or also large numbers (an overflow, an hi that rounded up to infinity: explained
 // below), the lane that holds it recomputes it as a chain of fp32 FMAs.
@@ -40,7 +40,7 @@ constexpr int kSpWStages = 7, kSpBStages = 2;
 constexpr int kSpWBytes = 128 * 32 * 4;             // 128 weight rows x 32 k, fp32
 constexpr int kSpBBytes = 3 * kTileRows * kBK * 2;  // three planes of up to 128 rows x 64 k, bf16
 constexpr int kSpRing = 16;  // the weights' producer is at most 7 items (W stages) ahead of the splitters, those 2 of the MMAs, those 2 of the drain
-constexpr int kSpSmem = kSpBStages * kSpBBytes + kSpWStages * kSpWBytes + 1024 /*alignment*/ + 512 /*barriers*/;
+constexpr int kSpSmem = kSpBStages * kSpBBytes + kSpWStages * kSpWBytes + 1024 /*alignment*/ + 576 /*barriers*/;
 constexpr uint32_t kSpRest = 256, kSpA = 384;       // tensor-memory columns: hi*hi at 0 and 128, the rest, four A stages of 3 x 8
 
 struct SplitMaps {
@@ -55,6 +55,7 @@ struct SplitParams {
   int P, E, F, H, tp, lag;
   const float *recv, *wg, *wu, *wd;
   const __nv_bfloat16* recv_planes;  // [3][P * 128][recv_pitch]
+  const uint2* group_large;          // [P] a byte for each of a tile's eight groups of 16 rows
   __nv_bfloat16* inter;              // [3][P * 128][inter_pitch]
   int recv_pitch, inter_pitch;
   float* out;              // [P * 128, H]
@@ -71,6 +72,7 @@ struct SplitShared {
   unsigned long long rest_full, rest_empty;
   unsigned long long item_bar[kSpRing];
   unsigned long long drain;
+  int item_large[kSpRing];  // bit i: group i of the item's tile holds large numbers
   int item_ring[kSpRing];  // item | (rows of its tile / 16, rounded up) << kSpRowShift, or -1
   int w_fills;
   uint32_t b_fills[2];     // of each B stage
@@ -78,18 +80,27 @@ struct SplitShared {
   int abort_flag;
   int last_cta;
 };
-static_assert(sizeof(SplitShared) <= 512, "barriers behind the stages");
+static_assert(sizeof(SplitShared) <= 576, "barriers behind the stages");
 constexpr int kSpRowShift = 23;
 constexpr int kSpDrain64 = 256;  // from sums of this length on, hi*hi is drained every 64 k instead of 32
 template <uint32_t V> struct Const { static constexpr uint32_t value = V; };
 
-// Three bf16 numbers whose sum is x (exactly, for |x| of at least 2^-109; below, the last ones run out of exponents).
-// Infinities and NaN stand in hi alone, and a finite x that would round up to infinity is cut instead.
+// bf16 has fp32's exponents, so the last of three parts of a number below 2^-109 would have none left.  Weights are split times 2^16
+// (down to fp32's smallest that keeps every bit), and so are the rows and the intermediate of a group of 16 rows, or, where one of
+// its x is 2^32 and more, times 2^-16, so that their sums keep their range: the products come out times 2^32 or as they are.
+// Without the scales, off by (relative, H 512, F 1024; fp32 FMAs 5.9e-7, with them 2.4e-7): Wd of size 2^-115 1.1e-6, of 2^-120 3.5e-5, of 2^-125
+// 1.1e-3.  They take 1 to 2 % (T 1000, H 1024, 16 experts, F 2048 233.5 -> 236.7 us, T 300, H 400, F 500 49.4 -> 50.5).
+constexpr float kUp = 65536.0f, kDown = 1.0f / 65536.0f, kLargeRow = 4294967296.0f;
+constexpr int kSplitRows = 16;  // rows of a group
+__device__ __forceinline__ float group_scale(int large) { return large ? kDown : kUp; }
+__device__ __forceinline__ float group_result(int large) { return large ? 1.0f : kDown * kDown; }  // what a sum of a group's products is to be multiplied by
+
+// Three bf16 numbers whose sum is x, if hi is finite.  A finite element of the intermediate for which it would not be has kBits, a NaN
+// that no conversion gives, in its place and its own bits in the other two (store_top).
+constexpr unsigned short kBits = 0x7fc1;
 __device__ __forceinline__ void split3(float x, __nv_bfloat16& hi, __nv_bfloat16& mid, __nv_bfloat16& lo) {
   hi = __float2bfloat16_rn(x);
-  const bool top = (__bfloat16_as_ushort(hi) & 0x7f80u) == 0x7f80u;
-  if (top && fabsf(x) <= FLT_MAX) hi = __ushort_as_bfloat16((unsigned short)(__float_as_uint(x) >> 16));
-  const float r = top && !(fabsf(x) <= FLT_MAX) ? 0.0f : x - __bfloat162float(hi);
+  const float r = x - __bfloat162float(hi);
   mid = __float2bfloat16_rn(r);
   lo = __float2bfloat16_rn(r - __bfloat162float(mid));
 }
@@ -111,6 +122,17 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
   lo = pack2(minus_low(a, mid), b - __uint_as_float(mid & 0xffff0000u));
 }
 
+__device__ __forceinline__ unsigned long long mul_x2(unsigned long long v, float by) {
+  unsigned long long d;
+  asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%2, %2};\n\tmul.rn.f32x2 %0, %1, t;\n\t}" : "=l"(d) : "l"(v), "f"(by));
+  return d;
+}
+// The same of two weights' bits, times kUp.
+__device__ __forceinline__ void split_pair_up(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  const unsigned long long v = mul_x2((unsigned long long)b << 32 | a, kUp);
+  split_pair(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)), hi, mid, lo);
+}
+
 // A operand in tensor memory: D[128, N] (+)= A[128, 16] * B[N, 16]^T.
 __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -129,11 +151,10 @@ __device__ __forceinline__ void add_x2(unsigned long long& acc, uint32_t lo, uin
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Rows of the pool to planes [3][rows][pitch].  A CTA takes rows of one tile; rows nobody wrote to are left out.
-constexpr int kSplitRows = 16;
 __global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ x, const int* __restrict__ tile_expert,
                                                          const int* __restrict__ tile_count, const int* __restrict__ rows_done,
                                                          int total_rows, int E, int H, int pitch, size_t plane,
-                                                         __nv_bfloat16* __restrict__ out) {
+                                                         __nv_bfloat16* __restrict__ out, unsigned char* __restrict__ group_large) {
   pdl_wait();
   pdl_trigger();
   const int tile = blockIdx.x / (kTileRows / kSplitRows), r0 = blockIdx.x % (kTileRows / kSplitRows) * kSplitRows;
@@ -143,17 +164,27 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict
   if (tile_count != nullptr && *rows_done >= total_rows) rows = min(kTileRows, tile_count[tile]);
   rows = min(rows - r0, kSplitRows);
   const int quads = H / 4;
-  for (int i = threadIdx.x; i < rows * quads; i += 256) {
-    const int r = i / quads, c = (i - r * quads) * 4;
-    const size_t row = (size_t)tile * kTileRows + r0 + r;
-    const float4 v = *reinterpret_cast<const float4*>(x + row * H + c);
-    const float f[4] = {v.x, v.y, v.z, v.w};
-    __align__(8) __nv_bfloat16 s[3][4];
+  auto split = [&](float scale) {  // whether one of them is large
+    bool large = false;
+    for (int i = threadIdx.x; i < rows * quads; i += 256) {
+      const int r = i / quads, c = (i - r * quads) * 4;
+      const size_t row = (size_t)tile * kTileRows + r0 + r;
+      const float4 v = *reinterpret_cast<const float4*>(x + row * H + c);
+      const float f[4] = {v.x, v.y, v.z, v.w};
+      __align__(8) __nv_bfloat16 s[3][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) split3(f[j], s[0][j], s[1][j], s[2][j]);
+      for (int j = 0; j < 4; ++j) {
+        split3(f[j] * scale, s[0][j], s[1][j], s[2][j]);
+        large |= fabsf(f[j]) >= kLargeRow;
+      }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2*>(out + q * plane + row * pitch + c) = *reinterpret_cast<const uint2*>(s[q]);
-  }
+      for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2*>(out + q * plane + row * pitch + c) = *reinterpret_cast<const uint2*>(s[q]);
+    }
+    return large;
+  };
+  const int large = __syncthreads_or(split(kUp));
+  if (large) split(kDown);
+  if (threadIdx.x == 0) group_large[blockIdx.x] = large ? 1 : 0;
 }
 
 // Which of a warp's values that are not finite (bits of todo: rows h * 16 + 0...15 of the tile, and from bit 16 on the sixteen
@@ -168,7 +199,7 @@ struct Explain {
   int pitch, K;
   bool paired;                  // GEMM1
 };
-constexpr float kLarge = 1.0e18f;
+constexpr float kLarge = 1.0e18f, kLargePart = 1.0e13f;  // (of a weight; of a row's hi, which may stand for 2^16 times as much)
 __device__ __noinline__ uint32_t unexplained(const Explain& q, uint32_t todo) {
   const int lane = threadIdx.x % 32;
   constexpr uint32_t all = 0xffffffffu;
@@ -186,9 +217,9 @@ __device__ __noinline__ uint32_t unexplained(const Explain& q, uint32_t todo) {
         const uint32_t f[4] = {v.x << 16 & 0x7fff0000u, v.x & 0x7fff0000u, v.y << 16 & 0x7fff0000u, v.y & 0x7fff0000u};  // magnitudes' bits
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          nan = nan || f[j] > 0x7f800000u;
+          nan |= f[j] > 0x7f800000u && f[j] != (uint32_t)kBits << 16;
           if (f[j] == 0x7f800000u) row_inf |= bit;
-          else if (f[j] > __float_as_uint(kLarge)) row_large |= bit;
+          else if (f[j] > __float_as_uint(kLargePart)) row_large |= bit;
         }
       }
       if (__any_sync(all, nan)) {
@@ -235,15 +266,26 @@ __device__ __noinline__ float fp32_chain(const float* __restrict__ a, const floa
   return s;
 }
 // (a: written by other CTAs of this launch, so neither const __restrict__ nor any other way to the non-coherent loads)
-__device__ __noinline__ float fp32_chain_planes(const __nv_bfloat16* a, size_t plane, const float* b, int n) {
+__device__ __noinline__ float fp32_chain_planes(const __nv_bfloat16* a, size_t plane, float unscale, const float* b, int n) {
   float s = 0.0f;
   for (int k = 0; k < n; ++k) {
     const float hi = __bfloat162float(a[k]), mid = __bfloat162float(a[plane + k]), lo = __bfloat162float(a[2 * plane + k]);
-    s = __fmaf_rn(fabsf(hi) <= FLT_MAX ? hi + (mid + lo) : hi, b[k], s);
+    float v = (hi + (mid + lo)) * unscale;
+    if (!(fabsf(hi) <= FLT_MAX)) v = __float_as_uint(hi) >> 16 == kBits ? __uint_as_float(__float_as_uint(mid) | __float_as_uint(lo) >> 16) : hi;
+    s = __fmaf_rn(v, b[k], s);
   }
   return s;
 }
 constexpr float kNearTop = 3.38e38f;  // (bf16's largest finite number is 3.39e38: beyond that a number may round to infinity)
+// The parts of s, an element of the intermediate, in a group of this scale.
+__device__ __forceinline__ void store_top(float s, float scale, __nv_bfloat16* to, size_t plane) {
+  split3(s * scale, to[0], to[plane], to[2 * plane]);
+  if (fabsf(s) <= FLT_MAX && !(fabsf(s * scale) <= kNearTop)) {
+    to[0] = __ushort_as_bfloat16(kBits);
+    to[plane] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(s) >> 16));
+    to[2 * plane] = __ushort_as_bfloat16((unsigned short)__float_as_uint(s));
+  }
+}
 __device__ __forceinline__ bool is_finite(float v) { return fabsf(v) < FLT_MAX; }  // (or the largest, which a clamped number leaves)
 
 __global__ void __launch_bounds__(kSpThreads, 1)
@@ -345,6 +387,11 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
         }
         const int rows = counted ? min(kTileRows, prm.tile_count[it.tile]) : kTileRows;
         item_ring[slot] = item | (max(1, (rows + 15) / 16) << kSpRowShift);
+        {
+          const uint2 g = prm.group_large[it.tile];
+          auto bits = [](uint32_t w) { return (w & 1u) | (w >> 7 & 2u) | (w >> 14 & 4u) | (w >> 21 & 8u); };
+          *(volatile int*)&sh->item_large[slot] = (int)(bits(g.x) | bits(g.y) << 4);
+        }
         mbar_arrive(smem_u32(&sh->item_bar[slot]));
         const int KW = ((it.type == 0 ? H : F) + 31) / 32;
         for (int kw = 0; kw < KW; ++kw) {
@@ -513,8 +560,8 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const uint4 v = lds128(src + (((uint32_t)(half * 4 + u) << 4) ^ sw));
-            split_pair(__uint_as_float(v.x), __uint_as_float(v.y), hi[2 * u], mid[2 * u], lo[2 * u]);
-            split_pair(__uint_as_float(v.z), __uint_as_float(v.w), hi[2 * u + 1], mid[2 * u + 1], lo[2 * u + 1]);
+            split_pair_up(v.x, v.y, hi[2 * u], mid[2 * u], lo[2 * u]);
+            split_pair_up(v.z, v.w, hi[2 * u + 1], mid[2 * u + 1], lo[2 * u + 1]);
           }
           // (the split is done by the time the stage is free: the stages are two rounds of a splitter ahead of the MMAs)
           if (!warp_agrees(mbar_wait(smem_u32(&sh->a_empty[2 * set + half]), (mine & 1u) ^ 1u, abort_flag, wait_ns))) { fail_site = kWaitMbarMma; break; }
@@ -588,8 +635,10 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&sh->rest_empty));
+      const int large = *(volatile int*)&sh->item_large[local_item & (kSpRing - 1)] >> h;  // bits 0 and 4: of this warp's two groups
       const size_t row0 = (size_t)it.tile * kTileRows;
-      auto acc = [&](int i, int j) { return __uint_as_float((uint32_t)(sum[i][j >> 1] >> (32 * (j & 1)))); };
+      const float unscale[2] = {group_result(large & 1), group_result(large >> 4 & 1)};
+      auto acc = [&](int i, int j) { return __uint_as_float((uint32_t)(sum[i][j >> 1] >> (32 * (j & 1)))) * unscale[i]; };
       uint32_t bad = 0;  // results that are not finite
       auto exist = [&]() { return ((1u << min(max(rows - h * 16, 0), 16)) - 1u) | ((1u << min(max(rows - (h + 4) * 16, 0), 16)) - 1u) << 16; };
       if (it.type == 0) {
@@ -609,8 +658,10 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
             for (int n = 0; n < 2; ++n) {
               const float got = __shfl_xor_sync(0xffffffffu, up ? acc(i, j + n) : acc(i, j + n + 8), 16);
               const float g = up ? got : acc(i, j + n), u = up ? acc(i, j + n + 8) : got;
-              v[n] = g / (1.0f + expf(-g)) * u;
-              if (!is_finite(g) || !is_finite(u) || (fabsf(v[n]) > kNearTop && is_finite(v[n]))) bad |= 1u << (16 * i + j + n);
+              const float s = g / (1.0f + expf(-g)) * u;
+              v[n] = s * group_scale(large >> (4 * i) & 1);
+              if (!(fabsf(v[n]) <= kNearTop))  // (g or u not finite: v is not either; finite both, and their product: too large for the parts)
+                if (!is_finite(g) || !is_finite(u) || is_finite(s)) bad |= 1u << (16 * i + j + n);
             }
             uint32_t part[3];
             split_pair(v[0], v[1], part[0], part[1], part[2]);
@@ -633,12 +684,7 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
           const float* a = prm.recv + (row0 + r) * H;
           const size_t w = ((size_t)it.e * F + f) * H;
           const float g = fp32_chain(a, prm.wg + w, H), u = fp32_chain(a, prm.wu + w, H);
-          __nv_bfloat16 s0, s1, s2;
-          split3(g / (1.0f + expf(-g)) * u, s0, s1, s2);
-          __nv_bfloat16* const d = dst + r * pitch;
-          d[0] = s0;
-          d[plane] = s1;
-          d[2 * plane] = s2;
+          store_top(g / (1.0f + expf(-g)) * u, group_scale(large >> (4 * (at >> 4)) & 1), dst + r * pitch, plane);
         }
         __syncwarp();
         // This warp's part of the block is written: make it visible (also to the async proxy, which is how the GEMM2
@@ -668,7 +714,7 @@ ffn_split_kernel(const __grid_constant__ SplitMaps maps, const SplitParams prm) 
         }
         for (; bad != 0; bad &= bad - 1) {
           const int at = __ffs(bad) - 1, r = (4 * (at >> 4) + h) * 16 + (at & 15);
-          dst[(size_t)r * H] = fp32_chain_planes(prm.inter + (row0 + r) * prm.inter_pitch, plane,
+          dst[(size_t)r * H] = fp32_chain_planes(prm.inter + (row0 + r) * prm.inter_pitch, plane, 1.0f / group_scale(large >> (4 * (at >> 4)) & 1),
                                                  prm.wd + ((size_t)(it.e / prm.tp) * H + hc) * F * prm.tp + (size_t)(it.e % prm.tp) * F, F);
         }
         __syncwarp();
@@ -791,6 +837,7 @@ int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, cons
   q.recv = (const float*)recv;
   q.recv_planes = (const __nv_bfloat16*)p->s.recv_planes;
   q.recv_pitch = (int)hp;
+  q.group_large = (const uint2*)p->s.group_large;
   q.wg = (const float*)wg;
   q.wu = (const float*)wu;
   q.wd = (const float*)wd;
@@ -805,7 +852,7 @@ int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, cons
   q.lag = grid;
   mark(p, 3, st);
   if (launch_pdl(split_rows_kernel, dim3((unsigned)(p->P * (kTileRows / kSplitRows))), dim3(256), 0, st, (const float*)recv, tile_expert,
-                 tile_count, rows_done, q.total_rows, c.E, c.H, (int)hp, (size_t)pool * hp, (__nv_bfloat16*)p->s.recv_planes) != cudaSuccess)
+                 tile_count, rows_done, q.total_rows, c.E, c.H, (int)hp, (size_t)pool * hp, (__nv_bfloat16*)p->s.recv_planes, p->s.group_large) != cudaSuccess)
     return MOE_ERR_CUDA;
   static SmemAttrOnce once;
   if (ensure_dynamic_smem(ffn_split_kernel, kSpSmem, p->device, once) != cudaSuccess) return MOE_ERR_CUDA;

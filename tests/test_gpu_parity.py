@@ -398,6 +398,35 @@ def test_fp32_on_tensor_cores_tiles_of_few_rows(rows):
     assert torch.count_nonzero(out[128:256]) == 0
 
 
+# (x, Wg, Wu, Wd times powers of two): parts of numbers near the smallest exponents; rows of large numbers, whose parts are
+# scaled the other way; an intermediate beyond what the parts of a row of ordinary x can hold.
+@pytest.mark.parametrize("exps", [(0, 0, 0, 0), (0, 0, -120, 0), (0, 0, 0, -120), (-60, 0, 0, 0), (-112, 0, 115, 0), (0, -113, 0, 0), (40, -40, -40, 0), (60, 0, 0, -60),
+                                  (60, 0, 0, 0), (0, 57, 57, -100), (33, 0, 0, -40)], ids=str)
+def test_fp32_on_tensor_cores_over_the_range_of_exponents(exps):
+    T, H, F = 48, 132, 932
+    plan = B.Plan(B.make_config(T, H, 1, 1, 1, F, FP32, dispatch_mode=B.DISPATCH_ATOMIC_PAGED))
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x, wg, wu, wd = (torch.empty(s, device="cuda").normal_(0.0, 1.0 if s[0] == T else 0.1, generator=g) * 2.0 ** e
+                     for s, e in zip(((T, H), (1, F, H), (1, F, H), (1, H, F)), exps))
+    recv = torch.zeros((plan.P * 128, H), device="cuda")
+    recv[:T] = x
+    if exps[0] == 33:
+        recv[1:T] *= 2.0 ** -33              # one large row in a group of ordinary ones
+    te = torch.full((plan.P,), -1, dtype=torch.int32, device="cuda")
+    te[0] = 0
+    out = torch.zeros_like(recv)
+    plan.moe_expert_ffn(recv, te, wg, wu, wd, out, torch.tensor([T] + [0] * (plan.P - 1), dtype=torch.int32, device="cuda"),
+                        torch.full((1,), T, dtype=torch.int32, device="cuda"))
+    torch.cuda.synchronize()
+    assert plan.moe_last_status() == (0, 0)
+    gate = recv[:T].double() @ wg[0].double().T
+    want = (gate * torch.sigmoid(gate) * (recv[:T].double() @ wu[0].double().T)) @ wd[0].double().T
+    row = want.abs().amax(1, keepdim=True)
+    assert (row < 3.4e38).all() and torch.isfinite(out[:T]).all()
+    # 1e-6 per row as above; rows so small that fp32's own smallest steps show (2^-150 an element) by these besides
+    assert (((out[:T].double() - want) / row).norm(dim=1) <= 1e-6 * (want / row).norm(dim=1) + 2.0 ** -150 / row[:, 0] * H ** 0.5).all()
+
+
 def test_fp32_on_tensor_cores_infinities_and_nan():
     """What an infinity, a NaN, an overflow or a number that rounds up to bf16's infinity does to a row is what fp32 sums give."""
     T, H, F = 48, 72, 928

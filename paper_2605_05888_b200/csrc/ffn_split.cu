@@ -779,9 +779,10 @@ int split_pitch(int n) { return (n + 7) / 8 * 8; }  // of a plane's rows: 16 byt
 
 // Where the plain FMAs of ffn_fp32_kernel are the slower ones: experts of some rows, and either a fair amount of work (below,
 // both are a chain of launches and this one has one more to start up) or sums so long that the FMAs have too few CTAs for
-// their GEMM2.  Measured, whole layer, us, FMAs / this: rows x H x F of 6 to 22 M 34 / 38 (mean of twelve shapes, none faster by
-// more than 5 %), 30 M (132 x 128, 4 experts) 39.5 / 39.5, 26 M (912 x 624) 70 / 58, 77 M (284 x 536) 62 / 51, 375 M (412 x 508, 32
-// experts) 117 / 69, 1677 M (444 x 1568) 425 / 136, 4194 M (T 1000, 1024 x 2048, 16 experts) 737 / 206.  Long sums: 22 M (92 x 1216) 88
+// their GEMM2.  Measured, whole layer, this / FMAs, work = rows x H x F: up to 16 experts, H from 384, 24 to 40 M 0.79-0.97 (H 912 with
+// 4 experts 1.00-1.04), 40 to 50 M 0.80-0.86; H 128 to 256 24 to 34 M 0.96-1.21, 39 to 51 M 0.88-1.01; 32 experts 51 M (256 x 200)
+// 1.15, 80 M (448 x 400) 1.05, 92 M 0.88.  us, FMAs / this: 375 M (412 x 508, 32
+// experts) 117 / 69, 1677 M (444 x 1568) 425 / 136, 4194 M (T 1000, 1024 x 2048, 16 experts) 737 / 217.  Long sums: 22 M (92 x 1216) 88
 // / 50, 8 M (148 x 1432) 62 / 50.  Few rows per expert, where both stream weights and this splits all of them, the more experts the
 // worse.  This over FMAs at 8 / 12 / 16 / 24 rows per expert, six shapes each (512 x 1024, 1024 x 2048, 448 x 400, 928 x 556, 1024 x
 // 512; last 256 x 2048, whose short sums have the most items for their work): 8 and 16 experts 0.65-0.92 / 0.67-0.91 / 0.60-0.85 / 0.59-0.93;
@@ -797,7 +798,8 @@ bool ffn_split_applies(const moe_config_t& c, int64_t P) {
   if (P > kMaxListTiles || items >= (1ll << kSpRowShift)) return false;  // the work list, the item ring's fields
   if (P > rows / kTileRows + c.E) return false;  // static regions of more tiles than the batch's rows fill: planes of all of them
   const int few = c.E <= 16 ? 8 : c.E > 64 && c.H < 384 ? 32 : 16;  // rows per expert from which on the tensor cores are the faster ones
-  return rows >= (long long)few * c.E && (rows * c.H * c.F >= 24000000ll || c.F >= 900);
+  const long long work = c.E > 16 ? 90000000ll : c.H >= 384 ? 24000000ll : 40000000ll;
+  return rows >= (long long)few * c.E && (rows * c.H * c.F >= work || c.F >= 900);
 }
 
 int launch_ffn_split(moe_plan* p, const void* recv, const int* tile_expert, const void* wg, const void* wu, const void* wd,

@@ -113,6 +113,11 @@ def test_fp32_workspace_holds_the_operands_parts_only_where_tensor_cores_read_th
     assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC, capacity_rows=256) > need(*static, 1, B.DISPATCH_ATOMIC_STATIC, capacity_rows=256)
     assert need(*static, 0, B.DISPATCH_ATOMIC_STATIC, capacity_rows=384) == need(*static, 1, B.DISPATCH_ATOMIC_STATIC, capacity_rows=384)
     assert need(16, 256, 8, 2, 256, 0) == need(16, 256, 8, 2, 256, 1)      # (little work: FMAs)
+    for E, H, F, least in ((8, 380, 400, 40e6), (4, 384, 400, 24e6), (17, 512, 400, 90e6), (8, 4, 900, 1)):     # (little work)
+        rows = max(int(-(-least // (H * F))), 16 * E)
+        assert need(rows, H, E, 1, F, 0) > need(rows, H, E, 1, F, 1), (E, H)
+        if least > 1:
+            assert need(rows - 1, H, E, 1, F, 0) == need(rows - 1, H, E, 1, F, 1), (E, H)
     for E, H, rows_per_expert in ((8, 512, 8), (16, 512, 8), (17, 512, 16), (64, 256, 16), (65, 384, 16), (65, 380, 32), (256, 256, 32)):
         at, below = rows_per_expert * E, rows_per_expert * E - 1           # (few rows per expert: FMAs, the more experts the longer)
         assert need(at, H, E, 1, 1024, 0) > need(at, H, E, 1, 1024, 1), (E, H)

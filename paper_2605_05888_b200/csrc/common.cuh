@@ -24,7 +24,7 @@ enum WaitSite { kWaitTileTable = 1, kWaitMbarTma = 3, kWaitMbarMma = 4,
 struct Scratch {          // device pointers carved out of the caller's workspace
   int* status;            // [4]
   int* pool_next;         // [1]   paged mode: next free tile
-  int* scan_ticket;       // [1]   mode 0: CTAs of the scan kernel that finished
+  int* scan_ticket;       // [1]   mode 0: CTAs of the scan kernel that finished; mode 2, small batches: of the dispatch (zero between calls)
   int* rows_done;         // [1]   assignments whose rows are stored (global completion counter)
   int* tile_count;        // [P]   rows stored per tile (per-tile status counter)
   int* tile_table;        // [E * tiles_per_expert] paged mode: expert-local tile -> pool tile

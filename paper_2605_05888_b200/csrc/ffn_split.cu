@@ -20,10 +20,10 @@
 // split once, by split_rows_kernel in front.
 //
 // What infinities and NaN in the operands make of a sum, the hi*hi products say: hi of an infinity is one, hi of a number is zero
-// only if the number is (below 2^-118 also in a group of large rows), and their signs are the numbers' own; the other five (inf * mid has any sign, inf * 0 none)
-// are clamped to finite numbers before they are added, which changes nothing where hi*hi is infinite or NaN.  Where a value that is not
-// finite has no infinity or NaN behind it, or also large numbers (an overflow, an hi that rounded up to infinity: explained
-// below), the lane that holds it recomputes it as a chain of fp32 FMAs.
+// only if the number is (or, in a group of large rows, below 2^-118), and their signs are the numbers' own.  The other five (inf * mid
+// has any sign, inf * 0 none) are clamped to finite numbers before they are added, which changes nothing where hi*hi is infinite or
+// NaN.  Where a value that is not finite has no infinity or NaN behind it, or also large numbers (an overflow, an hi that rounded up
+// to infinity), the lane that holds it recomputes it as a chain of fp32 FMAs (unexplained, below).
 //
 // Roles (864 threads): warp 0 claims and publishes the items and loads weights, warp 1 MMA issuer and TMEM owner, warps 2-9
 // split weights (two sets of four, two A stages each), warps 10-25 drain accumulators and write results, warp 26 loads the
@@ -191,15 +191,15 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict
 // that lie 64 rows on) are what their operands' infinities and NaN make of them: the row's, and those of this lane's weight row and,
 // in GEMM1, of the one 16 lanes on.  Returns the others.  All 32 lanes.  Large numbers are those whose products may add up to an overflow.
 // Measured, layer, T 1000, H 1024, 16 experts, top-2, F 2048 (215 us as a rule), us, FMAs / every such value recomputed / this: one
-// row with a NaN 737 / 465 / 217, one infinity in one Wg 741 / 24589 / 352, in every Wg 737 / 48854 / 546, every row NaN 698 / 66874 / 289,
-// infinite 698 / - / 549, every Wg NaN 743 / - / 600.
+// row with a NaN 737 / 465 / 217, one infinity in one Wg 741 / 24589 / 362, in every Wg 737 / 48854 / 571, every row NaN 698 / 66874 / 305,
+// infinite 698 / - / 549, every Wg NaN 743 / - / 643.
 struct Explain {
   const __nv_bfloat16* rows;    // hi plane
   const float* w;
   int pitch, K;
   bool paired;                  // GEMM1
 };
-constexpr float kLarge = 1.0e18f, kLargePart = 1.0e13f;  // (of a weight; of a row's hi, which may stand for 2^16 times as much)
+constexpr float kLarge = 1.0e15f, kLargePart = 1.0e13f;  // (of a weight; of a row's hi, which may stand for 2^16 times as much: half a million products)
 __device__ __noinline__ uint32_t unexplained(const Explain& q, uint32_t todo) {
   const int lane = threadIdx.x % 32;
   constexpr uint32_t all = 0xffffffffu;
@@ -781,9 +781,8 @@ int split_pitch(int n) { return (n + 7) / 8 * 8; }  // of a plane's rows: 16 byt
 // both are a chain of launches and this one has one more to start up) or sums so long that the FMAs have too few CTAs for
 // their GEMM2.  Measured, whole layer, this / FMAs, work = rows x H x F: up to 16 experts, H from 384, 24 to 40 M 0.79-0.97 (H 912 with
 // 4 experts 1.00-1.04), 40 to 50 M 0.80-0.86; H 128 to 256 24 to 34 M 0.96-1.21, 39 to 51 M 0.88-1.01; 32 experts 51 M (256 x 200)
-// 1.15, 80 M (448 x 400) 1.05, 92 M 0.88.  us, FMAs / this: 375 M (412 x 508, 32
-// experts) 117 / 69, 1677 M (444 x 1568) 425 / 136, 4194 M (T 1000, 1024 x 2048, 16 experts) 737 / 217.  Long sums: 22 M (92 x 1216) 88
-// / 50, 8 M (148 x 1432) 62 / 50.  Few rows per expert, where both stream weights and this splits all of them, the more experts the
+// 1.15, 80 M (448 x 400) 1.05, 92 M 0.88.  us, FMAs / this: 375 M (412 x 508, 32 experts) 117 / 69, 1677 M (444 x 1568) 425 / 136, 4194 M (T
+// 1000, 1024 x 2048, 16 experts) 737 / 217.  Long sums: 22 M (92 x 1216) 88 / 50, 8 M (148 x 1432) 62 / 50.  Few rows per expert, where both stream weights and this splits all of them, the more experts the
 // worse.  This over FMAs at 8 / 12 / 16 / 24 rows per expert, six shapes each (512 x 1024, 1024 x 2048, 448 x 400, 928 x 556, 1024 x
 // 512; last 256 x 2048, whose short sums have the most items for their work): 8 and 16 experts 0.65-0.92 / 0.67-0.91 / 0.60-0.85 / 0.59-0.93;
 // 32 experts 0.92-1.11 / 0.86-1.12 / 0.68-0.88, 0.74; 64 1.09-1.28 / 0.83-1.15 / 0.75-0.92, 0.85; 128 1.17-1.42 / 0.95-1.18 / 0.79-0.99, 1.12

@@ -968,8 +968,8 @@ def test_paged_dispatch_where_its_small_batches_end(case):
 
 @pytest.mark.parametrize("case", [(1, 64, 1), (37, 64, 32), (511, 256, 8), (4096, 8, 1)], ids=lambda c: f"T{c[0]}_E{c[1]}_K{c[2]}")
 def test_paged_dispatch_counters_seen_from_another_stream_follow_the_rows(case):
-    """Whoever looks while a small dispatch runs: copies of the counters, each followed by a copy of a piece of every row, on a
-    second stream beside the dispatch (they wait for nothing).  Where the counters say so, the rows are there."""
+    """Whoever looks while a small dispatch runs: copies of rows_done, of the tiles' counters and of a piece of every row, in this
+    order, on a second stream beside the dispatch (they wait for nothing).  Where the counters say so, the rows are there."""
     T, E, K = case
     H = 8192
     w = inputs.Workload("watched", T=T, H=H, E=E, R=1, K=K, F=0, dtype=BF16, identity_experts=True)
@@ -985,7 +985,8 @@ def test_paged_dispatch_counters_seen_from_another_stream_follow_the_rows(case):
     side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=side):
         for i in range(looks):
-            seen[i].copy_(counters)
+            seen[i, -1:].copy_(counters[-1:])
+            seen[i, :-1].copy_(counters[:-1])
             rows[i].copy_(recv[:, -8:])
     early = late = 0
     for _ in range(20):
@@ -1005,6 +1006,29 @@ def test_paged_dispatch_counters_seen_from_another_stream_follow_the_rows(case):
         assert ((seen[:, :-1] == counters[:-1]).all(1) | (seen[:, -1] < T * K)).all()
         early, late = early + (~said).any().item(), late + said.any().item()
     assert early and late
+
+
+def test_paged_dispatch_replayed_from_a_graph():
+    """The small dispatch's ticket is back at zero after every call: a captured call gives the same tables and counters each time."""
+    w = inputs.Workload("graph_dispatch", T=300, H=264, E=12, R=1, K=4, F=0, dtype=BF16, identity_experts=True)
+    plan = Hh.make_plan(w, B.DISPATCH_ATOMIC_PAGED)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.empty((w.T, w.H), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    ids = torch.rand((w.T, w.E), device="cuda", generator=g).argsort(1)[:, :w.K].to(torch.int32).contiguous()
+    b = _dispatch_with_counters(w, plan, x, ids)
+    names = ("recv", "cnt", "te", "src", "slot", "tile_count", "rows_done")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.moe_dispatch(x, ids, *(b[n] for n in names))
+    for _ in range(3):
+        for n in names:
+            b[n].fill_(77)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert plan.moe_last_status() == (0, 0) and b["rows_done"].item() == w.T * w.K
+        flat = b["slot"].flatten().long()
+        assert torch.equal(b["tile_count"].long(), torch.bincount(flat // 128, minlength=plan.P))
+        assert torch.equal(b["recv"][flat], x.repeat_interleave(w.K, 0)) and torch.equal(b["te"][flat // 128], ids.flatten())
 
 
 @pytest.mark.parametrize("mode", MODES)

@@ -87,10 +87,10 @@ typedef struct {
                                    ffn_hot_min_tiles left at 0) - and for fp32 the tensor cores on
                                    operands split into three bf16 numbers each (closer to the sums
                                    in 64 bits than fp32 FMAs, over the whole range of exponents), or
-                                   fp32 FMAs for little work, for few
-                                   rows per expert (on average fewer than 8, with more than 16
-                                   experts 16, with more than 64 and H below 384 32) and for static
-                                   regions of more tiles than the batch can fill; 1: fp32 FMAs always (bf16: a plain
+                                   fp32 FMAs for little work, for few rows per expert (on average
+                                   fewer than 8, with more than 16 experts 16, with more than 64 and
+                                   H below 384 32) and for static regions of more tiles than the
+                                   batch can fill; 1: fp32 FMAs always (bf16: a plain
                                    SIMT kernel, the check path); 2: always CTA pairs (bf16).
                                    The tensor-core forms add up every result in the same order,
                                    so a row's bytes do not depend on which of them computes it,
@@ -100,7 +100,8 @@ typedef struct {
                                    of 5 and one of 6, and moe_expert_ffn's rows between calls with
                                    and without row counts.  Naming ffn_split (1 or 2) keeps the
                                    tensor-core forms, and a token's bytes, at every batch size
-                                   (fp32: ffn_kernel 1 keeps the FMAs)                         */
+                                   (dtype fp32: with 0 a row's last bits depend on which of the two
+                                   kernels the batch gets; 1 keeps the FMAs' at every batch size) */
   int32_t ffn_split;            /* 1: one launch per expert GEMM; 2: both GEMMs in one persistent
                                    launch (per-tile status counters gate GEMM2); 0: choose
                                    (one launch when E <= 64; with more, smaller experts two
@@ -173,7 +174,8 @@ int moe_workspace_bytes(const moe_config_t* cfg, size_t* out_bytes);
  * work.  (dtype fp32: as long as the same configuration needs with ffn_kernel 1 is enough; below
  * moe_workspace_bytes() the plan's experts are computed as with ffn_kernel 1.  Likewise for a router
  * that holds several sets of logits, from T*E*H = 3.2e8 on: with room for one set, and 1 KB, it
- * computes every chain, or filters all rows: see route_filter.)  Runs on the current CUDA device.  *out is freed by moe_plan_destroy. */
+ * computes every chain, or filters all rows: see route_filter.)  Runs on the current CUDA device.
+ * *out is freed by moe_plan_destroy. */
 int moe_plan_create(const moe_config_t* cfg, void* d_workspace, size_t bytes, moe_plan_t** out);
 int moe_plan_destroy(moe_plan_t* plan);
 
